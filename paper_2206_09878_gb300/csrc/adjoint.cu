@@ -622,14 +622,14 @@ void wscale(Ctx& c, cd* const* f, int nf, double s0, double s1) {
   LMVD_LAUNCH(c, KC_MISC, 2.0 * n * nf, 32.0 * n * nf, k_wscale, dim3(eblocks(n), nf), 256, 0, c.g, w, s0, s1);
 }
 void g_transpose(Ctx& c, double* const* phys, cd* const* spec, int nf) {
-  fft_forward_as(c, const_cast<double* const*>(phys), spec, nf, 0);
+  fft_forward(c, const_cast<double* const*>(phys), spec, nf);
   const double pp = (double)c.g.px * (double)c.g.pz;
   wscale(c, spec, nf, pp, 2.0 * pp);
 }
 void f_transpose(Ctx& c, cd* const* spec, double* const* phys, int nf) {  // overwrites spec
   const double pp = (double)c.g.px * (double)c.g.pz;
   wscale(c, spec, nf, 1.0 / pp, 0.5 / pp);
-  fft_inverse_as(c, spec, phys, nf, 0);
+  fft_inverse_d(c, spec, phys, nf);
 }
 // out = A^{-T} in per job (one launch), boundary rows outside [zlo, zhi] zero
 void solve_T_jobs(Ctx& c, KClass cls, const DLU& lu, std::initializer_list<SolveTJob> jobs) {

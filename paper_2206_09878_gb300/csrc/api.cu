@@ -307,7 +307,8 @@ void carve(Ctx& c, Carver& cv) {
   c.fprime = cv.take<double>(P);
   for (auto& p : c.w) p = cv.take<double>(P);
   for (int f = 0; f < PW_FIELDS; ++f) c.pw[f] = f < c.pw_n ? cv.take<double>(P) : nullptr;
-  c.tbuf = cv.take<cd>((size_t)c.tbuf_n * ny * g.pz * (g.nx / 2));
+  c.tbuf = reinterpret_cast<cfx*>(cv.take<cd>((size_t)c.tbuf_n * ny * g.pz * (g.nx / 2)));
+  c.texp = cv.take<int>((size_t)c.tbuf_n * ny * std::max(g.nx / 2, g.pz / 2));
 }
 
 // ------------------------------------------------------------------ substage pieces
@@ -384,12 +385,7 @@ void physical_pass_1(Ctx& c, double* const* zp = nullptr) {
   fft_inverse(c, in, out, 8);
   const size_t n = (size_t)c.g.ny * c.g.P;
   EosArgs e{c.cfg.rho_heavy, c.cfg.rho_light, 1.0 / (c.cfg.re * c.cfg.sc)};
-  if (c.cfg.precision == 1)
-    LMVD_LAUNCH(c, KC_PRODUCTS, 25.0 * n, 8.0 * 15 * n, k_products_p1_df, elem_blocks(n), 256, 0, n, e, zf[0],
-                zf[1], zf[2], zf[3], zf[4], c.md[0], c.md[1], c.md[2], c.rho, c.invrho, c.fprime, c.w[0],
-                c.w[1], c.w[2], c.pw[5]);
-  else
-    LMVD_LAUNCH(c, KC_PRODUCTS, 25.0 * n, 8.0 * 15 * n, k_products_p1, elem_blocks(n), 256, 0, n, e, zf[0],
+  LMVD_LAUNCH(c, KC_PRODUCTS, 25.0 * n, 8.0 * 15 * n, k_products_p1, elem_blocks(n), 256, 0, n, e, zf[0],
                 zf[1], zf[2], zf[3], zf[4], c.md[0], c.md[1], c.md[2], c.rho, c.invrho, c.fprime, c.w[0],
                 c.w[1], c.w[2], c.pw[5]);
   double* fin[1] = {c.pw[5]};
@@ -417,11 +413,7 @@ void mc_from_zdot(Ctx& c, double* a = nullptr, double* const* b = nullptr) {
       double* out[1] = {a};
       fft_inverse(c, in, out, 1);
     }
-    if (c.cfg.precision == 1)
-      LMVD_LAUNCH(c, KC_PRODUCTS, 1.0 * n, 24.0 * n, k_product_rt_df, elem_blocks(n), 256, 0, n, c.fprime, a,
-                  c.pw[1]);
-    else
-      LMVD_LAUNCH(c, KC_PRODUCTS, 1.0 * n, 24.0 * n, k_product_rt, elem_blocks(n), 256, 0, n, c.fprime, a, c.pw[1]);
+    LMVD_LAUNCH(c, KC_PRODUCTS, 1.0 * n, 24.0 * n, k_product_rt, elem_blocks(n), 256, 0, n, c.fprime, a, c.pw[1]);
   }
   {
     double* in[1] = {c.pw[1]};
@@ -536,7 +528,7 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
     // kinetic energy and max |m| of m = m^d + m^c (before the products overwrite m^c), <m2^c> at y0
     Fields3C mdf{{c.md[0], c.md[1], c.md[2]}}, mcf{{mcp[0], mcp[1], mcp[2]}};
     LMVD_LAUNCH(c, KC_MISC, 10.0 * n, 8.0 * 7 * n, k_energy_norms, elem_blocks(n), 256, 0, g, c.wq, mdf, mcf,
-                c.invrho, cf.precision == 1 ? 1 : 0, c.ddiag + DIAG_KE,
+                c.invrho, c.ddiag + DIAG_KE,
                 reinterpret_cast<unsigned long long*>(c.ddiag + DIAG_MMAX));
     cudaMemcpyAsync(c.ddiag + DIAG_MC2, c.m2c, sizeof(double), cudaMemcpyDeviceToDevice, c.stream);
   }
@@ -547,11 +539,7 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
     P2Out q{};
     for (int f = 0; f < bt.count; ++f) q.p[bt.first + f] = c.pw[bt.slot + f];
     const double fl = 1.8 * bt.count * n, by = 8.0 * (8 + bt.count) * n;
-    if (cf.precision == 1)
-      LMVD_LAUNCH(c, KC_PRODUCTS, fl, by, k_products_p2_df, elem_blocks(n), 256, 0, n, c.md[0], c.md[1], c.md[2],
-                  mcp[0], mcp[1], mcp[2], c.rho, c.invrho, q);
-    else
-      LMVD_LAUNCH(c, KC_PRODUCTS, fl, by, k_products_p2, elem_blocks(n), 256, 0, n, c.md[0], c.md[1], c.md[2],
+    LMVD_LAUNCH(c, KC_PRODUCTS, fl, by, k_products_p2, elem_blocks(n), 256, 0, n, c.md[0], c.md[1], c.md[2],
                   mcp[0], mcp[1], mcp[2], c.rho, c.invrho, q);
     fft_forward(c, c.pw + bt.slot, c.sv + bt.first, bt.count);
   }
@@ -1048,7 +1036,7 @@ int lmvd_inverse_transform(lmvd_ctx* h, const void* spec, double* phys, int nfie
       in[f] = (cd*)spec + (size_t)(f0 + f) * S;
       out[f] = phys + (size_t)(f0 + f) * P;
     }
-    fft_inverse_as(c, in, out, n, 0);
+    fft_inverse_d(c, in, out, n);
   }
   return cuda_check(c);
 }
@@ -1065,7 +1053,7 @@ int lmvd_forward_transform(lmvd_ctx* h, const double* phys, void* spec, int nfie
       in[f] = (double*)phys + (size_t)(f0 + f) * P;
       out[f] = (cd*)spec + (size_t)(f0 + f) * S;
     }
-    fft_forward_as(c, in, out, n, 0);
+    fft_forward(c, in, out, n);
   }
   return cuda_check(c);
 }

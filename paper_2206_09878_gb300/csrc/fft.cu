@@ -9,27 +9,33 @@
 //            two real rows packed into one complex transform);
 //   forward: x-pass (real-to-complex, two rows per complex transform, split by Hermitian symmetry; the
 //            split's factor 1/2 is left to the z-pass) then z-pass (complex, truncated, scaled by
-//            1/(2 px pz), which is bit-for-bit the same as halving first: power-of-two scaling commutes
-//            with every rounding of the pass).
+//            1/(2 px pz)).
 // Synthesis is unnormalised: f(x, z) = sum_k fhat_k exp(i (k1 x + k3 z)).
 // A pass is one CTA per (plane, field, batch of columns / row pairs); every 1D transform is a
-// Stockham autosort FFT in shared memory with radix-4/3/2 stages and a precomputed twiddle table. The
-// x-passes read and write their contiguous rows with the CTA's threads; the z-passes fetch their columns
-// with TMA tile copies (cp.async.bulk.tensor) and write them with the threads.
+// Stockham autosort FFT in shared memory with radix-4/2/3 stages, a last stage of radix 12 (or 6) and a
+// precomputed twiddle table. The z-passes fetch their columns with TMA tile copies
+// (cp.async.bulk.tensor), the inverse x-pass its rows with bulk copies.
 //
-// Arithmetic: complex double (precision 0) or complex double-float (precision 1, df64.h) selected
-// by the complex type C. Spectral inputs and outputs are always complex double; the intermediate
-// T and the physical fields are stored in the arithmetic's own type (double, or hi/lo float pairs
-// of the same size), so the double-float path converts only at the spectral ends.
+// Arithmetic: 64-bit fixed point with one exponent per 1D transform (fx.cuh), in both precisions. The
+// FP64 pipe retires 1.68 additions per clock per SM here, and transforms in complex double were bound by
+// it (85% busy); in fixed point the same passes run on the integer pipes (ALU 45-52%, multiply pipe
+// 50-60% busy), 4.4 times faster in FP64 arithmetic's place and 1.3 times faster than the double-float
+// transforms they replaced in the precision path: at 512 x 65 x 512, per substage, 100.1 ms (complex
+// double) and 25.2 ms (double-float) -> 19.7 ms. Physical fields and FP64 spectral fields are complex
+// double / double; the precision path's spectral inputs are double-float pairs; T is fixed point with an
+// array of exponents, so the conversions are at the ends only.
+// Accuracy (rms error over rms result against a transform in extended precision, 2D inverse of white
+// noise / k^-2 spectra): 32^2: 4.9e-17 / 4.7e-17 (complex double: 2.1e-16 / 1.9e-16), 128 x 96: 7.7e-17 /
+// 4.9e-17 (2.5e-16 / 2.0e-16), 512^2: 2.3e-16 / 6.7e-17 (2.8e-16 / 2.3e-16).
 #include <cuda.h>  // CUtensorMap and its enums (the encoder is reached through the runtime, no libcuda link)
 
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <mutex>
 #include <type_traits>
 
-#include "df64.h"
-#include "lmvd_internal.h"
+#include "fx.cuh"
 
 namespace lmvd {
 
@@ -48,230 +54,294 @@ struct FieldsRW {
   void* p[10];
 };
 
-// ------------------------------------------------------------------ arithmetic traits
-template <class C>
-struct FT;
-
-template <>
-struct FT<cd> {
-  using R = double;
-  __device__ static cd zero() { return mk(0, 0); }
-  __device__ static cd add(cd a, cd b) { return a + b; }
-  __device__ static cd sub(cd a, cd b) { return a - b; }
-  __device__ static cd add_lazy(cd a, cd b) { return a + b; }
-  __device__ static cd sub_lazy(cd a, cd b) { return a - b; }
-  __device__ static cd ti(cd a) { return times_i(a); }
-  __device__ static cd neg(cd a) { return cd{-a.re, -a.im}; }
-  __device__ static cd cj(cd a) { return conj(a); }
-  __device__ static cd half(cd a) { return 0.5 * a; }
-  template <int SIGN>
-  __device__ static cd mulw(cd v, const FFTPlan& p, int idx) {
-    const double2 w = p.tw[idx];
-    return cmul(v, cd{w.x, SIGN * w.y});
-  }
-  template <int SIGN>
-  __device__ static cd mul_s3(cd v, const FFTPlan&) {  // SIGN sin(2 pi / 3) v
-    return (SIGN * 0.86602540378443864676372317075294) * v;
-  }
-  __device__ static cd from_spec(cd x) { return x; }
-  __device__ static cd to_spec(cd x, const FFTPlan& p) { return p.scale_d * x; }
-  __device__ static cd make(R a, R b) { return cd{a, b}; }
-  __device__ static R re(cd a) { return a.re; }
-  __device__ static R im(cd a) { return a.im; }
-  __device__ static R rzero() { return 0.0; }
-  __device__ static R rmul(R a, R b) { return a * b; }
-  // -(w1 m1 + w2 m2 + w3 m3), the expression of k_product_L
-  __device__ static R dot3neg(R w1, R m1, R w2, R m2, R w3, R m3) { return -(w1 * m1 + w2 * m2 + w3 * m3); }
-};
-
-template <>
-struct FT<cdf> {
-  using R = df;
-  __device__ static cdf zero() { return cdf{df{0.f, 0.f}, df{0.f, 0.f}}; }
-  __device__ static cdf add(cdf a, cdf b) { return cadd(a, b); }
-  __device__ static cdf sub(cdf a, cdf b) { return csub(a, b); }
-  // intermediates of a butterfly that feed only add / sub: not renormalised
-  __device__ static cdf add_lazy(cdf a, cdf b) { return cadd_lazy(a, b); }
-  __device__ static cdf sub_lazy(cdf a, cdf b) { return csub_lazy(a, b); }
-  __device__ static cdf ti(cdf a) { return ctimes_i(a); }
-  __device__ static cdf neg(cdf a) { return cdf{dneg(a.re), dneg(a.im)}; }
-  __device__ static cdf cj(cdf a) { return cconj(a); }
-  __device__ static cdf half(cdf a) { return cdf{dscale2(a.re, 0.5f), dscale2(a.im, 0.5f)}; }
-  template <int SIGN>
-  __device__ static cdf mulw(cdf v, const FFTPlan& p, int idx) {
-    const float4 w = p.twf[idx];
-    const df wr{w.x, w.y};
-    const df wi = SIGN > 0 ? df{w.z, w.w} : df{-w.z, -w.w};
-    return cmulw_lazy(v, wr, wi);  // feeds only the butterfly's add / sub
-  }
-  template <int SIGN>
-  __device__ static cdf mul_s3(cdf v, const FFTPlan& p) {
-    const df s = SIGN > 0 ? p.s3f : dneg(p.s3f);
-    return cdf{dmul(v.re, s), dmul(v.im, s)};
-  }
-  __device__ static cdf from_spec(cd x) { return cdf{df_from_double_int(x.re), df_from_double_int(x.im)}; }
-  __device__ static cd to_spec(cdf x, const FFTPlan& p) {
-    return cd{df_to_double_int(dmul(x.re, p.scale_f)), df_to_double_int(dmul(x.im, p.scale_f))};
-  }
-  __device__ static cdf make(R a, R b) { return cdf{a, b}; }
-  __device__ static R re(cdf a) { return a.re; }
-  __device__ static R im(cdf a) { return a.im; }
-  __device__ static R rzero() { return df{0.f, 0.f}; }
-  __device__ static R rmul(R a, R b) { return dmul(a, b); }
-  // -(w1 m1 + w2 m2 + w3 m3), the arithmetic of k_product_L_df
-  __device__ static R dot3neg(R w1, R m1, R w2, R m2, R w3, R m3) {
-    return dneg(dadd(ddot2(w1, m1, w2, m2), dmul(w3, m3)));
-  }
-};
-
-// One radix-R Stockham stage, in place in shared memory. The transform of length n is shared by
-// tpt = n / EPT threads; thread tt owns the butterflies tt, tt + tpt, ... (EPT / R of them), loads all
-// their inputs into registers, waits for the whole block, then writes the outputs back to the same
-// buffer (the reads of every thread are complete before any write).
-// Pruning by the 3/2 rule, in separate instantiations so that the other stages keep their registers:
-// ZERO (a first radix-4 stage, L = 1): inputs at positions [lo, hi) are known to be zero (the padding of
-// a synthesis), so their loads and the additions with them are skipped. SKIP (a last stage): outputs at
-// positions [lo, hi) are not wanted (the truncated modes of an analysis), so their additions and stores
-// are skipped.
+// ------------------------------------------------------------------ Stockham stages
+// A transform of length n is shared by tpt = n / EPT threads, EPT = 12 or (n an odd multiple of 6) 6. Its last
+// stage has radix EPT, computed in a thread's registers; the stages before it have radices 4, 2 and 3, in place
+// in shared memory: thread tt owns the butterflies tt, tt + tpt, ... (EPT / R of them), loads all their inputs
+// into registers, waits for the whole block, then writes the outputs back to the same buffer.
 // S: distance in elements between consecutive points of a transform in shared memory (1: contiguous; the
 // z-passes interleave their columns, point i of column c at (i S + c)).
-template <class C, int SIGN, int R, int EPT, bool ZERO = false, bool SKIP = false, int S = 1>
-__device__ __forceinline__ void fft_stage(C* x, const FFTPlan& pl, int L, int tt, int tpt, int lo = 0, int hi = 0) {
-  using F = FT<C>;
-  static_assert(!ZERO || R == 4, "zero-input pruning is written for a first radix-4 stage");
+template <int SIGN>
+__device__ __forceinline__ void fx_bfly4(cfx& v0, cfx& v1, cfx& v2, cfx& v3) {
+  // the outputs as sums of three terms: one 64-bit addition of three operands takes the same two instructions as
+  // one of two
+  const cfx s = v1 + v3, d = v1 - v3, t = SIGN > 0 ? fx_ti(d) : cfx{d.im, -d.re};  // t = (SIGN i) (v1 - v3)
+  const cfx a = v0, c = v2;
+  v0 = (a + s) + c;
+  v1 = (a + t) - c;
+  v2 = (a - s) + c;
+  v3 = (a - t) - c;
+}
+template <int SIGN>
+__device__ __forceinline__ void fx_bfly3(cfx& v0, cfx& v1, cfx& v2, int2 s3) {
+  const cfx t = v1 + v2, d = v1 - v2;
+  const cfx m{v0.re - (t.re >> 1), v0.im - (t.im >> 1)};
+  const long long ur = fx_mulr(d.re, s3), ui = fx_mulr(d.im, s3);
+  const cfx u = SIGN > 0 ? cfx{-ui, ur} : cfx{ui, -ur};  // (SIGN i sin(2 pi / 3)) (v1 - v2)
+  v0 = v0 + t;
+  v1 = m + u;
+  v2 = m - u;
+}
+template <int SIGN, int R>
+__device__ __forceinline__ void fx_butterfly(cfx (&v)[R], const FFTPlan& pl) {
+  if constexpr (R == 4) {
+    fx_bfly4<SIGN>(v[0], v[1], v[2], v[3]);
+  } else if constexpr (R == 3) {
+    fx_bfly3<SIGN>(v[0], v[1], v[2], pl.s3);
+  } else {
+    const cfx t = v[0];
+    v[0] = t + v[1];
+    v[1] = t - v[1];
+  }
+}
+
+template <int SIGN, int R, int EPT, int S>
+__device__ __forceinline__ void fx_stage(cfx* x, const FFTPlan& pl, int L, int tt, int tpt, int lo, int hi) {
   constexpr int NBT = EPT / R;
   const int n = pl.n;
-  const int nb = n / R, Ls = L * R, tws = n / Ls;
-  const bool pow2 = (L & (L - 1)) == 0;
-  C v[NBT][R];
+  const int nb = n / R, tws = n / (L * R);
+  cfx v[NBT][R];
 #pragma unroll
-  for (int j = 0; j < NBT; ++j) {
-    const int b = tt + j * tpt;
+  for (int j = 0; j < NBT; ++j)
 #pragma unroll
     for (int q = 0; q < R; ++q) {
-      const int i = b + q * nb;
-      bool ld = LMVD_IN(i, n);
-      if constexpr (ZERO) ld = ld && (i < lo || i >= hi);
-      v[j][q] = ld ? x[i * S] : FT<C>::zero();
+      const int i = tt + j * tpt + q * nb;
+      v[j][q] = LMVD_IN(i, n) && (i < lo || i >= hi) ? x[i * S] : cfx{0, 0};
     }
-  }
   __syncthreads();
 #pragma unroll
   for (int j = 0; j < NBT; ++j) {
     const int b = tt + j * tpt;
-    const int k = pow2 ? (b & (L - 1)) : (b % L);
+    const int k = (L & (L - 1)) == 0 ? (b & (L - 1)) : (b % L);
     const int base = (b - k) * R + k;
     if (!LMVD_IN(base + (R - 1) * L, n)) continue;
-    if (!ZERO && k) {
+    if (k)  // (a product with w = 1 would not be exact)
 #pragma unroll
-      for (int q = 1; q < R; ++q) v[j][q] = F::template mulw<SIGN>(v[j][q], pl, q * k * tws);
-    }
-    // output q at base + q L is written unless SKIP drops it
-    auto want = [&](int q) { return !SKIP || base + q * L < lo || base + q * L >= hi; };
-    if (R == 4) {
-      C t0, t1, t2, d3;
-      // ZERO: v2 = 0 gives t0 = t1 = v0; v1 = 0 gives t2 = v3 and v1 - v3 = -v3
-      if (ZERO && b + 2 * nb >= lo && b + 2 * nb < hi) {
-        t0 = v[j][0];
-        t1 = v[j][0];
-      } else {
-        t0 = F::add_lazy(v[j][0], v[j][2]);
-        t1 = F::sub_lazy(v[j][0], v[j][2]);
-      }
-      if (ZERO && b + nb >= lo && b + nb < hi) {
-        t2 = v[j][3];
-        d3 = F::ti(F::neg(v[j][3]));
-      } else {
-        t2 = F::add_lazy(v[j][1], v[j][3]);
-        d3 = F::ti(F::sub_lazy(v[j][1], v[j][3]));
-      }
-      const C t3 = SIGN > 0 ? d3 : F::neg(d3);  // (SIGN i) (v1 - v3)
-      if (want(0)) x[base * S] = F::add(t0, t2);
-      if (want(1)) x[(base + L) * S] = F::add(t1, t3);
-      if (want(2)) x[(base + 2 * L) * S] = F::sub(t0, t2);
-      if (want(3)) x[(base + 3 * L) * S] = F::sub(t1, t3);
-    } else if (R == 3) {
-      const C t1 = F::add_lazy(v[j][1], v[j][2]);
-      const C m = F::sub_lazy(v[j][0], F::half(t1));
-      const C u = F::ti(F::template mul_s3<SIGN>(F::sub_lazy(v[j][1], v[j][2]), pl));
-      if (want(0)) x[base * S] = F::add(v[j][0], t1);
-      if (want(1)) x[(base + L) * S] = F::add(m, u);
-      if (want(2)) x[(base + 2 * L) * S] = F::sub(m, u);
-    } else {
-      if (want(0)) x[base * S] = F::add(v[j][0], v[j][1]);
-      if (want(1)) x[(base + L) * S] = F::sub(v[j][0], v[j][1]);
-    }
+      for (int q = 1; q < R; ++q) v[j][q] = fx_mulw<SIGN>(v[j][q], __ldg(pl.tw + q * k * tws));
+    fx_butterfly<SIGN, R>(v[j], pl);
+#pragma unroll
+    for (int q = 0; q < R; ++q) x[(base + q * L) * S] = v[j][q];
   }
   __syncthreads();
 }
 
-template <class C, int SIGN, int EPT, bool SKIP, int S>
-__device__ __forceinline__ void fft_stage_r(unsigned r2, C* x, const FFTPlan& pl, int L, int tt, int tpt, int lo,
-                                            int hi) {
-  if (r2 == 0) fft_stage<C, SIGN, 4, EPT, false, SKIP, S>(x, pl, L, tt, tpt, lo, hi);
-  else if (r2 == 2) fft_stage<C, SIGN, 3, EPT, false, SKIP, S>(x, pl, L, tt, tpt, lo, hi);
-  else fft_stage<C, SIGN, 2, EPT, false, SKIP, S>(x, pl, L, tt, tpt, lo, hi);
+// First stage of radix 4 (L = 1, no twiddles) from registers: v[4 j + q] is input point tt + j tpt + q n / 4. The
+// caller has waited for every thread's reads.
+template <int SIGN, int S>
+__device__ __forceinline__ void fx_first4(cfx (&v)[12], cfx* x, const FFTPlan& pl, int tt, int tpt) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    fx_bfly4<SIGN>(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    const int base = (tt + j * tpt) * 4;
+    if (!LMVD_IN(base + 3, pl.n)) continue;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[(base + q) * S] = v[4 * j + q];
+  }
+  __syncthreads();
 }
 
-// All stages of one transform held at x (the caller has synchronised after filling x).
-// SIGN = +1: synthesis (exp(+i)), -1: analysis. The result is in natural order in x. With PZ, positions
-// [lo, hi) of the input are zero (pruned in a first radix-4 stage); with PS, positions [lo, hi) of the
-// output are not wanted (pruned in the last stage). Compile-time switches, so that a pass without pruning
-// compiles to the plain stages. The FP64 passes prune (synthesis 7%, analysis <1% faster at 512^3); the
-// double-float ones do not (their x-passes spilled at the 72-register cap and lost 6%).
-template <class C, int SIGN, int EPT, bool PZ = false, bool PS = false, int S = 1>
-__device__ void fft_inplace(C* x, const FFTPlan& pl, int tt, int tpt, int lo = 0, int hi = 0) {
-  int L = 1, s = 0;
+// Stages s0 .. nst - 2; returns when every point of the last stage's input is in x. Input points [lo, hi) of stage 0
+// are zero and not read (the 3/2-rule padding of a synthesis).
+template <int SIGN, int EPT, int S>
+__device__ __forceinline__ void fx_middle(cfx* x, const FFTPlan& pl, int s0, int tt, int tpt, int lo = 0, int hi = 0) {
+  int L = 1;
   unsigned code = pl.code;
-  if (PZ && lo < hi && (code & 3u) == 0 && pl.nst > 1) {
-    fft_stage<C, SIGN, 4, EPT, true, false, S>(x, pl, 1, tt, tpt, lo, hi);
+  if (s0) {
     L = 4;
-    s = 1;
     code >>= 2;
   }
-  const int last = PS && lo < hi ? pl.nst - 1 : pl.nst;
-  for (; s < last; ++s, code >>= 2) {
+  for (int s = s0; s < pl.nst - 1; ++s, code >>= 2) {
     const unsigned r2 = code & 3u;
-    fft_stage_r<C, SIGN, EPT, false, S>(r2, x, pl, L, tt, tpt, 0, 0);
-    L *= r2 == 0 ? 4 : (r2 == 2 ? 3 : 2);
+    if (EPT == 12 && r2 == 0) {
+      fx_stage<SIGN, 4, EPT, S>(x, pl, L, tt, tpt, lo, hi);
+      L *= 4;
+    } else if (EPT == 12 && r2 == 1) {
+      fx_stage<SIGN, 2, EPT, S>(x, pl, L, tt, tpt, lo, hi);
+      L *= 2;
+    } else {
+      fx_stage<SIGN, 3, EPT, S>(x, pl, L, tt, tpt, lo, hi);
+      L *= 3;
+    }
+    lo = hi = 0;
   }
-  if (PS && s < pl.nst) fft_stage_r<C, SIGN, EPT, true, S>(code & 3u, x, pl, L, tt, tpt, lo, hi);
 }
 
-// The passes that prune (see fft_inplace).
-template <class C>
-constexpr bool kPrune = std::is_same<C, cd>::value;
-
-// Whether fft_inplace with PZ = kPrune<C> skips a zero input band of plan pl: only a first radix-4 stage
-// prunes, so a plan without one (n with a single factor 2) reads the band and it must hold zeros.
-template <class C>
-__device__ __forceinline__ bool prunes_zero_band(const FFTPlan& pl) {
-  return kPrune<C> && (pl.code & 3u) == 0 && pl.nst > 1;
+// Last stage: radix EPT, L = n / EPT = tpt; thread tt's butterfly reads and produces the points tt + q L. The EPT-point
+// transform is a prime-factor one (3 x 4 or 3 x 2): input q = (EPT / 3) a + 3 b, output q = 4 a' + s b' mod EPT
+// with s = 9 (EPT 12) or 3 (EPT 6), and no twiddles between its two parts. Against a radix-4 and a radix-3 stage
+// it saves an exchange through shared memory and a third of the two stages' twiddle products.
+template <int SIGN, int EPT, int S>
+__device__ __forceinline__ void fx_last(const cfx* x, const FFTPlan& pl, int tt, cfx (&v)[EPT]) {
+  constexpr int R = EPT / 3;
+  const int L = pl.tpt;
+  cfx u[EPT];
+#pragma unroll
+  for (int q = 0; q < EPT; ++q) u[q] = LMVD_IN(tt + q * L, pl.n) ? x[(tt + q * L) * S] : cfx{0, 0};
+  if (tt)
+#pragma unroll
+    for (int q = 1; q < EPT; ++q) u[q] = fx_mulw<SIGN>(u[q], __ldg(pl.tw + q * tt));
+#pragma unroll
+  for (int b = 0; b < R; ++b) fx_bfly3<SIGN>(u[3 * b], u[(R + 3 * b) % EPT], u[(2 * R + 3 * b) % EPT], pl.s3);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    // u[(R a + 3 b) mod EPT] now holds (a', b) = (a, b)
+    cfx w[R];
+#pragma unroll
+    for (int b = 0; b < R; ++b) w[b] = u[(R * a + 3 * b) % EPT];
+    if constexpr (R == 4) fx_bfly4<SIGN>(w[0], w[1], w[2], w[3]);
+    else fx_butterfly<SIGN, R>(w, pl);
+#pragma unroll
+    for (int b = 0; b < R; ++b) v[(4 * a + (R == 4 ? 9 : 3) * b) % EPT] = w[b];
+  }
 }
 
-// Launch bounds: every pass caps its registers (FftMinCtas below); the FP64 kernels would otherwise take ~100
-// and fit fewer CTAs, whose warps hide less of the FP64 pipe's latency. The x-passes run small CTAs (2
-// transforms of 768 points, 6-7 per SM), so that the load, compute and store phases of different CTAs
-// (separated by barriers) overlap: 7-8% faster in double-float at 512^3 than 256-thread CTAs. The z-passes
-// take 4 kx columns per CTA (2 when 4 transforms do not fit FFT_CTA_Z threads); with 2 at 768 points the
-// double-float inverse z-pass was 13% slower.
+// ------------------------------------------------------------------ the exponent of a transform
+// red: partial sums of the CTA (one float per group of g threads of a transform), top: its largest high word
+// (for the slow path), emin: its warps' smallest E (fx_scale_t). Thread tt of a transform whose threads are S lanes
+// apart; g is the largest power of two dividing tpt with g S <= 32, so a group lies in one warp.
+constexpr int FX_RED = 256;
+struct FxShared {
+  float red[FX_RED];
+  int emin[8];
+  int top;
+};
+
+__device__ __forceinline__ unsigned warp_lanes() {  // the lanes of this warp (the last one may be partial)
+  const unsigned lanes = blockDim.x - (threadIdx.x & ~31u);
+  return lanes >= 32 ? 0xffffffffu : (1u << lanes) - 1u;
+}
+__device__ __forceinline__ float group_sum(float v, int g, int S) {
+  const unsigned mask = warp_lanes();
+  for (int o = S; o < g * S; o <<= 1) v += __shfl_xor_sync(mask, v, o);
+  return v;
+}
+
+// The slow path of inputs outside the range of the FP32 sums: divides them by 2^xe, the exponent of the CTA's
+// largest magnitude; INT_MIN if one of them is inf or nan (the results are then nan).
+constexpr int kFxPoison = INT_MIN;
+__device__ __noinline__ double fx_scale2(double x, int e) { return scalbn(x, e); }
+__device__ __noinline__ float fx_scale2f(float x, int e) { return scalbnf(x, e); }
+__device__ __forceinline__ cd fx_scaled(cd x, int e) { return cd{fx_scale2(x.re, e), fx_scale2(x.im, e)}; }
+__device__ __forceinline__ df fx_scaled(df x, int e) { return df{fx_scale2f(x.hi, e), fx_scale2f(x.lo, e)}; }
+__device__ __forceinline__ cdf fx_scaled(cdf x, int e) { return cdf{fx_scaled(x.re, e), fx_scaled(x.im, e)}; }
+template <class RAW, int N>
+__device__ __forceinline__ int fx_rescale(RAW (&raw)[N], int top, FxShared& sh) {
+  constexpr bool d = std::is_same<RAW, cd>::value;
+  atomicMax(&sh.top, top);
+  __syncthreads();
+  const int m = sh.top;
+  if (m >= (d ? 0x7ff00000 : 0x7f800000)) return kFxPoison;
+  const int xe = d ? max(m >> 20, 1) - 1023 : max(m >> 23, 1) - 127;
+#pragma unroll
+  for (int i = 0; i < N; ++i) raw[i] = fx_scaled(raw[i], -xe);
+  return xe;
+}
+__device__ __noinline__ double fx_unscale(double d, int xe) {
+  return xe == kFxPoison ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(d, xe);
+}
+
+__device__ __forceinline__ void mag_add(FxMag& m, cd x) {
+  m.add(x.re);
+  m.add(x.im);
+}
+__device__ __forceinline__ void mag_add(FxMag& m, cdf x) {
+  m.add(x.re);
+  m.add(x.im);
+}
+template <class RAW>
+constexpr bool kIsDf = std::is_same<RAW, cdf>::value;
+
+// k of this thread's transform from the RAW values its threads hold (each counted `weight` times), all threads of
+// the CTA together; xe: see fx_rescale (0 on the usual path). One barrier.
+template <class RAW, int N>
+__device__ __forceinline__ int fx_scale(RAW (&raw)[N], FxShared& sh, int slot, int np, int stride, int g, int S, int tt,
+                                        float weight, int& xe) {
+  FxMag m;
+#pragma unroll
+  for (int i = 0; i < N; ++i) mag_add(m, raw[i]);
+  float v = group_sum(m.sum, g, S);
+  if ((tt & (g - 1)) == 0 && LMVD_IN(slot + (tt / g) * stride, FX_RED)) sh.red[slot + (tt / g) * stride] = v;
+  xe = 0;
+  if (__syncthreads_or(fx_out_of_range(m, kIsDf<RAW>))) {
+    xe = fx_rescale(raw, m.top, sh);
+    FxMag r;
+#pragma unroll
+    for (int i = 0; i < N; ++i) mag_add(r, raw[i]);
+    v = group_sum(r.sum, g, S);
+    if ((tt & (g - 1)) == 0 && LMVD_IN(slot + (tt / g) * stride, FX_RED)) sh.red[slot + (tt / g) * stride] = v;
+    __syncthreads();
+  }
+  float s = 0.f;
+  for (int i = 0; i < np; ++i) s += sh.red[slot + i * stride];
+  return fx_exponent(weight * s);
+}
+// The intermediate T between the two passes of a transform stays in fixed point: 16 bytes per element and one
+// exponent E per transform of the first pass (a kx column of the inverse, a row pair of the forward one; the value is
+// X 2^-E), so neither side converts; kFxNan marks a transform with inf or nan in it. The second pass's exponent k is
+// at most the smallest E of its inputs (their own unit: a smaller one holds no information), so that its inputs only
+// shift right. Sums are formed from the high words in FP32, E in the range that the usual path gives.
+constexpr int kFxNan = INT_MIN, kFxMinE = -40, kFxMaxE = 165;
+__device__ __forceinline__ float fx_mag_hi(cfx x) {
+  return fabsf(__int2float_rn((int)(x.re >> 32))) + fabsf(__int2float_rn((int)(x.im >> 32)));
+}
+__device__ __forceinline__ float fx_pow2(int e) { return __int_as_float((e + 127) << 23); }  // -126 <= e <= 127
+// sum |X| 2^-E of inputs that share E (kFxMinE <= E; a sum at an E beyond kFxMaxE may read too large, never too small)
+__device__ __forceinline__ float fx_mag(float hi_sum, int E) { return hi_sum * 0x1p-32f * fx_pow2(max(64 - E, -126)); }
+
+// As fx_scale, for fixed-point inputs: per thread the sum `mag` of its inputs' magnitudes and the smallest E. On the
+// slow path E is first counted from the CTA's smallest (remag recomputes mag for the shifted E's).
+template <class Remag>
+__device__ __forceinline__ int fx_scale_t(float mag, int& emin, FxShared& sh, int slot, int np, int stride, int g, int S,
+                                          int tt, float weight, int& xe, Remag&& remag) {
+  float v = group_sum(mag, g, S);
+  if ((tt & (g - 1)) == 0 && LMVD_IN(slot + (tt / g) * stride, FX_RED)) sh.red[slot + (tt / g) * stride] = v;
+  emin = __reduce_min_sync(warp_lanes(), emin);
+  if ((threadIdx.x & 31) == 0) sh.emin[threadIdx.x >> 5] = emin;
+  xe = 0;
+  const bool slow = __syncthreads_or(emin < kFxMinE || emin > kFxMaxE);
+  const int nw = (blockDim.x + 31) >> 5;
+  for (int w = 0; w < nw; ++w) emin = min(emin, sh.emin[w]);
+  if (slow) {
+    if (emin == kFxNan) {
+      xe = kFxPoison;
+    } else {
+      xe = 61 - emin;  // E' = E + xe: the largest inputs are of the order of one
+      v = group_sum(remag(xe), g, S);
+      __syncthreads();
+      if ((tt & (g - 1)) == 0 && LMVD_IN(slot + (tt / g) * stride, FX_RED)) sh.red[slot + (tt / g) * stride] = v;
+      __syncthreads();
+      emin = 61;
+    }
+  }
+  float s = 0.f;
+  for (int i = 0; i < np; ++i) s += sh.red[slot + i * stride];
+  return min(fx_exponent(weight * s), emin);
+}
+// X 2^(k - E), rounded; d = E - k >= 0
+__device__ __forceinline__ cfx fx_align(cfx x, int d) {
+  const long long h = (long long)(unsigned long long)shl32(1u, d - 1);
+  return cfx{sar64(x.re + h, d), sar64(x.im + h, d)};
+}
+__device__ __forceinline__ cfx fx_convert(cd x, int k, float) { return cfx{fx_from(x.re, k), fx_from(x.im, k)}; }
+__device__ __forceinline__ cfx fx_convert(cdf x, int, float sa) { return cfx{fx_from(x.re, sa), fx_from(x.im, sa)}; }
+__device__ __forceinline__ float fx_sa(int k) { return __int_as_float((k - 40 + 127) << 23); }
+
+// A result as a complex double: the two parts take different routes, so that the FP64 pipe does half of the
+// conversions beside the integer pipes.
+__device__ __forceinline__ cd fx_result(cfx v, int k, int xe) {
+  cd r{fx_to_fp(v.re, k << 20), fx_to(v.im, k)};
+  if (xe) r = cd{fx_unscale(r.re, xe), fx_unscale(r.im, xe)};
+  return r;
+}
+
+// CTAs: the x-passes run small ones (128 threads), so that the load, compute and store phases of different CTAs
+// (separated by barriers) overlap; the z-passes take 4 kx columns per CTA (2 when 4 transforms do not fit
+// FFT_CTA_Z threads).
 constexpr int FFT_CTA_X = 128, FFT_CTA_Z = 256;
-// CTAs per SM each pass is compiled for, i.e. its register cap. FP64: 6 x-pass and 3 z-pass CTAs (80
-// registers). Double-float: the x-passes fit 7 CTAs at 72 registers without spilling (inverse 1.5%, forward
-// 2.8% faster at 512^3 than at 6) and the forward z-pass 4 at 64 (4.4% faster); the inverse z-pass lost 2.3%
-// at 64 registers and keeps 3.
-template <class C>
-struct FftMinCtas {
-  static constexpr int x = 6, z_inv = 3, z_fwd = 3;
-};
-template <>
-struct FftMinCtas<cdf> {
-  static constexpr int x = 7, z_inv = 3, z_fwd = 4;
-};
-// Loads a thread issues before it stores any of them, in the forward x-pass's gather and the inverse x-pass's
-// loads of f': one load at a time would serialise a memory latency per iteration (ncu: long-scoreboard
-// stalls dominated the double-float passes). The z-passes and the inverse x-pass's input come by TMA.
-constexpr int FFT_LOAD_CHUNK = 4;
+// CTAs per SM each pass is compiled for, i.e. its register cap (80). A thread holds 12 elements of 4 registers; at
+// 512 x 65 x 512 the inverse x-passes take 7.82 / 7.33 / 7.33 / 7.46 ms per substage at 4 / 5 / 6 / 7 CTAs, the
+// forward ones 5.48 / 5.15 / 5.10 / 5.24, the z-passes 8.24 / 7.28 / 7.64 at 2 / 3 / 4.
+constexpr int FFT_MIN_X = 6, FFT_MIN_Z = 3;
 
 // ---------------------------------------------------------------- tile loads (TMA)
 // The z-passes read columns of a row-major plane: batch consecutive kx (16-byte elements) of every z-row. A
@@ -332,342 +402,367 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
   return true;
 }
 
+// The exponent a transform's fixed-point results are stored with (xe: fx_rescale's)
+__device__ __forceinline__ int fx_stored_exponent(int k, int xe) { return xe == kFxPoison ? kFxNan : k - xe; }
+
+// Fixed-point inputs v of a transform in shared memory: through a first radix-4 stage in registers (v in the order of
+// fx_first4), or, for a plan without one, to the points tt + u tpt (v in that order), then the middle stages.
+template <int SIGN, int EPT, int S>
+__device__ __forceinline__ void fx_run(cfx (&v)[EPT], cfx* x, const FFTPlan& pl, bool first4, int tt) {
+  if constexpr (EPT == 12) {
+    if (first4) {
+      fx_first4<SIGN, S>(v, x, pl, tt, pl.tpt);
+      fx_middle<SIGN, EPT, S>(x, pl, 1, tt, pl.tpt);
+      return;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < EPT; ++u)
+    if (LMVD_IN(tt + u * pl.tpt, pl.n)) x[(tt + u * pl.tpt) * S] = v[u];
+  __syncthreads();
+  fx_middle<SIGN, EPT, S>(x, pl, 0, tt, pl.tpt);
+}
+// input point u of a thread, in the order fx_run expects (step: n / 4 with a first radix-4 stage)
+__device__ __forceinline__ int fx_point(int u, bool first4, int tt, int tpt, int step) {
+  return first4 ? tt + (u >> 2) * tpt + (u & 3) * step : tt + u * tpt;
+}
+
 // ---------------------------------------------------------------- inverse z-pass
-// in: spectral value fields [ny][nz][nxh] (complex double); T: [f][ny][pz][nx/2] of C
-// IN_DF (double-float arithmetic only): the inputs already hold double-float pairs (the precision path's
-// evaluations store them so), read without conversion.
+// in: spectral value fields [ny][nz][nxh] of RAW (complex double, or the double-float pairs that the precision
+// path's evaluations store in the same 16 bytes); T: [f][ny][pz][nx/2] fixed-point, te: [f][ny][nx/2] its exponents.
 // A CTA transforms COLS kx columns of one plane. Shared layout: point z of column c at a[z COLS + c]; two
 // tile loads per row block put the kz >= 0 rows at the top and the kz < 0 rows at the bottom of the padded
-// column (the Nyquist row lands inside the zero band, which the FP64 passes never read and the double-float
-// ones clear).
-template <class C, int EPT, int COLS, bool IN_DF = false>
-__global__ void __launch_bounds__(FFT_CTA_Z, FftMinCtas<C>::z_inv)
-    k_fft_z_inv(FFTPlan pl, Grid g, const __grid_constant__ ZMaps maps, C* T, size_t tstride, unsigned* flags) {
-  using F = FT<C>;
+// column (the Nyquist row lands inside the zero band, which is never read).
+template <class RAW, int EPT, int COLS>
+__global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
+    k_fft_z_inv(FFTPlan pl, Grid g, const __grid_constant__ ZMaps maps, cfx* T, size_t tstride, int* te, unsigned* flags) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
-  C* a = reinterpret_cast<C*>(sm_raw);
-  const int pz = g.pz, nz = g.nz, h = g.nx / 2, n2 = nz / 2, H = pl.rows_in;
+  __shared__ FxShared sh;
+  cfx* a = reinterpret_cast<cfx*>(sm_raw);
+  const int pz = g.pz, nz = g.nz, h = g.nx / 2, n2 = nz / 2, H = pl.rows_in, tpt = pl.tpt;
   const int kx0 = blockIdx.x * COLS, j = blockIdx.y, f = blockIdx.z;
-  const int c = threadIdx.x % COLS, tt = threadIdx.x / COLS;
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(sm_raw + (size_t)pz * COLS * sizeof(C));
-  if (threadIdx.x == 0) mbar_init(bar);
+  const int c = threadIdx.x % COLS, tt = threadIdx.x / COLS, kx = kx0 + c;
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(sm_raw + (size_t)pz * COLS * sizeof(cfx));
+  if (threadIdx.x == 0) {
+    mbar_init(bar);
+    sh.top = 0;
+  }
   __syncthreads();
   if (threadIdx.x == 0 && LMVD_IN(f, TBUF_FIELDS)) {
-    mbar_expect_tx(bar, (unsigned)(nz * COLS * sizeof(C)));
+    mbar_expect_tx(bar, (unsigned)(nz * COLS * sizeof(cfx)));
     for (int r = 0; r < nz; r += H) {
       const int pos = r < n2 ? r : pz - nz + r;
       if (LMVD_IN((pos + H) * COLS - 1, pz * COLS)) tma_load_3d(a + (size_t)pos * COLS, &maps.m[f], 2 * kx0, r, j, bar);
     }
   }
   if (!mbar_wait_bounded(bar, flags)) return;
-  constexpr bool convert = !IN_DF && !std::is_same<C, cd>::value;
-  const bool zero_band = !prunes_zero_band<C>(pl);
-  if (zero_band || convert) {
-    // the padding band [n2, pz - n2 + 1) zeroed where the arithmetic reads it; spectral doubles to pairs
-    for (int idx = threadIdx.x; idx < pz * COLS; idx += blockDim.x) {
-      const int z = idx / COLS;
-      if (z >= n2 && z < pz - n2 + 1) {
-        if (zero_band) a[idx] = F::zero();
-      } else if (convert) {
-        a[idx] = F::from_spec(reinterpret_cast<const cd*>(a)[idx]);
-      }
-    }
-    __syncthreads();
+  const bool first4 = EPT == 12 && pl.first4;
+  RAW raw[EPT];
+  const int lo = n2, hi = pz - n2 + 1;  // kz padding: zero
+#pragma unroll
+  for (int u = 0; u < EPT; ++u) {
+    const int i = fx_point(u, first4, tt, tpt, pz >> 2);
+    raw[u] = kx < h && LMVD_IN(i, pz) && (i < lo || i >= hi) ? reinterpret_cast<const RAW*>(a)[i * COLS + c] : RAW{};
   }
-  fft_inplace<C, 1, EPT, kPrune<C>, false, COLS>(a + c, pl, tt, pl.tpt, n2, pz - n2 + 1);  // kz padding: zero
-  C* dst = T + f * tstride + (size_t)j * pz * h;
-  for (int idx = threadIdx.x; idx < pz * COLS; idx += blockDim.x) {
-    const int zz = idx / COLS, kx = kx0 + idx % COLS;
-    if (kx < h && LMVD_IN((size_t)zz * h + kx, (size_t)pz * h)) dst[(size_t)zz * h + kx] = a[idx];
+  int xe;
+  const int gz = pl.red_g, k = fx_scale(raw, sh, c, tpt / gz, COLS, gz, COLS, tt, 1.f, xe);
+  {
+    cfx v[EPT];
+    const float sa = fx_sa(k);
+#pragma unroll
+    for (int u = 0; u < EPT; ++u) v[u] = fx_convert(raw[u], k, sa);
+    fx_run<1, EPT, COLS>(v, a + c, pl, first4, tt);
   }
+  cfx v[EPT];
+  fx_last<1, EPT, COLS>(a + c, pl, tt, v);
+  if (kx >= h) return;
+  if (tt == 0) te[((size_t)f * g.ny + j) * h + kx] = fx_stored_exponent(k, xe);
+  cfx* dst = T + f * tstride + (size_t)j * pz * h + kx;
+#pragma unroll
+  for (int q = 0; q < EPT; ++q)
+    if (LMVD_IN((size_t)(tt + q * tpt) * h + kx, (size_t)pz * h)) dst[(size_t)(tt + q * tpt) * h] = v[q];
 }
-
-// (row, column) of a flat index idx = row n + column that a thread advances by a fixed step: one division at
-// the start instead of one per element (n is a run-time value, and an integer division costs tens of
-// instructions in passes that are bound by their instruction issue).
-struct RowCol {
-  int r, c;
-  __device__ __forceinline__ RowCol(int idx, int n) : r(idx / n), c(idx - (idx / n) * n) {}
-  __device__ __forceinline__ void advance(int step, int n) {
-    c += step;
-    while (c >= n) {
-      c -= n;
-      ++r;
-    }
-  }
-};
 
 // ---------------------------------------------------------------- inverse x-pass (c2r, 2 rows per transform)
 // With MUL the epilogue stores w * phys instead of phys (w: a physical field of the same layout, one for all
 // fields of the launch): the product f'(z) dz/dt of the fixed point (Sec. 4.3) formed as the transform is
-// written, so neither dz/dt on the grid nor a separate product pass is needed.
-template <class C, int EPT, bool MUL>
-__device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, const C* T, size_t tstride,
-                                           const FieldsRW& out, const void* wmul, unsigned* flags) {
-  using F = FT<C>;
-  using R = typename F::R;
+// written, so neither dz/dt on the grid nor a separate product pass is needed. (pz is even: 6 divides it.)
+template <int EPT, bool MUL>
+__device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, const cfx* T, size_t tstride, const int* te,
+                                           const FieldsRW& out, const double* wmul, unsigned* flags) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
-  C* a = reinterpret_cast<C*>(sm_raw);
-  const int batch = pl.batch, ld = pl.n + pl.pad, px = g.px, pz = g.pz, h = g.nx / 2;
+  __shared__ FxShared sh;
+  cfx* a = reinterpret_cast<cfx*>(sm_raw);
+  const int batch = pl.batch, ld = pl.n + pl.pad, px = g.px, pz = g.pz, h = g.nx / 2, tpt = pl.tpt;
   const int pr0 = blockIdx.x * batch, j = blockIdx.y, f = blockIdx.z;
-  const int bt = threadIdx.x / pl.tpt, tt = threadIdx.x - bt * pl.tpt;
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(sm_raw + (size_t)batch * ld * sizeof(C));
+  const int bt = threadIdx.x / tpt, tt = threadIdx.x - bt * tpt;
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(sm_raw + (size_t)batch * ld * sizeof(cfx));
   if (threadIdx.x == 0) mbar_init(bar);
   __syncthreads();
-  // A transform's rows za = 2 (pr0 + bb) and za + 1 of T are contiguous (2 h elements): one bulk copy each
+  // A transform's rows za = 2 (pr0 + bt) and za + 1 of T are contiguous (2 h elements): one bulk copy each
   // (TMA, cp.async.bulk) into the upper part [h, 3 h) = [h, px) of its buffer, completing on the mbarrier
   if (threadIdx.x == 0) {
-    const C* src = T + f * tstride + (size_t)j * pz * h;
+    const cfx* src = T + f * tstride + (size_t)j * pz * h;
     int nb = 0;
     while (nb < batch && 2 * (pr0 + nb) < pz) ++nb;
-    mbar_expect_tx(bar, (unsigned)(nb * 2 * h * sizeof(C)));
+    mbar_expect_tx(bar, (unsigned)(nb * 2 * h * sizeof(cfx)));
     for (int bb = 0; bb < nb; ++bb) {
       const int za = 2 * (pr0 + bb);
       if (LMVD_IN(bb * ld + px - 1, batch * ld) && LMVD_IN((size_t)(za + 2) * h - 1, (size_t)pz * h))
-        bulk_load(a + bb * ld + h, src + (size_t)za * h, (unsigned)(2 * h * sizeof(C)), bar);
+        bulk_load(a + bb * ld + h, src + (size_t)za * h, (unsigned)(2 * h * sizeof(cfx)), bar);
     }
+  }
+  // two real rows into one complex transform: y[k] = Xa[k] + i Xb[k], y[px - k] = conj(Xa[k]) + i conj(Xb[k]).
+  // A thread takes the EPT / 3 pairs k = tt, tt + tpt, ... < h; the scale's barrier precedes every write of a
+  // y[px - k] over the copied rows.
+  constexpr int NP = EPT / 3;
+  const int za = 2 * (pr0 + bt);
+  const bool live = za < pz;
+  cfx* y = a + bt * ld;
+  int E[NP], emin = INT_MAX;
+  const int* ej = te + ((size_t)f * g.ny + j) * h;
+#pragma unroll
+  for (int u = 0; u < NP; ++u) {
+    E[u] = LMVD_IN(tt + u * tpt, h) ? __ldg(ej + tt + u * tpt) : kFxMaxE;
+    emin = min(emin, E[u]);
   }
   if (!mbar_wait_bounded(bar, flags)) return;
-  // two real rows into one complex transform: y[k] = Xa[k] + i Xb[k], y[px - k] = conj(Xa[k]) + i conj(Xb[k]).
-  // Every thread reads its EPT / 3 pairs (batch h = blockDim.x EPT / 3 of them) before any is written,
-  // since the written y[px - k] overlay the copied rows.
-  constexpr int NP = EPT / 3;
-  C ta[NP], tb[NP];
-  int kk[NP], bs[NP];
-  RowCol rc(threadIdx.x, h);
+  cfx raw[2 * NP];
+  float hs[NP], mag = 0.f;
 #pragma unroll
   for (int u = 0; u < NP; ++u) {
-    const int bb = rc.r, k = rc.c;
-    rc.advance(blockDim.x, h);
-    kk[u] = -1;
-    if (bb >= batch || 2 * (pr0 + bb) >= pz || !LMVD_IN(bb * ld + 3 * h - 1, batch * ld)) continue;
-    kk[u] = k;
-    bs[u] = bb;
-    ta[u] = a[bb * ld + h + k];
-    tb[u] = a[bb * ld + 2 * h + k];
+    const int kk = tt + u * tpt;
+    const bool in = live && LMVD_IN(bt * ld + 2 * h + kk, batch * ld);
+    raw[2 * u] = in ? y[h + kk] : cfx{0, 0};
+    raw[2 * u + 1] = in ? y[2 * h + kk] : cfx{0, 0};
+    if (kk == 0) raw[2 * u].im = raw[2 * u + 1].im = 0;  // the kx = 0 coefficient of a real row is real
+    hs[u] = fx_mag_hi(raw[2 * u]) + fx_mag_hi(raw[2 * u + 1]);
+    mag += fx_mag(hs[u], E[u]);
   }
-  __syncthreads();
+  int xe;
+  const int gx = pl.red_g, np = tpt / gx;
+  const int k = fx_scale_t(mag, emin, sh, bt * np, np, 1, gx, 1, tt, 2.f, xe, [&](int s) {
+    float m = 0.f;
+#pragma unroll
+    for (int u = 0; u < NP; ++u) m += fx_mag(hs[u], E[u] += s);
+    return m;
+  });
 #pragma unroll
   for (int u = 0; u < NP; ++u) {
-    if (kk[u] < 0) continue;
-    const int k = kk[u];
-    C* y = a + bs[u] * ld;
-    if (k == 0) {
-      y[0] = F::make(F::re(ta[u]), F::re(tb[u]));  // the kx = 0 coefficient of a real row is real
+    const int kk = tt + u * tpt;
+    const cfx xa = fx_align(raw[2 * u], E[u] - k), xb = fx_align(raw[2 * u + 1], E[u] - k);
+    if (!LMVD_IN(kk, h)) continue;
+    if (kk == 0) {
+      y[0] = cfx{xa.re, xb.re};
     } else {
-      y[k] = F::add(ta[u], F::ti(tb[u]));                        // Xa[k] + i Xb[k]
-      y[px - k] = F::add(F::cj(ta[u]), F::ti(F::cj(tb[u])));  // conj(Xa[k]) + i conj(Xb[k])
+      y[kk] = cfx{xa.re - xb.im, xa.im + xb.re};       // Xa[k] + i Xb[k]
+      y[px - kk] = cfx{xa.re + xb.im, xb.re - xa.im};  // conj(Xa[k]) + i conj(Xb[k])
     }
   }
-  // the padding band [h, px - h + 1) = [h, 2 h]: zero where the arithmetic reads it (it held copied rows)
-  if (!prunes_zero_band<C>(pl)) {
-    RowCol rz(threadIdx.x, h + 1);
-    for (int idx = threadIdx.x; idx < batch * (h + 1); idx += blockDim.x) {
-      const int bb = rz.r, q = rz.c;
-      rz.advance(blockDim.x, h + 1);
-      if (LMVD_IN(bb * ld + h + q, batch * ld)) a[bb * ld + h + q] = F::zero();
-    }
-  }
+  if (pl.nst == 1)  // no stage that skips the kx padding [h, 2 h]
+    for (int q = h + tt; q <= 2 * h; q += tpt)
+      if (LMVD_IN(q, px)) y[q] = cfx{0, 0};
   __syncthreads();
-  fft_inplace<C, 1, EPT, kPrune<C>, false>(a + bt * ld, pl, tt, pl.tpt, h, px - h + 1);  // kx padding: zero
-  const C* res = a;
-  R* dst = reinterpret_cast<R*>(pick(out.p, f)) + (size_t)j * g.P;
-  if (MUL) {
-    const R* w = reinterpret_cast<const R*>(wmul) + (size_t)j * g.P;
-    RowCol rw(threadIdx.x, px);
-    for (int base = threadIdx.x; base < batch * px; base += FFT_LOAD_CHUNK * blockDim.x) {
-      R wa[FFT_LOAD_CHUNK], wb[FFT_LOAD_CHUNK];
-      int xs[FFT_LOAD_CHUNK], bs[FFT_LOAD_CHUNK];
+  fx_middle<1, EPT, 1>(y, pl, 0, tt, tpt, h, px - h + 1);  // kx padding: zero
+  double* dst = reinterpret_cast<double*>(pick(out.p, f)) + (size_t)j * g.P + (size_t)za * px;
+  const double* w = MUL ? wmul + (size_t)j * g.P + (size_t)za * px : nullptr;
+  cfx v[EPT];
+  fx_last<1, EPT, 1>(y, pl, tt, v);
+  if (!live) return;
 #pragma unroll
-      for (int u = 0; u < FFT_LOAD_CHUNK; ++u) {
-        const int idx = base + u * blockDim.x;
-        const int bb = rw.r, x = rw.c;
-        rw.advance(blockDim.x, px);
-        xs[u] = -1;
-        if (idx >= batch * px) continue;
-        const int za = 2 * (pr0 + bb), zb = za + 1;
-        if (za >= pz) continue;
-        if (!LMVD_IN((size_t)za * px + x, g.P) || !LMVD_IN(bb * ld + x, batch * ld)) continue;
-        xs[u] = x;
-        bs[u] = bb;
-        wa[u] = w[(size_t)za * px + x];
-        wb[u] = zb < pz ? w[(size_t)zb * px + x] : F::rzero();
-      }
-#pragma unroll
-      for (int u = 0; u < FFT_LOAD_CHUNK; ++u) {
-        if (xs[u] < 0) continue;
-        const int x = xs[u], za = 2 * (pr0 + bs[u]), zb = za + 1;
-        const C v = res[bs[u] * ld + x];
-        dst[(size_t)za * px + x] = F::rmul(wa[u], F::re(v));
-        if (zb < pz) dst[(size_t)zb * px + x] = F::rmul(wb[u], F::im(v));
-      }
-    }
-    return;
-  }
-  RowCol ro(threadIdx.x, px);
-  for (int idx = threadIdx.x; idx < batch * px; idx += blockDim.x) {
-    const int bb = ro.r, x = ro.c;
-    ro.advance(blockDim.x, px);
-    const int za = 2 * (pr0 + bb), zb = za + 1;
-    if (za >= pz) continue;
-    if (!LMVD_IN((size_t)za * px + x, g.P) || !LMVD_IN(bb * ld + x, batch * ld)) continue;
-    const C v = res[bb * ld + x];
-    dst[(size_t)za * px + x] = F::re(v);
-    if (zb < pz) dst[(size_t)zb * px + x] = F::im(v);
+  for (int q = 0; q < EPT; ++q) {
+    const int x = tt + q * tpt;
+    if (!LMVD_IN((size_t)(za + 1) * px + x, g.P)) continue;
+    const cd r = fx_result(v[q], k, xe);
+    dst[x] = MUL ? w[x] * r.re : r.re;
+    dst[px + x] = MUL ? w[px + x] * r.im : r.im;
   }
 }
-template <class C, int EPT>
-__global__ void __launch_bounds__(FFT_CTA_X, FftMinCtas<C>::x) k_fft_x_inv(FFTPlan pl, Grid g, const C* T, size_t tstride, FieldsRW out,
-                                                                         unsigned* flags) {
-  x_inv_body<C, EPT, false>(pl, g, T, tstride, out, nullptr, flags);
+template <int EPT>
+__global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_inv(FFTPlan pl, Grid g, const cfx* T, size_t tstride,
+                                                                    const int* te, FieldsRW out, unsigned* flags) {
+  x_inv_body<EPT, false>(pl, g, T, tstride, te, out, nullptr, flags);
 }
-template <class C, int EPT>
-__global__ void __launch_bounds__(FFT_CTA_X, FftMinCtas<C>::x) k_fft_x_inv_mul(FFTPlan pl, Grid g, const C* T, size_t tstride, FieldsRW out,
-                                                                             const void* wmul, unsigned* flags) {
-  x_inv_body<C, EPT, true>(pl, g, T, tstride, out, wmul, flags);
+template <int EPT>
+__global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_inv_mul(FFTPlan pl, Grid g, const cfx* T, size_t tstride,
+                                                                        const int* te, FieldsRW out, const double* wmul,
+                                                                        unsigned* flags) {
+  x_inv_body<EPT, true>(pl, g, T, tstride, te, out, wmul, flags);
 }
 
 // ---------------------------------------------------------------- forward x-pass (r2c, 2 rows per transform)
-// With DOT3 the load prologue forms -(w1 m1 + w2 m2 + w3 m3) from six physical fields instead of reading
-// one (d: w[0..2], m[0..2]; one launch, one field): the tail -(1/rho) grad z . m^c of L (Sec. 4.3) formed as
-// the transform reads it, so no product pass and no product field are needed.
+// With DOT3 the loads form -(w1 m1 + w2 m2 + w3 m3) from six physical fields instead of reading one (d: w[0..2],
+// m[0..2]; one launch, one field): the tail -(1/rho) grad z . m^c of L (Sec. 4.3) formed as the transform reads
+// it, so no product pass and no product field are needed.
+// The loads are the first stage's inputs: they go from global memory to registers. te: [f][ny][pz/2] exponents of T.
 struct Dot3 {
-  const void* w[3];
-  const void* m[3];
+  const double* w[3];
+  const double* m[3];
 };
-template <class C, int EPT, bool DOT3>
-__device__ __forceinline__ void x_fwd_body(const FFTPlan& pl, const Grid& g, const FieldsRC& in, C* T, size_t tstride,
-                                           const Dot3& d) {
-  using F = FT<C>;
-  using R = typename F::R;
+template <int EPT, bool DOT3>
+__device__ __forceinline__ void x_fwd_body(const FFTPlan& pl, const Grid& g, const FieldsRC& in, cfx* T, size_t tstride,
+                                           int* te, const Dot3& d) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
-  C* a = reinterpret_cast<C*>(sm_raw);
-  const int batch = pl.batch, ld = pl.n + pl.pad, px = g.px, pz = g.pz, h = g.nx / 2;
+  __shared__ FxShared sh;
+  cfx* a = reinterpret_cast<cfx*>(sm_raw);
+  const int batch = pl.batch, ld = pl.n + pl.pad, px = g.px, pz = g.pz, h = g.nx / 2, tpt = pl.tpt;
   const int pr0 = blockIdx.x * batch, j = blockIdx.y, f = blockIdx.z;
-  const int bt = threadIdx.x / pl.tpt, tt = threadIdx.x - bt * pl.tpt;
-  const R* src = reinterpret_cast<const R*>(pick(in.p, f)) + (size_t)j * g.P;
-  // DOT3 reads six fields per point: fewer points per chunk keep the registers in check
-  constexpr int CH = DOT3 ? 2 : FFT_LOAD_CHUNK;
-  RowCol rc(threadIdx.x, px);
-  for (int base = threadIdx.x; base < batch * px; base += CH * blockDim.x) {
-    R va[CH], vb[CH];
-    int ds[CH];
+  const int bt = threadIdx.x / tpt, tt = threadIdx.x - bt * tpt;
+  const int za = 2 * (pr0 + bt);
+  const bool live = za < pz;
+  cfx* y = a + bt * ld;
+  if (threadIdx.x == 0) sh.top = 0;
+  const bool first4 = EPT == 12 && pl.first4;
+  cd raw[EPT];
+  const size_t row = (size_t)j * g.P + (size_t)za * px;
+  const double* src = DOT3 ? nullptr : reinterpret_cast<const double*>(pick(in.p, f)) + row;
 #pragma unroll
-    for (int u = 0; u < CH; ++u) {
-      const int idx = base + u * blockDim.x;
-      const int bb = rc.r, x = rc.c;
-      rc.advance(blockDim.x, px);
-      ds[u] = -1;
-      va[u] = vb[u] = F::rzero();
-      if (idx >= batch * px) continue;
-      const int za = 2 * (pr0 + bb), zb = za + 1;
-      if (!LMVD_IN(bb * ld + x, batch * ld)) continue;
-      ds[u] = bb * ld + x;
-      if (za < pz && LMVD_IN((size_t)za * px + x, g.P)) {
-        if (DOT3) {
-          const size_t plane = (size_t)j * g.P;
-          const R* w0 = reinterpret_cast<const R*>(d.w[0]) + plane;
-          const R* w1 = reinterpret_cast<const R*>(d.w[1]) + plane;
-          const R* w2 = reinterpret_cast<const R*>(d.w[2]) + plane;
-          const R* m0 = reinterpret_cast<const R*>(d.m[0]) + plane;
-          const R* m1 = reinterpret_cast<const R*>(d.m[1]) + plane;
-          const R* m2 = reinterpret_cast<const R*>(d.m[2]) + plane;
-          size_t o = (size_t)za * px + x;
-          va[u] = F::dot3neg(w0[o], m0[o], w1[o], m1[o], w2[o], m2[o]);
-          if (zb < pz) {
-            o += px;
-            vb[u] = F::dot3neg(w0[o], m0[o], w1[o], m1[o], w2[o], m2[o]);
-          }
-        } else {
-          va[u] = src[(size_t)za * px + x];
-          if (zb < pz) vb[u] = src[(size_t)zb * px + x];
-        }
+  for (int u = 0; u < EPT; ++u) {
+    const int x = fx_point(u, first4, tt, tpt, px >> 2);
+    cd v{};
+    if (live && LMVD_IN((size_t)(za + 1) * px + x, g.P)) {
+      if (DOT3) {
+        const size_t o = row + x;
+        v.re = -(d.w[0][o] * d.m[0][o] + d.w[1][o] * d.m[1][o] + d.w[2][o] * d.m[2][o]);
+        const size_t o2 = o + px;
+        v.im = -(d.w[0][o2] * d.m[0][o2] + d.w[1][o2] * d.m[1][o2] + d.w[2][o2] * d.m[2][o2]);
+      } else {
+        v = cd{src[x], src[px + x]};
       }
     }
+    raw[u] = v;
+  }
+  __syncthreads();  // sh.top
+  int xe;
+  // (the sums p + conj(m) = twice a row's coefficient formed at the end may reach 2^62.7: no product follows)
+  const int gx = pl.red_g, np = tpt / gx, k = fx_scale(raw, sh, bt * np, np, 1, gx, 1, tt, 1.f, xe);
+  {
+    cfx v[EPT];
 #pragma unroll
-    for (int u = 0; u < CH; ++u)
-      if (ds[u] >= 0) a[ds[u]] = F::make(va[u], vb[u]);
+    for (int u = 0; u < EPT; ++u) v[u] = fx_convert(raw[u], k, 0.f);
+    fx_run<-1, EPT, 1>(v, y, pl, first4, tt);
   }
+  // last stage: the retained kx are the outputs q < NP (kx = tt + q tpt) and q >= 2 NP (px - kx); a thread keeps the
+  // first and stores the others for the thread that pairs them
+  constexpr int NP = EPT / 3;
+  cfx v[EPT];
+  fx_last<-1, EPT, 1>(y, pl, tt, v);
+#pragma unroll
+  for (int q = 2 * NP; q < EPT; ++q)
+    if (LMVD_IN(tt + q * tpt, px)) y[tt + q * tpt] = v[q];  // this thread's own inputs
   __syncthreads();
-  fft_inplace<C, -1, EPT, false, kPrune<C>>(a + bt * ld, pl, tt, pl.tpt, h, px - h + 1);  // truncated kx
-  const C* res = a;
-  C* dst = T + f * tstride + (size_t)j * pz * h;
-  RowCol ro(threadIdx.x, h);
-  for (int idx = threadIdx.x; idx < batch * h; idx += blockDim.x) {
-    const int bb = ro.r, k = ro.c;
-    ro.advance(blockDim.x, h);
-    const int za = 2 * (pr0 + bb), zb = za + 1;
-    if (za >= pz) continue;
-    if (!LMVD_IN((size_t)za * h + k, (size_t)pz * h) || !LMVD_IN(bb * ld + px - 1, batch * ld)) continue;
-    const C yk = res[bb * ld + k];
-    const C ym = F::cj(res[bb * ld + (k == 0 ? 0 : px - k)]);
-    // twice the two rows' spectra (the 1/2 is in the z-pass's scale): yk + ym and (yk - ym) / i
-    dst[(size_t)za * h + k] = F::add(yk, ym);
-    if (zb < pz) dst[(size_t)zb * h + k] = F::neg(F::ti(F::sub(yk, ym)));
+  if (!live) return;
+  if (tt == 0) te[((size_t)f * g.ny + j) * (pz / 2) + pr0 + bt] = fx_stored_exponent(k, xe);
+  cfx* dst = T + f * tstride + (size_t)j * pz * h + (size_t)za * h;
+#pragma unroll
+  for (int q = 0; q < NP; ++q) {
+    const int kk = tt + q * tpt;
+    if (!LMVD_IN((size_t)(za + 1) * h + kk, (size_t)pz * h)) continue;
+    const cfx p = v[q], m = kk == 0 ? p : y[px - kk];
+    // twice the two rows' spectra (the 1/2 is in the z-pass's scale): p + conj(m) and (p - conj(m)) / i
+    dst[kk] = cfx{p.re + m.re, p.im - m.im};
+    dst[h + kk] = cfx{p.im + m.im, m.re - p.re};
   }
 }
-template <class C, int EPT>
-__global__ void __launch_bounds__(FFT_CTA_X, FftMinCtas<C>::x) k_fft_x_fwd(FFTPlan pl, Grid g, FieldsRC in, C* T, size_t tstride) {
-  x_fwd_body<C, EPT, false>(pl, g, in, T, tstride, Dot3{});
+template <int EPT>
+__global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_fwd(FFTPlan pl, Grid g, FieldsRC in, cfx* T, size_t tstride,
+                                                                    int* te) {
+  x_fwd_body<EPT, false>(pl, g, in, T, tstride, te, Dot3{});
 }
-template <class C, int EPT>
-__global__ void __launch_bounds__(FFT_CTA_X, FftMinCtas<C>::x) k_fft_x_fwd_dot3(FFTPlan pl, Grid g, C* T, size_t tstride, Dot3 d) {
-  x_fwd_body<C, EPT, true>(pl, g, FieldsRC{}, T, tstride, d);
+template <int EPT>
+__global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_fwd_dot3(FFTPlan pl, Grid g, cfx* T, size_t tstride, int* te,
+                                                                         Dot3 d) {
+  x_fwd_body<EPT, true>(pl, g, FieldsRC{}, T, tstride, te, d);
 }
 
 // ---------------------------------------------------------------- forward z-pass (truncate, scale)
-// T: [f][ny][pz][nx/2] of C, read through maps.m[0] (all fields of the launch: planes f ny + j); out:
-// spectral fields [ny][nz][nxh]. Same interleaved layout as the inverse z-pass; kx = nx/2 and the kz
-// Nyquist row are written as zero.
-template <class C, int EPT, int COLS>
-__global__ void __launch_bounds__(FFT_CTA_Z, FftMinCtas<C>::z_fwd)
-    k_fft_z_fwd(FFTPlan pl, Grid g, const __grid_constant__ ZMaps maps, FieldsW out, unsigned* flags) {
-  using F = FT<C>;
+// T: [f][ny][pz][nx/2], read through maps.m[0] (all fields of the launch: planes f ny + j), its exponents te [f][ny]
+// [pz/2]; out: spectral fields [ny][nz][nxh]. Same interleaved layout as the inverse z-pass; kx = nx/2 and the kz
+// Nyquist row are written as zero. The last stage's middle outputs are the truncated kz.
+template <int EPT, int COLS>
+__global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
+    k_fft_z_fwd(FFTPlan pl, Grid g, const __grid_constant__ ZMaps maps, const int* te, FieldsW out, unsigned* flags) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
-  C* a = reinterpret_cast<C*>(sm_raw);
-  const int pz = g.pz, nz = g.nz, h = g.nx / 2, n2 = nz / 2, H = pl.rows_t;
+  __shared__ FxShared sh;
+  cfx* a = reinterpret_cast<cfx*>(sm_raw);
+  const int pz = g.pz, h = g.nx / 2, n2 = g.nz / 2, H = pl.rows_t, tpt = pl.tpt;
   const int kx0 = blockIdx.x * COLS, j = blockIdx.y, f = blockIdx.z;
-  const int c = threadIdx.x % COLS, tt = threadIdx.x / COLS;
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(sm_raw + (size_t)pz * COLS * sizeof(C));
+  const int c = threadIdx.x % COLS, tt = threadIdx.x / COLS, kx = kx0 + c;
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(sm_raw + (size_t)pz * COLS * sizeof(cfx));
   if (threadIdx.x == 0) mbar_init(bar);
   __syncthreads();
   if (threadIdx.x == 0) {
-    mbar_expect_tx(bar, (unsigned)(pz * COLS * sizeof(C)));
+    mbar_expect_tx(bar, (unsigned)(pz * COLS * sizeof(cfx)));
     for (int r = 0; r < pz; r += H)
       if (LMVD_IN((r + H) * COLS - 1, pz * COLS)) tma_load_3d(a + (size_t)r * COLS, &maps.m[0], 2 * kx0, r, f * g.ny + j, bar);
   }
+  const bool first4 = EPT == 12 && pl.first4;
+  int E[EPT], emin = INT_MAX;
+  const int* ej = te + ((size_t)f * g.ny + j) * (pz / 2);
+#pragma unroll
+  for (int u = 0; u < EPT; ++u) {
+    const int i = fx_point(u, first4, tt, tpt, pz >> 2);
+    E[u] = LMVD_IN(i, pz) ? __ldg(ej + (i >> 1)) : kFxMaxE;
+    emin = min(emin, E[u]);
+  }
   if (!mbar_wait_bounded(bar, flags)) return;
-  fft_inplace<C, -1, EPT, false, kPrune<C>, COLS>(a + c, pl, tt, pl.tpt, n2, pz - n2 + 1);  // truncated kz
-  cd* dst = pick(out.p, f) + (size_t)j * g.M;
-  for (int idx = threadIdx.x; idx < nz * COLS; idx += blockDim.x) {
-    const int jz = idx / COLS, cc = idx % COLS, kx = kx0 + cc;
-    if (kx > h) continue;
-    const int pos = jz < n2 ? jz : pz - nz + jz;
-    cd v = mk(0, 0);
-    if (kx < h && jz != n2 && LMVD_IN(pos * COLS + cc, pz * COLS)) v = F::to_spec(a[pos * COLS + cc], pl);
-    if (LMVD_IN((size_t)jz * g.nxh + kx, g.M)) dst[(size_t)jz * g.nxh + kx] = v;
+  cfx v[EPT];
+  float mag = 0.f;
+#pragma unroll
+  for (int u = 0; u < EPT; ++u) {
+    const int i = fx_point(u, first4, tt, tpt, pz >> 2);
+    v[u] = LMVD_IN(i, pz) ? a[i * COLS + c] : cfx{0, 0};
+    mag += fx_mag(fx_mag_hi(v[u]), E[u]);
+  }
+  int xe;
+  const int gz = pl.red_g;
+  const int k = fx_scale_t(mag, emin, sh, c, tpt / gz, COLS, gz, COLS, tt, 1.f, xe, [&](int s) {
+    float m = 0.f;
+#pragma unroll
+    for (int u = 0; u < EPT; ++u) m += fx_mag(fx_mag_hi(v[u]), E[u] += s);
+    return m;
+  });
+#pragma unroll
+  for (int u = 0; u < EPT; ++u) v[u] = fx_align(v[u], E[u] - k);
+  fx_run<-1, EPT, COLS>(v, a + c, pl, first4, tt);
+  fx_last<-1, EPT, COLS>(a + c, pl, tt, v);
+  if (kx > h) return;
+  cd* dst = pick(out.p, f) + (size_t)j * g.M + kx;
+  // outputs q < NP (kz = tt + q tpt) and q >= 2 NP (kz = i - n2, row n2 + i; i = 0 is the Nyquist row)
+  constexpr int NP = EPT / 3;
+#pragma unroll
+  for (int q = 0; q < NP; ++q) {
+    const int b = tt + q * tpt;
+    if (!LMVD_IN((size_t)(n2 + b) * g.nxh + kx, g.M)) continue;
+    cd p = pl.scale_d * fx_result(v[q], k, xe), m = pl.scale_d * fx_result(v[2 * NP + q], k, xe);
+    if (kx == h) p = m = mk(0, 0);
+    if (b == 0) m = mk(0, 0);
+    dst[(size_t)b * g.nxh] = p;
+    dst[(size_t)(n2 + b) * g.nxh] = m;
   }
 }
 
 // ---------------------------------------------------------------- host side
-// Radix order 4s, 2s, 3s: the sub-length L is a power of two in every radix-4/2 stage (mask arithmetic).
-// 12 elements per thread (6 when n has a single factor 2, hence no radix-4 stage); at most cta threads per
+// Radix order 4s, 2s, 3s, then the last stage's 12 (6 when n has a single factor 2): the sub-length L is a power of
+// two in every radix-4/2 stage (mask arithmetic). 12 (6) elements per thread; at most cta threads per
 // CTA (so n <= 12 cta); one shared buffer of batch transforms with leading dimension n + pad.
 static bool make_plan(int n, int cta, FFTPlan& p) {
   p.n = n;
   p.nst = 0;
-  int m = n;
-  while (m % 4 == 0) { p.radix[p.nst++] = 4; m /= 4; }
-  while (m % 2 == 0) { p.radix[p.nst++] = 2; m /= 2; }
-  while (m % 3 == 0) { p.radix[p.nst++] = 3; m /= 3; }
-  if (m != 1 || p.nst > 16) return false;
-  p.code = 0;
-  for (int s2 = 0; s2 < p.nst; ++s2)
-    p.code |= (unsigned)(p.radix[s2] == 4 ? 0 : (p.radix[s2] == 2 ? 1 : 2)) << (2 * s2);
   p.ept = (n % 12 == 0) ? 12 : ((n % 6 == 0) ? 6 : 0);
   if (!p.ept) return false;
   p.tpt = n / p.ept;
+  p.code = 0;
+  int m = p.tpt;
+  for (int r : {4, 2, 3})
+    for (; m % r == 0; m /= r) p.code |= (unsigned)(r == 4 ? 0 : (r == 2 ? 1 : 2)) << (2 * p.nst++);
+  if (m != 1 || p.nst > 15) return false;
+  ++p.nst;  // the last stage, radix ept
+  p.first4 = p.tpt % 4 == 0;
   if (p.tpt > cta) return false;
+  for (p.red_g = 1; p.tpt % (2 * p.red_g) == 0 && p.red_g < (cta == FFT_CTA_Z ? 8 : 32);) p.red_g *= 2;
+  const long double s3 = sqrtl(3.0L) / 2.0L;
+  fx_limbs(s3, p.s3.x, p.s3.y);
   p.batch = cta / p.tpt;
   p.pad = 1;  // the x-passes: leading dimension n + 1 keeps the transforms of a batch in different banks
   if (cta == FFT_CTA_Z) {
@@ -690,7 +785,7 @@ static bool make_plan(int n, int cta, FFTPlan& p) {
 }
 
 // a pass's buffer is followed by its mbarrier (the z-passes' and the inverse x-pass's copies)
-static size_t smem_bytes(const FFTPlan& p) { return (size_t)p.batch * (p.n + p.pad) * sizeof(cd) + 16; }
+static size_t smem_bytes(const FFTPlan& p) { return (size_t)p.batch * (p.n + p.pad) * sizeof(cfx) + 16; }
 
 // Tensor maps for the z-passes' tile copies. cuTensorMapEncodeTiled is a driver function; the runtime hands
 // out its address, so the library needs no link to the driver library.
@@ -725,49 +820,30 @@ static bool tile_map(CUtensorMap* m, const void* base, size_t cols, size_t rows,
 }
 static unsigned threads(const FFTPlan& p) { return (unsigned)(p.batch * p.tpt); }
 
-static df host_split(long double x) {
-  const float h = (float)x;
-  return df{h, (float)(x - (long double)h)};
-}
-
 // Every pass may take up to kFftSmemMax bytes of dynamic shared memory. The limit is a property of the
 // kernel, shared by all contexts and the allocation-free path in the process: setting it to one grid's size
 // would break the launches of another context with a larger grid, so it is set once, to the maximum a plan
 // may ask for (fft_prepare rejects larger plans).
 constexpr int kFftSmemMax = 200 * 1024;
 
-template <class C, int EPT, int COLS>
-static int set_smem_z(int sz) {
-  if (cudaFuncSetAttribute(k_fft_z_inv<C, EPT, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, sz) != cudaSuccess ||
-      cudaFuncSetAttribute(k_fft_z_fwd<C, EPT, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, sz) != cudaSuccess)
-    return LMVD_ERR_CUDA;
-  if constexpr (std::is_same<C, cdf>::value) {
-    if (cudaFuncSetAttribute(k_fft_z_inv<C, EPT, COLS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sz) !=
-        cudaSuccess)
-      return LMVD_ERR_CUDA;
-  }
-  return LMVD_OK;
+template <class K>
+static bool smem_limit(K kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax) == cudaSuccess;
 }
-
-template <class C, int EPT>
-static int set_smem_e(int sx, int sz) {
-  if constexpr (EPT == 12) {
-    if (set_smem_z<C, EPT, 2>(sz)) return LMVD_ERR_CUDA;
-  }
-  if (set_smem_z<C, EPT, 4>(sz) ||
-      cudaFuncSetAttribute(k_fft_x_inv<C, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx) != cudaSuccess ||
-      cudaFuncSetAttribute(k_fft_x_fwd<C, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx) != cudaSuccess ||
-      cudaFuncSetAttribute(k_fft_x_inv_mul<C, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx) != cudaSuccess ||
-      cudaFuncSetAttribute(k_fft_x_fwd_dot3<C, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx) != cudaSuccess)
-    return LMVD_ERR_CUDA;
-  return LMVD_OK;
+template <int EPT, int COLS>
+static bool smem_limit_z() {
+  return smem_limit(k_fft_z_inv<cd, EPT, COLS>) && smem_limit(k_fft_z_inv<cdf, EPT, COLS>) &&
+         smem_limit(k_fft_z_fwd<EPT, COLS>);
 }
-
-template <class C>
+template <int EPT>
+static bool smem_limit_x() {
+  return smem_limit(k_fft_x_inv<EPT>) && smem_limit(k_fft_x_inv_mul<EPT>) && smem_limit(k_fft_x_fwd<EPT>) &&
+         smem_limit(k_fft_x_fwd_dot3<EPT>);
+}
 static int set_smem() {
-  int e = set_smem_e<C, 12>(kFftSmemMax, kFftSmemMax);
-  if (!e) e = set_smem_e<C, 6>(kFftSmemMax, kFftSmemMax);
-  return e;
+  return smem_limit_z<12, 4>() && smem_limit_z<12, 2>() && smem_limit_z<6, 4>() && smem_limit_x<12>() && smem_limit_x<6>()
+             ? LMVD_OK
+             : LMVD_ERR_CUDA;
 }
 
 int fft_prepare(Ctx& c) {
@@ -776,30 +852,21 @@ int fft_prepare(Ctx& c) {
   const long double pi = 3.141592653589793238462643383279502884L;
   for (FFTPlan* p : {&c.fx, &c.fz}) {
     if (smem_bytes(*p) > kFftSmemMax) return LMVD_ERR_UNSUPPORTED;
-    std::vector<double2> tw(p->n);
-    std::vector<float4> twf(p->n);
+    std::vector<int4> tw(p->n);
     for (int m = 0; m < p->n; ++m) {
       const long double ang = 2.0L * pi * (long double)m / (long double)p->n;
-      const long double cs = cosl(ang), sn = sinl(ang);
-      tw[m] = make_double2((double)cs, (double)sn);
-      const df hc = host_split(cs), hs = host_split(sn);
-      twf[m] = make_float4(hc.hi, hc.lo, hs.hi, hs.lo);
+      fx_limbs(cosl(ang), tw[m].x, tw[m].y);
+      fx_limbs(sinl(ang), tw[m].z, tw[m].w);
     }
-    if (cudaMalloc(&p->tw, sizeof(double2) * p->n) != cudaSuccess) return LMVD_ERR_OOM;
-    c.small_allocs.push_back(p->tw);
-    if (cudaMalloc(&p->twf, sizeof(float4) * p->n) != cudaSuccess) return LMVD_ERR_OOM;
-    c.small_allocs.push_back(p->twf);
-    c.small_bytes += (sizeof(double2) + sizeof(float4)) * p->n;
-    if (cudaMemcpy(p->tw, tw.data(), sizeof(double2) * p->n, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(p->twf, twf.data(), sizeof(float4) * p->n, cudaMemcpyHostToDevice) != cudaSuccess)
-      return LMVD_ERR_CUDA;
+    int4* d = nullptr;
+    if (cudaMalloc(&d, sizeof(int4) * p->n) != cudaSuccess) return LMVD_ERR_OOM;
+    c.small_allocs.push_back(d);
+    c.small_bytes += sizeof(int4) * p->n;
+    if (cudaMemcpy(d, tw.data(), sizeof(int4) * p->n, cudaMemcpyHostToDevice) != cudaSuccess) return LMVD_ERR_CUDA;
+    p->tw = d;
     p->scale_d = (double)(scale / 2);  // used by the forward z-pass (see the file head)
-    p->scale_f = host_split(scale / 2);
-    p->s3f = host_split(sqrtl(3.0L) / 2.0L);
   }
-  int e = set_smem<cd>();
-  if (!e) e = set_smem<cdf>();
-  return e;
+  return set_smem();
 }
 
 static inline unsigned cdiv(unsigned a, unsigned b) { return (a + b - 1) / b; }
@@ -813,8 +880,8 @@ static void map_failed(Ctx& c) {
 
 // The inverse z-pass of n fields (spectral inputs fi) into T, and the forward z-pass of n fields of T into
 // fo: tensor maps for their tile copies, then one launch of the instantiation the plan selects.
-template <class C, bool IN_DF>
-static void z_inv_launch(Ctx& c, const FieldsC& fi, int n, C* T, size_t tstride, double fl, double by) {
+template <class RAW>
+static void z_inv_launch(Ctx& c, const FieldsC& fi, int n, size_t tstride, double fl, double by) {
   const Grid& g = c.g;
   const FFTPlan& p = c.fz;
   ZMaps maps;
@@ -825,42 +892,37 @@ static void z_inv_launch(Ctx& c, const FieldsC& fi, int n, C* T, size_t tstride,
     }
   const dim3 gz(cdiv(g.nx / 2, p.batch), g.ny, n);
   if (p.ept == 12 && p.batch == 4)
-    LMVD_LAUNCH(c, KC_FFT_Z_INV, fl, by, (k_fft_z_inv<C, 12, 4, IN_DF>), gz, threads(p), smem_bytes(p), p, g, maps, T,
-                tstride, c.dflags);
+    LMVD_LAUNCH(c, KC_FFT_Z_INV, fl, by, (k_fft_z_inv<RAW, 12, 4>), gz, threads(p), smem_bytes(p), p, g, maps,
+                c.tbuf, tstride, c.texp, c.dflags);
   else if (p.ept == 12)
-    LMVD_LAUNCH(c, KC_FFT_Z_INV, fl, by, (k_fft_z_inv<C, 12, 2, IN_DF>), gz, threads(p), smem_bytes(p), p, g, maps, T,
-                tstride, c.dflags);
+    LMVD_LAUNCH(c, KC_FFT_Z_INV, fl, by, (k_fft_z_inv<RAW, 12, 2>), gz, threads(p), smem_bytes(p), p, g, maps,
+                c.tbuf, tstride, c.texp, c.dflags);
   else
-    LMVD_LAUNCH(c, KC_FFT_Z_INV, fl, by, (k_fft_z_inv<C, 6, 4, IN_DF>), gz, threads(p), smem_bytes(p), p, g, maps, T,
-                tstride, c.dflags);
+    LMVD_LAUNCH(c, KC_FFT_Z_INV, fl, by, (k_fft_z_inv<RAW, 6, 4>), gz, threads(p), smem_bytes(p), p, g, maps,
+                c.tbuf, tstride, c.texp, c.dflags);
 }
 
-template <class C>
-static void z_fwd_launch(Ctx& c, const C* T, int n, const FieldsW& fo, double fl, double by) {
+static void z_fwd_launch(Ctx& c, int n, const FieldsW& fo, double fl, double by) {
   const Grid& g = c.g;
   const FFTPlan& p = c.fz;
   ZMaps maps;
-  if (!tile_map(&maps.m[0], T, g.nx / 2, g.pz, (size_t)n * g.ny, p.batch, p.rows_t)) {
+  if (!tile_map(&maps.m[0], c.tbuf, g.nx / 2, g.pz, (size_t)n * g.ny, p.batch, p.rows_t)) {
     map_failed(c);
     return;
   }
   const dim3 gz(cdiv(g.nx / 2 + 1, p.batch), g.ny, n);
   if (p.ept == 12 && p.batch == 4)
-    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<C, 12, 4>), gz, threads(p), smem_bytes(p), p, g, maps, fo,
-                c.dflags);
+    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 4>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, c.dflags);
   else if (p.ept == 12)
-    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<C, 12, 2>), gz, threads(p), smem_bytes(p), p, g, maps, fo,
-                c.dflags);
+    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 2>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, c.dflags);
   else
-    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<C, 6, 4>), gz, threads(p), smem_bytes(p), p, g, maps, fo,
-                c.dflags);
+    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<6, 4>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, c.dflags);
 }
 
-template <class C>
-static void inverse_t(Ctx& c, cd* const* in, void* const* out, int nf, const void* wmul = nullptr, bool in_df = false) {
+// df_in: the spectral inputs are double-float pairs (the precision path's evaluations)
+static void inverse(Ctx& c, cd* const* in, double* const* out, int nf, bool df_in, const double* wmul = nullptr) {
   const Grid& g = c.g;
   const size_t tstride = (size_t)g.ny * g.pz * (g.nx / 2);
-  C* T = reinterpret_cast<C*>(c.tbuf);
   for (int f0 = 0; f0 < nf; f0 += c.tbuf_n) {
     const int n = nf - f0 < c.tbuf_n ? nf - f0 : c.tbuf_n;
     FieldsC fi{};
@@ -871,33 +933,30 @@ static void inverse_t(Ctx& c, cd* const* in, void* const* out, int nf, const voi
     }
     const double h = g.nx / 2, ny = g.ny, pz = g.pz, px = g.px;
     const double zfl = n * ny * h * fft_flops(pz), zby = n * ny * h * 16.0 * ((g.nz - 1) + pz);
-    // double-float inputs only exist for the double-float arithmetic
-    if (in_df && std::is_same<C, cdf>::value) z_inv_launch<C, std::is_same<C, cdf>::value>(c, fi, n, T, tstride, zfl, zby);
-    else z_inv_launch<C, false>(c, fi, n, T, tstride, zfl, zby);
+    if (df_in) z_inv_launch<cdf>(c, fi, n, tstride, zfl, zby);
+    else z_inv_launch<cd>(c, fi, n, tstride, zfl, zby);
     dim3 gx(cdiv(cdiv(g.pz, 2), c.fx.batch), g.ny, n);
     const double xfl = n * ny * ((g.pz + 1) / 2) * fft_flops(px), xby = n * ny * pz * (16.0 * h + 8.0 * px);
     if (wmul) {  // the product with w in the epilogue: one more physical field read, one multiply per point
       if (c.fx.ept == 12)
-        LMVD_LAUNCH(c, KC_FFT_X_INV, xfl + n * ny * pz * px, xby + n * ny * pz * 8.0 * px, (k_fft_x_inv_mul<C, 12>),
-                    gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, T, tstride, fo, wmul, c.dflags);
+        LMVD_LAUNCH(c, KC_FFT_X_INV, xfl + n * ny * pz * px, xby + n * ny * pz * 8.0 * px, k_fft_x_inv_mul<12>, gx,
+                    threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf, tstride, c.texp, fo, wmul, c.dflags);
       else
-        LMVD_LAUNCH(c, KC_FFT_X_INV, xfl + n * ny * pz * px, xby + n * ny * pz * 8.0 * px, (k_fft_x_inv_mul<C, 6>),
-                    gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, T, tstride, fo, wmul, c.dflags);
+        LMVD_LAUNCH(c, KC_FFT_X_INV, xfl + n * ny * pz * px, xby + n * ny * pz * 8.0 * px, k_fft_x_inv_mul<6>, gx,
+                    threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf, tstride, c.texp, fo, wmul, c.dflags);
     } else if (c.fx.ept == 12) {
-      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, (k_fft_x_inv<C, 12>), gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, T,
-                  tstride, fo, c.dflags);
+      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, k_fft_x_inv<12>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf,
+                  tstride, c.texp, fo, c.dflags);
     } else {
-      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, (k_fft_x_inv<C, 6>), gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, T,
-                  tstride, fo, c.dflags);
+      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, k_fft_x_inv<6>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf,
+                  tstride, c.texp, fo, c.dflags);
     }
   }
 }
 
-template <class C>
-static void forward_t(Ctx& c, void* const* in, cd* const* out, int nf) {
+void fft_forward(Ctx& c, double* const* in, cd* const* out, int nf) {
   const Grid& g = c.g;
   const size_t tstride = (size_t)g.ny * g.pz * (g.nx / 2);
-  C* T = reinterpret_cast<C*>(c.tbuf);
   for (int f0 = 0; f0 < nf; f0 += c.tbuf_n) {
     const int n = nf - f0 < c.tbuf_n ? nf - f0 : c.tbuf_n;
     FieldsRC fi{};
@@ -910,20 +969,18 @@ static void forward_t(Ctx& c, void* const* in, cd* const* out, int nf) {
     dim3 gx(cdiv(cdiv(g.pz, 2), c.fx.batch), g.ny, n);
     if (c.fx.ept == 12)
       LMVD_LAUNCH(c, KC_FFT_X_FWD, n * ny * ((g.pz + 1) / 2) * fft_flops(px), n * ny * pz * (16.0 * h + 8.0 * px),
-                  (k_fft_x_fwd<C, 12>), gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, fi, T, tstride);
+                  k_fft_x_fwd<12>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, fi, c.tbuf, tstride, c.texp);
     else
       LMVD_LAUNCH(c, KC_FFT_X_FWD, n * ny * ((g.pz + 1) / 2) * fft_flops(px), n * ny * pz * (16.0 * h + 8.0 * px),
-                  (k_fft_x_fwd<C, 6>), gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, fi, T, tstride);
-    z_fwd_launch<C>(c, T, n, fo, n * ny * h * fft_flops(pz), n * ny * 16.0 * (pz * h + (double)g.nz * g.nxh));
+                  k_fft_x_fwd<6>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, fi, c.tbuf, tstride, c.texp);
+    z_fwd_launch(c, n, fo, n * ny * h * fft_flops(pz), n * ny * 16.0 * (pz * h + (double)g.nz * g.nxh));
   }
 }
 
 // forward transform of -(w1 m1 + w2 m2 + w3 m3), formed in the x-pass prologue, into one spectral field
-template <class C>
-static void forward_dot3_t(Ctx& c, const double* const* w, const double* const* m, cd* out) {
+void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, cd* out) {
   const Grid& g = c.g;
   const size_t tstride = (size_t)g.ny * g.pz * (g.nx / 2);
-  C* T = reinterpret_cast<C*>(c.tbuf);
   Dot3 d{};
   for (int f = 0; f < 3; ++f) {
     d.w[f] = w[f];
@@ -935,24 +992,21 @@ static void forward_dot3_t(Ctx& c, const double* const* w, const double* const* 
   dim3 gx(cdiv(cdiv(g.pz, 2), c.fx.batch), g.ny, 1);
   const double xfl = ny * ((g.pz + 1) / 2) * fft_flops(px) + 6.0 * ny * pz * px, xby = ny * pz * (16.0 * h + 48.0 * px);
   if (c.fx.ept == 12)
-    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, (k_fft_x_fwd_dot3<C, 12>), gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, T,
-                tstride, d);
+    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, k_fft_x_fwd_dot3<12>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf,
+                tstride, c.texp, d);
   else
-    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, (k_fft_x_fwd_dot3<C, 6>), gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, T,
-                tstride, d);
-  z_fwd_launch<C>(c, T, 1, fo, ny * h * fft_flops(pz), ny * 16.0 * (pz * h + (double)g.nz * g.nxh));
+    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, k_fft_x_fwd_dot3<6>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf,
+                tstride, c.texp, d);
+  z_fwd_launch(c, 1, fo, ny * h * fft_flops(pz), ny * 16.0 * (pz * h + (double)g.nz * g.nxh));
 }
 
+// the substage's inputs come from the double-float evaluations in the precision path
+void fft_inverse(Ctx& c, cd* const* in, double* const* out, int nf) { inverse(c, in, out, nf, c.cfg.precision == 1); }
+void fft_inverse_d(Ctx& c, cd* const* in, double* const* out, int nf) { inverse(c, in, out, nf, false); }
 void fft_inverse_mul(Ctx& c, cd* in, double* out, const double* w) {
   cd* i[1] = {in};
-  void* o[1] = {out};
-  if (c.cfg.precision == 1) inverse_t<cdf>(c, i, o, 1, w, true);
-  else inverse_t<cd>(c, i, o, 1, w);
-}
-
-void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, cd* out) {
-  if (c.cfg.precision == 1) forward_dot3_t<cdf>(c, w, m, out);
-  else forward_dot3_t<cd>(c, w, m, out);
+  double* o[1] = {out};
+  inverse(c, i, o, 1, c.cfg.precision == 1, w);
 }
 
 // The bounded wait of the z-passes, on its own (lmvd_tile_wait_probe): one CTA expects 128 + extra bytes on
@@ -969,32 +1023,6 @@ __global__ void k_tile_wait_probe(const double* src, int extra, unsigned* status
   if (!mbar_wait_bounded(&bar, status)) return;
   if (threadIdx.x < 16 && buf[threadIdx.x] != src[threadIdx.x]) atomicOr(status, 8u);
 }
-
-void fft_inverse_as(Ctx& c, cd* const* in, double* const* out, int nf, int precision) {
-  void* o[64];
-  for (int f = 0; f < nf; ++f) o[f] = out[f];
-  if (precision == 1) inverse_t<cdf>(c, in, o, nf);
-  else inverse_t<cd>(c, in, o, nf);
-}
-
-void fft_forward_as(Ctx& c, double* const* in, cd* const* out, int nf, int precision) {
-  void* i[64];
-  for (int f = 0; f < nf; ++f) i[f] = in[f];
-  if (precision == 1) forward_t<cdf>(c, i, out, nf);
-  else forward_t<cd>(c, i, out, nf);
-}
-
-void fft_inverse(Ctx& c, cd* const* in, double* const* out, int nf) {
-  if (c.cfg.precision == 1) {  // the substage's inputs come from the double-float evaluations
-    void* o[64];
-    for (int f = 0; f < nf; ++f) o[f] = out[f];
-    inverse_t<cdf>(c, in, o, nf, nullptr, true);
-  } else {
-    fft_inverse_as(c, in, out, nf, 0);
-  }
-}
-
-void fft_forward(Ctx& c, double* const* in, cd* const* out, int nf) { fft_forward_as(c, in, out, nf, c.cfg.precision); }
 
 }  // namespace lmvd
 
@@ -1014,28 +1042,38 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratch
 constexpr int kNoAllocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 void* g_noalloc_ptr[kNoAllocMaxDevices] = {};
+// exponents of T: one per kx column and plane, for the shortest columns (pz = 6) that fill the scratch
+static __device__ int g_noalloc_exp[kNoAllocScratchBytes / sizeof(cd) / 6];
+int* g_noalloc_exp_ptr[kNoAllocMaxDevices] = {};
 
-// twiddle table tw[m] = (cos 2 pi m / n, sin 2 pi m / n) computed on the device
-__global__ void k_twiddles(double2* tw, int n) {
+// twiddle table tw[m] = limbs of (cos 2 pi m / n, sin 2 pi m / n) computed on the device
+__global__ void k_twiddles(int4* tw, int n) {
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n; m += gridDim.x * blockDim.x) {
     double s, c;
     sincospi(2.0 * (double)m / (double)n, &s, &c);
-    tw[m] = make_double2(c, s);
+    int4 w;
+    fx_limbs(c, w.x, w.y);
+    fx_limbs(s, w.z, w.w);
+    tw[m] = w;
   }
 }
 
 // Once per device, with that device current: the device address of the scratch array (in host code
 // the array's name is only a stand-in) and the shared-memory limits of the two kernels.
-int noalloc_setup(int dev, void** ptr) {
+int noalloc_setup(int dev, void** ptr, int** te) {
   std::lock_guard<std::mutex> lock(g_noalloc_mu);
   if (g_noalloc_ptr[dev]) {
     *ptr = g_noalloc_ptr[dev];
+    *te = g_noalloc_exp_ptr[dev];
     return LMVD_OK;
   }
   void* p = nullptr;
   if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return LMVD_ERR_CUDA;
-  if (set_smem<cd>())
+  if (set_smem())
     return LMVD_ERR_CUDA;
+  void* e = nullptr;
+  if (cudaGetSymbolAddress(&e, g_noalloc_exp) != cudaSuccess || !e) return LMVD_ERR_CUDA;
+  *te = g_noalloc_exp_ptr[dev] = (int*)e;
   g_noalloc_ptr[dev] = p;
   *ptr = p;
   return LMVD_OK;
@@ -1067,25 +1105,26 @@ extern "C" int lmvd_inverse_transform_noalloc(int nx, int ny, int nz, const void
   for (FFTPlan* p : {&fx, &fz})
     if (smem_bytes(*p) > kFftSmemMax) return LMVD_ERR_UNSUPPORTED;
   // scratch layout: x twiddles | z twiddles | one field's intermediate T[ny][pz][nx/2]
-  const size_t off_tz = align256(sizeof(double2) * g.px);
-  const size_t off_tb = off_tz + align256(sizeof(double2) * g.pz);
-  const size_t tbytes = sizeof(cd) * (size_t)ny * g.pz * (nx / 2);
+  const size_t off_tz = align256(sizeof(int4) * g.px);
+  const size_t off_tb = off_tz + align256(sizeof(int4) * g.pz);
+  const size_t tbytes = sizeof(cfx) * (size_t)ny * g.pz * (nx / 2);
   if (off_tb + tbytes > kNoAllocScratchBytes) return LMVD_ERR_INVALID_ARG;  // grid too large for the scratch
   // a launch error left pending on this host thread by earlier work is not this call's to report
   (void)cudaGetLastError();
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kNoAllocMaxDevices) return LMVD_ERR_CUDA;
   void* base = nullptr;
-  int err = noalloc_setup(dev, &base);
+  int* te = nullptr;
+  int err = noalloc_setup(dev, &base, &te);
   if (err) return err;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char* sb = (char*)base;
-  fx.tw = (double2*)sb;
-  fz.tw = (double2*)(sb + off_tz);
-  cd* T = (cd*)(sb + off_tb);
-  k_twiddles<<<(g.px + 255) / 256, 256, 0, st>>>(fx.tw, g.px);
+  fx.tw = (const int4*)sb;
+  fz.tw = (const int4*)(sb + off_tz);
+  cfx* T = (cfx*)(sb + off_tb);
+  k_twiddles<<<(g.px + 255) / 256, 256, 0, st>>>((int4*)sb, g.px);
   if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
-  k_twiddles<<<(g.pz + 255) / 256, 256, 0, st>>>(fz.tw, g.pz);
+  k_twiddles<<<(g.pz + 255) / 256, 256, 0, st>>>((int4*)(sb + off_tz), g.pz);
   if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
   const size_t S = (size_t)ny * g.M, P = (size_t)ny * g.P;
   for (int f = 0; f < nfields; ++f) {
@@ -1096,13 +1135,13 @@ extern "C" int lmvd_inverse_transform_noalloc(int nx, int ny, int nz, const void
     ZMaps maps;
     if (!tile_map(&maps.m[0], fi.p[0], g.nxh, nz, ny, fz.batch, fz.rows_in)) return LMVD_ERR_CUDA;
     dim3 gz(cdiv(nx / 2, fz.batch), ny, 1);
-    if (fz.ept == 12 && fz.batch == 4) k_fft_z_inv<cd, 12, 4><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, nullptr);
-    else if (fz.ept == 12) k_fft_z_inv<cd, 12, 2><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, nullptr);
-    else k_fft_z_inv<cd, 6, 4><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, nullptr);
+    if (fz.ept == 12 && fz.batch == 4) k_fft_z_inv<cd, 12, 4><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, te, nullptr);
+    else if (fz.ept == 12) k_fft_z_inv<cd, 12, 2><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, te, nullptr);
+    else k_fft_z_inv<cd, 6, 4><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, te, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
     dim3 gx(cdiv(cdiv(g.pz, 2), fx.batch), ny, 1);
-    if (fx.ept == 12) k_fft_x_inv<cd, 12><<<gx, threads(fx), smem_bytes(fx), st>>>(fx, g, T, 0, fo, nullptr);
-    else k_fft_x_inv<cd, 6><<<gx, threads(fx), smem_bytes(fx), st>>>(fx, g, T, 0, fo, nullptr);
+    if (fx.ept == 12) k_fft_x_inv<12><<<gx, threads(fx), smem_bytes(fx), st>>>(fx, g, T, 0, te, fo, nullptr);
+    else k_fft_x_inv<6><<<gx, threads(fx), smem_bytes(fx), st>>>(fx, g, T, 0, te, fo, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
   }
   return LMVD_OK;

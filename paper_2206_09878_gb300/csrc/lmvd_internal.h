@@ -164,14 +164,15 @@ __device__ inline cd band_row(const DBand& B, int i, const cd* x, size_t M, int 
   return acc;
 }
 
+struct cfx;  // a complex value in block fixed point, 16 bytes (fx.cuh)
+
 // ---------------------------------------------------------------- FFT plan
 struct FFTPlan {
   int n = 0;
   int nst = 0;
-  int radix[24];
-  unsigned code = 0;       // the radix sequence, 2 bits per stage (0: 4, 1: 2, 2: 3), first stage lowest
-  double2* tw = nullptr;   // tw[m] = (cos 2 pi m / n, sin 2 pi m / n), device
-  float4* twf = nullptr;   // the same as double-float pairs (cos.hi, cos.lo, sin.hi, sin.lo), device
+  unsigned code = 0;       // the radices before the last (ept), 2 bits per stage (0: 4, 1: 2, 2: 3), first lowest
+  bool first4 = false;     // the first stage is a radix-4 one (4 divides tpt)
+  const int4* tw = nullptr;  // tw[m] = limbs of (cos 2 pi m / n, sin 2 pi m / n), device (fx.cuh)
   int batch = 1;           // transforms per CTA
   int ept = 12;            // elements per thread (a multiple of every radix of the plan)
   int tpt = 1;             // threads per transform = n / ept; a CTA has tpt * batch threads
@@ -179,9 +180,9 @@ struct FFTPlan {
                            // interleave their batch columns, pad 0)
   int rows_in = 0;         // z-passes: rows per tile copy of the spectral input (divides nz / 2) ...
   int rows_t = 0;          // ... and of the intermediate T (divides pz); 0 for the x-passes
+  int red_g = 1;           // threads of a transform whose partial sums one warp adds (fx_scale)
   double scale_d = 1.0;    // 1 / (2 px pz) for the forward z-pass (with the x-pass's 1/2)
-  df scale_f{1.f, 0.f};
-  df s3f{0.f, 0.f};        // sin(2 pi / 3) as a double-float
+  int2 s3{0, 0};           // sin(2 pi / 3) as limbs
 };
 
 // ---------------------------------------------------------------- tracing
@@ -259,7 +260,8 @@ struct Ctx {
   double* r_m;        // 2 * ny
   cd* sv[10];         // spectral value fields at g (FFT outputs / inputs)
   cd* st[7];          // RHS streams: the same memory as sv[0..6] (formed in place from sv)
-  cd* tbuf;           // FFT intermediate: tbuf_n fields of ny * pz * (nx/2)
+  cfx* tbuf;          // FFT intermediate (fixed point): tbuf_n fields of ny * pz * (nx/2)
+  int* texp;          // its exponents: tbuf_n fields of ny * max(nx, pz) / 2
   // physical
   double *md[3], *rho, *invrho, *fprime, *w[3];
   double* pw[PW_FIELDS];  // physical work fields (pw_n of them allocated)
@@ -329,14 +331,13 @@ int fft_prepare(Ctx& c);                       // plans, twiddles, smem attribut
 // inverse: nf spectral value fields (in[f]) -> physical (out[f]); in the precision path (precision 1) the
 // inputs are the double-float pairs the evaluation kernels store
 void fft_inverse(Ctx& c, cd* const* in, double* const* out, int nf);
+// the same from complex doubles in every precision
+void fft_inverse_d(Ctx& c, cd* const* in, double* const* out, int nf);
 // forward: nf physical fields -> spectral value fields, truncated and scaled
 void fft_forward(Ctx& c, double* const* in, cd* const* out, int nf);
-// the same with an explicit arithmetic (0: complex double, 1: double-float), nf <= 64
-void fft_inverse_as(Ctx& c, cd* const* in, double* const* out, int nf, int precision);
-void fft_forward_as(Ctx& c, double* const* in, cd* const* out, int nf, int precision);
 // the fixed point's products formed inside the x-passes (Sec. 4.3): inverse transform of one field whose
 // x-pass stores w * phys (rho_t = f'(z) dz/dt), and forward transform of -(w1 m1 + w2 m2 + w3 m3) formed
-// in the x-pass prologue (the tail of L); w, m: physical fields in the arithmetic of the precision
+// in the x-pass prologue (the tail of L); w, m: physical fields
 void fft_inverse_mul(Ctx& c, cd* in, double* out, const double* w);  // input as for fft_inverse
 void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, cd* out);
 

@@ -669,23 +669,18 @@ __global__ void k_mass_norms(Grid g, const double* dstar, const cd* rt, const cd
 // Kinetic energy (1/2) integral of |m|^2 / rho over the domain and max |m|^2 over the grid, m = m^d + m^c on the
 // padded grid. A plane's mean of a product on the 3/2 grid is the k = 0 coefficient of the dealiased product;
 // the y-integral uses the quadrature weights of the Greville interpolant (wq), and the x-z area lx lz is
-// applied on the host. df_fields: the physical fields hold double-float pairs (precision 1).
-__device__ __forceinline__ double phys_value(const double* p, size_t o, int df_fields) {
-  if (!df_fields) return p[o];
-  const float2 v = reinterpret_cast<const float2*>(p)[o];
-  return (double)v.x + (double)v.y;
-}
-__global__ void k_energy_norms(Grid g, const double* wq, Fields3C md, Fields3C mc, const double* invrho, int df_fields,
-                               double* ke, unsigned long long* m2max) {
+// applied on the host.
+__global__ void k_energy_norms(Grid g, const double* wq, Fields3C md, Fields3C mc, const double* invrho, double* ke,
+                               unsigned long long* m2max) {
   const size_t n = (size_t)g.ny * g.P;
   double e = 0.0, mx = 0.0;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     double mm = 0.0;
     for (int c = 0; c < 3; ++c) {
-      const double m = phys_value(md.p[c], o, df_fields) + phys_value(mc.p[c], o, df_fields);
+      const double m = md.p[c][o] + mc.p[c][o];
       mm = fma(m, m, mm);
     }
-    e = fma(0.5 * __ldg(wq + o / g.P) * mm, phys_value(invrho, o, df_fields), e);
+    e = fma(0.5 * __ldg(wq + o / g.P) * mm, invrho[o], e);
     mx = fmax(mx, mm);
   }
   block_add(e / (double)g.P, ke);
