@@ -83,7 +83,7 @@ __global__ void k_wscale(Grid g, FieldsW10 f, double s0, double s1) {
 
 // out = A^{-T} in for job blockIdx.y, shared or per-mode factors; rows of the result outside [zlo, zhi]
 // are zero (boundary rows whose forward right-hand side is a constant). out may alias in. Nyquist modes
-// are set to zero. k_solve_T_cd: one thread per mode; k_solve_T_re: one thread per (mode, real part).
+// are set to zero. k_solve_T_cd: one thread per mode; k_solve_T_piped: one thread per (mode, real part).
 struct SolveTJob {
   const cd* in;
   cd* out;
@@ -92,23 +92,30 @@ struct SolveTJob {
 struct SolveTJobs {
   SolveTJob j[8];
 };
-template <class V>
-__device__ void solve_T_job(const Grid& g, const DLU& lu, const SolveTJob& jb) {
-  constexpr int TPM = sizeof(V) == sizeof(cd) ? 1 : 2;
-  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (t >= TPM * g.M) return;
-  const int m = (int)(t / TPM), comp = (int)(t % TPM);
-  const size_t M = g.M;
-  V* out = reinterpret_cast<V*>(jb.out);
-  if (is_nyquist(g, m)) {
-    for (int i = 0; i < lu.n; ++i) out[vidx<V>(i, M, m, comp)] = vzero<V>();
+__global__ void k_solve_T_cd(Grid g, DLU lu, SolveTJobs jobs) {
+  const size_t m = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (m >= g.M) return;
+  const SolveTJob& jb = jobs.j[blockIdx.y];
+  if (is_nyquist(g, (int)m)) {
+    for (int i = 0; i < lu.n; ++i) jb.out[(size_t)i * g.M + m] = mk(0, 0);
     return;
   }
-  band_solve_T_v<V>(lu, m, lu.mstride ? factor_mode(g, m) : 0, comp, reinterpret_cast<const V*>(jb.in), out, M,
-                    jb.zlo, jb.zhi);
+  band_solve_T_v<cd>(lu, (int)m, lu.mstride ? factor_mode(g, (int)m) : 0, 0, jb.in, jb.out, g.M, jb.zlo, jb.zhi);
 }
-__global__ void k_solve_T_cd(Grid g, DLU lu, SolveTJobs jobs) { solve_T_job<cd>(g, lu, jobs.j[blockIdx.y]); }
-__global__ void k_solve_T_re(Grid g, DLU lu, SolveTJobs jobs) { solve_T_job<double>(g, lu, jobs.j[blockIdx.y]); }
+__global__ void __launch_bounds__(128) k_solve_T_piped(Grid g, DLU lu, const __grid_constant__ SolveTJobs jobs) {
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (t >= 2 * g.M) return;
+  const int m = (int)(t >> 1);
+  const SolveTJob& jb = jobs.j[blockIdx.y];
+  const long long rs = 2ll * g.M;
+  double* out = reinterpret_cast<double*>(jb.out) + t;
+  if (is_nyquist(g, m)) {
+    for (int i = 0; i < lu.n; ++i) out[i * rs] = 0.0;
+    return;
+  }
+  band_solve_T_piped(lu, lu.mstride ? factor_mode(g, m) : 0, reinterpret_cast<const double*>(jb.in) + t, out, rs, jb.zlo,
+                     jb.zhi);
+}
 
 // ------------------------------------------------------------------ update (step 6) adjoint
 struct AdjUpd {
@@ -640,7 +647,7 @@ void solve_T_jobs(Ctx& c, KClass cls, const DLU& lu, std::initializer_list<Solve
   const int tpm = solve_split(c.g);
   const dim3 grid((unsigned)((tpm * c.g.M + TPB - 1) / TPB), n);
   if (tpm == 2)
-    LMVD_LAUNCH(c, cls, n * lu.flops_per_mode * c.g.M, 32.0 * rowsM * n, k_solve_T_re, grid, TPB, 0, c.g, lu, sj);
+    LMVD_LAUNCH(c, cls, n * lu.flops_per_mode * c.g.M, 32.0 * rowsM * n, k_solve_T_piped, grid, TPB, 0, c.g, lu, sj);
   else
     LMVD_LAUNCH(c, cls, n * lu.flops_per_mode * c.g.M, 32.0 * rowsM * n, k_solve_T_cd, grid, TPB, 0, c.g, lu, sj);
 }

@@ -140,6 +140,15 @@ int half_width(const RowBand& m) {
   return K;
 }
 
+// the rows around the middle one with the same number of factors
+BandInterior band_interior(const std::vector<int>& cnt) {
+  const int n = (int)cnt.size();
+  BandInterior b{cnt[n / 2], n / 2, n / 2 + 1};
+  while (b.r0 > 0 && cnt[b.r0 - 1] == b.n) --b.r0;
+  while (b.r1 < n && cnt[b.r1] == b.n) ++b.r1;
+  return b;
+}
+
 int upload_lu(Ctx& c, const BandLU& f, DLU& d) {
   double *lo, *up, *invd;
   int *nl, *nu;
@@ -149,7 +158,7 @@ int upload_lu(Ctx& c, const BandLU& f, DLU& d) {
   if (!e) e = upload(c, f.nl, &nl);
   if (!e) e = upload(c, f.nu, &nu);
   if (e) return e;
-  d = DLU{lo, up, invd, nl, nu, f.n, f.K, 0, 0.0};
+  d = DLU{lo, up, invd, nl, nu, f.n, f.K, 0, band_interior(f.nl), band_interior(f.nu), 0.0};
   for (int i = 0; i < f.n; ++i) d.flops_per_mode += 4.0 * (f.nl[i] + f.nu[i]) + 2.0;
   return LMVD_OK;
 }
@@ -253,7 +262,7 @@ int factor_per_mode(Ctx& c, const PerMode& pm, int K, DLU& out) {
   if (e) return e;
   LMVD_LAUNCH(c, KC_MISC, 0, 8.0 * n * (2 * K + 1) * Mh, k_factor, (unsigned)((Mh + TPB_MODE - 1) / TPB_MODE),
               TPB_MODE, 0, c.g, n, K, A2, A0, A1, dnl, dnu, lo, up, invd);
-  out = DLU{lo, up, invd, dnl, dnu, n, K, Mh, 0.0};
+  out = DLU{lo, up, invd, dnl, dnu, n, K, Mh, band_interior(nl), band_interior(nu), 0.0};
   for (int i = 0; i < n; ++i) out.flops_per_mode += 4.0 * (nl[i] + nu[i]) + 2.0;
   return cuda_check(c);
 }
@@ -339,26 +348,49 @@ void eval_jobs(Ctx& c, std::initializer_list<EvalJob> jobs) {
 
 // out = A^{-1} in (+ add) for each job; shared or per-mode factors; one or two threads per mode
 // (solve_split)
-void solve_modes(Ctx& c, KClass cls, std::initializer_list<SolveJob> jobs, const DLU& lu) {
-  SolveJobs sj{};
-  int n = 0;
-  double arrays = 0;
-  for (const SolveJob& j : jobs) {
-    sj.j[n++] = j;
-    arrays += j.add ? 3 : 2;
-  }
-  const double rowsM = (double)lu.n * c.g.M;
-  const double factors = lu.mstride ? 8.0 * (2 * lu.K + 1) * rowsM * n : 0.0;
-  const int tpm = solve_split(c.g);
-  const unsigned blocks = (unsigned)((tpm * c.g.M + TPB_MODE - 1) / TPB_MODE);
-  if (tpm == 2)
-    LMVD_LAUNCH(c, cls, n * lu.flops_per_mode * c.g.M, 16.0 * arrays * rowsM + factors, k_solve_re, dim3(blocks, n),
-                TPB_MODE, 0, c.g, lu, sj);
-  else
-    LMVD_LAUNCH(c, cls, n * lu.flops_per_mode * c.g.M, 16.0 * arrays * rowsM + factors, k_solve_cd, dim3(blocks, n),
-                TPB_MODE, 0, c.g, lu, sj);
+struct SolveReq {
+  SolveJob job;
+  const DLU* lu;
+};
+PipedJob piped(const Ctx& c, const SolveReq& r) {
+  return PipedJob{reinterpret_cast<const double*>(r.job.in), reinterpret_cast<const double*>(r.job.add),
+                  reinterpret_cast<double*>(r.job.out), 0, (int)c.g.M, *r.lu};
 }
-void solve_interp(Ctx& c, std::initializer_list<SolveJob> jobs, const DLU& lu) { solve_modes(c, KC_SOLVE, jobs, lu); }
+// means: also the plane means in place in (mm1_new, mm3_new) with lu_means
+void solve_modes(Ctx& c, KClass cls, std::initializer_list<SolveReq> reqs, bool means = false) {
+  double fl = 0, by = 0;
+  for (const SolveReq& r : reqs) {
+    const double rowsM = (double)r.lu->n * c.g.M;
+    fl += r.lu->flops_per_mode * c.g.M;
+    by += 16.0 * (r.job.add ? 3 : 2) * rowsM + (r.lu->mstride ? 8.0 * (2 * r.lu->K + 1) * rowsM : 0.0);
+  }
+  const bool split = solve_split(c.g) == 2;
+  PipedJobs pj{};
+  int n = 0;
+  if (split)
+    for (const SolveReq& r : reqs) pj.j[n++] = piped(c, r);
+  if (means) pj.j[n++] = PipedJob{c.mm1_new, nullptr, c.mm1_new, c.mm3_new - c.mm1_new, 0, c.lu_means};
+  if (n)
+    LMVD_LAUNCH(c, cls, split ? fl : 0.0, split ? by : 0.0, k_solve_piped,
+                dim3(split ? (unsigned)((2 * c.g.M + TPB_MODE - 1) / TPB_MODE) : 1u, n), TPB_MODE, 0, c.g, pj);
+  if (split) return;
+  // one launch per run of jobs with the same factors
+  for (const SolveReq* r = reqs.begin(); r != reqs.end();) {
+    SolveJobs sj{};
+    int k = 0;
+    const SolveReq* q = r;
+    double f1 = 0, b1 = 0;
+    for (; q != reqs.end() && q->lu == r->lu; ++q) {
+      sj.j[k++] = q->job;
+      const double rowsM = (double)q->lu->n * c.g.M;
+      f1 += q->lu->flops_per_mode * c.g.M;
+      b1 += 16.0 * (q->job.add ? 3 : 2) * rowsM + (q->lu->mstride ? 8.0 * (2 * q->lu->K + 1) * rowsM : 0.0);
+    }
+    LMVD_LAUNCH(c, cls, f1, b1, k_solve_cd, dim3(mode_blocks(c.g), k), TPB_MODE, 0, c.g, *r->lu, sj);
+    r = q;
+  }
+}
+void solve_interp(Ctx& c, SolveJob job) { solve_modes(c, KC_SOLVE, {SolveReq{job, &c.lu_interp}}); }
 
 // steps 1-2: m^d and z-derived fields in physical space; rho, 1/rho, f', grad z / rho; R_z.
 // zp: where z, dz/dx, dz/dz, dz/dy, lap z land on the physical grid (work fields by default; the adjoint
@@ -391,7 +423,7 @@ void physical_pass_1(Ctx& c, double* const* zp = nullptr) {
   double* fin[1] = {c.pw[5]};
   cd* fout[1] = {c.sv[0]};
   fft_forward(c, fin, fout, 1);
-  solve_interp(c, {SolveJob{c.sv[0], nullptr, c.Rz}}, c.lu_interp);
+  solve_interp(c, SolveJob{c.sv[0], nullptr, c.Rz});
 }
 
 // rho_t = P[f'(z) zdot] and m^c = C(rho_t) (B coefficients), then m^c on the physical grid.
@@ -420,12 +452,12 @@ void mc_from_zdot(Ctx& c, double* a = nullptr, double* const* b = nullptr) {
     cd* out[1] = {c.sv[1]};
     fft_forward(c, in, out, 1);
   }
-  solve_interp(c, {SolveJob{c.sv[1], nullptr, c.rt}}, c.lu_interp);
+  solve_interp(c, SolveJob{c.sv[1], nullptr, c.rt});
   {
     const double rowsM = (double)(c.g.ny + 1) * c.g.M;
     LMVD_LAUNCH(c, KC_MC_SOLVE, rowsM * 4.0 * c.Bs[1].w, rowsM * 16.0 * 2, k_mc_rhs,
                 dim3(mode_blocks(c.g), row_chunks(c.g, c.g.ny + 1)), TPB_MODE, 0, c.g, c.Bs[1], c.rt, c.m2c);
-    solve_modes(c, KC_MC_SOLVE, {SolveJob{c.m2c, nullptr, c.m2c}}, c.lu_mc);
+    solve_modes(c, KC_MC_SOLVE, {SolveReq{SolveJob{c.m2c, nullptr, c.m2c}, &c.lu_mc}});
     LMVD_LAUNCH(c, KC_MC_SOLVE, rowsM * 20.0, rowsM * 16.0 * 5, k_mc_post,
                 dim3(mode_blocks(c.g), row_chunks(c.g, c.g.ny)), TPB_MODE, 0, c.g, c.dstar, c.rt, c.m1c, c.m2c,
                 c.m3c);
@@ -445,7 +477,7 @@ void fp_apply(Ctx& c, double* a = nullptr, double* const* b = nullptr) {
   const double* w[3] = {c.w[0], c.w[1], c.w[2]};
   const double* m[3] = {bb[0], bb[1], bb[2]};
   fft_forward_dot3(c, w, m, c.sv[3]);
-  solve_interp(c, {SolveJob{c.sv[3], c.Rz, c.zdot}}, c.lu_interp);
+  solve_interp(c, SolveJob{c.sv[3], c.Rz, c.zdot});
 }
 
 // Reading R6: n_startup fixed-point applications from dz/dt = 0, then the Taylor back-fill of the history.
@@ -549,11 +581,10 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
   for (int f = 0; f < 7; ++f) stw.p[f] = c.st[f];
   LMVD_LAUNCH(c, KC_RHS_COMBINE, 90.0 * S, 16.0 * 17 * S, k_rhs_combine, elem_blocks(S), 256, 0, g, 1.0 / cf.re,
               1.0 / (cf.fr * cf.fr), svc, stw);
-  solve_interp(c,
-               {SolveJob{c.st[1], nullptr, c.st[1]}, SolveJob{c.st[2], nullptr, c.st[2]},
-                SolveJob{c.st[3], nullptr, c.st[3]}, SolveJob{c.st[4], nullptr, c.st[4]},
-                SolveJob{c.st[5], nullptr, c.st[5]}, SolveJob{c.st[6], nullptr, c.st[6]}},
-               c.lu_interp);
+  const DLU* li = &c.lu_interp;
+  solve_modes(c, KC_SOLVE, {SolveReq{SolveJob{c.st[1], nullptr, c.st[1]}, li}, SolveReq{SolveJob{c.st[2], nullptr, c.st[2]}, li},
+                            SolveReq{SolveJob{c.st[3], nullptr, c.st[3]}, li}, SolveReq{SolveJob{c.st[4], nullptr, c.st[4]}, li},
+                            SolveReq{SolveJob{c.st[5], nullptr, c.st[5]}, li}, SolveReq{SolveJob{c.st[6], nullptr, c.st[6]}, li}});
   Fields7C stc{};
   for (int f = 0; f < 7; ++f) stc.p[f] = c.st[f];
   if (cf.precision == 1) {
@@ -577,17 +608,15 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
   u.m2 = c.m2; u.r_phi = c.r_phi; u.r_phi_prev = c.r_phi_prev;
   u.mm1 = c.mm1; u.mm3 = c.mm3; u.r_m = c.r_m; u.r_m_prev = c.r_m_prev;
   u.om_new = c.om_new; u.z_new = c.z_new; u.m2_new = c.m2_new; u.mm1_new = c.mm1_new; u.mm3_new = c.mm3_new;
-  LMVD_LAUNCH(c, KC_UPDATE, S * (12.0 * c.B0g.w + 20.0), 16.0 * 7 * S, k_update_om_z_rhs,
-              dim3(mode_blocks(g), row_chunks(g, g.ny), 2), TPB_MODE, 0, g, c.B0g, u);
-  solve_modes(c, KC_UPDATE, {SolveJob{c.om_new, nullptr, c.om_new}}, c.lu_interp);
-  solve_modes(c, KC_UPDATE, {SolveJob{c.z_new, nullptr, c.z_new}}, c.lu_neumann);
-  LMVD_LAUNCH(c, KC_UPDATE, 0, 0, k_update_means, 1, 32, 0, g, c.B0g, c.lu_means, u);
-  {
-    const double Sp = (double)(g.ny + 1) * g.M;
-    LMVD_LAUNCH(c, KC_UPDATE, Sp * (8.0 * c.Ss0.w + 10.0), 16.0 * 4 * Sp, k_update_m2_rhs,
-                dim3(mode_blocks(g), row_chunks(g, g.ny + 1)), TPB_MODE, 0, g, c.Ss0, c.Ss2, u);
-    solve_modes(c, KC_UPDATE, {SolveJob{c.m2_new, nullptr, c.m2_new}}, c.lu_md);
-  }
+  const double Sp = (double)(g.ny + 1) * g.M;
+  LMVD_LAUNCH(c, KC_UPDATE, S * (12.0 * c.B0g.w + 20.0) + Sp * (8.0 * c.Ss0.w + 10.0), 16.0 * 7 * S + 16.0 * 4 * Sp,
+              k_update_rhs, dim3(std::max(mode_blocks(g), (unsigned)(2 * g.ny + TPB_MODE - 1) / TPB_MODE),
+                                 row_chunks(g, g.ny + 1), 4),
+              TPB_MODE, 0, g, c.B0g, c.Ss0, c.Ss2, u);
+  solve_modes(c, KC_UPDATE, {SolveReq{SolveJob{c.om_new, nullptr, c.om_new}, &c.lu_interp},
+                             SolveReq{SolveJob{c.z_new, nullptr, c.z_new}, &c.lu_neumann},
+                             SolveReq{SolveJob{c.m2_new, nullptr, c.m2_new}, &c.lu_md}},
+              true);
   // failure detection: any non-finite value in the new state sets the device status word
   {
     CheckJobs cj{};

@@ -107,10 +107,14 @@ RowBand collocation(const Knots& k, const std::vector<double>& pts, int deriv) {
     // keep the window inside [0, n)
     int c0 = std::max(0, std::min(first, k.n - m.w));
     m.c0[i] = c0;
+    // a basis function whose support ends at the point has value zero there; rounding of the point leaves ~1e-45,
+    // which would widen the row's band
+    double top = 0.0;
+    for (double v : vals) top = std::max(top, std::fabs(v));
     for (int r = 0; r < k.order; ++r) {
       int j = first + r;
       if (j < 0 || j >= k.n) continue;
-      m.v[(size_t)i * m.w + (j - c0)] = vals[r];
+      m.v[(size_t)i * m.w + (j - c0)] = std::fabs(vals[r]) < 1e-30 * top ? 0.0 : vals[r];
     }
   }
   return m;

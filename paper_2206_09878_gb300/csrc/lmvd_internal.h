@@ -86,6 +86,9 @@ struct DBand {
 // mstride = 0, element (i, q) at [i * K + q]; per-mode factors: element (i, q) of factor mode mf at
 // [(i * K + q) * mstride + mf], where A(k) depends on kz only through kz^2, so only the modes with
 // kz >= 0 are stored (factor_mode): mstride = (nz/2 + 1) * nxh.
+struct BandInterior {
+  int n, r0, r1;  // rows [r0, r1) all have n factors (around the middle row)
+};
 struct DLU {
   const double* lo;
   const double* up;
@@ -94,6 +97,7 @@ struct DLU {
   const int* nu;
   int n, K;
   size_t mstride;
+  BandInterior lin, uin;  // of L and of U
   double flops_per_mode;  // host-side: flops of one complex solve (sum over rows of 4 (nl + nu) + 2)
 };
 

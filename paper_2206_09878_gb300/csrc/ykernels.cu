@@ -352,24 +352,32 @@ void launch_rhs_eval_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& 
 // ------------------------------------------------------------------ banded solves
 // job blockIdx.y: out = A^{-1} in (+ add), factors shared or per mode (DLU.mstride); used for the
 // collocation (interpolation) solves and the per-mode systems. out may alias in. Nyquist modes are set to
-// zero. k_solve_cd: one thread per mode; k_solve_re: one thread per (mode, real part), see band_solve_v.
-template <class V>
-__device__ void solve_job(const Grid& g, const DLU& lu, const SolveJob& jb) {
-  constexpr int TPM = sizeof(V) == sizeof(cd) ? 1 : 2;
-  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (t >= TPM * g.M) return;
-  const int m = (int)(t / TPM), comp = (int)(t % TPM);
-  const size_t M = g.M;
-  V* out = reinterpret_cast<V*>(jb.out);
-  if (is_nyquist(g, m)) {
-    for (int i = 0; i < lu.n; ++i) out[vidx<V>(i, M, m, comp)] = vzero<V>();
+// zero. k_solve_cd: one thread per mode (band_solve_v).
+__global__ void k_solve_cd(Grid g, DLU lu, SolveJobs jobs) {
+  const size_t m = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (m >= g.M) return;
+  const SolveJob& jb = jobs.j[blockIdx.y];
+  if (is_nyquist(g, (int)m)) {
+    for (int i = 0; i < lu.n; ++i) jb.out[(size_t)i * g.M + m] = mk(0, 0);
     return;
   }
-  band_solve_v<V>(lu, m, lu.mstride ? factor_mode(g, m) : 0, comp, reinterpret_cast<const V*>(jb.in),
-                  reinterpret_cast<const V*>(jb.add), out, M);
+  band_solve_v<cd>(lu, (int)m, lu.mstride ? factor_mode(g, (int)m) : 0, 0, jb.in, jb.add, jb.out, g.M);
 }
-__global__ void k_solve_cd(Grid g, DLU lu, SolveJobs jobs) { solve_job<cd>(g, lu, jobs.j[blockIdx.y]); }
-__global__ void k_solve_re(Grid g, DLU lu, SolveJobs jobs) { solve_job<double>(g, lu, jobs.j[blockIdx.y]); }
+// One thread per (mode, real part), loads pipelined (band_solve_piped); a job may have its own factors, and a job of
+// real columns (modes = 0: the plane means) has one thread per column, `part` elements apart.
+__global__ void __launch_bounds__(128) k_solve_piped(Grid g, const __grid_constant__ PipedJobs jobs) {
+  const PipedJob& jb = jobs.j[blockIdx.y];
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  const int m = (int)(t >> 1), comp = (int)(t & 1);
+  if (m >= (jb.modes ? jb.modes : 1)) return;
+  const long long o = jb.modes ? (long long)t : comp * jb.part, rs = jb.modes ? 2ll * jb.modes : 1;
+  const DLU lu = jb.lu;
+  if (jb.modes && is_nyquist(g, m)) {
+    for (int i = 0; i < lu.n; ++i) jb.out[o + i * rs] = 0.0;
+    return;
+  }
+  band_solve_piped(lu, lu.mstride ? factor_mode(g, m) : 0, jb.in + o, jb.add ? jb.add + o : nullptr, jb.out + o, rs);
+}
 
 // ------------------------------------------------------------------ m^c from rho_t
 // Eq. COM_fourier + CF_fourier with m_par eliminated: rows 1..ny-1 collocate
@@ -516,17 +524,44 @@ __global__ void k_rhs_eval(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, D
 // Dirichlet rows (interpolation LU); z (blockIdx.z = 1): values at g advanced with (dz/dt)^{k_f},
 // Neumann rows dz/dy(+-1) = 0 (Neumann LU). This kernel writes the right-hand sides; rows split over
 // gridDim.y chunks.
-__global__ void k_update_om_z_rhs(Grid g, DBand B0g, UpdateArgs a) {
+// m2^d (Eq. phi_poisson, blockIdx.z = 2): phi2 = (B*'' - k^2 B*) m2^d at g*_2 .. g*_{ny-2} advanced with RHS_phi2, four
+// boundary rows (no-slip or potential matching) with zero right-hand side; k = 0: m2^d = 0. Plane means <m1>, <m3>
+// (blockIdx.z = 3, one thread per row and component): values at g advanced, boundary rows zero.
+__global__ void k_update_rhs(Grid g, DBand B0g, DBand Ss0, DBand Ss2, UpdateArgs a) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= (int)g.M) return;
-  const size_t M = g.M;
   const int ny = g.ny;
   const int job = blockIdx.z;
-  cd* out = job == 0 ? a.om_new : a.z_new;
-  int r0, r1;
-  row_range(ny, blockIdx.y, gridDim.y, r0, r1);
-  const bool zero = is_nyquist(g, m) || (job == 0 && m == 0);
   const double dt = a.dt, al = a.al, be = a.be;
+  if (job == 3) {
+    if (blockIdx.y != 0 || m >= 2 * ny) return;
+    const int c = m / ny, i = m - c * ny;
+    const double v = i > 0 && i < ny - 1 ? band_row_real(B0g, i, c == 0 ? a.mm1 : a.mm3) +
+                                               dt * (al * a.r_m[m] + be * a.r_m_prev[m])
+                                         : 0.0;
+    (c == 0 ? a.mm1_new : a.mm3_new)[i] = v;
+    return;
+  }
+  if (m >= (int)g.M) return;
+  const size_t M = g.M;
+  cd* out = job == 0 ? a.om_new : (job == 1 ? a.z_new : a.m2_new);
+  int r0, r1;
+  row_range(job == 2 ? ny + 1 : ny, blockIdx.y, gridDim.y, r0, r1);
+  const bool zero = is_nyquist(g, m) || (job != 1 && m == 0);
+  if (job == 2) {
+    double k1 = 0.0, k3 = 0.0;
+    if (!zero) wavenumbers(g, m, k1, k3);
+    const double k2 = k1 * k1 + k3 * k3;
+    for (int i = r0; i < r1; ++i) {
+      cd v = mk(0, 0);
+      if (!zero && i >= 2 && i <= ny - 2) {
+        const size_t o = (size_t)i * M + m;
+        const cd phi = band_row(Ss2, i, a.m2, M, m) - k2 * band_row(Ss0, i, a.m2, M, m);
+        v = phi + dt * (al * a.r_phi[o] + be * a.r_phi_prev[o]);
+      }
+      out[(size_t)i * M + m] = v;
+    }
+    return;
+  }
   for (int i = r0; i < r1; ++i) {
     cd v = mk(0, 0);
     if (!zero && i > 0 && i < ny - 1) {
@@ -542,67 +577,6 @@ __global__ void k_update_om_z_rhs(Grid g, DBand B0g, UpdateArgs a) {
           v = fma_rc(__ldg(w + q), zz, v);
         }
       }
-    }
-    out[(size_t)i * M + m] = v;
-  }
-}
-
-// Plane means <m1>, <m3>: values at g advanced, no-slip Dirichlet rows (one thread per component).
-__global__ void k_update_means(Grid g, DBand B0g, DLU lu_i, UpdateArgs a) {
-  const int c = threadIdx.x;
-  if (c > 1) return;
-  const int ny = g.ny;
-  const double* cur = c == 0 ? a.mm1 : a.mm3;
-  double* out = c == 0 ? a.mm1_new : a.mm3_new;
-  const double* r = a.r_m + c * ny;
-  const double* rp = a.r_m_prev + c * ny;
-  // real solve through the complex routine with a 1-mode stride
-  double win[KMAX];
-  for (int q = 0; q < KMAX; ++q) win[q] = 0.0;
-  for (int i = 0; i < ny; ++i) {
-    double v = 0.0;
-    if (i > 0 && i < ny - 1) v = band_row_real(B0g, i, cur) + a.dt * (a.al * r[i] + a.be * rp[i]);
-    const int nl = lu_i.nl[i];
-    for (int q = 1; q <= nl; ++q) v -= lu_lo(lu_i, i, q, 0) * win[q - 1];
-    for (int q = KMAX - 1; q > 0; --q) win[q] = win[q - 1];
-    win[0] = v;
-    out[i] = v;
-  }
-  for (int q = 0; q < KMAX; ++q) win[q] = 0.0;
-  for (int i = ny - 1; i >= 0; --i) {
-    double v = out[i];
-    const int nu = lu_i.nu[i];
-    for (int q = 1; q <= nu; ++q) v -= lu_up(lu_i, i, q, 0) * win[q - 1];
-    v *= lu_i.invd[i];
-    for (int q = KMAX - 1; q > 0; --q) win[q] = win[q - 1];
-    win[0] = v;
-    out[i] = v;
-  }
-}
-
-// m2^d (Eq. phi_poisson): phi2 = (B*'' - k^2 B*) m2^d at g*_2 .. g*_{ny-2} advanced with RHS_phi2, four
-// boundary rows (no-slip or potential matching) with zero right-hand side; k = 0: m2^d = 0. This kernel
-// writes the right-hand side into m2_new (rows split over gridDim.y chunks); the banded solve with the
-// per-mode factors then runs in place.
-__global__ void k_update_m2_rhs(Grid g, DBand Ss0, DBand Ss2, UpdateArgs a) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= (int)g.M) return;
-  const size_t M = g.M;
-  const int ny = g.ny;
-  int r0, r1;
-  row_range(ny + 1, blockIdx.y, gridDim.y, r0, r1);
-  cd* out = a.m2_new;
-  const bool zero = m == 0 || is_nyquist(g, m);
-  double k1 = 0.0, k3 = 0.0;
-  if (!zero) wavenumbers(g, m, k1, k3);
-  const double k2 = k1 * k1 + k3 * k3;
-  const double dt = a.dt, al = a.al, be = a.be;
-  for (int i = r0; i < r1; ++i) {
-    cd v = mk(0, 0);
-    if (!zero && i >= 2 && i <= ny - 2) {
-      const size_t o = (size_t)i * M + m;
-      const cd phi = band_row(Ss2, i, a.m2, M, m) - k2 * band_row(Ss0, i, a.m2, M, m);
-      v = phi + dt * (al * a.r_phi[o] + be * a.r_phi_prev[o]);
     }
     out[(size_t)i * M + m] = v;
   }

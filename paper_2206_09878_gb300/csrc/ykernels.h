@@ -33,6 +33,19 @@ struct SolveJob {
 struct SolveJobs {
   SolveJob j[8];
 };
+// a job of k_solve_piped: modes spectral columns (2 modes real ones, interleaved), or, with modes = 0, two real
+// columns `part` elements apart
+struct PipedJob {
+  const double* in;
+  const double* add;  // may be null
+  double* out;
+  long long part;
+  int modes;
+  DLU lu;
+};
+struct PipedJobs {
+  PipedJob j[6];
+};
 struct UpdateArgs {
   double dt, al, be;
   const cd *om, *r_om, *r_om_prev, *z, *zdot, *zdot_prev, *m2, *r_phi, *r_phi_prev;
@@ -72,15 +85,13 @@ void launch_eval_df(int w, dim3 grid, int tpb, cudaStream_t st, const Grid& g, c
 void launch_rhs_eval_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B1g, const DBand& B2g,
                         const DBand* Bs, const Fields7C& stc, cd* r_om, cd* r_phi, double* r_m);
 __global__ void k_solve_cd(Grid g, DLU lu, SolveJobs jobs);
-__global__ void k_solve_re(Grid g, DLU lu, SolveJobs jobs);
+__global__ void k_solve_piped(Grid g, const __grid_constant__ PipedJobs jobs);
 __global__ void k_mc_rhs(Grid g, DBand Bs1, const cd* rt, cd* m2c);
 __global__ void k_mc_post(Grid g, const double* dstar, const cd* rt, cd* m1c, cd* m2c, cd* m3c);
 __global__ void k_rhs_combine(Grid g, double mu, double grav, Fields10C sv, Fields7 st);
 __global__ void k_rhs_eval(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, DBand Bs2, DBand Bs3, Fields7C st,
                            cd* r_om, cd* r_phi, double* r_m);
-__global__ void k_update_om_z_rhs(Grid g, DBand B0g, UpdateArgs a);
-__global__ void k_update_means(Grid g, DBand B0g, DLU lu_i, UpdateArgs a);
-__global__ void k_update_m2_rhs(Grid g, DBand Ss0, DBand Ss2, UpdateArgs a);
+__global__ void k_update_rhs(Grid g, DBand B0g, DBand Ss0, DBand Ss2, UpdateArgs a);
 __global__ void k_bdf(size_t n, double a0, double a1, double a2, double a3, double idt, const cd* z, const cd* h0,
                       const cd* h1, const cd* h2, cd* out);
 __global__ void k_backfill(size_t n, double c0, double c1, double c2, const cd* z, const cd* zdot, cd* h0, cd* h1,
