@@ -235,7 +235,8 @@ PerMode md_system(const RowBand& Ss0, const RowBand& Ss1, const RowBand& Ss2, in
   return p;
 }
 
-int factor_per_mode(Ctx& c, const PerMode& pm, int K, DLU& out) {
+// mean_rows: the k = 0 mode's factors solve x_i - x_{i+1} = r_i, x_{n-1} = r_{n-1} (Eq. mc_mean) instead of x = r
+int factor_per_mode(Ctx& c, const PerMode& pm, int K, bool mean_rows, DLU& out) {
   std::vector<int> nl, nu;
   DiagBand pattern = pm.A0;  // union of the non-zero patterns of A0 and A1 (A2 is the other argument)
   for (size_t i = 0; i < pattern.a.size(); ++i)
@@ -246,6 +247,8 @@ int factor_per_mode(Ctx& c, const PerMode& pm, int K, DLU& out) {
     return LMVD_ERR_UNSUPPORTED;
   }
   const int n = pm.A2.n;
+  if (mean_rows)
+    for (int i = 0; i < n - 1; ++i) nu[i] = std::max(nu[i], 1);
   double *A2, *A0, *A1, *lo, *up, *invd;
   int *dnl, *dnu;
   int e = upload(c, pm.A2.a, &A2);
@@ -261,7 +264,7 @@ int factor_per_mode(Ctx& c, const PerMode& pm, int K, DLU& out) {
     e = device_alloc(c, (void**)&invd, sizeof(double) * (size_t)n * Mh);
   if (e) return e;
   LMVD_LAUNCH(c, KC_MISC, 0, 8.0 * n * (2 * K + 1) * Mh, k_factor, (unsigned)((Mh + TPB_MODE - 1) / TPB_MODE),
-              TPB_MODE, 0, c.g, n, K, A2, A0, A1, dnl, dnu, lo, up, invd);
+              TPB_MODE, 0, c.g, n, K, A2, A0, A1, dnl, dnu, lo, up, invd, mean_rows ? 1 : 0);
   out = DLU{lo, up, invd, dnl, dnu, n, K, Mh, band_interior(nl), band_interior(nu), 0.0};
   for (int i = 0; i < n; ++i) out.flops_per_mode += 4.0 * (nl[i] + nu[i]) + 2.0;
   return cuda_check(c);
@@ -421,29 +424,37 @@ void physical_pass_1(Ctx& c, double* const* zp = nullptr) {
                 zf[1], zf[2], zf[3], zf[4], c.md[0], c.md[1], c.md[2], c.rho, c.invrho, c.fprime, c.w[0],
                 c.w[1], c.w[2], c.pw[5]);
   double* fin[1] = {c.pw[5]};
-  cd* fout[1] = {c.sv[0]};
+  cd* fout[1] = {c.sv[SV_RZ]};
   fft_forward(c, fin, fout, 1);
-  solve_interp(c, SolveJob{c.sv[0], nullptr, c.Rz});
+  solve_interp(c, SolveJob{c.sv[SV_RZ], nullptr, c.Rz});
 }
 
-// rho_t = P[f'(z) zdot] and m^c = C(rho_t) (B coefficients), then m^c on the physical grid.
-// a: where zdot lands on the physical grid; b: where m^c lands (work fields by default).
-void mc_from_zdot(Ctx& c, double* a = nullptr, double* const* b = nullptr) {
+// The fixed point works on values at the Greville points: the tail of L is a forward transform, whose values v plus
+// those of R_z (sv[SV_RZ], kept from pass 1) are the values of the next dz/dt (sv[SV_ZDOT]), and the next application
+// transforms values. Its B-spline coefficients A^{-1} v are only formed where they are asked for, instead of solving
+// with A and evaluating with the same A in every application.
+void zdot_values(Ctx& c) { eval_jobs(c, {EvalJob{c.B0g, c.zdot, c.sv[SV_ZDOT], 0}}); }
+void zdot_coefficients(Ctx& c) { solve_interp(c, SolveJob{c.sv[SV_ZDOT], nullptr, c.zdot}); }
+
+// rho_t = P[f'(z) zdot] and m^c = C(rho_t), then m^c on the physical grid, from the values of zdot (from_eval: they
+// are zdot_values' output, double-float pairs in the precision path). m2^c in B coefficients; m1^c and m3^c too with
+// `coefficients`. a: where zdot lands on the physical grid; b: where m^c lands (work fields by default).
+void mc_from_zdot(Ctx& c, bool from_eval, bool coefficients, double* a = nullptr, double* const* b = nullptr) {
   const size_t n = (size_t)c.g.ny * c.g.P;
   const bool keep_a = a != nullptr;  // the adjoint's tape keeps dz/dt on the grid: separate product pass
-  if (!a) a = c.pw[0];
   double* bb[3] = {c.pw[0], c.pw[1], c.pw[2]};
   if (b)
     for (int f = 0; f < 3; ++f) bb[f] = b[f];
-  eval_jobs(c, {EvalJob{c.B0g, c.zdot, c.sv[0], 0}});
+  const bool df_in = from_eval && c.cfg.precision == 1;
   if (!keep_a) {
     // rho_t = f' dz/dt formed in the epilogue of the inverse x-pass (dz/dt on the grid is not stored)
-    fft_inverse_mul(c, c.sv[0], c.pw[1], c.fprime);
+    fft_inverse_mul(c, c.sv[SV_ZDOT], c.pw[1], c.fprime, df_in);
   } else {
     {
-      cd* in[1] = {c.sv[0]};
+      cd* in[1] = {c.sv[SV_ZDOT]};
       double* out[1] = {a};
-      fft_inverse(c, in, out, 1);
+      if (df_in) fft_inverse(c, in, out, 1);
+      else fft_inverse_d(c, in, out, 1);
     }
     LMVD_LAUNCH(c, KC_PRODUCTS, 1.0 * n, 24.0 * n, k_product_rt, elem_blocks(n), 256, 0, n, c.fprime, a, c.pw[1]);
   }
@@ -456,28 +467,40 @@ void mc_from_zdot(Ctx& c, double* a = nullptr, double* const* b = nullptr) {
   {
     const double rowsM = (double)(c.g.ny + 1) * c.g.M;
     LMVD_LAUNCH(c, KC_MC_SOLVE, rowsM * 4.0 * c.Bs[1].w, rowsM * 16.0 * 2, k_mc_rhs,
-                dim3(mode_blocks(c.g), row_chunks(c.g, c.g.ny + 1)), TPB_MODE, 0, c.g, c.Bs[1], c.rt, c.m2c);
+                dim3(mode_blocks(c.g), row_chunks(c.g, c.g.ny + 1)), TPB_MODE, 0, c.g, c.Bs[1], c.dstar, c.rt, c.m2c);
     solve_modes(c, KC_MC_SOLVE, {SolveReq{SolveJob{c.m2c, nullptr, c.m2c}, &c.lu_mc}});
-    LMVD_LAUNCH(c, KC_MC_SOLVE, rowsM * 20.0, rowsM * 16.0 * 5, k_mc_post,
-                dim3(mode_blocks(c.g), row_chunks(c.g, c.g.ny)), TPB_MODE, 0, c.g, c.dstar, c.rt, c.m1c, c.m2c,
-                c.m3c);
+    if (coefficients)
+      LMVD_LAUNCH(c, KC_MC_SOLVE, rowsM * 20.0, rowsM * 16.0 * 5, k_mc_post,
+                  dim3(mode_blocks(c.g), row_chunks(c.g, c.g.ny)), TPB_MODE, 0, c.g, c.dstar, c.rt, c.m1c, c.m2c,
+                  c.m3c);
   }
-  eval_jobs(c, {EvalJob{c.B0g, c.m1c, c.sv[0], 0}, EvalJob{c.Sg0, c.m2c, c.sv[1], 0}, EvalJob{c.B0g, c.m3c, c.sv[2], 0}});
-  cd* in[3] = {c.sv[0], c.sv[1], c.sv[2]};
+  // values of m^c: m1^c, m3^c = i (k1, k3) / k^2 (rho_t + D* m2^c) need the values of rho_t, which are the forward
+  // transform's, and those of D* m2^c, which is the derivative of m2^c
+  const double SM = (double)c.g.ny * c.g.M, fl = SM * (8.0 * c.Sg0.w + 12.0), by = SM * 16.0 * 5;
+  const dim3 grid(mode_blocks(c.g), row_chunks(c.g, c.g.ny));
+  if (c.cfg.precision == 1)
+    LMVD_LAUNCH_CALL(c, KC_EVAL, fl, by,
+                     launch_mc_values_df(c.cfg.spline_order, grid, TPB_MODE, c.stream, c.g, c.Sg0, c.Sg1, c.sv[1], c.m2c,
+                                         c.sv[0], c.sv[2], c.sv[3]));
+  else
+    LMVD_LAUNCH(c, KC_EVAL, fl, by, k_mc_values, grid, TPB_MODE, 0, c.g, c.Sg0, c.Sg1, c.sv[1], c.m2c, c.sv[0], c.sv[2],
+                c.sv[3]);
+  cd* in[3] = {c.sv[0], c.sv[2], c.sv[3]};
   fft_inverse(c, in, bb, 3);
 }
 
-// one application of the fixed point (Eq. y_k): zdot <- L(z) zdot + R_z
-void fp_apply(Ctx& c, double* a = nullptr, double* const* b = nullptr) {
-  mc_from_zdot(c, a, b);
+// one application of the fixed point (Eq. y_k) on the values of zdot: zdot <- L(z) zdot + R_z; with `coefficients` also
+// its B coefficients
+void fp_apply(Ctx& c, bool from_eval, bool coefficients, double* a = nullptr, double* const* b = nullptr) {
+  mc_from_zdot(c, from_eval, false, a, b);
   double* bb[3] = {c.pw[0], c.pw[1], c.pw[2]};
   if (b)
     for (int f = 0; f < 3; ++f) bb[f] = b[f];
   // the tail -(grad z / rho) . m^c formed in the prologue of the forward x-pass
   const double* w[3] = {c.w[0], c.w[1], c.w[2]};
   const double* m[3] = {bb[0], bb[1], bb[2]};
-  fft_forward_dot3(c, w, m, c.sv[3]);
-  solve_interp(c, SolveJob{c.sv[3], c.Rz, c.zdot});
+  fft_forward_dot3(c, w, m, c.sv[SV_RZ], c.sv[SV_ZDOT]);
+  if (coefficients) zdot_coefficients(c);
 }
 
 // Reading R6: n_startup fixed-point applications from dz/dt = 0, then the Taylor back-fill of the history.
@@ -488,10 +511,11 @@ void startup(Ctx& c, const Tape* tape = nullptr, cd* iterates = nullptr) {
   const size_t S = (size_t)c.g.ny * c.g.M;
   physical_pass_1(c, tape ? tape->zp : nullptr);
   cudaMemsetAsync(c.zdot, 0, sizeof(cd) * S, c.stream);
+  cudaMemsetAsync(c.sv[SV_ZDOT], 0, sizeof(cd) * S, c.stream);
   for (int it = 0; it < c.cfg.n_startup; ++it) {
     if (iterates)
       cudaMemcpyAsync(iterates + (size_t)it * S, c.zdot, sizeof(cd) * S, cudaMemcpyDeviceToDevice, c.stream);
-    fp_apply(c);
+    fp_apply(c, false, iterates || it == c.cfg.n_startup - 1);
   }
   const double dt = c.cfg.dt;
   LMVD_LAUNCH(c, KC_MISC, 12.0 * S, 80.0 * S, k_backfill, elem_blocks(S), 256, 0, S, 0.5 * dt, dt, 1.5 * dt, c.z,
@@ -529,16 +553,17 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
   nvtxRangePop();
   nvtxRangePushA("step 3: fixed point, m^c");
   if (c.diag_on) cudaMemsetAsync(c.ddiag, 0, sizeof(double) * DIAG_N, c.stream);
+  zdot_values(c);
   for (int k = 0; k < cf.kf; ++k) {
     // diagnostics: the change of this application (the previous iterate kept in sv[9], unused until pass 2)
     if (c.diag_on && k < KF_MAX_ADJ + 1)
       cudaMemcpyAsync(c.sv[9], c.zdot, sizeof(cd) * S, cudaMemcpyDeviceToDevice, c.stream);
-    fp_apply(c, tape ? tape->a[k] : nullptr, tape ? tape->b[k] : nullptr);
+    fp_apply(c, k == 0, c.diag_on || k == cf.kf - 1, tape ? tape->a[k] : nullptr, tape ? tape->b[k] : nullptr);
     if (c.diag_on && k < KF_MAX_ADJ + 1)
       LMVD_LAUNCH(c, KC_MISC, 6.0 * S, 32.0 * S, k_diff_norms, elem_blocks(S), 256, 0, S, c.zdot, c.sv[9],
                   c.ddiag + 2 + 2 * k);
   }
-  mc_from_zdot(c, tape ? tape->a[cf.kf] : nullptr, tape ? tape->b[cf.kf] : nullptr);
+  mc_from_zdot(c, cf.kf == 0, true, tape ? tape->a[cf.kf] : nullptr, tape ? tape->b[cf.kf] : nullptr);
   if (c.diag_on) {
     LMVD_LAUNCH(c, KC_MISC, 20.0 * S, 16.0 * 5 * S, k_mass_norms, elem_blocks(S), 256, 0, g, c.dstar, c.rt, c.m1c,
                 c.m2c, c.m3c, c.ddiag);
@@ -753,7 +778,8 @@ int startup_record(Ctx& c, const Tape* tape, cd* iterates) {
 }
 int fp_record(Ctx& c, const cd* zdot_in, double* a, double* const* b) {
   cudaMemcpyAsync(c.zdot, zdot_in, sizeof(cd) * c.g.ny * c.g.M, cudaMemcpyDeviceToDevice, c.stream);
-  fp_apply(c, a, b);
+  zdot_values(c);
+  fp_apply(c, true, true, a, b);
   return cudaGetLastError() == cudaSuccess ? LMVD_OK : LMVD_ERR_CUDA;
 }
 }  // namespace lmvd
@@ -862,8 +888,8 @@ int lmvd_create(const lmvd_config* cfg, void* stream, lmvd_ctx** out) {
     // per-mode LUs of the m^c and m2^d systems
     const int Ks = std::max({half_width(Ss0), half_width(Ss1), half_width(Ss2)});
     if (Ks > KMAX) throw std::runtime_error("band");
-    if (!err) err = factor_per_mode(c, mc_system(Ss0, Ss1, Ss2, Ks, cfg->bc_mode), Ks, c.lu_mc);
-    if (!err) err = factor_per_mode(c, md_system(Ss0, Ss1, Ss2, Ks, cfg->bc_mode), Ks, c.lu_md);
+    if (!err) err = factor_per_mode(c, mc_system(Ss0, Ss1, Ss2, Ks, cfg->bc_mode), Ks, true, c.lu_mc);
+    if (!err) err = factor_per_mode(c, md_system(Ss0, Ss1, Ss2, Ks, cfg->bc_mode), Ks, false, c.lu_md);
     // plane means <m1>, <m3>: Dirichlet rows (walls) or Neumann rows (potential matching)
     c.lu_means = cfg->bc_mode == 1 ? c.lu_neumann : c.lu_interp;
   } catch (const std::exception&) {

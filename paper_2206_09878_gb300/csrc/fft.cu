@@ -678,10 +678,12 @@ __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_fwd_dot3(FFTPlan
 // ---------------------------------------------------------------- forward z-pass (truncate, scale)
 // T: [f][ny][pz][nx/2], read through maps.m[0] (all fields of the launch: planes f ny + j), its exponents te [f][ny]
 // [pz/2]; out: spectral fields [ny][nz][nxh]. Same interleaved layout as the inverse z-pass; kx = nx/2 and the kz
-// Nyquist row are written as zero. The last stage's middle outputs are the truncated kz.
+// Nyquist row are written as zero. The last stage's middle outputs are the truncated kz. add (may be null, one field):
+// a spectral field added to the result.
 template <int EPT, int COLS>
 __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
-    k_fft_z_fwd(FFTPlan pl, Grid g, const __grid_constant__ ZMaps maps, const int* te, FieldsW out, unsigned* flags) {
+    k_fft_z_fwd(FFTPlan pl, Grid g, const __grid_constant__ ZMaps maps, const int* te, FieldsW out, const cd* add,
+                unsigned* flags) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
   __shared__ FxShared sh;
   cfx* a = reinterpret_cast<cfx*>(sm_raw);
@@ -737,8 +739,14 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
     cd p = pl.scale_d * fx_result(v[q], k, xe), m = pl.scale_d * fx_result(v[2 * NP + q], k, xe);
     if (kx == h) p = m = mk(0, 0);
     if (b == 0) m = mk(0, 0);
-    dst[(size_t)b * g.nxh] = p;
-    dst[(size_t)(n2 + b) * g.nxh] = m;
+    const size_t op = (size_t)b * g.nxh, om = (size_t)(n2 + b) * g.nxh;
+    if (add) {
+      const cd* q0 = add + (size_t)j * g.M + kx;
+      if (kx < h) p = p + q0[op];
+      if (kx < h && b != 0) m = m + q0[om];
+    }
+    dst[op] = p;
+    dst[om] = m;
   }
 }
 
@@ -902,7 +910,7 @@ static void z_inv_launch(Ctx& c, const FieldsC& fi, int n, size_t tstride, doubl
                 c.tbuf, tstride, c.texp, c.dflags);
 }
 
-static void z_fwd_launch(Ctx& c, int n, const FieldsW& fo, double fl, double by) {
+static void z_fwd_launch(Ctx& c, int n, const FieldsW& fo, double fl, double by, const cd* add = nullptr) {
   const Grid& g = c.g;
   const FFTPlan& p = c.fz;
   ZMaps maps;
@@ -912,11 +920,14 @@ static void z_fwd_launch(Ctx& c, int n, const FieldsW& fo, double fl, double by)
   }
   const dim3 gz(cdiv(g.nx / 2 + 1, p.batch), g.ny, n);
   if (p.ept == 12 && p.batch == 4)
-    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 4>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, c.dflags);
+    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 4>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, add,
+                c.dflags);
   else if (p.ept == 12)
-    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 2>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, c.dflags);
+    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 2>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, add,
+                c.dflags);
   else
-    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<6, 4>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, c.dflags);
+    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<6, 4>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, add,
+                c.dflags);
 }
 
 // df_in: the spectral inputs are double-float pairs (the precision path's evaluations)
@@ -977,8 +988,8 @@ void fft_forward(Ctx& c, double* const* in, cd* const* out, int nf) {
   }
 }
 
-// forward transform of -(w1 m1 + w2 m2 + w3 m3), formed in the x-pass prologue, into one spectral field
-void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, cd* out) {
+// add + the forward transform of -(w1 m1 + w2 m2 + w3 m3), formed in the x-pass prologue, into one spectral field
+void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, const cd* add, cd* out) {
   const Grid& g = c.g;
   const size_t tstride = (size_t)g.ny * g.pz * (g.nx / 2);
   Dot3 d{};
@@ -997,16 +1008,16 @@ void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, cd
   else
     LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, k_fft_x_fwd_dot3<6>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf,
                 tstride, c.texp, d);
-  z_fwd_launch(c, 1, fo, ny * h * fft_flops(pz), ny * 16.0 * (pz * h + (double)g.nz * g.nxh));
+  z_fwd_launch(c, 1, fo, ny * h * fft_flops(pz), ny * 16.0 * (pz * h + 2.0 * g.nz * g.nxh), add);
 }
 
 // the substage's inputs come from the double-float evaluations in the precision path
 void fft_inverse(Ctx& c, cd* const* in, double* const* out, int nf) { inverse(c, in, out, nf, c.cfg.precision == 1); }
 void fft_inverse_d(Ctx& c, cd* const* in, double* const* out, int nf) { inverse(c, in, out, nf, false); }
-void fft_inverse_mul(Ctx& c, cd* in, double* out, const double* w) {
+void fft_inverse_mul(Ctx& c, cd* in, double* out, const double* w, bool df_in) {
   cd* i[1] = {in};
   double* o[1] = {out};
-  inverse(c, i, o, 1, c.cfg.precision == 1, w);
+  inverse(c, i, o, 1, df_in, w);
 }
 
 // The bounded wait of the z-passes, on its own (lmvd_tile_wait_probe): one CTA expects 128 + extra bytes on

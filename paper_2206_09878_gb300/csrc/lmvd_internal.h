@@ -231,6 +231,8 @@ struct Tape {
 struct AdjWork;
 
 // ---------------------------------------------------------------- context
+// the value fields that hold R_z and dz/dt at the Greville points during the fixed point
+constexpr int SV_RZ = 4, SV_ZDOT = 5;
 struct Ctx {
   lmvd_config cfg;
   Grid g;
@@ -262,7 +264,7 @@ struct Ctx {
   double *mm1_new, *mm3_new;
   cd *Rz, *zdot, *rt, *m1c, *m2c, *m3c, *r_om, *r_phi;
   double* r_m;        // 2 * ny
-  cd* sv[10];         // spectral value fields at g (FFT outputs / inputs)
+  cd* sv[10];         // spectral value fields at g (FFT outputs / inputs); see SV_RZ, SV_ZDOT
   cd* st[7];          // RHS streams: the same memory as sv[0..6] (formed in place from sv)
   cfx* tbuf;          // FFT intermediate (fixed point): tbuf_n fields of ny * pz * (nx/2)
   int* texp;          // its exponents: tbuf_n fields of ny * max(nx, pz) / 2
@@ -342,7 +344,8 @@ void fft_forward(Ctx& c, double* const* in, cd* const* out, int nf);
 // the fixed point's products formed inside the x-passes (Sec. 4.3): inverse transform of one field whose
 // x-pass stores w * phys (rho_t = f'(z) dz/dt), and forward transform of -(w1 m1 + w2 m2 + w3 m3) formed
 // in the x-pass prologue (the tail of L); w, m: physical fields
-void fft_inverse_mul(Ctx& c, cd* in, double* out, const double* w);  // input as for fft_inverse
-void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, cd* out);
+// (df_in: the input is double-float pairs; the tail's spectrum is added to `add`'s)
+void fft_inverse_mul(Ctx& c, cd* in, double* out, const double* w, bool df_in);
+void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, const cd* add, cd* out);
 
 }  // namespace lmvd

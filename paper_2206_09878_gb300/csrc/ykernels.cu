@@ -263,6 +263,41 @@ __global__ void __launch_bounds__(128) k_eval_df(Grid g, EvalJobs jobs) {
   }
 }
 
+// k_mc_values in double-float (values as double-float pairs); WS: width of the order-(p+1) bands
+template <int WS>
+__global__ void __launch_bounds__(128) k_mc_values_df(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const cd* m2c, cd* v1,
+                                                      cd* v2, cd* v3) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= (int)g.M) return;
+  const size_t M = g.M;
+  int r0, r1;
+  row_range(g.ny, blockIdx.y, gridDim.y, r0, r1);
+  if (m == 0 || is_nyquist(g, m)) {  // k = 0: one mode, kept in FP64
+    for (int i = r0; i < r1; ++i) {
+      const size_t o = (size_t)i * M + m;
+      put_df(v1, o, mk(0, 0));
+      put_df(v2, o, m == 0 ? band_row(Sg0, i, m2c, M, 0) : mk(0, 0));
+      put_df(v3, o, mk(0, 0));
+    }
+    return;
+  }
+  double k1, k3;
+  wavenumbers(g, m, k1, k3);
+  const double ik2 = 1.0 / (k1 * k1 + k3 * k3);
+  const df a1 = df_of(k1 * ik2), a3 = df_of(k3 * ik2);
+  DfWin<WS> win;
+  for (int i = r0; i < r1; ++i) {
+    const size_t o = (size_t)i * M + m;
+    win.seek(m2c, M, m, __ldg(Sg0.c0 + i), Sg0.cols);
+    if (i + 1 < r1) win.prefetch(m2c, M, m, __ldg(Sg0.c0 + i + 1), Sg0.cols);
+    const cdf t = cdf_add_lazy(cd_to_cdf(rtv[o]), win.dot(Sg1, i));
+    const df tr = drenorm(t.re), ti = drenorm(t.im);
+    put_df(v1, o, cdf{dmul(a1, dneg(ti)), dmul(a1, tr)});
+    put_df(v2, o, win.dot(Sg0, i));
+    put_df(v3, o, cdf{dmul(a3, dneg(ti)), dmul(a3, tr)});
+  }
+}
+
 // k_rhs_eval in double-float; the k = 0 mean right-hand sides stay in FP64 (one mode). WB: band width of the
 // order-p space (B1g, B2g at g; Bs0..Bs3 at g*). Two sweeps: R_Omega2 (two windows), then R_phi2 (four).
 template <int WB>
@@ -339,6 +374,15 @@ void launch_eval_df(int w, dim3 grid, int tpb, cudaStream_t st, const Grid& g, c
 #undef LMVD_EV
   }
 }
+void launch_mc_values_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& Sg0, const DBand& Sg1,
+                         const cd* rtv, const cd* m2c, cd* v1, cd* v2, cd* v3) {
+  switch (p) {
+#define LMVD_MV(P) \
+    case P: k_mc_values_df<P + 1><<<grid, tpb, 0, st>>>(g, Sg0, Sg1, rtv, m2c, v1, v2, v3); break;
+    LMVD_MV(4) LMVD_MV(5) LMVD_MV(6) LMVD_MV(7) LMVD_MV(8)
+#undef LMVD_MV
+  }
+}
 void launch_rhs_eval_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B1g, const DBand& B2g,
                         const DBand* Bs, const Fields7C& stc, cd* r_om, cd* r_phi, double* r_m) {
   switch (p) {
@@ -386,21 +430,24 @@ __global__ void __launch_bounds__(128) k_solve_piped(Grid g, const __grid_consta
 // Then m_par = i (rho_t + D* m2^c) / k (exact mass conservation in B-coefficient space) and
 // Eq. mc_recon m1^c = k1/k m_par, m3^c = k3/k m_par.
 // k = 0 (Eq. mc_mean): D* <m2^c> = -<rho_t> with <m2^c>(+1) = 0; <m1^c> = <m3^c> = 0.
-// Three launches: k_mc_rhs (right-hand side into m2c), the banded solve (in place, per-mode factors),
-// k_mc_post (m1c, m3c; the k = 0 mean).
+// k_mc_rhs writes the right-hand side into m2c, the banded solve runs in place with per-mode factors (those of k = 0
+// are the summation of Eq. mc_mean), k_mc_values gives the values of m^c at g for the transforms, k_mc_post the
+// coefficients of m1^c and m3^c.
 
 // rows 0..ny split over gridDim.y chunks
-__global__ void k_mc_rhs(Grid g, DBand Bs1, const cd* rt, cd* m2c) {
+__global__ void k_mc_rhs(Grid g, DBand Bs1, const double* dstar, const cd* rt, cd* m2c) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
   const int ny = g.ny;
   int r0, r1;
   row_range(ny + 1, blockIdx.y, gridDim.y, r0, r1);
-  const bool zero = m == 0 || is_nyquist(g, m);
+  const bool zero = is_nyquist(g, m);
   for (int i = r0; i < r1; ++i) {
     cd v = mk(0, 0);
-    if (!zero && i > 0 && i < ny) {
+    if (m == 0) {
+      if (i < ny) v = (1.0 / __ldg(dstar + i)) * rt[(size_t)i * M];
+    } else if (!zero && i > 0 && i < ny) {
       const cd d = band_row(Bs1, i, rt, M, m);
       v = mk(-d.re, -d.im);
     }
@@ -408,27 +455,16 @@ __global__ void k_mc_rhs(Grid g, DBand Bs1, const cd* rt, cd* m2c) {
   }
 }
 
-// rows 0..ny-1 split over gridDim.y chunks; the k = 0 mode is one serial pass (chunk 0)
-__global__ void k_mc_post(Grid g, const double* dstar, const cd* rt, cd* m1c, cd* m2c, cd* m3c) {
+// rows 0..ny-1 split over gridDim.y chunks
+__global__ void k_mc_post(Grid g, const double* dstar, const cd* rt, cd* m1c, const cd* m2c, cd* m3c) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
   const int ny = g.ny;
   int r0, r1;
   row_range(ny, blockIdx.y, gridDim.y, r0, r1);
-  if (is_nyquist(g, m)) {
+  if (m == 0 || is_nyquist(g, m)) {
     for (int i = r0; i < r1; ++i) m1c[(size_t)i * M + m] = m3c[(size_t)i * M + m] = mk(0, 0);
-    return;
-  }
-  if (m == 0) {
-    if (blockIdx.y != 0) return;
-    cd c = mk(0, 0);
-    m2c[(size_t)ny * M] = c;
-    for (int i = ny - 1; i >= 0; --i) {
-      c = c + (1.0 / __ldg(dstar + i)) * rt[(size_t)i * M];
-      m2c[(size_t)i * M] = c;
-      m1c[(size_t)i * M] = m3c[(size_t)i * M] = mk(0, 0);
-    }
     return;
   }
   double k1, k3;
@@ -441,6 +477,36 @@ __global__ void k_mc_post(Grid g, const double* dstar, const cd* rt, cd* m1c, cd
     const cd mpar = ik * times_i(rt[(size_t)i * M + m] + dm);
     m1c[(size_t)i * M + m] = (k1 * ik) * mpar;
     m3c[(size_t)i * M + m] = (k3 * ik) * mpar;
+  }
+}
+
+// Values of m^c at g: v2 = B* m2^c, (v1, v3) = i (k1, k3) / k^2 (rho_t + d m2^c / dy) with rtv the values of rho_t; zero
+// v1, v3 at k = 0. Rows split over gridDim.y chunks.
+__global__ void k_mc_values(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const cd* m2c, cd* v1, cd* v2, cd* v3) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= (int)g.M) return;
+  const size_t M = g.M;
+  int r0, r1;
+  row_range(g.ny, blockIdx.y, gridDim.y, r0, r1);
+  const bool zero = is_nyquist(g, m);
+  double a1 = 0.0, a3 = 0.0;
+  if (m != 0 && !zero) {
+    double k1, k3;
+    wavenumbers(g, m, k1, k3);
+    const double ik2 = 1.0 / (k1 * k1 + k3 * k3);
+    a1 = k1 * ik2;
+    a3 = k3 * ik2;
+  }
+  for (int i = r0; i < r1; ++i) {
+    const size_t o = (size_t)i * M + m;
+    cd w = mk(0, 0), t = mk(0, 0);
+    if (!zero) {
+      w = band_row(Sg0, i, m2c, M, m);
+      if (m != 0) t = times_i(rtv[o] + band_row(Sg1, i, m2c, M, m));
+    }
+    v1[o] = a1 * t;
+    v2[o] = w;
+    v3[o] = a3 * t;
   }
 }
 
@@ -702,9 +768,9 @@ __global__ void k_sanitize(Grid g, int rows, cd* f, int zero_mean) {
 // LU (no pivoting) of A(k) = A2 - k^2 A0 + k A1 for the factor modes (kx, kz >= 0), mf = jz * nxh + kx,
 // jz = 0..nz/2 (stride Mh = (nz/2 + 1) nxh); A2, A0, A1 in diagonal band storage (half-width K, shared),
 // profile nl/nu shared; entries outside the profile are stored as zeros. k = 0 and Nyquist modes get
-// identity factors.
+// identity factors, or with mean_rows the k = 0 mode those of x_i - x_{i+1} = r_i (x_{n-1} = r_{n-1}).
 __global__ void k_factor(Grid g, int n, int K, const double* A2, const double* A0, const double* A1, const int* nl,
-                         const int* nu, double* lo, double* up, double* invd) {
+                         const int* nu, double* lo, double* up, double* invd, int mean_rows) {
   const size_t Mh = (size_t)(g.nz / 2 + 1) * g.nxh;
   const int mf = blockIdx.x * blockDim.x + threadIdx.x;
   if (mf >= (int)Mh) return;
@@ -714,6 +780,7 @@ __global__ void k_factor(Grid g, int n, int K, const double* A2, const double* A
     for (int i = 0; i < n; ++i) {
       for (int q = 0; q < K; ++q) lo[(size_t)(i * K + q) * Mh + mf] = up[(size_t)(i * K + q) * Mh + mf] = 0.0;
       invd[(size_t)i * Mh + mf] = 1.0;
+      if (mean_rows && mf == 0 && i < n - 1) up[(size_t)(i * K) * Mh] = -1.0;
     }
     return;
   }

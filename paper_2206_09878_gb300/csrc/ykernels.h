@@ -82,12 +82,15 @@ void launch_eval_p1_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g
                        const DBand& B2g, const DBand& Sg0, const DBand& Sg1, const cd* z, const cd* om, const cd* m2,
                        const double* mm1, const double* mm3, const Fields8& out);
 void launch_eval_df(int w, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const EvalJobs& jobs);
+void launch_mc_values_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& Sg0, const DBand& Sg1,
+                         const cd* rtv, const cd* m2c, cd* v1, cd* v2, cd* v3);
 void launch_rhs_eval_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B1g, const DBand& B2g,
                         const DBand* Bs, const Fields7C& stc, cd* r_om, cd* r_phi, double* r_m);
 __global__ void k_solve_cd(Grid g, DLU lu, SolveJobs jobs);
 __global__ void k_solve_piped(Grid g, const __grid_constant__ PipedJobs jobs);
-__global__ void k_mc_rhs(Grid g, DBand Bs1, const cd* rt, cd* m2c);
-__global__ void k_mc_post(Grid g, const double* dstar, const cd* rt, cd* m1c, cd* m2c, cd* m3c);
+__global__ void k_mc_rhs(Grid g, DBand Bs1, const double* dstar, const cd* rt, cd* m2c);
+__global__ void k_mc_post(Grid g, const double* dstar, const cd* rt, cd* m1c, const cd* m2c, cd* m3c);
+__global__ void k_mc_values(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const cd* m2c, cd* v1, cd* v2, cd* v3);
 __global__ void k_rhs_combine(Grid g, double mu, double grav, Fields10C sv, Fields7 st);
 __global__ void k_rhs_eval(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, DBand Bs2, DBand Bs3, Fields7C st,
                            cd* r_om, cd* r_phi, double* r_m);
@@ -98,7 +101,7 @@ __global__ void k_backfill(size_t n, double c0, double c1, double c2, const cd* 
                            cd* h2);
 __global__ void k_sanitize(Grid g, int rows, cd* f, int zero_mean);
 __global__ void k_factor(Grid g, int n, int K, const double* A2, const double* A0, const double* A1, const int* nl,
-                         const int* nu, double* lo, double* up, double* invd);
+                         const int* nu, double* lo, double* up, double* invd, int mean_rows);
 
 // pointwise.cu: physical-space products (Sec. 2.1, 4.3, 5)
 struct EosArgs {
