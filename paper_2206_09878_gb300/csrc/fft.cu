@@ -19,9 +19,9 @@
 // Arithmetic: 64-bit fixed point with one exponent per 1D transform (fx.cuh), in both precisions. The
 // FP64 pipe retires 1.68 additions per clock per SM here, and transforms in complex double were bound by
 // it (85% busy); in fixed point the same passes run on the integer pipes (ALU 45-52%, multiply pipe
-// 50-60% busy), 4.4 times faster in FP64 arithmetic's place and 1.3 times faster than the double-float
+// 50-60% busy), 5.3 times faster in FP64 arithmetic's place and 1.3 times faster than the double-float
 // transforms they replaced in the precision path: at 512 x 65 x 512, per substage, 100.1 ms (complex
-// double) and 25.2 ms (double-float) -> 19.7 ms. Physical fields and FP64 spectral fields are complex
+// double) and 25.2 ms (double-float) -> 18.8 ms. Physical fields and FP64 spectral fields are complex
 // double / double; the precision path's spectral inputs are double-float pairs; T is fixed point with an
 // array of exponents, so the conversions are at the ends only.
 // Accuracy (rms error over rms result against a transform in extended precision, 2D inverse of white
@@ -95,32 +95,37 @@ __device__ __forceinline__ void fx_butterfly(cfx (&v)[R], const FFTPlan& pl) {
   }
 }
 
+// The sub-length L divides tpt (the radices before the last multiply to tpt), so a thread's butterflies share k = tt mod
+// L and their twiddles, which are fetched before the barrier.
 template <int SIGN, int R, int EPT, int S>
-__device__ __forceinline__ void fx_stage(cfx* x, const FFTPlan& pl, int L, int tt, int tpt, int lo, int hi) {
+__device__ __forceinline__ void fx_stage(cfx* x, const FFTPlan& pl, int L, int tt, int tpt) {
   constexpr int NBT = EPT / R;
   const int n = pl.n;
-  const int nb = n / R, tws = n / (L * R);
+  const int nb = n / R;
+  const int k = (L & (L - 1)) == 0 ? (tt & (L - 1)) : (tt % L);
+  const int kt = k * (n / (L * R));
+  int4 w[R];
+#pragma unroll
+  for (int q = 1; q < R; ++q) w[q] = __ldg(pl.tw + q * kt);
   cfx v[NBT][R];
 #pragma unroll
   for (int j = 0; j < NBT; ++j)
 #pragma unroll
     for (int q = 0; q < R; ++q) {
       const int i = tt + j * tpt + q * nb;
-      v[j][q] = LMVD_IN(i, n) && (i < lo || i >= hi) ? x[i * S] : cfx{0, 0};
+      v[j][q] = LMVD_IN(i, n) ? x[i * S] : cfx{0, 0};
     }
   __syncthreads();
+  cfx* y = x + ((tt - k) * R + k) * S;
 #pragma unroll
   for (int j = 0; j < NBT; ++j) {
-    const int b = tt + j * tpt;
-    const int k = (L & (L - 1)) == 0 ? (b & (L - 1)) : (b % L);
-    const int base = (b - k) * R + k;
-    if (!LMVD_IN(base + (R - 1) * L, n)) continue;
+    if (!LMVD_IN((tt - k) * R + k + j * tpt * R + (R - 1) * L, n)) continue;
     if (k)  // (a product with w = 1 would not be exact)
 #pragma unroll
-      for (int q = 1; q < R; ++q) v[j][q] = fx_mulw<SIGN>(v[j][q], __ldg(pl.tw + q * k * tws));
+      for (int q = 1; q < R; ++q) v[j][q] = fx_mulw<SIGN>(v[j][q], w[q]);
     fx_butterfly<SIGN, R>(v[j], pl);
 #pragma unroll
-    for (int q = 0; q < R; ++q) x[(base + q * L) * S] = v[j][q];
+    for (int q = 0; q < R; ++q) y[(j * tpt * R + q * L) * S] = v[j][q];
   }
   __syncthreads();
 }
@@ -140,10 +145,9 @@ __device__ __forceinline__ void fx_first4(cfx (&v)[12], cfx* x, const FFTPlan& p
   __syncthreads();
 }
 
-// Stages s0 .. nst - 2; returns when every point of the last stage's input is in x. Input points [lo, hi) of stage 0
-// are zero and not read (the 3/2-rule padding of a synthesis).
+// Stages s0 .. nst - 2; returns when every point of the last stage's input is in x.
 template <int SIGN, int EPT, int S>
-__device__ __forceinline__ void fx_middle(cfx* x, const FFTPlan& pl, int s0, int tt, int tpt, int lo = 0, int hi = 0) {
+__device__ __forceinline__ void fx_middle(cfx* x, const FFTPlan& pl, int s0, int tt, int tpt) {
   int L = 1;
   unsigned code = pl.code;
   if (s0) {
@@ -153,16 +157,15 @@ __device__ __forceinline__ void fx_middle(cfx* x, const FFTPlan& pl, int s0, int
   for (int s = s0; s < pl.nst - 1; ++s, code >>= 2) {
     const unsigned r2 = code & 3u;
     if (EPT == 12 && r2 == 0) {
-      fx_stage<SIGN, 4, EPT, S>(x, pl, L, tt, tpt, lo, hi);
+      fx_stage<SIGN, 4, EPT, S>(x, pl, L, tt, tpt);
       L *= 4;
     } else if (EPT == 12 && r2 == 1) {
-      fx_stage<SIGN, 2, EPT, S>(x, pl, L, tt, tpt, lo, hi);
+      fx_stage<SIGN, 2, EPT, S>(x, pl, L, tt, tpt);
       L *= 2;
     } else {
-      fx_stage<SIGN, 3, EPT, S>(x, pl, L, tt, tpt, lo, hi);
+      fx_stage<SIGN, 3, EPT, S>(x, pl, L, tt, tpt);
       L *= 3;
     }
-    lo = hi = 0;
   }
 }
 
@@ -240,14 +243,8 @@ __device__ __noinline__ double fx_unscale(double d, int xe) {
   return xe == kFxPoison ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(d, xe);
 }
 
-__device__ __forceinline__ void mag_add(FxMag& m, cd x) {
-  m.add(x.re);
-  m.add(x.im);
-}
-__device__ __forceinline__ void mag_add(FxMag& m, cdf x) {
-  m.add(x.re);
-  m.add(x.im);
-}
+__device__ __forceinline__ void mag_add(FxMag& m, cd x) { m.add(x.re, x.im); }
+__device__ __forceinline__ void mag_add(FxMag& m, cdf x) { m.add(x.re, x.im); }
 template <class RAW>
 constexpr bool kIsDf = std::is_same<RAW, cdf>::value;
 
@@ -339,8 +336,8 @@ __device__ __forceinline__ cd fx_result(cfx v, int k, int xe) {
 // FFT_CTA_Z threads).
 constexpr int FFT_CTA_X = 128, FFT_CTA_Z = 256;
 // CTAs per SM each pass is compiled for, i.e. its register cap (80). A thread holds 12 elements of 4 registers; at
-// 512 x 65 x 512 the inverse x-passes take 7.82 / 7.33 / 7.33 / 7.46 ms per substage at 4 / 5 / 6 / 7 CTAs, the
-// forward ones 5.48 / 5.15 / 5.10 / 5.24, the z-passes 8.24 / 7.28 / 7.64 at 2 / 3 / 4.
+// 512 x 65 x 512 the inverse x-passes take 7.06 / 6.95 / 7.05 ms per substage at 5 / 6 / 7 CTAs, the forward ones
+// 4.97 / 4.91 / 5.21, the z-passes 8.22 / 7.11 at 2 / 3 (4: 5% slower than 3).
 constexpr int FFT_MIN_X = 6, FFT_MIN_Z = 3;
 
 // ---------------------------------------------------------------- tile loads (TMA)
@@ -470,7 +467,11 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
     cfx v[EPT];
     const float sa = fx_sa(k);
 #pragma unroll
-    for (int u = 0; u < EPT; ++u) v[u] = fx_convert(raw[u], k, sa);
+    for (int u = 0; u < EPT; ++u) {
+      const int i = fx_point(u, first4, tt, tpt, pz >> 2);
+      v[u] = cfx{0, 0};
+      if (i < lo || i >= hi) v[u] = fx_convert(raw[u], k, sa);  // (whole warps skip the padding)
+    }
     fx_run<1, EPT, COLS>(v, a + c, pl, first4, tt);
   }
   cfx v[EPT];
@@ -559,11 +560,13 @@ __device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, con
       y[px - kk] = cfx{xa.re + xb.im, xb.re - xa.im};  // conj(Xa[k]) + i conj(Xb[k])
     }
   }
-  if (pl.nst == 1)  // no stage that skips the kx padding [h, 2 h]
-    for (int q = h + tt; q <= 2 * h; q += tpt)
-      if (LMVD_IN(q, px)) y[q] = cfx{0, 0};
+  // the kx padding [h, 2 h] (a first stage of its own that skips it instead was 3% slower: instruction cache)
+#pragma unroll
+  for (int u = 0; u < NP; ++u)
+    if (LMVD_IN(h + tt + u * tpt, px)) y[h + tt + u * tpt] = cfx{0, 0};
+  if (tt == 0 && LMVD_IN(2 * h, px)) y[2 * h] = cfx{0, 0};
   __syncthreads();
-  fx_middle<1, EPT, 1>(y, pl, 0, tt, tpt, h, px - h + 1);  // kx padding: zero
+  fx_middle<1, EPT, 1>(y, pl, 0, tt, tpt);
   double* dst = reinterpret_cast<double*>(pick(out.p, f)) + (size_t)j * g.P + (size_t)za * px;
   const double* w = MUL ? wmul + (size_t)j * g.P + (size_t)za * px : nullptr;
   cfx v[EPT];

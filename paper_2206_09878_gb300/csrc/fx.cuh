@@ -75,15 +75,17 @@ __host__ __device__ inline void fx_limbs(F w, int& hi, int& lo) {
 struct FxMag {
   float sum = 0.f;
   int top = 0;  // largest |high word|
-  __device__ __forceinline__ void add(double x) {
-    const int t = __double2hiint(x) & 0x7fffffff;
-    top = max(top, t);
-    sum += __int_as_float(max(t - 0x38000000, 0) << 3);
+  __device__ __forceinline__ void add(double x, double y) {
+    const int t = __double2hiint(x) & 0x7fffffff, u = __double2hiint(y) & 0x7fffffff;
+    top = __vimax3_s32(top, t, u);
+    sum += __int_as_float(__viaddmax_s32(t, -0x38000000, 0) << 3);
+    sum += __int_as_float(__viaddmax_s32(u, -0x38000000, 0) << 3);
   }
-  __device__ __forceinline__ void add(df x) {
-    const float a = fabsf(x.hi);
-    top = max(top, __float_as_int(a));
+  __device__ __forceinline__ void add(df x, df y) {
+    const float a = fabsf(x.hi), b = fabsf(y.hi);
+    top = __vimax3_s32(top, __float_as_int(a), __float_as_int(b));
     sum += a;
+    sum += b;
   }
 };
 // Sums in [kFxTiny, kFxHuge) (or all-zero inputs) need no rescaling; outside, or with inf / nan, the slow path
