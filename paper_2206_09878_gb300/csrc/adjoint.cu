@@ -518,7 +518,13 @@ int adj_upload_band(AdjWork& A, const RowBand& m, DBand& d) {
   if (cudaMemcpy(c0, m.c0.data(), sizeof(int) * m.c0.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(v, m.v.data(), sizeof(double) * m.v.size(), cudaMemcpyHostToDevice) != cudaSuccess)
     return LMVD_ERR_CUDA;
-  d = DBand{c0, v, m.rows, m.w, nullptr, m.cols};
+  const std::vector<int> n = entry_counts(m);
+  int* cnt = nullptr;
+  if (cudaMalloc(&cnt, sizeof(int) * n.size()) != cudaSuccess) return LMVD_ERR_OOM;
+  A.small.push_back(cnt);
+  A.small_bytes += sizeof(int) * n.size();
+  if (cudaMemcpy(cnt, n.data(), sizeof(int) * n.size(), cudaMemcpyHostToDevice) != cudaSuccess) return LMVD_ERR_CUDA;
+  d = DBand{c0, v, m.rows, m.w, nullptr, m.cols, cnt};
   return LMVD_OK;
 }
 

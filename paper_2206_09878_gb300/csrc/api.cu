@@ -116,6 +116,10 @@ int upload_band(Ctx& c, const RowBand& m, DBand& d) {
   if (e) return e;
   e = upload(c, m.v, &v);
   if (e) return e;
+  int* cnt;
+  e = upload(c, entry_counts(m), &cnt);
+  if (e) return e;
+  d.cnt = cnt;
   std::vector<df> split(m.v.size());
   for (size_t q = 0; q < m.v.size(); ++q) {
     const float hi = (float)m.v[q];
@@ -236,7 +240,7 @@ PerMode md_system(const RowBand& Ss0, const RowBand& Ss1, const RowBand& Ss2, in
 }
 
 // mean_rows: the k = 0 mode's factors solve x_i - x_{i+1} = r_i, x_{n-1} = r_{n-1} (Eq. mc_mean) instead of x = r
-int factor_per_mode(Ctx& c, const PerMode& pm, int K, bool mean_rows, DLU& out) {
+int factor_per_mode(Ctx& c, const PerMode& pm, int K, bool mean_rows, DLU& out, DRows* rows = nullptr) {
   std::vector<int> nl, nu;
   DiagBand pattern = pm.A0;  // union of the non-zero patterns of A0 and A1 (A2 is the other argument)
   for (size_t i = 0; i < pattern.a.size(); ++i)
@@ -267,6 +271,7 @@ int factor_per_mode(Ctx& c, const PerMode& pm, int K, bool mean_rows, DLU& out) 
               TPB_MODE, 0, c.g, n, K, A2, A0, A1, dnl, dnu, lo, up, invd, mean_rows ? 1 : 0);
   out = DLU{lo, up, invd, dnl, dnu, n, K, Mh, band_interior(nl), band_interior(nu), 0.0};
   for (int i = 0; i < n; ++i) out.flops_per_mode += 4.0 * (nl[i] + nu[i]) + 2.0;
+  if (rows) *rows = DRows{A2, A0, A1, n, K};
   return cuda_check(c);
 }
 
@@ -604,8 +609,8 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
   for (int f = 0; f < 10; ++f) svc.p[f] = c.sv[f];
   Fields7 stw{};
   for (int f = 0; f < 7; ++f) stw.p[f] = c.st[f];
-  LMVD_LAUNCH(c, KC_RHS_COMBINE, 90.0 * S, 16.0 * 17 * S, k_rhs_combine, elem_blocks(S), 256, 0, g, 1.0 / cf.re,
-              1.0 / (cf.fr * cf.fr), svc, stw);
+  LMVD_LAUNCH(c, KC_RHS_COMBINE, 60.0 * S, 16.0 * 17 * S, k_rhs_combine, dim3(mode_blocks(g), row_chunks(g, g.ny)),
+              TPB_MODE, 0, g, 1.0 / cf.re, 1.0 / (cf.fr * cf.fr), svc, stw);
   const DLU* li = &c.lu_interp;
   solve_modes(c, KC_SOLVE, {SolveReq{SolveJob{c.st[1], nullptr, c.st[1]}, li}, SolveReq{SolveJob{c.st[2], nullptr, c.st[2]}, li},
                             SolveReq{SolveJob{c.st[3], nullptr, c.st[3]}, li}, SolveReq{SolveJob{c.st[4], nullptr, c.st[4]}, li},
@@ -633,14 +638,16 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
   u.m2 = c.m2; u.r_phi = c.r_phi; u.r_phi_prev = c.r_phi_prev;
   u.mm1 = c.mm1; u.mm3 = c.mm3; u.r_m = c.r_m; u.r_m_prev = c.r_m_prev;
   u.om_new = c.om_new; u.z_new = c.z_new; u.m2_new = c.m2_new; u.mm1_new = c.mm1_new; u.mm3_new = c.mm3_new;
+  u.md = c.md_rows;
   const double Sp = (double)(g.ny + 1) * g.M;
-  LMVD_LAUNCH(c, KC_UPDATE, S * (12.0 * c.B0g.w + 20.0) + Sp * (8.0 * c.Ss0.w + 10.0), 16.0 * 7 * S + 16.0 * 4 * Sp,
-              k_update_rhs, dim3(std::max(mode_blocks(g), (unsigned)(2 * g.ny + TPB_MODE - 1) / TPB_MODE),
-                                 row_chunks(g, g.ny + 1), 4),
-              TPB_MODE, 0, g, c.B0g, c.Ss0, c.Ss2, u);
-  solve_modes(c, KC_UPDATE, {SolveReq{SolveJob{c.om_new, nullptr, c.om_new}, &c.lu_interp},
+  LMVD_LAUNCH_CALL(c, KC_UPDATE, S * (4.0 * c.B0g.w + 24.0) + Sp * 6.0, 16.0 * (3 * S + 4 * S + 3 * Sp),
+                   launch_update_rhs(cf.spline_order,
+                                     dim3(std::max(mode_blocks(g), (unsigned)(2 * g.ny + TPB_MODE - 1) / TPB_MODE),
+                                          row_chunks(g, g.ny + 1), 4),
+                                     TPB_MODE, c.stream, g, c.B0g, u));
+  solve_modes(c, KC_UPDATE, {SolveReq{SolveJob{c.om_new, c.om, c.om_new}, &c.lu_interp},
                              SolveReq{SolveJob{c.z_new, nullptr, c.z_new}, &c.lu_neumann},
-                             SolveReq{SolveJob{c.m2_new, nullptr, c.m2_new}, &c.lu_md}},
+                             SolveReq{SolveJob{c.m2_new, c.m2, c.m2_new}, &c.lu_md}},
               true);
   // failure detection: any non-finite value in the new state sets the device status word
   {
@@ -889,7 +896,7 @@ int lmvd_create(const lmvd_config* cfg, void* stream, lmvd_ctx** out) {
     const int Ks = std::max({half_width(Ss0), half_width(Ss1), half_width(Ss2)});
     if (Ks > KMAX) throw std::runtime_error("band");
     if (!err) err = factor_per_mode(c, mc_system(Ss0, Ss1, Ss2, Ks, cfg->bc_mode), Ks, true, c.lu_mc);
-    if (!err) err = factor_per_mode(c, md_system(Ss0, Ss1, Ss2, Ks, cfg->bc_mode), Ks, false, c.lu_md);
+    if (!err) err = factor_per_mode(c, md_system(Ss0, Ss1, Ss2, Ks, cfg->bc_mode), Ks, false, c.lu_md, &c.md_rows);
     // plane means <m1>, <m3>: Dirichlet rows (walls) or Neumann rows (potential matching)
     c.lu_means = cfg->bc_mode == 1 ? c.lu_neumann : c.lu_interp;
   } catch (const std::exception&) {

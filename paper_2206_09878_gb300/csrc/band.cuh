@@ -342,7 +342,8 @@ __device__ inline double band_row_real(const DBand& B, int i, const double* x) {
   if (!LMVD_IN(i, B.rows)) return acc;
   const int c = B.c0[i];
   const double* v = B.v + (size_t)i * B.w;
-  for (int q = 0; q < B.w; ++q)
+  const int n = __ldg(B.cnt + i);
+  for (int q = 0; q < n; ++q)
     if (LMVD_IN(c + q, B.cols)) acc = fma(__ldg(v + q), x[c + q], acc);
   return acc;
 }

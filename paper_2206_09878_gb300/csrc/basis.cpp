@@ -220,6 +220,14 @@ std::vector<double> greville_quadrature(const Knots& k, const RowBand& B0g) {
   return w;
 }
 
+std::vector<int> entry_counts(const RowBand& m) {
+  std::vector<int> n(m.rows, 0);
+  for (int i = 0; i < m.rows; ++i)
+    for (int q = 0; q < m.w; ++q)
+      if (m.v[(size_t)i * m.w + q] != 0.0) n[i] = q + 1;
+  return n;
+}
+
 BandLU band_lu(const DiagBand& A) {
   BandLU f;
   const int n = A.n, K = A.K;

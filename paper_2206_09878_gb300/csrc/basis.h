@@ -57,6 +57,8 @@ struct BandLU {
   std::vector<int> nl, nu;
 };
 BandLU band_lu(const DiagBand& A);
+// entries of each row up to its last non-zero one
+std::vector<int> entry_counts(const RowBand& m);
 // Weights w_i with sum_i w_i f(g_i) = integral over [y0, y1] of the order-p spline that interpolates f at
 // the Greville points g_i: w = A^{-T} b, A the collocation matrix (B0g), b_j = (t_{j+p} - t_j) / p the
 // integral of B_j.

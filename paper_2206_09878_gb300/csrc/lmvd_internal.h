@@ -81,6 +81,12 @@ struct DBand {
   int rows, w;
   const df* vf;
   int cols;  // rows of the array a row of the band reads (index checks of the checked build)
+  const int* cnt;  // entries of a row up to its last non-zero one (at a knot the last basis function is zero)
+};
+// Rows of the m2^d system, A(k) = A2 - k^2 A0 + k A1, in diagonal band storage (2 K + 1 entries a row)
+struct DRows {
+  const double *A2, *A0, *A1;
+  int n, K;
 };
 // LU factors of band systems, K entries per row (zeros outside the profile nl / nu). Shared factors:
 // mstride = 0, element (i, q) at [i * K + q]; per-mode factors: element (i, q) of factor mode mf at
@@ -145,17 +151,19 @@ __host__ __device__ inline void row_range(int rows, int c, int nc, int& r0, int&
   r1 = (int)((long long)rows * (c + 1) / nc);
 }
 
-// Row chunks for the evaluation kernels: enough threads for about 1024 per SM when the grid has few
-// Fourier modes, at least 8 rows per thread.
+// Row chunks for the evaluation kernels: about 2^17 threads when the grid has few
+// Fourier modes (more repeat the per-mode FP64 work of a chunk's start: 1% of a substage at 128 modes), at least 2 rows per thread. (With 8 a thread's rows were the time of a launch on the smallest grids: one
+// warp's FP64 instruction takes 64 cycles whatever else runs. 32 x 33 x 32: pass-1 evaluation 58 -> 27 us, right-hand
+// sides 76 -> 24 us.)
 inline unsigned row_chunks(const Grid& g, int rows) {
-  const size_t want = ((size_t)152 * 1024 + g.M - 1) / g.M;
-  const size_t cap = (size_t)(rows / 8 > 1 ? rows / 8 : 1);
+  const size_t want = (((size_t)1 << 17) + g.M - 1) / g.M;
+  const size_t cap = (size_t)(rows / 2 > 1 ? rows / 2 : 1);
   const size_t ch = want < cap ? want : cap;
   return (unsigned)(ch > 1 ? ch : 1);
 }
 
-// Threads per mode of the banded-solve kernels: 2 (one per real part) when the grid has fewer than 65536
-// Fourier modes per row, else 1 (see band_solve_v).
+// Threads per mode of the banded-solve kernels: 2 (one per real part, band_solve_piped) when the grid has fewer than
+// 65536 Fourier modes per row, else 1 (band_solve_v).
 inline int solve_split(const Grid& g) { return g.M < 65536 ? 2 : 1; }
 
 __device__ inline cd band_row(const DBand& B, int i, const cd* x, size_t M, int m) {
@@ -163,7 +171,8 @@ __device__ inline cd band_row(const DBand& B, int i, const cd* x, size_t M, int 
   if (!LMVD_IN(i, B.rows) || !LMVD_IN(m, M)) return acc;
   const int c = B.c0[i];
   const double* v = B.v + (size_t)i * B.w;
-  for (int q = 0; q < B.w; ++q)
+  const int n = __ldg(B.cnt + i);
+  for (int q = 0; q < n; ++q)
     if (LMVD_IN(c + q, B.cols)) acc = fma_rc(__ldg(v + q), x[(size_t)(c + q) * M + m], acc);
   return acc;
 }
@@ -245,6 +254,7 @@ struct Ctx {
   double* dstar = nullptr;  // ny entries: (D* c)_i = dstar[i] (c_{i+1} - c_i)
   DLU lu_interp, lu_neumann, lu_mc, lu_md;
   DLU lu_means;  // lu_interp (walls) or lu_neumann (potential matching): not owned
+  DRows md_rows;              // the m2^d system (its boundary rows are evaluated by the RK update)
   FFTPlan fx, fz;
 
   // memory arena

@@ -32,7 +32,7 @@ __global__ void k_eval_p1(Grid g, DBand B0g, DBand B1g, DBand B2g, DBand Sg0, DB
   double k1, k3;
   wavenumbers(g, m, k1, k3);
   const double k2 = k1 * k1 + k3 * k3;
-  const double ik2 = m == 0 ? 0.0 : 1.0 / k2;
+  const double ik2 = m == 0 ? 0.0 : 1.0 / k2, a1 = k1 * ik2, a3 = k3 * ik2;
   for (int i = r0; i < r1; ++i) {
     const size_t o = (size_t)i * M + m;
     const cd zg = band_row(B0g, i, z, M, m);
@@ -42,7 +42,7 @@ __global__ void k_eval_p1(Grid g, DBand B0g, DBand B1g, DBand B2g, DBand Sg0, DB
     out.p[1][o] = k1 * times_i(zg);
     out.p[2][o] = k3 * times_i(zg);
     out.p[3][o] = zy;
-    out.p[4][o] = (-k2) * zg + zyy;
+    out.p[4][o] = fma_rc(-k2, zg, zyy);
     if (m == 0) {
       out.p[5][o] = mk(band_row_real(B0g, i, mm1), 0.0);
       out.p[6][o] = mk(0, 0);
@@ -50,9 +50,9 @@ __global__ void k_eval_p1(Grid g, DBand B0g, DBand B1g, DBand B2g, DBand Sg0, DB
     } else {
       const cd dm2 = band_row(Sg1, i, m2, M, m);
       const cd omg = band_row(B0g, i, om, M, m);
-      out.p[5][o] = ik2 * times_i(k1 * dm2 - k3 * omg);
+      out.p[5][o] = times_i(fma_rc(a1, dm2, (-a3) * omg));
       out.p[6][o] = band_row(Sg0, i, m2, M, m);
-      out.p[7][o] = ik2 * times_i(k3 * dm2 + k1 * omg);
+      out.p[7][o] = times_i(fma_rc(a3, dm2, a1 * omg));
     }
   }
 }
@@ -519,37 +519,48 @@ __global__ void k_mc_values(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const c
 // so only st1..st6 need B-spline coefficients (st0 is already the value at g).
 // k = 0: st1 = <C12>, st2 = mu <u1>, st4 = <C23>, st5 = mu <u3> carry the mean equations
 // (Eq. mean_m1m3); the k = 0 values of all seven streams vanish otherwise.
+// One thread per mode and row chunk: the multipliers are formed once per mode.
 __global__ void k_rhs_combine(Grid g, double mu, double grav, Fields10C sv, Fields7 st) {
-  const size_t n = (size_t)g.ny * g.M;
-  for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
-    const int m = (int)(o % g.M);
-    cd r[7];
-    for (int q = 0; q < 7; ++q) r[q] = mk(0, 0);
-    if (!is_nyquist(g, m)) {
-      const cd C11 = sv.p[0][o], C12 = sv.p[1][o], C13 = sv.p[2][o], C22 = sv.p[3][o], C23 = sv.p[4][o],
-               C33 = sv.p[5][o], u1 = sv.p[6][o], u2 = sv.p[7][o], u3 = sv.p[8][o], rho = sv.p[9][o];
-      if (m == 0) {
-        r[1] = C12;
-        r[2] = mu * u1;
-        r[4] = C23;
-        r[5] = mu * u3;
-      } else {
-        double k1, k3;
-        wavenumbers(g, m, k1, k3);
-        const double k2 = k1 * k1 + k3 * k3;
-        const cd w13 = times_i(k3 * u1 - k1 * u3);        // i k3 u1 - i k1 u3
-        const cd d13 = times_i(k1 * u1 + k3 * u3);        // i k1 u1 + i k3 u3
-        const cd c1223 = times_i(k1 * C12 + k3 * C23);    // i k1 C12 + i k3 C23
-        r[0] = (-k1 * k3) * C11 + (k1 * k1 - k3 * k3) * C13 + (k1 * k3) * C33 - (mu * k2) * w13;
-        r[1] = times_i(k3 * C12 - k1 * C23);
-        r[2] = mu * w13;
-        r[3] = (-k2) * (c1223 - grav * rho) + (mu * k2 * k2) * u2;
-        r[4] = (-k2) * C22 + (k1 * k1) * C11 + (2.0 * k1 * k3) * C13 + (k3 * k3) * C33 + (mu * k2) * d13;
-        r[5] = mk(-c1223.re, -c1223.im) - (mu * k2) * u2;
-        r[6] = (-mu) * d13;
-      }
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= (int)g.M) return;
+  const size_t M = g.M;
+  int r0, r1;
+  row_range(g.ny, blockIdx.y, gridDim.y, r0, r1);
+  if (is_nyquist(g, m)) {
+    for (int i = r0; i < r1; ++i)
+      for (int q = 0; q < 7; ++q) st.p[q][(size_t)i * M + m] = mk(0, 0);
+    return;
+  }
+  if (m == 0) {
+    for (int i = r0; i < r1; ++i) {
+      const size_t o = (size_t)i * M;
+      const cd C12 = sv.p[1][o], C23 = sv.p[4][o], u1 = sv.p[6][o], u3 = sv.p[8][o];
+      st.p[0][o] = st.p[3][o] = st.p[6][o] = mk(0, 0);
+      st.p[1][o] = C12;
+      st.p[2][o] = mu * u1;
+      st.p[4][o] = C23;
+      st.p[5][o] = mu * u3;
     }
-    for (int q = 0; q < 7; ++q) st.p[q][o] = r[q];
+    return;
+  }
+  double k1, k3;
+  wavenumbers(g, m, k1, k3);
+  const double k11 = k1 * k1, k33 = k3 * k3, k13 = k1 * k3, k2 = k11 + k33, kd = k11 - k33, m2 = mu * k2, m4 = m2 * k2;
+  for (int i = r0; i < r1; ++i) {
+    const size_t o = (size_t)i * M + m;
+    const cd C11 = sv.p[0][o], C12 = sv.p[1][o], C13 = sv.p[2][o], C22 = sv.p[3][o], C23 = sv.p[4][o], C33 = sv.p[5][o],
+             u1 = sv.p[6][o], u2 = sv.p[7][o], u3 = sv.p[8][o], rho = sv.p[9][o];
+    const cd w13 = times_i(fma_rc(k3, u1, (-k1) * u3));      // i k3 u1 - i k1 u3
+    const cd d13 = times_i(fma_rc(k1, u1, k3 * u3));         // i k1 u1 + i k3 u3
+    const cd c1223 = times_i(fma_rc(k1, C12, k3 * C23));     // i k1 C12 + i k3 C23
+    const cd nc = mk(-c1223.re, -c1223.im);
+    st.p[0][o] = fma_rc(-m2, w13, fma_rc(kd, C13, k13 * (C33 - C11)));
+    st.p[1][o] = times_i(fma_rc(k3, C12, (-k1) * C23));
+    st.p[2][o] = mu * w13;
+    st.p[3][o] = fma_rc(m4, u2, k2 * fma_rc(grav, rho, nc));
+    st.p[4][o] = fma_rc(m2, d13, fma_rc(k33, C33, fma_rc(2.0 * k13, C13, fma_rc(k11, C11, (-k2) * C22))));
+    st.p[5][o] = fma_rc(-m2, u2, nc);
+    st.p[6][o] = (-mu) * d13;
   }
 }
 
@@ -585,66 +596,109 @@ __global__ void k_rhs_eval(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, D
 }
 
 // ------------------------------------------------------------------ RK2 update (step 6)
-// Midpoint RK2 in low-storage form at the collocation points, X^{s+1} = X^s + dt (al R^s + be R^{s-1}),
-// followed by the boundary-row solves (banded solves in place). Omega2 (blockIdx.z = 0): values at g,
-// Dirichlet rows (interpolation LU); z (blockIdx.z = 1): values at g advanced with (dz/dt)^{k_f},
-// Neumann rows dz/dy(+-1) = 0 (Neumann LU). This kernel writes the right-hand sides; rows split over
-// gridDim.y chunks.
-// m2^d (Eq. phi_poisson, blockIdx.z = 2): phi2 = (B*'' - k^2 B*) m2^d at g*_2 .. g*_{ny-2} advanced with RHS_phi2, four
-// boundary rows (no-slip or potential matching) with zero right-hand side; k = 0: m2^d = 0. Plane means <m1>, <m3>
-// (blockIdx.z = 3, one thread per row and component): values at g advanced, boundary rows zero.
-__global__ void k_update_rhs(Grid g, DBand B0g, DBand Ss0, DBand Ss2, UpdateArgs a) {
+// Midpoint RK2 in low-storage form at the collocation points, X^{s+1} = X^s + dt (al R^s + be R^{s-1}), with boundary
+// rows:
+//  * Omega2 (blockIdx.z = 0) and m2^d (blockIdx.z = 2) in increments of the coefficients: the interior rows of their
+//    solves are those that evaluate X^s, so evaluating X^s and solving is X^s itself, and X^{s+1} = X^s + A^{-1} r with r
+//    the increments and, in the boundary rows, minus those rows applied to X^s. Omega2: increments at g, Dirichlet
+//    rows (interpolation LU). m2^d (Eq. phi_poisson): increments of phi2 = (B*'' - k^2 B*) m2^d at g*_2 .. g*_{ny-2}, four
+//    boundary rows of A(k) (no-slip or potential matching); k = 0: zero.
+//  * z (blockIdx.z = 1): t = z + dt (al zdot + be zdot_prev) evaluated at g, Neumann rows dz/dy = 0 (Neumann LU). Its
+//    coefficients would be t but for the walls; but the next guess divides differences of z by dt, so z keeps the
+//    rounding of an evaluation and a solve. Each t is formed once and kept in a window of W coefficients.
+//  * plane means <m1>, <m3> (blockIdx.z = 3, one thread per row and component): values at g advanced, boundary rows zero.
+// This kernel writes the right-hand sides into the new fields; rows split over gridDim.y chunks.
+template <int W>
+__global__ void k_update_rhs(Grid g, DBand B0g, const __grid_constant__ UpdateArgs a) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   const int ny = g.ny;
   const int job = blockIdx.z;
-  const double dt = a.dt, al = a.al, be = a.be;
+  const double dal = a.dt * a.al, dbe = a.dt * a.be;
   if (job == 3) {
     if (blockIdx.y != 0 || m >= 2 * ny) return;
     const int c = m / ny, i = m - c * ny;
     const double v = i > 0 && i < ny - 1 ? band_row_real(B0g, i, c == 0 ? a.mm1 : a.mm3) +
-                                               dt * (al * a.r_m[m] + be * a.r_m_prev[m])
+                                               (dal * a.r_m[m] + dbe * a.r_m_prev[m])
                                          : 0.0;
     (c == 0 ? a.mm1_new : a.mm3_new)[i] = v;
     return;
   }
   if (m >= (int)g.M) return;
   const size_t M = g.M;
-  cd* out = job == 0 ? a.om_new : (job == 1 ? a.z_new : a.m2_new);
+  const int rows = job == 2 ? ny + 1 : ny;
   int r0, r1;
-  row_range(job == 2 ? ny + 1 : ny, blockIdx.y, gridDim.y, r0, r1);
-  const bool zero = is_nyquist(g, m) || (job != 1 && m == 0);
-  if (job == 2) {
-    double k1 = 0.0, k3 = 0.0;
-    if (!zero) wavenumbers(g, m, k1, k3);
-    const double k2 = k1 * k1 + k3 * k3;
+  row_range(rows, blockIdx.y, gridDim.y, r0, r1);
+  cd* out = job == 0 ? a.om_new : (job == 1 ? a.z_new : a.m2_new);
+  if (is_nyquist(g, m) || (job != 1 && m == 0)) {
+    for (int i = r0; i < r1; ++i) out[(size_t)i * M + m] = mk(0, 0);
+    return;
+  }
+  if (job == 1) {
+    auto t = [&](int i) {
+      if (!LMVD_IN(i, B0g.cols)) return mk(0, 0);
+      const size_t o = (size_t)i * M + m;
+      return a.z[o] + a.dt * (a.al * a.zdot[o] + a.be * a.zdot_prev[o]);
+    };
+    cd w[W];
+    int c = -(1 << 30);
     for (int i = r0; i < r1; ++i) {
       cd v = mk(0, 0);
-      if (!zero && i >= 2 && i <= ny - 2) {
-        const size_t o = (size_t)i * M + m;
-        const cd phi = band_row(Ss2, i, a.m2, M, m) - k2 * band_row(Ss0, i, a.m2, M, m);
-        v = phi + dt * (al * a.r_phi[o] + be * a.r_phi_prev[o]);
+      if (i > 0 && i < ny - 1 && LMVD_IN(i, B0g.rows)) {
+        const int ci = __ldg(B0g.c0 + i);
+        if (ci == c + 1) {
+#pragma unroll
+          for (int q = 0; q + 1 < W; ++q) w[q] = w[q + 1];
+          w[W - 1] = t(ci + W - 1);
+        } else if (ci != c) {
+#pragma unroll
+          for (int q = 0; q < W; ++q) w[q] = t(ci + q);
+        }
+        c = ci;
+        const int n = __ldg(B0g.cnt + i);
+#pragma unroll
+        for (int q = 0; q < W; ++q)
+          if (q < n) v = fma_rc(__ldg(B0g.v + (size_t)i * W + q), w[q], v);
       }
       out[(size_t)i * M + m] = v;
     }
     return;
   }
+  const cd* x = job == 0 ? a.om : a.m2;
+  const cd* r = job == 0 ? a.r_om : a.r_phi;
+  const cd* rp = job == 0 ? a.r_om_prev : a.r_phi_prev;
+  const int nb = job == 0 ? 1 : 2;  // boundary rows at each end
   for (int i = r0; i < r1; ++i) {
-    cd v = mk(0, 0);
-    if (!zero && i > 0 && i < ny - 1) {
-      if (job == 0) {
-        const size_t o = (size_t)i * M + m;
-        v = band_row(B0g, i, a.om, M, m) + dt * (al * a.r_om[o] + be * a.r_om_prev[o]);
-      } else {
-        const int c = B0g.c0[i];
-        const double* w = B0g.v + (size_t)i * B0g.w;
-        for (int q = 0; q < B0g.w; ++q) {
-          const size_t o = (size_t)(c + q) * M + m;
-          const cd zz = a.z[o] + dt * (al * a.zdot[o] + be * a.zdot_prev[o]);
-          v = fma_rc(__ldg(w + q), zz, v);
-        }
+    const size_t o = (size_t)i * M + m;
+    cd v;
+    if (i >= nb && i < rows - nb) {
+      const cd p = rp[o], q = r[o];
+      v = mk(fma(dal, q.re, dbe * p.re), fma(dal, q.im, dbe * p.im));
+    } else if (job == 0) {
+      v = band_row(B0g, i, x, M, m);
+      v = mk(-v.re, -v.im);
+    } else {
+      double k1, k3;
+      wavenumbers(g, m, k1, k3);
+      const double k2 = k1 * k1 + k3 * k3, k = sqrt(k2);
+      v = mk(0, 0);
+      for (int q = -a.md.K; q <= a.md.K; ++q) {
+        const int j = i + q;
+        if (j < 0 || j >= a.md.n) continue;
+        const size_t e = (size_t)i * (2 * a.md.K + 1) + q + a.md.K;
+        const double c = __ldg(a.md.A2 + e) - k2 * __ldg(a.md.A0 + e) + k * __ldg(a.md.A1 + e);
+        if (LMVD_IN(j, ny + 1)) v = fma_rc(-c, x[(size_t)j * M + m], v);
       }
     }
-    out[(size_t)i * M + m] = v;
+    out[o] = v;
+  }
+}
+
+void launch_update_rhs(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B0g, const UpdateArgs& a) {
+  switch (p) {
+#define LMVD_UP(P) \
+    case P: k_update_rhs<P><<<grid, tpb, 0, st>>>(g, B0g, a); break;
+    LMVD_UP(4) LMVD_UP(5) LMVD_UP(6) LMVD_UP(7) LMVD_UP(8)
+#undef LMVD_UP
   }
 }
 

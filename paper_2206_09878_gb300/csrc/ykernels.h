@@ -52,6 +52,7 @@ struct UpdateArgs {
   const double *mm1, *mm3, *r_m, *r_m_prev;
   cd *om_new, *z_new, *m2_new;
   double *mm1_new, *mm3_new;
+  DRows md;
 };
 
 struct CheckJob {
@@ -94,7 +95,7 @@ __global__ void k_mc_values(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const c
 __global__ void k_rhs_combine(Grid g, double mu, double grav, Fields10C sv, Fields7 st);
 __global__ void k_rhs_eval(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, DBand Bs2, DBand Bs3, Fields7C st,
                            cd* r_om, cd* r_phi, double* r_m);
-__global__ void k_update_rhs(Grid g, DBand B0g, DBand Ss0, DBand Ss2, UpdateArgs a);
+void launch_update_rhs(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B0g, const UpdateArgs& a);
 __global__ void k_bdf(size_t n, double a0, double a1, double a2, double a3, double idt, const cd* z, const cd* h0,
                       const cd* h1, const cd* h2, cd* out);
 __global__ void k_backfill(size_t n, double c0, double c1, double c2, const cd* z, const cd* zdot, cd* h0, cd* h1,
