@@ -154,41 +154,21 @@ __global__ void k_adj_update_om_z_post(Grid g, DBand B0gT, AdjUpd a) {
     }
   }
 }
-__global__ void k_adj_update_means(Grid g, DBand B0gT, DLU lu, AdjUpd a) {
-  const int c = threadIdx.x;
-  if (c > 1) return;
+// Plane means, one CTA: v = A^{-T} ybar per component (threads 0 and 1; boundary rows zero), then the transposed
+// evaluation and the RK coefficients over the rows.
+__global__ void __launch_bounds__(128) k_adj_update_means(Grid g, DBand B0gT, DLU lu, AdjUpd a) {
   const int ny = g.ny;
-  const double* yb = c == 0 ? a.omm1 : a.omm3;
-  double* mmb = c == 0 ? a.mm1 : a.mm3;
-  double* v = reinterpret_cast<double*>(c == 0 ? a.scr0 : a.scr1);  // ny doubles of scratch
-  double win[KMAX];
-  for (int q = 0; q < KMAX; ++q) win[q] = 0.0;
-  for (int i = 0; i < ny; ++i) {  // U^T sweep
-    double x = yb[i];
-    for (int r = 1; r <= lu.K; ++r)
-      if (i - r >= 0) x -= lu_up(lu, i - r, r, 0) * win[r - 1];
-    x *= lu.invd[i];
-    for (int q = KMAX - 1; q > 0; --q) win[q] = win[q - 1];
-    win[0] = x;
-    v[i] = x;
-  }
-  for (int q = 0; q < KMAX; ++q) win[q] = 0.0;
-  for (int i = ny - 1; i >= 0; --i) {  // L^T sweep
-    double x = v[i];
-    for (int q = 1; q <= lu.K; ++q)
-      if (i + q < ny) x -= lu_lo(lu, i + q, q, 0) * win[q - 1];
-    for (int q = KMAX - 1; q > 0; --q) win[q] = win[q - 1];
-    win[0] = x;
-    v[i] = x;
-  }
-  v[0] = 0.0;
-  v[ny - 1] = 0.0;
-  for (int j = 0; j < ny; ++j) {
-    double t = 0.0;
-    for (int q = 0; q < B0gT.w; ++q) t += B0gT.v[(size_t)j * B0gT.w + q] * v[B0gT.c0[j] + q];
-    mmb[j] += t;
-    a.rm[c * ny + j] += a.dt * a.al * v[j];
-    a.rmp[c * ny + j] += a.dt * a.be * v[j];
+  double* v0 = reinterpret_cast<double*>(a.scr0);  // ny doubles of scratch each
+  double* v1 = reinterpret_cast<double*>(a.scr1);
+  if (threadIdx.x < 2)
+    band_solve_T_piped(lu, 0, threadIdx.x == 0 ? a.omm1 : a.omm3, threadIdx.x == 0 ? v0 : v1, 1, 1, ny - 2);
+  __syncthreads();
+  for (int t = threadIdx.x; t < 2 * ny; t += blockDim.x) {
+    const int c = t / ny, j = t - c * ny;
+    const double* v = c == 0 ? v0 : v1;
+    (c == 0 ? a.mm1 : a.mm3)[j] += band_row_real(B0gT, j, v);
+    a.rm[t] += a.dt * a.al * v[j];
+    a.rmp[t] += a.dt * a.be * v[j];
   }
 }
 
@@ -220,19 +200,23 @@ struct Sv10C {
   const cd* p[10];
 };
 
+// rows split over gridDim.y chunks
 __global__ void k_adj_rhs_eval(Grid g, DBand B1gT, DBand B2gT, DBand Bs0T, DBand Bs1T, DBand Bs2T, DBand Bs3T,
                                const cd* rom, const cd* rphi, const double* rm, St7 st) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
   const int ny = g.ny;
-  for (int q = 0; q < 7; ++q)
-    for (int i = 0; i < ny; ++i) st.p[q][(size_t)i * M + m] = mk(0, 0);
+  int j0, j1;
+  row_range(ny, blockIdx.y, gridDim.y, j0, j1);
+  if (m == 0 || is_nyquist(g, m))
+    for (int q = 0; q < 7; ++q)
+      for (int i = j0; i < j1; ++i) st.p[q][(size_t)i * M + m] = mk(0, 0);
   if (is_nyquist(g, m)) return;
   if (m == 0) {
     const double* r1 = rm;
     const double* r3 = rm + ny;
-    for (int j = 0; j < ny; ++j) {
+    for (int j = j0; j < j1; ++j) {
       const size_t o = (size_t)j * M;
       st.p[1][o] = mk(band_row_real(B1gT, j, r1), 0.0);
       st.p[2][o] = mk(band_row_real(B2gT, j, r1), 0.0);
@@ -241,7 +225,7 @@ __global__ void k_adj_rhs_eval(Grid g, DBand B1gT, DBand B2gT, DBand Bs0T, DBand
     }
     return;
   }
-  for (int j = 0; j < ny; ++j) {
+  for (int j = j0; j < j1; ++j) {
     const size_t o = (size_t)j * M + m;
     st.p[0][o] = rom[o];
     st.p[1][o] = band_row(B1gT, j, rom, M, m);
@@ -364,56 +348,55 @@ struct Sv8C {
   const cd* p[8];
 };
 
-// transpose of k_eval_p1: accumulates into zbar, ombar, m2bar and the means
+// transpose of k_eval_p1, in two launches: the per-mode combinations of the eight fields, in place (each value once,
+// not once per band entry that reads it): v0 <- what multiplies B0g z, v5 and v7 <- what multiplies B0g Omega2 and Sg1
+// m2 (at k = 0 v5 and v7 stay the plane means'); then the transposed evaluations, accumulated into zbar, ombar, m2bar
+// and the means. Rows split over gridDim.y chunks.
+struct Sv8 {
+  cd* p[8];
+};
+__global__ void k_adj_p1_combine(Grid g, Sv8 v) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= (int)g.M || is_nyquist(g, m)) return;
+  const size_t M = g.M;
+  int r0, r1;
+  row_range(g.ny, blockIdx.y, gridDim.y, r0, r1);
+  double k1, k3;
+  wavenumbers(g, m, k1, k3);
+  const double k2 = k1 * k1 + k3 * k3, ik2 = m == 0 ? 0.0 : 1.0 / k2, a1 = k1 * ik2, a3 = k3 * ik2;
+  for (int i = r0; i < r1; ++i) {
+    const size_t o = (size_t)i * M + m;
+    v.p[0][o] = fma_rc(-k2, v.p[4][o], v.p[0][o] - times_i(fma_rc(k1, v.p[1][o], k3 * v.p[2][o])));
+    if (m == 0) continue;
+    const cd x = v.p[5][o], y = v.p[7][o];
+    v.p[5][o] = times_i(fma_rc(a3, x, (-a1) * y));
+    const cd d = fma_rc(a1, x, a3 * y);
+    v.p[7][o] = mk(d.im, -d.re);  // -i d
+  }
+}
 __global__ void k_adj_eval_p1(Grid g, DBand B0gT, DBand B1gT, DBand B2gT, DBand Sg0T, DBand Sg1T, Sv8C v, cd* zb,
                               cd* omb, cd* m2b, double* mm1b, double* mm3b) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M || is_nyquist(g, m)) return;
   const size_t M = g.M;
   const int ny = g.ny;
-  double k1, k3;
-  wavenumbers(g, m, k1, k3);
-  const double k2 = k1 * k1 + k3 * k3;
-  const double ik2 = m == 0 ? 0.0 : 1.0 / k2;
-  auto at = [&](int f, int i) { return v.p[f][(size_t)i * M + m]; };
-  for (int j = 0; j < ny; ++j) {
-    cd acc = mk(0, 0);
-    for (int q = 0; q < B0gT.w; ++q) {
-      const int i = B0gT.c0[j] + q;
-      const cd t0 = at(0, i) - times_i(k1 * at(1, i) + k3 * at(2, i)) - k2 * at(4, i);
-      acc = acc + __ldg(B0gT.v + (size_t)j * B0gT.w + q) * t0;
-    }
-    acc = acc + band_row(B1gT, j, v.p[3], M, m) + band_row(B2gT, j, v.p[4], M, m);
-    zb[(size_t)j * M + m] = zb[(size_t)j * M + m] + acc;
+  int r0, r1;
+  row_range(ny, blockIdx.y, gridDim.y, r0, r1);
+  for (int j = r0; j < r1; ++j) {
+    const size_t o = (size_t)j * M + m;
+    zb[o] = zb[o] + (band_row(B0gT, j, v.p[0], M, m) + band_row(B1gT, j, v.p[3], M, m) + band_row(B2gT, j, v.p[4], M, m));
     if (m == 0) {
-      double a1 = 0.0, a3 = 0.0;
-      for (int q = 0; q < B0gT.w; ++q) {
-        const int i = B0gT.c0[j] + q;
-        const double bv = __ldg(B0gT.v + (size_t)j * B0gT.w + q);
-        a1 += bv * at(5, i).re;
-        a3 += bv * at(7, i).re;
-      }
-      mm1b[j] += a1;
-      mm3b[j] += a3;
+      mm1b[j] += band_row(B0gT, j, v.p[5], M, 0).re;
+      mm3b[j] += band_row(B0gT, j, v.p[7], M, 0).re;
     } else {
-      cd ao = mk(0, 0);
-      for (int q = 0; q < B0gT.w; ++q) {
-        const int i = B0gT.c0[j] + q;
-        const cd oi = ik2 * times_i(k3 * at(5, i) - k1 * at(7, i));
-        ao = ao + __ldg(B0gT.v + (size_t)j * B0gT.w + q) * oi;
-      }
-      omb[(size_t)j * M + m] = omb[(size_t)j * M + m] + ao;
+      omb[o] = omb[o] + band_row(B0gT, j, v.p[5], M, m);
     }
   }
   if (m == 0) return;
-  for (int j = 0; j <= ny; ++j) {
-    cd acc = band_row(Sg0T, j, v.p[6], M, m);
-    for (int q = 0; q < Sg1T.w; ++q) {
-      const int i = Sg1T.c0[j] + q;
-      const cd di = (-ik2) * times_i(k1 * at(5, i) + k3 * at(7, i));
-      acc = acc + __ldg(Sg1T.v + (size_t)j * Sg1T.w + q) * di;
-    }
-    m2b[(size_t)j * M + m] = m2b[(size_t)j * M + m] + acc;
+  row_range(ny + 1, blockIdx.y, gridDim.y, r0, r1);
+  for (int j = r0; j < r1; ++j) {
+    const size_t o = (size_t)j * M + m;
+    m2b[o] = m2b[o] + (band_row(Sg0T, j, v.p[6], M, m) + band_row(Sg1T, j, v.p[7], M, m));
   }
 }
 
@@ -745,14 +728,14 @@ int adjoint_impl(Ctx& c) {
   solve_T_jobs(c, KC_UPDATE, c.lu_neumann, {SolveTJob{A.oz, u.scr1, 1, ny - 2}});
   LMVD_LAUNCH(c, KC_UPDATE, 0, 0, k_adj_update_om_z_post, dim3(mblocks(g), row_chunks(g, ny), 2), TPB, 0, g, A.B0gT,
               u);
-  LMVD_LAUNCH(c, KC_UPDATE, 0, 0, k_adj_update_means, 1, 32, 0, g, A.B0gT, c.lu_means, u);
+  LMVD_LAUNCH(c, KC_UPDATE, 0, 0, k_adj_update_means, 1, 128, 0, g, A.B0gT, c.lu_means, u);
   solve_T_jobs(c, KC_UPDATE, c.lu_md, {SolveTJob{A.om2, u.scrp, 2, ny - 2}});
   LMVD_LAUNCH(c, KC_UPDATE, 0, 0, k_adj_update_m2_post, dim3(mblocks(g), row_chunks(g, ny + 1)), TPB, 0, g, A.Ss0T,
               A.Ss2T, u);
   // step 5: RHS streams, collocation solves, transforms, products of pass 2
   St7 stw{};
   for (int q = 0; q < 7; ++q) stw.p[q] = A.st[q];
-  LMVD_LAUNCH(c, KC_RHS_EVAL, 0, 0, k_adj_rhs_eval, mblocks(g), TPB, 0, g, A.B1gT, A.B2gT, A.BsT[0], A.BsT[1],
+  LMVD_LAUNCH(c, KC_RHS_EVAL, 0, 0, k_adj_rhs_eval, dim3(mblocks(g), row_chunks(g, ny)), TPB, 0, g, A.B1gT, A.B2gT, A.BsT[0], A.BsT[1],
               A.BsT[2], A.BsT[3], A.rom, A.rphi, A.rm, stw);
   solve_T_jobs(c, KC_SOLVE, c.lu_interp,
                {SolveTJob{A.st[1], A.st[1], 0, ny - 1}, SolveTJob{A.st[2], A.st[2], 0, ny - 1},
@@ -822,8 +805,10 @@ int pass1_T(Ctx& c, AdjWork& A) {
               wbc, A.pb[8], mdbc, pbw);
   g_transpose(c, A.pb, A.sv, 8);
   Sv8C v8{};
-  for (int q = 0; q < 8; ++q) v8.p[q] = A.sv[q];
-  LMVD_LAUNCH(c, KC_EVAL_P1, 0, 0, k_adj_eval_p1, mblocks(g), TPB, 0, g, A.B0gT, A.B1gT, A.B2gT, A.Sg0T, A.Sg1T, v8,
+  Sv8 w8{};
+  for (int q = 0; q < 8; ++q) v8.p[q] = w8.p[q] = A.sv[q];
+  LMVD_LAUNCH(c, KC_EVAL_P1, 0, 0, k_adj_p1_combine, dim3(mblocks(g), row_chunks(g, g.ny)), TPB, 0, g, w8);
+  LMVD_LAUNCH(c, KC_EVAL_P1, 0, 0, k_adj_eval_p1, dim3(mblocks(g), row_chunks(g, g.ny)), TPB, 0, g, A.B0gT, A.B1gT, A.B2gT, A.Sg0T, A.Sg1T, v8,
               A.z, A.om, A.m2, A.mm1, A.mm3);
   // lmvd_set_state zeroes these entries of the state, so the substage does not depend on them
   LMVD_LAUNCH(c, KC_MISC, 0, 0, k_sanitize, eblocks(S), 256, 0, g, g.ny, A.z, 0);
