@@ -462,7 +462,7 @@ def cufft_comparison(L, w, stream, df_prof=None, steps=None, kf=4, reps=5):
             del real, spec_c, zbuf, spec_o
             torch.cuda.empty_cache()
     if df_prof and steps:
-        n_inv, n_fwd = 8 + 4 * (kf + 1), 12 + 2 * kf
+        n_inv, n_fwd = 8 + 4 * (kf + 1), 11 + 2 * kf
         out["lmvd_df_inverse"] = (df_prof["fft_z_inverse"][0] + df_prof["fft_x_inverse"][0]) / steps / n_inv
         out["lmvd_df_forward"] = (df_prof["fft_x_forward"][0] + df_prof["fft_z_forward"][0]) / steps / n_fwd
     return {"unit": "ms per field", "grid": [nx, ny, nz], "padded": [px, ny, pz], **out,

@@ -78,9 +78,9 @@ extern "C" {
  *               Omega2 = 0, d<m1>/dy = d<m3>/dy = 0, dz/dy = 0, <m2^c>(y1) = 0. Both modes put the
  *               boundary rows first and last in each per-mode system and factor it without pivoting.
  * memory_layout: 0 = automatic (the full layout unless its workspace would take more than 85% of the
- *               free device memory), 1 = full, 2 = lean (6 instead of 10 physical work fields, the products
+ *               free device memory), 1 = full, 2 = lean (6 instead of 9 physical work fields, the products
  *               of the RHS formed in three batches instead of one, a 2-field instead of 4-field transform
- *               intermediate: the same results in about 43 GB less at 768 x 769 x 768).
+ *               intermediate: the same results in about 35 GB less at 768 x 769 x 768).
  */
 typedef struct {
   int nx, ny, nz, spline_order;

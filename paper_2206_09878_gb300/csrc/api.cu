@@ -495,9 +495,10 @@ void mc_from_zdot(Ctx& c, bool from_eval, bool coefficients, double* a = nullptr
 }
 
 // one application of the fixed point (Eq. y_k) on the values of zdot: zdot <- L(z) zdot + R_z; with `coefficients` also
-// its B coefficients
-void fp_apply(Ctx& c, bool from_eval, bool coefficients, double* a = nullptr, double* const* b = nullptr) {
-  mc_from_zdot(c, from_eval, false, a, b);
+// its B coefficients, with `mc_coefficients` those of the m^c it formed
+void fp_apply(Ctx& c, bool from_eval, bool coefficients, bool mc_coefficients, double* a = nullptr,
+              double* const* b = nullptr) {
+  mc_from_zdot(c, from_eval, mc_coefficients, a, b);
   double* bb[3] = {c.pw[0], c.pw[1], c.pw[2]};
   if (b)
     for (int f = 0; f < 3; ++f) bb[f] = b[f];
@@ -520,7 +521,8 @@ void startup(Ctx& c, const Tape* tape = nullptr, cd* iterates = nullptr) {
   for (int it = 0; it < c.cfg.n_startup; ++it) {
     if (iterates)
       cudaMemcpyAsync(iterates + (size_t)it * S, c.zdot, sizeof(cd) * S, cudaMemcpyDeviceToDevice, c.stream);
-    fp_apply(c, false, iterates || it == c.cfg.n_startup - 1);
+    const bool last = it == c.cfg.n_startup - 1;  // the fields it leaves can be read (lmvd_get_field)
+    fp_apply(c, false, iterates || last, last);
   }
   const double dt = c.cfg.dt;
   LMVD_LAUNCH(c, KC_MISC, 12.0 * S, 80.0 * S, k_backfill, elem_blocks(S), 256, 0, S, 0.5 * dt, dt, 1.5 * dt, c.z,
@@ -563,7 +565,7 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
     // diagnostics: the change of this application (the previous iterate kept in sv[9], unused until pass 2)
     if (c.diag_on && k < KF_MAX_ADJ + 1)
       cudaMemcpyAsync(c.sv[9], c.zdot, sizeof(cd) * S, cudaMemcpyDeviceToDevice, c.stream);
-    fp_apply(c, k == 0, c.diag_on || k == cf.kf - 1, tape ? tape->a[k] : nullptr, tape ? tape->b[k] : nullptr);
+    fp_apply(c, k == 0, c.diag_on || k == cf.kf - 1, false, tape ? tape->a[k] : nullptr, tape ? tape->b[k] : nullptr);
     if (c.diag_on && k < KF_MAX_ADJ + 1)
       LMVD_LAUNCH(c, KC_MISC, 6.0 * S, 32.0 * S, k_diff_norms, elem_blocks(S), 256, 0, S, c.zdot, c.sv[9],
                   c.ddiag + 2 + 2 * k);
@@ -581,11 +583,11 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
   nvtxRangePop();
   nvtxRangePushA("steps 4-5: pass 2, RHS");
   // steps 4-5: products with m = m^d + m^c, forward transforms, RHS streams, collocation solves, RHS.
-  // The ten products overwrite m^c where it sits in pw[0..2] (each point's inputs are read before its
-  // outputs are written): one batch into pw[0..9] in the full layout; in the lean one (6 work fields)
-  // C11-C13 and C22-C33 through pw[3..5], then u and rho into pw[0..3].
+  // The nine products overwrite m^c where it sits in pw[0..2] (each point's inputs are read before its
+  // outputs are written): one batch into pw[0..8] in the full layout; in the lean one (6 work fields)
+  // C11 - C22 .. C13 and C23, C33 - C22 through pw[3..5], then u and rho into pw[0..3].
   struct Batch { int first, count, slot; };
-  const Batch full[1] = {{0, 10, 0}}, lean[3] = {{0, 3, 3}, {3, 3, 3}, {6, 4, 0}};
+  const Batch full[1] = {{0, 9, 0}}, lean[3] = {{0, 3, 3}, {3, 2, 3}, {5, 4, 0}};
   if (c.diag_on) {
     // kinetic energy and max |m| of m = m^d + m^c (before the products overwrite m^c), <m2^c> at y0
     Fields3C mdf{{c.md[0], c.md[1], c.md[2]}}, mcf{{mcp[0], mcp[1], mcp[2]}};
@@ -594,8 +596,8 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
                 reinterpret_cast<unsigned long long*>(c.ddiag + DIAG_MMAX));
     cudaMemcpyAsync(c.ddiag + DIAG_MC2, c.m2c, sizeof(double), cudaMemcpyDeviceToDevice, c.stream);
   }
-  const Batch* batches = c.pw_n >= 10 ? full : lean;
-  const int nb = c.pw_n >= 10 ? 1 : 3;
+  const Batch* batches = c.pw_n >= PW_FIELDS ? full : lean;
+  const int nb = c.pw_n >= PW_FIELDS ? 1 : 3;
   for (int b = 0; b < nb; ++b) {
     const Batch& bt = batches[b];
     P2Out q{};
@@ -605,11 +607,11 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
                   mcp[0], mcp[1], mcp[2], c.rho, c.invrho, q);
     fft_forward(c, c.pw + bt.slot, c.sv + bt.first, bt.count);
   }
-  Fields10C svc{};
-  for (int f = 0; f < 10; ++f) svc.p[f] = c.sv[f];
+  Fields9C svc{};
+  for (int f = 0; f < 9; ++f) svc.p[f] = c.sv[f];
   Fields7 stw{};
   for (int f = 0; f < 7; ++f) stw.p[f] = c.st[f];
-  LMVD_LAUNCH(c, KC_RHS_COMBINE, 60.0 * S, 16.0 * 17 * S, k_rhs_combine, dim3(mode_blocks(g), row_chunks(g, g.ny)),
+  LMVD_LAUNCH(c, KC_RHS_COMBINE, 56.0 * S, 16.0 * 16 * S, k_rhs_combine, dim3(mode_blocks(g), row_chunks(g, g.ny)),
               TPB_MODE, 0, g, 1.0 / cf.re, 1.0 / (cf.fr * cf.fr), svc, stw);
   const DLU* li = &c.lu_interp;
   solve_modes(c, KC_SOLVE, {SolveReq{SolveJob{c.st[1], nullptr, c.st[1]}, li}, SolveReq{SolveJob{c.st[2], nullptr, c.st[2]}, li},
@@ -786,7 +788,7 @@ int startup_record(Ctx& c, const Tape* tape, cd* iterates) {
 int fp_record(Ctx& c, const cd* zdot_in, double* a, double* const* b) {
   cudaMemcpyAsync(c.zdot, zdot_in, sizeof(cd) * c.g.ny * c.g.M, cudaMemcpyDeviceToDevice, c.stream);
   zdot_values(c);
-  fp_apply(c, true, true, a, b);
+  fp_apply(c, true, true, true, a, b);
   return cudaGetLastError() == cudaSuccess ? LMVD_OK : LMVD_ERR_CUDA;
 }
 }  // namespace lmvd

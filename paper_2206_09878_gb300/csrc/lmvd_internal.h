@@ -53,7 +53,7 @@ constexpr int KMAX = 8;   // widest band (each side) of any y-system LU supporte
 // streams overwrite the first seven spectral value fields. When that layout would not leave room on the
 // device (768 x 769 x 768), lmvd_create uses the lean one: TBUF_LEAN and PW_LEAN fields.
 constexpr int TBUF_FIELDS = 4;
-constexpr int PW_FIELDS = 10;
+constexpr int PW_FIELDS = 9;
 constexpr int TBUF_LEAN = 2;
 constexpr int PW_LEAN = 6;
 constexpr int WMAX = 9;   // widest row of a collocation matrix (spline order <= 9)

@@ -46,24 +46,25 @@ __global__ void k_product_L(size_t n, const double* w1, const double* w2, const 
     out[o] = -(w1[o] * m1[o] + w2[o] * m2[o] + w3[o] * m3[o]);
 }
 
-// m = m^d + m^c; outputs C11, C12, C13, C22, C23, C33 (C_ij = -m_i m_j / rho), u1, u2, u3 (u = m / rho), rho;
-// a null output pointer is skipped (the outputs are formed in batches)
+// m = m^d + m^c, u = m / rho, C_ij = -m_i m_j / rho; outputs C11 - C22, C12, C13, C23, C33 - C22, u1, u2, u3, rho (an
+// isotropic part of C is a gradient and cancels in both curls, so C22 needs no transform of its own); a null output
+// pointer is skipped (the outputs are formed in batches)
 __global__ void k_products_p2(size_t n, const double* md1, const double* md2, const double* md3, const double* mc1,
                               const double* mc2, const double* mc3, const double* rho, const double* invrho, P2Out q) {
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const double ir = invrho[o];
     const double a = md1[o] + mc1[o], b = md2[o] + mc2[o], c = md3[o] + mc3[o];
     const double ua = a * ir, ub = b * ir, uc = c * ir;
-    if (q.p[0]) q.p[0][o] = -a * ua;
+    const double c22 = b * ub;
+    if (q.p[0]) q.p[0][o] = fma(-a, ua, c22);
     if (q.p[1]) q.p[1][o] = -a * ub;
     if (q.p[2]) q.p[2][o] = -a * uc;
-    if (q.p[3]) q.p[3][o] = -b * ub;
-    if (q.p[4]) q.p[4][o] = -b * uc;
-    if (q.p[5]) q.p[5][o] = -c * uc;
-    if (q.p[6]) q.p[6][o] = ua;
-    if (q.p[7]) q.p[7][o] = ub;
-    if (q.p[8]) q.p[8][o] = uc;
-    if (q.p[9]) q.p[9][o] = rho[o];
+    if (q.p[3]) q.p[3][o] = -b * uc;
+    if (q.p[4]) q.p[4][o] = fma(-c, uc, c22);
+    if (q.p[5]) q.p[5][o] = ua;
+    if (q.p[6]) q.p[6][o] = ub;
+    if (q.p[7]) q.p[7][o] = uc;
+    if (q.p[8]) q.p[8][o] = rho[o];
   }
 }
 

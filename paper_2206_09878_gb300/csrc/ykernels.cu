@@ -511,16 +511,16 @@ __global__ void k_mc_values(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const c
 }
 
 // ------------------------------------------------------------------ RHS streams (Eq. DNS_system)
-// sv[0..9] = C11, C12, C13, C22, C23, C33, u1, u2, u3, rho at the Greville points (values).
-// With H_i = d_j C_ij + mu lap u_i - g rho delta_i2 (the (1/3) grad div u part of the viscous force is
-// a gradient and cancels in both curls):
+// sv[0..8] = C11 - C22, C12, C13, C23, C33 - C22, u1, u2, u3, rho at the Greville points (values).
+// With H_i = d_j C_ij + mu lap u_i - g rho delta_i2 (the (1/3) grad div u part of the viscous force and C22 delta_ij
+// are gradients and cancel in both curls):
 //   RHS_Omega2 = i k3 H1 - i k1 H3 = st0 + d/dy st1 + d2/dy2 st2,
 //   RHS_phi2 = -k^2 H2 - d/dy (i k1 H1 + i k3 H3) = st3 + d/dy st4 + d2/dy2 st5 + d3/dy3 st6,
 // so only st1..st6 need B-spline coefficients (st0 is already the value at g).
 // k = 0: st1 = <C12>, st2 = mu <u1>, st4 = <C23>, st5 = mu <u3> carry the mean equations
 // (Eq. mean_m1m3); the k = 0 values of all seven streams vanish otherwise.
 // One thread per mode and row chunk: the multipliers are formed once per mode.
-__global__ void k_rhs_combine(Grid g, double mu, double grav, Fields10C sv, Fields7 st) {
+__global__ void k_rhs_combine(Grid g, double mu, double grav, Fields9C sv, Fields7 st) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -534,7 +534,7 @@ __global__ void k_rhs_combine(Grid g, double mu, double grav, Fields10C sv, Fiel
   if (m == 0) {
     for (int i = r0; i < r1; ++i) {
       const size_t o = (size_t)i * M;
-      const cd C12 = sv.p[1][o], C23 = sv.p[4][o], u1 = sv.p[6][o], u3 = sv.p[8][o];
+      const cd C12 = sv.p[1][o], C23 = sv.p[3][o], u1 = sv.p[5][o], u3 = sv.p[7][o];
       st.p[0][o] = st.p[3][o] = st.p[6][o] = mk(0, 0);
       st.p[1][o] = C12;
       st.p[2][o] = mu * u1;
@@ -548,17 +548,17 @@ __global__ void k_rhs_combine(Grid g, double mu, double grav, Fields10C sv, Fiel
   const double k11 = k1 * k1, k33 = k3 * k3, k13 = k1 * k3, k2 = k11 + k33, kd = k11 - k33, m2 = mu * k2, m4 = m2 * k2;
   for (int i = r0; i < r1; ++i) {
     const size_t o = (size_t)i * M + m;
-    const cd C11 = sv.p[0][o], C12 = sv.p[1][o], C13 = sv.p[2][o], C22 = sv.p[3][o], C23 = sv.p[4][o], C33 = sv.p[5][o],
-             u1 = sv.p[6][o], u2 = sv.p[7][o], u3 = sv.p[8][o], rho = sv.p[9][o];
+    const cd D11 = sv.p[0][o], C12 = sv.p[1][o], C13 = sv.p[2][o], C23 = sv.p[3][o], D33 = sv.p[4][o], u1 = sv.p[5][o],
+             u2 = sv.p[6][o], u3 = sv.p[7][o], rho = sv.p[8][o];
     const cd w13 = times_i(fma_rc(k3, u1, (-k1) * u3));      // i k3 u1 - i k1 u3
     const cd d13 = times_i(fma_rc(k1, u1, k3 * u3));         // i k1 u1 + i k3 u3
     const cd c1223 = times_i(fma_rc(k1, C12, k3 * C23));     // i k1 C12 + i k3 C23
     const cd nc = mk(-c1223.re, -c1223.im);
-    st.p[0][o] = fma_rc(-m2, w13, fma_rc(kd, C13, k13 * (C33 - C11)));
+    st.p[0][o] = fma_rc(-m2, w13, fma_rc(kd, C13, k13 * (D33 - D11)));
     st.p[1][o] = times_i(fma_rc(k3, C12, (-k1) * C23));
     st.p[2][o] = mu * w13;
     st.p[3][o] = fma_rc(m4, u2, k2 * fma_rc(grav, rho, nc));
-    st.p[4][o] = fma_rc(m2, d13, fma_rc(k33, C33, fma_rc(2.0 * k13, C13, fma_rc(k11, C11, (-k2) * C22))));
+    st.p[4][o] = fma_rc(m2, d13, fma_rc(k33, D33, fma_rc(2.0 * k13, C13, k11 * D11)));
     st.p[5][o] = fma_rc(-m2, u2, nc);
     st.p[6][o] = (-mu) * d13;
   }

@@ -13,8 +13,8 @@ struct Fields7 {
 struct Fields7C {
   const cd* p[7];
 };
-struct Fields10C {
-  const cd* p[10];
+struct Fields9C {
+  const cd* p[9];
 };
 struct EvalJob {
   DBand B;
@@ -92,7 +92,7 @@ __global__ void k_solve_piped(Grid g, const __grid_constant__ PipedJobs jobs);
 __global__ void k_mc_rhs(Grid g, DBand Bs1, const double* dstar, const cd* rt, cd* m2c);
 __global__ void k_mc_post(Grid g, const double* dstar, const cd* rt, cd* m1c, const cd* m2c, cd* m3c);
 __global__ void k_mc_values(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const cd* m2c, cd* v1, cd* v2, cd* v3);
-__global__ void k_rhs_combine(Grid g, double mu, double grav, Fields10C sv, Fields7 st);
+__global__ void k_rhs_combine(Grid g, double mu, double grav, Fields9C sv, Fields7 st);
 __global__ void k_rhs_eval(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, DBand Bs2, DBand Bs3, Fields7C st,
                            cd* r_om, cd* r_phi, double* r_m);
 void launch_update_rhs(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B0g, const UpdateArgs& a);
@@ -116,7 +116,7 @@ __global__ void k_product_rt(size_t n, const double* fprime, const double* zdot,
 __global__ void k_product_L(size_t n, const double* w1, const double* w2, const double* w3, const double* m1,
                             const double* m2, const double* m3, double* out);
 struct P2Out {
-  double* p[10];
+  double* p[9];
 };
 __global__ void k_products_p2(size_t n, const double* md1, const double* md2, const double* md3, const double* mc1,
                               const double* mc2, const double* mc3, const double* rho, const double* invrho, P2Out o);

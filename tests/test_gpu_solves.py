@@ -38,6 +38,21 @@ def test_state_matches_oracle(L, p, ny, bc):
     assert all(v <= 1e-12 for v in e.values()), e
 
 
+@pytest.mark.parametrize("precision", [0, 1])
+def test_fields_after_the_start_up(L, precision):
+    """rho_t and m^c of the last start-up application can be read and conserve mass (to rounding: an m^c of
+    double-float transforms is still solved for in FP64)."""
+    from _pairs import make_pair, to_torch
+    S, ctx, st, cfg = make_pair(L, "rt32", precision=precision)
+    ctx.set_state(to_torch(st))
+    rt, m1, m2, m3 = (ctx.field(f).cpu().numpy() for f in (L.LMVD_FIELD_RHO_T, L.LMVD_FIELD_MC1, L.LMVD_FIELD_MC2,
+                                                           L.LMVD_FIELD_MC3))
+    ctx.close()
+    for m in (m1, m2, m3):
+        assert np.abs(m).max() > 0
+    assert np.linalg.norm(S.mass_residual(rt, (m1, m2, m3))) <= 1e-12 * np.linalg.norm(rt)
+
+
 @pytest.mark.parametrize("p,ny", [(4, 10), (5, 24), (7, 30), (8, 45)])
 def test_adjoint_directional_derivative(L, p, ny):
     from _pairs import make_pair, to_torch
