@@ -159,7 +159,7 @@ __device__ __forceinline__ void fx_middle(cfx* x, const FFTPlan& pl, int s0, int
     if (EPT == 12 && r2 == 0) {
       fx_stage<SIGN, 4, EPT, S>(x, pl, L, tt, tpt);
       L *= 4;
-    } else if (EPT == 12 && r2 == 1) {
+    } else if (r2 == 1) {
       fx_stage<SIGN, 2, EPT, S>(x, pl, L, tt, tpt);
       L *= 2;
     } else {
@@ -757,19 +757,19 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
 // Radix order 4s, 2s, 3s, then the last stage's 12 (6 when n has a single factor 2): the sub-length L is a power of
 // two in every radix-4/2 stage (mask arithmetic). 12 (6) elements per thread; at most cta threads per
 // CTA (so n <= 12 cta); one shared buffer of batch transforms with leading dimension n + pad.
-static bool make_plan(int n, int cta, FFTPlan& p) {
+static bool make_plan(int n, int cta, FFTPlan& p, int ept = 0) {
   p.n = n;
   p.nst = 0;
-  p.ept = (n % 12 == 0) ? 12 : ((n % 6 == 0) ? 6 : 0);
-  if (!p.ept) return false;
+  p.ept = ept ? ept : (n % 12 == 0) ? 12 : ((n % 6 == 0) ? 6 : 0);
+  if (!p.ept || n % p.ept) return false;
   p.tpt = n / p.ept;
   p.code = 0;
   int m = p.tpt;
-  for (int r : {4, 2, 3})
-    for (; m % r == 0; m /= r) p.code |= (unsigned)(r == 4 ? 0 : (r == 2 ? 1 : 2)) << (2 * p.nst++);
+  for (int r : {4, 2, 3})  // (6 elements per thread hold no radix-4 butterflies)
+    for (; m % r == 0 && !(r == 4 && p.ept == 6); m /= r) p.code |= (unsigned)(r == 4 ? 0 : (r == 2 ? 1 : 2)) << (2 * p.nst++);
   if (m != 1 || p.nst > 15) return false;
   ++p.nst;  // the last stage, radix ept
-  p.first4 = p.tpt % 4 == 0;
+  p.first4 = p.ept == 12 && p.tpt % 4 == 0;
   if (p.tpt > cta) return false;
   for (p.red_g = 1; p.tpt % (2 * p.red_g) == 0 && p.red_g < (cta == FFT_CTA_Z ? 8 : 32);) p.red_g *= 2;
   const long double s3 = sqrtl(3.0L) / 2.0L;
@@ -793,6 +793,21 @@ static bool make_plan(int n, int cta, FFTPlan& p) {
     if (!p.rows_in || !p.rows_t) return false;
   }
   return true;
+}
+
+// A launch with few transforms is a chain of one thread's instructions (about 250 per element, one or two warps per
+// SM), so it takes the plan with 6 elements per thread where there is one (twice the threads, radix-2 stages for radix-4
+// ones). 32 x 33 x 32, per substage: the four passes 0.128 / 0.167 / 0.150 / 0.143 -> 0.119 / 0.141 / 0.137 / 0.133 ms,
+// 72 x 61 x 48: 0.187 / 0.244 / 0.220 / 0.200 -> 0.155 / 0.218 / 0.184 / 0.169. The line: fewer than 384 threads per SM
+// with 12 elements each (128: 72 x 61 x 48 loses 4%, 512: 64 x 65 x 64 loses 1%).
+constexpr double FFT_SMALL_THREADS = 152 * 384;
+static const FFTPlan& pick_plan(const FFTPlan& full, const FFTPlan& small, double transforms) {
+  return small.n && transforms * full.tpt < FFT_SMALL_THREADS ? small : full;
+}
+static void make_small_plan(const FFTPlan& full, int cta, FFTPlan& p) {
+  if (full.ept != 12 || !make_plan(full.n, cta, p, 6)) p.n = 0;
+  p.tw = full.tw;
+  p.scale_d = full.scale_d;
 }
 
 // a pass's buffer is followed by its mbarrier (the z-passes' and the inverse x-pass's copies)
@@ -877,6 +892,8 @@ int fft_prepare(Ctx& c) {
     p->tw = d;
     p->scale_d = (double)(scale / 2);  // used by the forward z-pass (see the file head)
   }
+  make_small_plan(c.fx, FFT_CTA_X, c.fx6);
+  make_small_plan(c.fz, FFT_CTA_Z, c.fz6);
   return set_smem();
 }
 
@@ -894,7 +911,7 @@ static void map_failed(Ctx& c) {
 template <class RAW>
 static void z_inv_launch(Ctx& c, const FieldsC& fi, int n, size_t tstride, double fl, double by) {
   const Grid& g = c.g;
-  const FFTPlan& p = c.fz;
+  const FFTPlan& p = pick_plan(c.fz, c.fz6, (double)(g.nx / 2) * g.ny * n);
   ZMaps maps;
   for (int f = 0; f < n; ++f)
     if (!tile_map(&maps.m[f], fi.p[f], g.nxh, g.nz, g.ny, p.batch, p.rows_in)) {
@@ -915,7 +932,7 @@ static void z_inv_launch(Ctx& c, const FieldsC& fi, int n, size_t tstride, doubl
 
 static void z_fwd_launch(Ctx& c, int n, const FieldsW& fo, double fl, double by, const cd* add = nullptr) {
   const Grid& g = c.g;
-  const FFTPlan& p = c.fz;
+  const FFTPlan& p = pick_plan(c.fz, c.fz6, (double)(g.nx / 2 + 1) * g.ny * n);
   ZMaps maps;
   if (!tile_map(&maps.m[0], c.tbuf, g.nx / 2, g.pz, (size_t)n * g.ny, p.batch, p.rows_t)) {
     map_failed(c);
@@ -949,20 +966,21 @@ static void inverse(Ctx& c, cd* const* in, double* const* out, int nf, bool df_i
     const double zfl = n * ny * h * fft_flops(pz), zby = n * ny * h * 16.0 * ((g.nz - 1) + pz);
     if (df_in) z_inv_launch<cdf>(c, fi, n, tstride, zfl, zby);
     else z_inv_launch<cd>(c, fi, n, tstride, zfl, zby);
-    dim3 gx(cdiv(cdiv(g.pz, 2), c.fx.batch), g.ny, n);
+    const FFTPlan& p = pick_plan(c.fx, c.fx6, 0.5 * g.pz * g.ny * n);
+    dim3 gx(cdiv(cdiv(g.pz, 2), p.batch), g.ny, n);
     const double xfl = n * ny * ((g.pz + 1) / 2) * fft_flops(px), xby = n * ny * pz * (16.0 * h + 8.0 * px);
     if (wmul) {  // the product with w in the epilogue: one more physical field read, one multiply per point
-      if (c.fx.ept == 12)
+      if (p.ept == 12)
         LMVD_LAUNCH(c, KC_FFT_X_INV, xfl + n * ny * pz * px, xby + n * ny * pz * 8.0 * px, k_fft_x_inv_mul<12>, gx,
-                    threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf, tstride, c.texp, fo, wmul, c.dflags);
+                    threads(p), smem_bytes(p), p, g, c.tbuf, tstride, c.texp, fo, wmul, c.dflags);
       else
         LMVD_LAUNCH(c, KC_FFT_X_INV, xfl + n * ny * pz * px, xby + n * ny * pz * 8.0 * px, k_fft_x_inv_mul<6>, gx,
-                    threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf, tstride, c.texp, fo, wmul, c.dflags);
-    } else if (c.fx.ept == 12) {
-      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, k_fft_x_inv<12>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf,
+                    threads(p), smem_bytes(p), p, g, c.tbuf, tstride, c.texp, fo, wmul, c.dflags);
+    } else if (p.ept == 12) {
+      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, k_fft_x_inv<12>, gx, threads(p), smem_bytes(p), p, g, c.tbuf,
                   tstride, c.texp, fo, c.dflags);
     } else {
-      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, k_fft_x_inv<6>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf,
+      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, k_fft_x_inv<6>, gx, threads(p), smem_bytes(p), p, g, c.tbuf,
                   tstride, c.texp, fo, c.dflags);
     }
   }
@@ -980,13 +998,14 @@ void fft_forward(Ctx& c, double* const* in, cd* const* out, int nf) {
       fo.p[f] = out[f0 + f];
     }
     const double h = g.nx / 2, ny = g.ny, pz = g.pz, px = g.px;
-    dim3 gx(cdiv(cdiv(g.pz, 2), c.fx.batch), g.ny, n);
-    if (c.fx.ept == 12)
+    const FFTPlan& p = pick_plan(c.fx, c.fx6, 0.5 * g.pz * g.ny * n);
+    dim3 gx(cdiv(cdiv(g.pz, 2), p.batch), g.ny, n);
+    if (p.ept == 12)
       LMVD_LAUNCH(c, KC_FFT_X_FWD, n * ny * ((g.pz + 1) / 2) * fft_flops(px), n * ny * pz * (16.0 * h + 8.0 * px),
-                  k_fft_x_fwd<12>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, fi, c.tbuf, tstride, c.texp);
+                  k_fft_x_fwd<12>, gx, threads(p), smem_bytes(p), p, g, fi, c.tbuf, tstride, c.texp);
     else
       LMVD_LAUNCH(c, KC_FFT_X_FWD, n * ny * ((g.pz + 1) / 2) * fft_flops(px), n * ny * pz * (16.0 * h + 8.0 * px),
-                  k_fft_x_fwd<6>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, fi, c.tbuf, tstride, c.texp);
+                  k_fft_x_fwd<6>, gx, threads(p), smem_bytes(p), p, g, fi, c.tbuf, tstride, c.texp);
     z_fwd_launch(c, n, fo, n * ny * h * fft_flops(pz), n * ny * 16.0 * (pz * h + (double)g.nz * g.nxh));
   }
 }
@@ -1003,13 +1022,14 @@ void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, co
   FieldsW fo{};
   fo.p[0] = out;
   const double h = g.nx / 2, ny = g.ny, pz = g.pz, px = g.px;
-  dim3 gx(cdiv(cdiv(g.pz, 2), c.fx.batch), g.ny, 1);
+  const FFTPlan& p = pick_plan(c.fx, c.fx6, 0.5 * g.pz * g.ny * 1);
+    dim3 gx(cdiv(cdiv(g.pz, 2), p.batch), g.ny, 1);
   const double xfl = ny * ((g.pz + 1) / 2) * fft_flops(px) + 6.0 * ny * pz * px, xby = ny * pz * (16.0 * h + 48.0 * px);
-  if (c.fx.ept == 12)
-    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, k_fft_x_fwd_dot3<12>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf,
+  if (p.ept == 12)
+    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, k_fft_x_fwd_dot3<12>, gx, threads(p), smem_bytes(p), p, g, c.tbuf,
                 tstride, c.texp, d);
   else
-    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, k_fft_x_fwd_dot3<6>, gx, threads(c.fx), smem_bytes(c.fx), c.fx, g, c.tbuf,
+    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, k_fft_x_fwd_dot3<6>, gx, threads(p), smem_bytes(p), p, g, c.tbuf,
                 tstride, c.texp, d);
   z_fwd_launch(c, 1, fo, ny * h * fft_flops(pz), ny * 16.0 * (pz * h + 2.0 * g.nz * g.nxh), add);
 }
@@ -1141,6 +1161,11 @@ extern "C" int lmvd_inverse_transform_noalloc(int nx, int ny, int nz, const void
   k_twiddles<<<(g.pz + 255) / 256, 256, 0, st>>>((int4*)(sb + off_tz), g.pz);
   if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
   const size_t S = (size_t)ny * g.M, P = (size_t)ny * g.P;
+  FFTPlan fx6, fz6;
+  make_small_plan(fx, FFT_CTA_X, fx6);
+  make_small_plan(fz, FFT_CTA_Z, fz6);
+  fx = pick_plan(fx, fx6, 0.5 * g.pz * ny);
+  fz = pick_plan(fz, fz6, (double)(nx / 2) * ny);
   for (int f = 0; f < nfields; ++f) {
     FieldsC fi{};
     FieldsRW fo{};

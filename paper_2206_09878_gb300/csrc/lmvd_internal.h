@@ -256,6 +256,7 @@ struct Ctx {
   DLU lu_means;  // lu_interp (walls) or lu_neumann (potential matching): not owned
   DRows md_rows;              // the m2^d system (its boundary rows are evaluated by the RK update)
   FFTPlan fx, fz;
+  FFTPlan fx6, fz6;  // the same lengths with 6 elements per thread, for launches with few transforms (n = 0: none)
 
   // memory arena
   void* arena = nullptr;
