@@ -100,7 +100,7 @@ __global__ void k_solve_T_cd(Grid g, DLU lu, SolveTJobs jobs) {
     for (int i = 0; i < lu.n; ++i) jb.out[(size_t)i * g.M + m] = mk(0, 0);
     return;
   }
-  band_solve_T_v<cd>(lu, (int)m, lu.mstride ? factor_mode(g, (int)m) : 0, 0, jb.in, jb.out, g.M, jb.zlo, jb.zhi);
+  band_solve_T_cd(lu, (int)m, lu.mstride ? factor_mode(g, (int)m) : 0, jb.in, jb.out, g.M, jb.zlo, jb.zhi);
 }
 __global__ void __launch_bounds__(128) k_solve_T_piped(Grid g, DLU lu, const __grid_constant__ SolveTJobs jobs) {
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;

@@ -17,54 +17,39 @@ __device__ inline double lu_invd(const DLU& f, int i, int mf) {
 }
 
 // Banded solves with the LU factors, for right-hand sides stored complex [row][mode]. Every y-system
-// matrix is real, so the real and imaginary parts of a right-hand side are independent recurrences. A
-// thread solves one element type V of one mode: V = cd (both parts; one thread per mode, each factor
-// loaded once per mode) or V = double (one part, comp 0 = real, 1 = imaginary; two threads per mode).
-// The second halves each thread's chain of dependent FP64 operations, which is what bounds these solves
-// when the grid has few Fourier modes (GB300 retires 2 FP64 lanes per clock per SM, so a lone warp's
-// dependent FP64 instruction costs ~64 cycles); with many modes the FP64 pipe is saturated either way
-// and the first reads half as many factor words. A warp's accesses stay contiguous in both (16 modes x
-// 2 parts, or 32 modes, of one row).
-__device__ inline double vfma(double s, double x, double acc) { return fma(s, x, acc); }
-__device__ inline cd vfma(double s, cd x, cd acc) { return fma_rc(s, x, acc); }
-template <class V>
-__device__ inline V vzero() {
-  return V{};
-}
-
-// Element (i, m) of a [row][mode] complex array seen as V: its index in V units
-template <class V>
-__device__ inline size_t vidx(int i, size_t M, int m, int comp) {
-  return sizeof(V) == sizeof(cd) ? (size_t)i * M + m : ((size_t)i * M + m) * 2 + comp;
-}
+// matrix is real, so the real and imaginary parts of a right-hand side are independent recurrences. With
+// many modes a thread solves both parts of one mode (band_solve_cd, band_solve_T_cd): the FP64 pipe is
+// saturated and each factor is loaded once per mode. With few modes it solves one part (band_solve_piped,
+// band_solve_T_piped), which halves each thread's chain of dependent FP64 operations, the bound there
+// (GB300 retires 2 FP64 lanes per clock per SM, so a lone warp's dependent FP64 instruction costs ~64
+// cycles). A warp's accesses stay contiguous in both (32 modes, or 16 modes x 2 parts, of one row).
 
 // L U x = in, then out = x (+ add). out may alias in; add may be null.
-template <class V>
-__device__ void band_solve_v(const DLU& f, int m, int mf, int comp, const V* in, const V* add, V* out, size_t M) {
+__device__ inline void band_solve_cd(const DLU& f, int m, int mf, const cd* in, const cd* add, cd* out, size_t M) {
   if (!LMVD_IN(m, M) || (f.mstride && !LMVD_IN(mf, f.mstride)) || !LMVD_IN(f.K, KMAX + 1)) return;
-  V win[KMAX];
+  cd win[KMAX];
 #pragma unroll
-  for (int q = 0; q < KMAX; ++q) win[q] = vzero<V>();
+  for (int q = 0; q < KMAX; ++q) win[q] = cd{};
   for (int i = 0; i < f.n; ++i) {
-    V v = in[vidx<V>(i, M, m, comp)];
+    cd v = in[(size_t)i * M + m];
     const int nl = __ldg(f.nl + i);
 #pragma unroll
     for (int q = 1; q <= KMAX; ++q)
-      if (q <= nl) v = vfma(-lu_lo(f, i, q, mf), win[q - 1], v);
+      if (q <= nl) v = fma_rc(-lu_lo(f, i, q, mf), win[q - 1], v);
 #pragma unroll
     for (int q = KMAX - 1; q > 0; --q) win[q] = win[q - 1];
     win[0] = v;
-    out[vidx<V>(i, M, m, comp)] = v;
+    out[(size_t)i * M + m] = v;
   }
 #pragma unroll
-  for (int q = 0; q < KMAX; ++q) win[q] = vzero<V>();
+  for (int q = 0; q < KMAX; ++q) win[q] = cd{};
   for (int i = f.n - 1; i >= 0; --i) {
-    const size_t o = vidx<V>(i, M, m, comp);
-    V v = out[o];
+    const size_t o = (size_t)i * M + m;
+    cd v = out[o];
     const int nu = __ldg(f.nu + i);
 #pragma unroll
     for (int r = 1; r <= KMAX; ++r)
-      if (r <= nu) v = vfma(-lu_up(f, i, r, mf), win[r - 1], v);
+      if (r <= nu) v = fma_rc(-lu_up(f, i, r, mf), win[r - 1], v);
     v = lu_invd(f, i, mf) * v;
 #pragma unroll
     for (int q = KMAX - 1; q > 0; --q) win[q] = win[q - 1];
@@ -75,7 +60,7 @@ __device__ void band_solve_v(const DLU& f, int m, int mf, int comp, const V* in,
 
 // The same solve for one real part, for grids with few Fourier modes (1 - 14 warps per SM): element i of the column is
 // at in[i rs], out[i rs] and add[i rs]. With so few warps nothing hides a load or an instruction of another warp, so a
-// row costs its latencies: 183 us for 129 rows at 128 x 128 modes as band_solve_v writes it (a value, its row's profile,
+// row costs its latencies: 183 us for 129 rows at 128 x 128 modes as band_solve_cd writes it (a value, its row's profile,
 // then its factors, one after the other; 300 instructions a row). All but a few rows at each end have the same
 // number of factors (DLU::lin, uin), so those rows run in a sweep that knows it: no tests, the window in registers,
 // pointers that walk, values and factors of the next 6 or 8 rows in flight: 65 us (m^c system, 3 factors per mode:
@@ -218,40 +203,39 @@ __device__ __forceinline__ void band_solve_piped(const DLU& f, int mf, const dou
 // the factors outside their profile are stored as zeros, so the sweeps run over K. Rows of the result
 // outside [zlo, zhi] are stored as zero (the recurrence itself uses the unmodified values). out may
 // alias in.
-template <class V>
-__device__ void band_solve_T_v(const DLU& f, int m, int mf, int comp, const V* in, V* out, size_t M, int zlo,
-                               int zhi) {
+__device__ inline void band_solve_T_cd(const DLU& f, int m, int mf, const cd* in, cd* out, size_t M, int zlo,
+                                       int zhi) {
   if (!LMVD_IN(m, M) || (f.mstride && !LMVD_IN(mf, f.mstride)) || !LMVD_IN(f.K, KMAX + 1)) return;
-  V win[KMAX];
+  cd win[KMAX];
 #pragma unroll
-  for (int q = 0; q < KMAX; ++q) win[q] = vzero<V>();
+  for (int q = 0; q < KMAX; ++q) win[q] = cd{};
   for (int i = 0; i < f.n; ++i) {
-    V v = in[vidx<V>(i, M, m, comp)];
+    cd v = in[(size_t)i * M + m];
 #pragma unroll
     for (int r = 1; r <= KMAX; ++r)
-      if (r <= f.K && i - r >= 0) v = vfma(-lu_up(f, i - r, r, mf), win[r - 1], v);
+      if (r <= f.K && i - r >= 0) v = fma_rc(-lu_up(f, i - r, r, mf), win[r - 1], v);
     v = lu_invd(f, i, mf) * v;
 #pragma unroll
     for (int q = KMAX - 1; q > 0; --q) win[q] = win[q - 1];
     win[0] = v;
-    out[vidx<V>(i, M, m, comp)] = v;
+    out[(size_t)i * M + m] = v;
   }
 #pragma unroll
-  for (int q = 0; q < KMAX; ++q) win[q] = vzero<V>();
+  for (int q = 0; q < KMAX; ++q) win[q] = cd{};
   for (int i = f.n - 1; i >= 0; --i) {
-    const size_t o = vidx<V>(i, M, m, comp);
-    V v = out[o];
+    const size_t o = (size_t)i * M + m;
+    cd v = out[o];
 #pragma unroll
     for (int q = 1; q <= KMAX; ++q)
-      if (q <= f.K && i + q < f.n) v = vfma(-lu_lo(f, i + q, q, mf), win[q - 1], v);
+      if (q <= f.K && i + q < f.n) v = fma_rc(-lu_lo(f, i + q, q, mf), win[q - 1], v);
 #pragma unroll
     for (int q = KMAX - 1; q > 0; --q) win[q] = win[q - 1];
     win[0] = v;
-    out[o] = (i < zlo || i > zhi) ? vzero<V>() : v;
+    out[o] = (i < zlo || i > zhi) ? cd{} : v;
   }
 }
 
-// band_solve_T_v for one real part (see band_solve_piped): the sweep with U^T uses row i - r's factor r, the one with
+// band_solve_T_cd for one real part (see band_solve_piped): the sweep with U^T uses row i - r's factor r, the one with
 // L^T row i + q's factor q; factors outside the profile are zeros and are skipped in the rows at the ends. Away from
 // the ends a row has the interior number of factors.
 template <bool UP>

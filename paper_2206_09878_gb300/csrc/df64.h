@@ -8,8 +8,8 @@
 // cancellation of the high parts, where its error stays below ~2^-47 of the operands' magnitudes
 // (the normwise bound an FFT or a pointwise product needs).
 //
-// On GB300 an FP32 FMA issues 63x faster than an FP64 FMA, so transforms and pointwise products in
-// this arithmetic run several times faster than in FP64 while staying within ~1e-14 relative error.
+// On GB300 an FP32 FMA issues 63x faster than an FP64 FMA, so the band evaluations of the precision path
+// run several times faster in this arithmetic than in FP64 while staying within ~1e-14 relative error.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -21,11 +21,6 @@ struct df {
 struct cdf {
   df re, im;  // 16 bytes, same footprint as a complex double
 };
-
-__host__ __device__ inline df df_from_double(double x) {
-  const float h = (float)x;
-  return df{h, (float)(x - (double)h)};
-}
 
 // Split of a double into hi + lo with integer operations only (no FP64 instruction): hi takes the
 // sign, exponent and the top 23 stored mantissa bits (truncation), lo the remaining 29 bits rounded
@@ -120,23 +115,14 @@ __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& 
   e = __fsub_rn(b, __fsub_rn(s, a));
 }
 
-__device__ __forceinline__ df dadd(df a, df b) {
-  float s, e, r, rl;
-  two_sum(a.hi, b.hi, s, e);
-  e = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
-  fast_two_sum(s, e, r, rl);
-  return df{r, rl};
-}
 // a + b without the final renormalisation: hi + lo is the sum to the same accuracy, but lo may exceed
-// ulp(hi) / 2. For intermediates that only feed another dadd (its TwoSum of the high parts is exact for
-// any operands and it renormalises its result).
+// ulp(hi) / 2. For intermediates whose consumer takes any pair (df_to_double_int adds the parts).
 __device__ __forceinline__ df dadd_lazy(df a, df b) {
   float s, e;
   two_sum(a.hi, b.hi, s, e);
   return df{s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
 }
 __device__ __forceinline__ df dneg(df a) { return df{-a.hi, -a.lo}; }
-__device__ __forceinline__ df dsub(df a, df b) { return dadd(a, dneg(b)); }
 __device__ __forceinline__ df dmul(df a, df b) {
   const float p = __fmul_rn(a.hi, b.hi);
   float e = __fmaf_rn(a.hi, b.hi, -p);
@@ -146,8 +132,6 @@ __device__ __forceinline__ df dmul(df a, df b) {
   fast_two_sum(p, e, r, rl);
   return df{r, rl};
 }
-// a * b for a power of two b (exact)
-__device__ __forceinline__ df dscale2(df a, float b) { return df{a.hi * b, a.lo * b}; }
 // a * b + c * d with one renormalisation
 __device__ __forceinline__ df ddot2(df a, df b, df c, df d) {
   const float p1 = __fmul_rn(a.hi, b.hi), e1 = __fmaf_rn(a.hi, b.hi, -p1);
@@ -162,33 +146,6 @@ __device__ __forceinline__ df ddot2(df a, df b, df c, df d) {
   float r, rl;
   fast_two_sum(s, t, r, rl);
   return df{r, rl};
-}
-// a * b + c * d without the final renormalisation (see dadd_lazy)
-__device__ __forceinline__ df ddot2_lazy(df a, df b, df c, df d) {
-  const float p1 = __fmul_rn(a.hi, b.hi), e1 = __fmaf_rn(a.hi, b.hi, -p1);
-  const float p2 = __fmul_rn(c.hi, d.hi), e2 = __fmaf_rn(c.hi, d.hi, -p2);
-  float s, e3;
-  two_sum(p1, p2, s, e3);
-  float t = __fadd_rn(__fadd_rn(e1, e2), e3);
-  t = __fmaf_rn(a.hi, b.lo, t);
-  t = __fmaf_rn(a.lo, b.hi, t);
-  t = __fmaf_rn(c.hi, d.lo, t);
-  t = __fmaf_rn(c.lo, d.hi, t);
-  return df{s, t};
-}
-
-// complex helpers
-__device__ __forceinline__ cdf cadd(cdf a, cdf b) { return cdf{dadd(a.re, b.re), dadd(a.im, b.im)}; }
-__device__ __forceinline__ cdf csub(cdf a, cdf b) { return cdf{dsub(a.re, b.re), dsub(a.im, b.im)}; }
-__device__ __forceinline__ cdf cadd_lazy(cdf a, cdf b) { return cdf{dadd_lazy(a.re, b.re), dadd_lazy(a.im, b.im)}; }
-__device__ __forceinline__ cdf csub_lazy(cdf a, cdf b) {
-  return cdf{dadd_lazy(a.re, dneg(b.re)), dadd_lazy(a.im, dneg(b.im))};
-}
-__device__ __forceinline__ cdf ctimes_i(cdf a) { return cdf{dneg(a.im), a.re}; }
-__device__ __forceinline__ cdf cconj(cdf a) { return cdf{a.re, dneg(a.im)}; }
-// v * (wr + i wi), not renormalised (the twiddle products feed only a butterfly's additions)
-__device__ __forceinline__ cdf cmulw_lazy(cdf v, df wr, df wi) {
-  return cdf{ddot2_lazy(v.re, wr, dneg(v.im), wi), ddot2_lazy(v.re, wi, v.im, wr)};
 }
 
 }  // namespace lmvd

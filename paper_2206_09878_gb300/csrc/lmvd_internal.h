@@ -66,8 +66,6 @@ __host__ __device__ inline cd mk(double r, double i) { return cd{r, i}; }
 __host__ __device__ inline cd operator+(cd a, cd b) { return cd{a.re + b.re, a.im + b.im}; }
 __host__ __device__ inline cd operator-(cd a, cd b) { return cd{a.re - b.re, a.im - b.im}; }
 __host__ __device__ inline cd operator*(double s, cd a) { return cd{s * a.re, s * a.im}; }
-__host__ __device__ inline cd cmul(cd a, cd b) { return cd{a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
-__host__ __device__ inline cd conj(cd a) { return cd{a.re, -a.im}; }
 __host__ __device__ inline cd times_i(cd a) { return cd{-a.im, a.re}; }         // i * a
 __host__ __device__ inline cd fma_rc(double s, cd x, cd acc) { return cd{fma(s, x.re, acc.re), fma(s, x.im, acc.im)}; }
 
@@ -163,7 +161,7 @@ inline unsigned row_chunks(const Grid& g, int rows) {
 }
 
 // Threads per mode of the banded-solve kernels: 2 (one per real part, band_solve_piped) when the grid has fewer than
-// 65536 Fourier modes per row, else 1 (band_solve_v).
+// 65536 Fourier modes per row, else 1 (band_solve_cd).
 inline int solve_split(const Grid& g) { return g.M < 65536 ? 2 : 1; }
 
 __device__ inline cd band_row(const DBand& B, int i, const cd* x, size_t M, int m) {

@@ -104,9 +104,9 @@ __device__ __forceinline__ cdf cd_to_cdf(cd x) { return cdf{df_from_double_int(x
 __device__ __forceinline__ cd cdf_to_cd(cdf x) {
   return cd{df_to_double_int(drenorm(x.re)), df_to_double_int(drenorm(x.im))};
 }
-// The values these evaluations produce feed only the precision path's inverse transforms, whose z-pass
-// works in double-float: they are stored as renormalised pairs (cdf, the same 16 bytes as a complex
-// double) and the z-pass reads them as they are (fft_inverse_df_in), so neither side converts.
+// The values these evaluations produce feed only the inverse transforms: they are stored as renormalised
+// pairs (cdf, the same 16 bytes as a complex double) and the z-pass converts the pairs to its fixed point
+// (fft_inverse, fft_inverse_mul with df_in), with fewer instructions than a double's bits need.
 __device__ __forceinline__ void put_df(cd* p, size_t o, cdf v) {
   reinterpret_cast<cdf*>(p)[o] = cdf{drenorm(v.re), drenorm(v.im)};
 }
@@ -396,7 +396,7 @@ void launch_rhs_eval_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& 
 // ------------------------------------------------------------------ banded solves
 // job blockIdx.y: out = A^{-1} in (+ add), factors shared or per mode (DLU.mstride); used for the
 // collocation (interpolation) solves and the per-mode systems. out may alias in. Nyquist modes are set to
-// zero. k_solve_cd: one thread per mode (band_solve_v).
+// zero. k_solve_cd: one thread per mode (band_solve_cd).
 __global__ void k_solve_cd(Grid g, DLU lu, SolveJobs jobs) {
   const size_t m = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (m >= g.M) return;
@@ -405,7 +405,7 @@ __global__ void k_solve_cd(Grid g, DLU lu, SolveJobs jobs) {
     for (int i = 0; i < lu.n; ++i) jb.out[(size_t)i * g.M + m] = mk(0, 0);
     return;
   }
-  band_solve_v<cd>(lu, (int)m, lu.mstride ? factor_mode(g, (int)m) : 0, 0, jb.in, jb.add, jb.out, g.M);
+  band_solve_cd(lu, (int)m, lu.mstride ? factor_mode(g, (int)m) : 0, jb.in, jb.add, jb.out, g.M);
 }
 // One thread per (mode, real part), loads pipelined (band_solve_piped); a job may have its own factors, and a job of
 // real columns (modes = 0: the plane means) has one thread per column, `part` elements apart.
