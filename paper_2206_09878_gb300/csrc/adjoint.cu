@@ -73,6 +73,7 @@ struct Fields10R {
 // ------------------------------------------------------------------ elementwise helpers
 // f[o] *= (kx == 0 ? s0 : s1); Nyquist slots set to zero. blockIdx.y selects the field.
 __global__ void k_wscale(Grid g, FieldsW10 f, double s0, double s1) {
+  grid_wait();
   cd* x = pick(f.p, (int)blockIdx.y);
   const size_t n = (size_t)g.ny * g.M;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
@@ -93,6 +94,7 @@ struct SolveTJobs {
   SolveTJob j[8];
 };
 __global__ void k_solve_T_cd(Grid g, DLU lu, SolveTJobs jobs) {
+  grid_wait();
   const size_t m = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (m >= g.M) return;
   const SolveTJob& jb = jobs.j[blockIdx.y];
@@ -103,6 +105,7 @@ __global__ void k_solve_T_cd(Grid g, DLU lu, SolveTJobs jobs) {
   band_solve_T_cd(lu, (int)m, lu.mstride ? factor_mode(g, (int)m) : 0, jb.in, jb.out, g.M, jb.zlo, jb.zhi);
 }
 __global__ void __launch_bounds__(128) k_solve_T_piped(Grid g, DLU lu, const __grid_constant__ SolveTJobs jobs) {
+  grid_wait();
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (t >= 2 * g.M) return;
   const int m = (int)(t >> 1);
@@ -132,6 +135,7 @@ struct AdjUpd {
 // LU, scr1 for z with the Neumann LU): transposed evaluation and the RK coefficients. Rows split over
 // gridDim.y chunks, job blockIdx.z (0: Omega2, 1: z).
 __global__ void k_adj_update_om_z_post(Grid g, DBand B0gT, AdjUpd a) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M || is_nyquist(g, m)) return;
   const size_t M = g.M;
@@ -157,6 +161,7 @@ __global__ void k_adj_update_om_z_post(Grid g, DBand B0gT, AdjUpd a) {
 // Plane means, one CTA: v = A^{-T} ybar per component (threads 0 and 1; boundary rows zero), then the transposed
 // evaluation and the RK coefficients over the rows.
 __global__ void __launch_bounds__(128) k_adj_update_means(Grid g, DBand B0gT, DLU lu, AdjUpd a) {
+  grid_wait();
   const int ny = g.ny;
   double* v0 = reinterpret_cast<double*>(a.scr0);  // ny doubles of scratch each
   double* v1 = reinterpret_cast<double*>(a.scr1);
@@ -175,6 +180,7 @@ __global__ void __launch_bounds__(128) k_adj_update_means(Grid g, DBand B0gT, DL
 // After v = A^{-T} m2^d-bar (per-mode factors, rows < 2 and > ny - 2 zero) in scrp: transposed phi2
 // evaluation and the RK coefficients. Rows 0..ny split over gridDim.y chunks.
 __global__ void k_adj_update_m2_post(Grid g, DBand Ss0T, DBand Ss2T, AdjUpd a) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M || m == 0 || is_nyquist(g, m)) return;
   const size_t M = g.M;
@@ -203,6 +209,7 @@ struct Sv10C {
 // rows split over gridDim.y chunks
 __global__ void k_adj_rhs_eval(Grid g, DBand B1gT, DBand B2gT, DBand Bs0T, DBand Bs1T, DBand Bs2T, DBand Bs3T,
                                const cd* rom, const cd* rphi, const double* rm, St7 st) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -239,6 +246,7 @@ __global__ void k_adj_rhs_eval(Grid g, DBand B1gT, DBand B2gT, DBand Bs0T, DBand
 
 // conj-transpose of the per-mode stream combination of k_rhs_combine
 __global__ void k_adj_rhs_combine(Grid g, double mu, double grav, St7 stb, FieldsW10 svb) {
+  grid_wait();
   const size_t n = (size_t)g.ny * g.M;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const int m = (int)(o % g.M);
@@ -278,6 +286,7 @@ __global__ void k_adj_rhs_combine(Grid g, double mu, double grav, St7 stb, Field
 // (that is, of m^c); accumulates the adjoints of m^d, 1/rho, rho.
 __global__ void k_adj_p2(size_t n, Fields10R pb, Fields3RC md, Fields3RC b, const double* ir, Fields3R mdb, double* irb,
                          double* rhob) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const double c11 = pb.p[0][o], c12 = pb.p[1][o], c13 = pb.p[2][o], c22 = pb.p[3][o], c23 = pb.p[4][o],
                  c33 = pb.p[5][o], u1 = pb.p[6][o], u2 = pb.p[7][o], u3 = pb.p[8][o], rb = pb.p[9][o];
@@ -300,6 +309,7 @@ __global__ void k_adj_p2(size_t n, Fields10R pb, Fields3RC md, Fields3RC b, cons
 
 // rho_t = f' a: abar = f' rtbar, f'bar += a rtbar
 __global__ void k_adj_rt(size_t n, const double* fp, const double* a, const double* rtb, double* ab, double* fpb) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const double t = rtb[o];
     fpb[o] += a[o] * t;
@@ -309,6 +319,7 @@ __global__ void k_adj_rt(size_t n, const double* fp, const double* a, const doub
 
 // l = -(w . b): bbar_i = -w_i lbar, wbar_i += -b_i lbar
 __global__ void k_adj_L(size_t n, Fields3RC w, Fields3RC b, const double* lb, Fields3R bb, Fields3R wb) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const double t = lb[o];
     for (int i = 0; i < 3; ++i) {
@@ -323,6 +334,7 @@ __global__ void k_adj_L(size_t n, Fields3RC w, Fields3RC b, const double* lb, Fi
 __global__ void k_adj_p1(size_t n, EosArgs e, Fields5RC zp, Fields3RC md, const double* rho, const double* ir,
                          const double* rhob, const double* irb, const double* fpb, Fields3RC wb, const double* rzb,
                          Fields3RC mdb, Fields10R pb) {
+  grid_wait();
   const double irlrh = 1.0 / (e.rl * e.rh);
   const double drho = e.rh - e.rl;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
@@ -356,6 +368,7 @@ struct Sv8 {
   cd* p[8];
 };
 __global__ void k_adj_p1_combine(Grid g, Sv8 v) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M || is_nyquist(g, m)) return;
   const size_t M = g.M;
@@ -376,6 +389,7 @@ __global__ void k_adj_p1_combine(Grid g, Sv8 v) {
 }
 __global__ void k_adj_eval_p1(Grid g, DBand B0gT, DBand B1gT, DBand B2gT, DBand Sg0T, DBand Sg1T, Sv8C v, cd* zb,
                               cd* omb, cd* m2b, double* mm1b, double* mm3b) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M || is_nyquist(g, m)) return;
   const size_t M = g.M;
@@ -411,6 +425,7 @@ __device__ inline cd adj_mc_q(const cd* m1b, const cd* m3b, size_t o, double k1,
 
 // rows 0..ny split over gridDim.y chunks
 __global__ void k_adj_mc_rhs(Grid g, const double* dstar, const cd* m1b, const cd* m2b, const cd* m3b, cd* scr) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -435,6 +450,7 @@ __global__ void k_adj_mc_rhs(Grid g, const double* dstar, const cd* m1b, const c
 // rows 0..ny-1 split over gridDim.y chunks; the k = 0 mode is one serial pass (chunk 0)
 __global__ void k_adj_mc_post(Grid g, DBand Bs1T, const double* dstar, const cd* m1b, const cd* m2b, const cd* m3b,
                               const cd* scr, cd* rtb) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -464,6 +480,7 @@ __global__ void k_adj_mc_post(Grid g, DBand Bs1T, const double* dstar, const cd*
 // BDF guess adjoint: zbar += a0/dt zdbar, zh_k bar += a_{k+1}/dt zdbar
 __global__ void k_adj_bdf(size_t n, double c0, double c1, double c2, double c3, const cd* zd, cd* z, cd* h0, cd* h1,
                           cd* h2) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const cd t = zd[o];
     z[o] = z[o] + c0 * t;
@@ -477,6 +494,7 @@ __global__ void k_adj_bdf(size_t n, double c0, double c1, double c2, double c3, 
 // sum c_q zh_q bar
 __global__ void k_adj_backfill(size_t n, double c0, double c1, double c2, const cd* h0, const cd* h1, const cd* h2,
                                const cd* zdp, cd* z, cd* zd) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const cd a = h0[o], b = h1[o], d = h2[o];
     z[o] = z[o] + (a + b + d);
@@ -485,6 +503,7 @@ __global__ void k_adj_backfill(size_t n, double c0, double c1, double c2, const 
 }
 
 __global__ void k_add(size_t n, cd* y, const cd* x) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x)
     y[o] = y[o] + x[o];
 }

@@ -433,6 +433,7 @@ __device__ __forceinline__ int fx_point(int u, bool first4, int tt, int tpt, int
 template <class RAW, int EPT, int COLS>
 __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
     k_fft_z_inv(FFTPlan pl, Grid g, const __grid_constant__ ZMaps maps, cfx* T, size_t tstride, int* te, unsigned* flags) {
+  grid_wait();
   extern __shared__ __align__(128) unsigned char sm_raw[];
   __shared__ FxShared sh;
   cfx* a = reinterpret_cast<cfx*>(sm_raw);
@@ -524,7 +525,7 @@ __device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, con
   const int* ej = te + ((size_t)f * g.ny + j) * h;
 #pragma unroll
   for (int u = 0; u < NP; ++u) {
-    E[u] = LMVD_IN(tt + u * tpt, h) ? __ldg(ej + tt + u * tpt) : kFxMaxE;
+    E[u] = LMVD_IN(tt + u * tpt, h) ? ej[tt + u * tpt] : kFxMaxE;
     emin = min(emin, E[u]);
   }
   if (!mbar_wait_bounded(bar, flags)) return;
@@ -584,12 +585,14 @@ __device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, con
 template <int EPT>
 __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_inv(FFTPlan pl, Grid g, const cfx* T, size_t tstride,
                                                                     const int* te, FieldsRW out, unsigned* flags) {
+  grid_wait();
   x_inv_body<EPT, false>(pl, g, T, tstride, te, out, nullptr, flags);
 }
 template <int EPT>
 __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_inv_mul(FFTPlan pl, Grid g, const cfx* T, size_t tstride,
                                                                         const int* te, FieldsRW out, const double* wmul,
                                                                         unsigned* flags) {
+  grid_wait();
   x_inv_body<EPT, true>(pl, g, T, tstride, te, out, wmul, flags);
 }
 
@@ -670,11 +673,13 @@ __device__ __forceinline__ void x_fwd_body(const FFTPlan& pl, const Grid& g, con
 template <int EPT>
 __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_fwd(FFTPlan pl, Grid g, FieldsRC in, cfx* T, size_t tstride,
                                                                     int* te) {
+  grid_wait();
   x_fwd_body<EPT, false>(pl, g, in, T, tstride, te, Dot3{});
 }
 template <int EPT>
 __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_fwd_dot3(FFTPlan pl, Grid g, cfx* T, size_t tstride, int* te,
                                                                          Dot3 d) {
+  grid_wait();
   x_fwd_body<EPT, true>(pl, g, FieldsRC{}, T, tstride, te, d);
 }
 
@@ -687,6 +692,7 @@ template <int EPT, int COLS>
 __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
     k_fft_z_fwd(FFTPlan pl, Grid g, const __grid_constant__ ZMaps maps, const int* te, FieldsW out, const cd* add,
                 unsigned* flags) {
+  grid_wait();
   extern __shared__ __align__(128) unsigned char sm_raw[];
   __shared__ FxShared sh;
   cfx* a = reinterpret_cast<cfx*>(sm_raw);
@@ -707,7 +713,7 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
 #pragma unroll
   for (int u = 0; u < EPT; ++u) {
     const int i = fx_point(u, first4, tt, tpt, pz >> 2);
-    E[u] = LMVD_IN(i, pz) ? __ldg(ej + (i >> 1)) : kFxMaxE;
+    E[u] = LMVD_IN(i, pz) ? ej[i >> 1] : kFxMaxE;
     emin = min(emin, E[u]);
   }
   if (!mbar_wait_bounded(bar, flags)) return;
@@ -1081,14 +1087,15 @@ static __device__ int g_noalloc_exp[kNoAllocScratchBytes / sizeof(cd) / 6];
 int* g_noalloc_exp_ptr[kNoAllocMaxDevices] = {};
 
 // twiddle table tw[m] = limbs of (cos 2 pi m / n, sin 2 pi m / n) computed on the device
-__global__ void k_twiddles(int4* tw, int n) {
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n; m += gridDim.x * blockDim.x) {
+__global__ void k_twiddles(int4* tx, int nx, int4* tz, int nz) {
+  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < nx + nz; m += gridDim.x * blockDim.x) {
+    const int i = m < nx ? m : m - nx, n = m < nx ? nx : nz;
     double s, c;
-    sincospi(2.0 * (double)m / (double)n, &s, &c);
+    sincospi(2.0 * (double)i / (double)n, &s, &c);
     int4 w;
     fx_limbs(c, w.x, w.y);
     fx_limbs(s, w.z, w.w);
-    tw[m] = w;
+    (m < nx ? tx : tz)[i] = w;
   }
 }
 
@@ -1156,9 +1163,7 @@ extern "C" int lmvd_inverse_transform_noalloc(int nx, int ny, int nz, const void
   fx.tw = (const int4*)sb;
   fz.tw = (const int4*)(sb + off_tz);
   cfx* T = (cfx*)(sb + off_tb);
-  k_twiddles<<<(g.px + 255) / 256, 256, 0, st>>>((int4*)sb, g.px);
-  if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
-  k_twiddles<<<(g.pz + 255) / 256, 256, 0, st>>>((int4*)(sb + off_tz), g.pz);
+  k_twiddles<<<cdiv(g.px + g.pz, 128), 128, 0, st>>>((int4*)sb, g.px, (int4*)(sb + off_tz), g.pz);
   if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
   const size_t S = (size_t)ny * g.M, P = (size_t)ny * g.P;
   FFTPlan fx6, fz6;
@@ -1174,13 +1179,14 @@ extern "C" int lmvd_inverse_transform_noalloc(int nx, int ny, int nz, const void
     ZMaps maps;
     if (!tile_map(&maps.m[0], fi.p[0], g.nxh, nz, ny, fz.batch, fz.rows_in)) return LMVD_ERR_CUDA;
     dim3 gz(cdiv(nx / 2, fz.batch), ny, 1);
+    // an ordinary launch: it reads the twiddles, which the kernel before may have written, through the read-only path
     if (fz.ept == 12 && fz.batch == 4) k_fft_z_inv<cd, 12, 4><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, te, nullptr);
     else if (fz.ept == 12) k_fft_z_inv<cd, 12, 2><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, te, nullptr);
     else k_fft_z_inv<cd, 6, 4><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, te, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
     dim3 gx(cdiv(cdiv(g.pz, 2), fx.batch), ny, 1);
-    if (fx.ept == 12) k_fft_x_inv<12><<<gx, threads(fx), smem_bytes(fx), st>>>(fx, g, T, 0, te, fo, nullptr);
-    else k_fft_x_inv<6><<<gx, threads(fx), smem_bytes(fx), st>>>(fx, g, T, 0, te, fo, nullptr);
+    if (fx.ept == 12) launch_next(k_fft_x_inv<12>, gx, threads(fx), smem_bytes(fx), st, fx, g, T, 0, te, fo, nullptr);
+    else launch_next(k_fft_x_inv<6>, gx, threads(fx), smem_bytes(fx), st, fx, g, T, 0, te, fo, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
   }
   return LMVD_OK;

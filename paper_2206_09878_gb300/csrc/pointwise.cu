@@ -17,6 +17,7 @@ __global__ void k_products_p1(size_t n, EosArgs e, const double* zp, const doubl
                               const double* zy, const double* lapz, const double* m1, const double* m2,
                               const double* m3, double* rho, double* invrho, double* fprime, double* w1, double* w2,
                               double* w3, double* rz) {
+  grid_wait();
   const double irlrh = 1.0 / (e.rl * e.rh);
   const double drho = e.rh - e.rl;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
@@ -35,15 +36,9 @@ __global__ void k_products_p1(size_t n, EosArgs e, const double* zp, const doubl
 
 // rho_t = f'(z) dz/dt
 __global__ void k_product_rt(size_t n, const double* fprime, const double* zdot, double* out) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x)
     out[o] = fprime[o] * zdot[o];
-}
-
-// L tail: -(1/rho) grad z . m^c
-__global__ void k_product_L(size_t n, const double* w1, const double* w2, const double* w3, const double* m1,
-                            const double* m2, const double* m3, double* out) {
-  for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x)
-    out[o] = -(w1[o] * m1[o] + w2[o] * m2[o] + w3[o] * m3[o]);
 }
 
 // m = m^d + m^c, u = m / rho, C_ij = -m_i m_j / rho; outputs C11 - C22, C12, C13, C23, C33 - C22, u1, u2, u3, rho (an
@@ -51,6 +46,7 @@ __global__ void k_product_L(size_t n, const double* w1, const double* w2, const 
 // pointer is skipped (the outputs are formed in batches)
 __global__ void k_products_p2(size_t n, const double* md1, const double* md2, const double* md3, const double* mc1,
                               const double* mc2, const double* mc3, const double* rho, const double* invrho, P2Out q) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const double ir = invrho[o];
     const double a = md1[o] + mc1[o], b = md2[o] + mc2[o], c = md3[o] + mc3[o];

@@ -19,6 +19,7 @@ LMVD_DEFINE_OOB_TAKE(yk)
 // threads, each with its own loads in flight.
 __global__ void k_eval_p1(Grid g, DBand B0g, DBand B1g, DBand B2g, DBand Sg0, DBand Sg1, const cd* z,
                           const cd* om, const cd* m2, const double* mm1, const double* mm3, Fields8 out) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -61,6 +62,7 @@ __global__ void k_eval_p1(Grid g, DBand B0g, DBand B1g, DBand B2g, DBand Sg0, DB
 // job blockIdx.y: out = B in (or out += B in), rows B.rows split into gridDim.z chunks; Nyquist modes
 // zero (or unchanged).
 __global__ void k_eval(Grid g, EvalJobs jobs) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const EvalJob& jb = jobs.j[blockIdx.y];
@@ -177,6 +179,7 @@ template <int WB, int WS>
 __global__ void __launch_bounds__(128) k_eval_p1_df(Grid g, DBand B0g, DBand B1g, DBand B2g, DBand Sg0, DBand Sg1,
                                                     const cd* z, const cd* om, const cd* m2, const double* mm1,
                                                     const double* mm3, Fields8 out) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -244,6 +247,7 @@ __global__ void __launch_bounds__(128) k_eval_p1_df(Grid g, DBand B0g, DBand B1g
 // band of the jobs
 template <int W>
 __global__ void __launch_bounds__(128) k_eval_df(Grid g, EvalJobs jobs) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const EvalJob& jb = jobs.j[blockIdx.y];
@@ -267,6 +271,7 @@ __global__ void __launch_bounds__(128) k_eval_df(Grid g, EvalJobs jobs) {
 template <int WS>
 __global__ void __launch_bounds__(128) k_mc_values_df(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const cd* m2c, cd* v1,
                                                       cd* v2, cd* v3) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -303,6 +308,7 @@ __global__ void __launch_bounds__(128) k_mc_values_df(Grid g, DBand Sg0, DBand S
 template <int WB>
 __global__ void __launch_bounds__(128) k_rhs_eval_df(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, DBand Bs2,
                                                      DBand Bs3, Fields7C st, cd* r_om, cd* r_phi, double* r_m) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -361,7 +367,7 @@ void launch_eval_p1_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g
                        const double* mm1, const double* mm3, const Fields8& out) {
   switch (p) {
 #define LMVD_P1(P) \
-    case P: k_eval_p1_df<P, P + 1><<<grid, tpb, 0, st>>>(g, B0g, B1g, B2g, Sg0, Sg1, z, om, m2, mm1, mm3, out); break;
+    case P: launch_next(k_eval_p1_df<P, P + 1>, grid, tpb, 0, st, g, B0g, B1g, B2g, Sg0, Sg1, z, om, m2, mm1, mm3, out); break;
     LMVD_P1(4) LMVD_P1(5) LMVD_P1(6) LMVD_P1(7) LMVD_P1(8)
 #undef LMVD_P1
   }
@@ -369,7 +375,7 @@ void launch_eval_p1_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g
 void launch_eval_df(int w, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const EvalJobs& jobs) {
   switch (w) {
 #define LMVD_EV(W) \
-    case W: k_eval_df<W><<<grid, tpb, 0, st>>>(g, jobs); break;
+    case W: launch_next(k_eval_df<W>, grid, tpb, 0, st, g, jobs); break;
     LMVD_EV(4) LMVD_EV(5) LMVD_EV(6) LMVD_EV(7) LMVD_EV(8) LMVD_EV(9)
 #undef LMVD_EV
   }
@@ -378,7 +384,7 @@ void launch_mc_values_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid&
                          const cd* rtv, const cd* m2c, cd* v1, cd* v2, cd* v3) {
   switch (p) {
 #define LMVD_MV(P) \
-    case P: k_mc_values_df<P + 1><<<grid, tpb, 0, st>>>(g, Sg0, Sg1, rtv, m2c, v1, v2, v3); break;
+    case P: launch_next(k_mc_values_df<P + 1>, grid, tpb, 0, st, g, Sg0, Sg1, rtv, m2c, v1, v2, v3); break;
     LMVD_MV(4) LMVD_MV(5) LMVD_MV(6) LMVD_MV(7) LMVD_MV(8)
 #undef LMVD_MV
   }
@@ -387,7 +393,7 @@ void launch_rhs_eval_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& 
                         const DBand* Bs, const Fields7C& stc, cd* r_om, cd* r_phi, double* r_m) {
   switch (p) {
 #define LMVD_RE(P) \
-    case P: k_rhs_eval_df<P><<<grid, tpb, 0, st>>>(g, B1g, B2g, Bs[0], Bs[1], Bs[2], Bs[3], stc, r_om, r_phi, r_m); break;
+    case P: launch_next(k_rhs_eval_df<P>, grid, tpb, 0, st, g, B1g, B2g, Bs[0], Bs[1], Bs[2], Bs[3], stc, r_om, r_phi, r_m); break;
     LMVD_RE(4) LMVD_RE(5) LMVD_RE(6) LMVD_RE(7) LMVD_RE(8)
 #undef LMVD_RE
   }
@@ -398,6 +404,7 @@ void launch_rhs_eval_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& 
 // collocation (interpolation) solves and the per-mode systems. out may alias in. Nyquist modes are set to
 // zero. k_solve_cd: one thread per mode (band_solve_cd).
 __global__ void k_solve_cd(Grid g, DLU lu, SolveJobs jobs) {
+  grid_wait();
   const size_t m = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (m >= g.M) return;
   const SolveJob& jb = jobs.j[blockIdx.y];
@@ -410,6 +417,7 @@ __global__ void k_solve_cd(Grid g, DLU lu, SolveJobs jobs) {
 // One thread per (mode, real part), loads pipelined (band_solve_piped); a job may have its own factors, and a job of
 // real columns (modes = 0: the plane means) has one thread per column, `part` elements apart.
 __global__ void __launch_bounds__(128) k_solve_piped(Grid g, const __grid_constant__ PipedJobs jobs) {
+  grid_wait();
   const PipedJob& jb = jobs.j[blockIdx.y];
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   const int m = (int)(t >> 1), comp = (int)(t & 1);
@@ -436,6 +444,7 @@ __global__ void __launch_bounds__(128) k_solve_piped(Grid g, const __grid_consta
 
 // rows 0..ny split over gridDim.y chunks
 __global__ void k_mc_rhs(Grid g, DBand Bs1, const double* dstar, const cd* rt, cd* m2c) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -457,6 +466,7 @@ __global__ void k_mc_rhs(Grid g, DBand Bs1, const double* dstar, const cd* rt, c
 
 // rows 0..ny-1 split over gridDim.y chunks
 __global__ void k_mc_post(Grid g, const double* dstar, const cd* rt, cd* m1c, const cd* m2c, cd* m3c) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -483,6 +493,7 @@ __global__ void k_mc_post(Grid g, const double* dstar, const cd* rt, cd* m1c, co
 // Values of m^c at g: v2 = B* m2^c, (v1, v3) = i (k1, k3) / k^2 (rho_t + d m2^c / dy) with rtv the values of rho_t; zero
 // v1, v3 at k = 0. Rows split over gridDim.y chunks.
 __global__ void k_mc_values(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const cd* m2c, cd* v1, cd* v2, cd* v3) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -521,6 +532,7 @@ __global__ void k_mc_values(Grid g, DBand Sg0, DBand Sg1, const cd* rtv, const c
 // (Eq. mean_m1m3); the k = 0 values of all seven streams vanish otherwise.
 // One thread per mode and row chunk: the multipliers are formed once per mode.
 __global__ void k_rhs_combine(Grid g, double mu, double grav, Fields9C sv, Fields7 st) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -569,6 +581,7 @@ __global__ void k_rhs_combine(Grid g, double mu, double grav, Fields9C sv, Field
 // Rows 0..ny (R_phi2 has ny + 1) are split into gridDim.y chunks.
 __global__ void k_rhs_eval(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, DBand Bs2, DBand Bs3, Fields7C st,
                            cd* r_om, cd* r_phi, double* r_m) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= (int)g.M) return;
   const size_t M = g.M;
@@ -610,6 +623,7 @@ __global__ void k_rhs_eval(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, D
 // This kernel writes the right-hand sides into the new fields; rows split over gridDim.y chunks.
 template <int W>
 __global__ void k_update_rhs(Grid g, DBand B0g, const __grid_constant__ UpdateArgs a) {
+  grid_wait();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   const int ny = g.ny;
   const int job = blockIdx.z;
@@ -696,7 +710,7 @@ __global__ void k_update_rhs(Grid g, DBand B0g, const __grid_constant__ UpdateAr
 void launch_update_rhs(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B0g, const UpdateArgs& a) {
   switch (p) {
 #define LMVD_UP(P) \
-    case P: k_update_rhs<P><<<grid, tpb, 0, st>>>(g, B0g, a); break;
+    case P: launch_next(k_update_rhs<P>, grid, tpb, 0, st, g, B0g, a); break;
     LMVD_UP(4) LMVD_UP(5) LMVD_UP(6) LMVD_UP(7) LMVD_UP(8)
 #undef LMVD_UP
   }
@@ -706,6 +720,7 @@ void launch_update_rhs(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g
 // Sets bit 0 of *flag if array blockIdx.y of the job list holds a non-finite double (inf or nan: all
 // exponent bits set). Integer tests on the bit pattern keep this off the FP64 pipe; one atomic per warp.
 __global__ void k_check_finite(CheckJobs jobs, unsigned* flag) {
+  grid_wait();
   const CheckJob jb = pick(jobs.j, (int)blockIdx.y);
   bool bad = false;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < jb.n; o += (size_t)gridDim.x * blockDim.x)
@@ -729,6 +744,7 @@ __device__ inline void block_add(double v, double* out) {
 
 // out[0] += |a - b|^2, out[1] += |a|^2 over n complex entries
 __global__ void k_diff_norms(size_t n, const cd* a, const cd* b, double* out) {
+  grid_wait();
   double d = 0.0, s = 0.0;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const cd x = a[o], y = b[o];
@@ -744,6 +760,7 @@ __global__ void k_diff_norms(size_t n, const cd* a, const cd* b, double* out) {
 // out[1] += |rho_t|^2, over all rows and modes (k = 0 included: D* <m2^c> = -<rho_t>)
 __global__ void k_mass_norms(Grid g, const double* dstar, const cd* rt, const cd* m1, const cd* m2, const cd* m3,
                              double* out) {
+  grid_wait();
   const size_t n = (size_t)g.ny * g.M;
   double d = 0.0, s = 0.0;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
@@ -766,6 +783,7 @@ __global__ void k_mass_norms(Grid g, const double* dstar, const cd* rt, const cd
 // applied on the host.
 __global__ void k_energy_norms(Grid g, const double* wq, Fields3C md, Fields3C mc, const double* invrho, double* ke,
                                unsigned long long* m2max) {
+  grid_wait();
   const size_t n = (size_t)g.ny * g.P;
   double e = 0.0, mx = 0.0;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
@@ -785,6 +803,7 @@ __global__ void k_energy_norms(Grid g, const double* wq, Fields3C md, Fields3C m
 // bit 1 of *flag if the last (the kf-th) fixed-point application, recorded at diag[2 kf], diag[2 kf + 1],
 // still changed dz/dt by half its size or more
 __global__ void k_fp_check(const double* diag, int kf, unsigned* flag) {
+  grid_wait();
   if (kf < 1) return;
   const double d = diag[2 * kf], s = diag[2 * kf + 1];
   if (d >= 0.25 * s && d > 0.0) atomicOr(flag, 2u);
@@ -794,6 +813,7 @@ __global__ void k_fp_check(const double* diag, int kf, unsigned* flag) {
 // BDF-like guess (Eq. dzdt_guesses): zdot = (a0 z^s + a1 z^{s-1} + a2 z^{s-2} + a3 z^{s-3}) / dt.
 __global__ void k_bdf(size_t n, double a0, double a1, double a2, double a3, double idt, const cd* z, const cd* h0,
                       const cd* h1, const cd* h2, cd* out) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x)
     out[o] = idt * (a0 * z[o] + a1 * h0[o] + a2 * h1[o] + a3 * h2[o]);
 }
@@ -801,6 +821,7 @@ __global__ void k_bdf(size_t n, double a0, double a1, double a2, double a3, doub
 // start-up history: zh_q = z - c_q dt zdot
 __global__ void k_backfill(size_t n, double c0, double c1, double c2, const cd* z, const cd* zdot, cd* h0, cd* h1,
                            cd* h2) {
+  grid_wait();
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const cd zz = z[o], d = zdot[o];
     h0[o] = zz - c0 * d;
@@ -811,6 +832,7 @@ __global__ void k_backfill(size_t n, double c0, double c1, double c2, const cd* 
 
 // zero the Nyquist slots of a spectral field and, if zero_mean, its k = 0 slot
 __global__ void k_sanitize(Grid g, int rows, cd* f, int zero_mean) {
+  grid_wait();
   const size_t n = (size_t)rows * g.M;
   for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
     const int m = (int)(o % g.M);
@@ -825,6 +847,7 @@ __global__ void k_sanitize(Grid g, int rows, cd* f, int zero_mean) {
 // identity factors, or with mean_rows the k = 0 mode those of x_i - x_{i+1} = r_i (x_{n-1} = r_{n-1}).
 __global__ void k_factor(Grid g, int n, int K, const double* A2, const double* A0, const double* A1, const int* nl,
                          const int* nu, double* lo, double* up, double* invd, int mean_rows) {
+  grid_wait();
   const size_t Mh = (size_t)(g.nz / 2 + 1) * g.nxh;
   const int mf = blockIdx.x * blockDim.x + threadIdx.x;
   if (mf >= (int)Mh) return;

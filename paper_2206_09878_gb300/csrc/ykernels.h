@@ -113,8 +113,6 @@ __global__ void k_products_p1(size_t n, EosArgs e, const double* zp, const doubl
                               const double* m3, double* rho, double* invrho, double* fprime, double* w1, double* w2,
                               double* w3, double* rz);
 __global__ void k_product_rt(size_t n, const double* fprime, const double* zdot, double* out);
-__global__ void k_product_L(size_t n, const double* w1, const double* w2, const double* w3, const double* m1,
-                            const double* m2, const double* m3, double* out);
 struct P2Out {
   double* p[9];
 };
