@@ -33,11 +33,14 @@ UNIT = "Mpoints*substages/s"
 # FP64 peak of GB300 from this pool's measurement: 0.596e12 DFMA/s at 1.99 GHz across 152 SMs is
 # 2 DFMA/clk/SM; at the 2070 MHz maximum SM clock: 152 * 2 * 2 flop * 2.07e9 = 1.259 TFLOP/s.
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# FP64-equivalent peak of double-float arithmetic on the FP32 pipe: a radix-2 butterfly (10 classic
-# flops: one complex multiply, two complex adds) costs 2 x 22 + 4 x 14 = 100 FP32 instructions in
-# df64.h (TwoSum-renormalised adds, FMA TwoProd products), i.e. 10 instructions per classic flop;
-# the FP32 pipe issues 152 SMs x 128 lanes x 2.07 GHz instructions per second.
+# FP64-equivalent peak of double-float arithmetic on the FP32 pipe (the precision path's band evaluations): ten
+# FP32 instructions (TwoSum-renormalised adds, FMA TwoProd products) per classic flop; the FP32 pipe issues
+# 152 SMs x 128 lanes x 2.07 GHz instructions per second.
 DF64_EQ_PEAK_TFLOPS = 152 * 128 * 2.07e9 / 10 / 1e12
+# The transforms compute in 64-bit fixed point on the integer pipes (csrc/fx.cuh), in both precisions. Their peak in
+# classic flops: a radix-2 butterfly (10 flops) takes one complex product of 12 multiply-adds 32 x 32 + 64 bits,
+# which the pipe retires at 30 lanes per clock per SM (measured), the slower of its pipes.
+FIXED_EQ_PEAK_TFLOPS = 152 * 30 / 12 * 10 * 2.07e9 / 1e12
 # Measured DRAM bytes (read + write) of the dominant kernel class over its algorithmic bytes, from one ncu
 # capture of a smaller case with the same transform length (512 x 33 x 512: 768-point x-transforms), keyed by
 # (precision, kernel class, transform length). The class fft_x_inverse holds k_fft_x_inv (19042-19412 /
@@ -68,7 +71,7 @@ def parse():
     ap.add_argument("--workload", default="rt512")
     ap.add_argument("--e2e-steps", type=int, default=2)
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--precision", type=int, default=0, help="0: FP64; 1: double-float transforms/products")
+    ap.add_argument("--precision", type=int, default=0, help="0: FP64; 1: double-float evaluations around the transforms")
     ap.add_argument("--no-variant", action="store_true", help="skip timing the other precision")
     ap.add_argument("--no-adjoint", action="store_true", help="skip the adjoint/forward cost ratio")
     ap.add_argument("--adjoint-workload", default="rt128")
@@ -335,7 +338,14 @@ def roofline_of(prof, ms_step_total, fp, grid, rates=None):
     else:
         peak, note = DF64_EQ_PEAK_TFLOPS, ("FP64-equivalent peak of double-float on the FP32 pipe: 152 SMs x 128 "
                                             "lanes x 2.07 GHz / 10 FP32 instructions per classic flop")
-    return {"kernel": top, "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+    fixed = {}
+    if top.startswith("fft"):
+        fixed = {"fixed_point_peak": FIXED_EQ_PEAK_TFLOPS,
+                 "fixed_point_frac": achieved / FIXED_EQ_PEAK_TFLOPS if achieved else None}
+        note += ("; the transforms run in 64-bit fixed point on the integer pipes, so this fraction may exceed 1: "
+                 "fixed_point_frac is against the integer multiply pipe (12 multiply-adds per radix-2 butterfly of 10 "
+                 "flops, 30 lanes per clock per SM measured, 152 SMs, 2.07 GHz)")
+    return {"kernel": top, "bound": "alu", **fixed, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak if achieved else None,
             "traffic": traffic_per_launch(fp, top, grid, tby / tn if tn else None),
             "traffic_note": "ncu dram__bytes_read.sum + dram__bytes_write.sum over the algorithmic bytes of the "
@@ -581,7 +591,7 @@ def run_cuda(args):
     w, config = workload_config(args.workload)
     config["parallelism"] = "replicas%d" % ws if ws > 1 else "single"
     config["precision"] = ("FP64 throughout" if args.precision == 0 else
-                           "double-float transforms and products, FP64 spectral steps")
+                           "double-float band evaluations, fixed-point transforms, FP64 elsewhere")
     npts = w["nx"] * w["ny"] * w["nz"]
     stream = torch.cuda.Stream()
     st = {k: torch.from_numpy(np.ascontiguousarray(v)) for k, v in rt_state(**w).items()}
@@ -615,8 +625,8 @@ def run_cuda(args):
         errs = {k: rel_err(f2[k], final[k]) for k in ("z", "om", "m2")}
         out["variant"] = {
             "precision": ("FP64 throughout" if other == 0 else
-                          "FP32-FFT: double-float (2 x FP32, error-free transformations) transforms and products, "
-                          "FP64 solves / RHS / update"),
+                          "double-float (2 x FP32, error-free transformations) band evaluations, fixed-point "
+                          "transforms, FP64 products / solves / RHS / update"),
             "value": v2, "unit": UNIT, "ms_per_step": r2["ms"] / args.steps, "clocks": r2["clocks"],
             "device_bytes": r2["device_bytes"],
             "roofline": roofline_of(r2["prof"], r2["ms"], other, (w["nx"], w["ny"], w["nz"]), rates),

@@ -6,8 +6,8 @@
  * Eq. dzdt_guesses, k_f fixed-point applications of L (Eq. y_k, Sec. 4.3), m^c from
  * Eq. COM_fourier / CF_fourier / mc_recon / mc_mean, the right-hand sides of Eq. DNS_system,
  * and the segregated midpoint RK2 update (Sec. 3.3). The adjoints of a substage and of the start-up
- * (the differentiation path) and a double-float precision path for the transforms and products are
- * part of the same library.
+ * (the differentiation path) and a double-float precision path for the B-spline evaluations are part
+ * of the same library.
  *
  * Conventions shared by every call
  * --------------------------------
@@ -65,11 +65,12 @@ extern "C" {
  * kf          : fixed-point applications of L per substage (Sec. 3.2).
  * beta_n, beta_p: free parameters of the guesses of Eq. dzdt_guesses (paper: 0 and -4).
  * n_startup   : fixed-point iterations from dz/dt = 0 used by lmvd_set_state without history.
- * precision   : 0 = FP64 throughout; 1 = transforms and physical-space products in double-float
- *               arithmetic on the FP32 units (pairs of floats, 48-bit significand, error-free
- *               TwoSum/TwoProd compensation), while every spectral step (collocation, m^c and m2^d
- *               solves, RHS assembly, the RK update and the state) and the EOS (rho, 1/rho, f'(z))
- *               stay FP64.
+ * precision   : 0 = FP64; 1 = the B-spline evaluations before and after the transforms in
+ *               double-float arithmetic on the FP32 units (pairs of floats, 48-bit significand,
+ *               error-free TwoSum/TwoProd compensation), everything else (products, EOS, collocation,
+ *               m^c and m2^d solves, RHS assembly, the RK update and the state) in FP64. In both the
+ *               transforms compute in 64-bit fixed point with one exponent per 1D transform, with
+ *               rounding errors below those of a binary64 FFT.
  * bc_mode     : boundary rows at y0 and y1. 0 = no-slip walls: Omega2 = 0, m2^d = dm2^d/dy = 0,
  *               m2^c = 0, <m1> = <m3> = 0, dz/dy = 0, <m2^c>(y1) = 0.
  *               1 = the paper's potential matching (Sec. 4.5, Eq. bc_both, md_bc) for a domain
@@ -217,9 +218,9 @@ int lmvd_forward_transform(lmvd_ctx* ctx, const double* phys, void* spec, int nf
 int lmvd_inverse_transform_noalloc(int nx, int ny, int nz, const void* spec, double* phys, int nfields,
                                    void* cuda_stream);
 
-/* Self-test of the precision path's conversions (precision = 1; no paper counterpart). The spectral
- * ends of its transforms split each FP64 value into a double-float pair and round pairs back, with
- * integer operations only; this runs the same device code on caller arrays:
+/* Self-test of the precision path's conversions (precision = 1; no paper counterpart). Its band
+ * evaluations split each FP64 value into a double-float pair and round pairs back, with integer
+ * operations only; this runs the same device code on caller arrays:
  *   (hi[i], lo[i]) = split of x[i]: hi the top 24 significand bits of x (truncated), lo the rest rounded
  *     to a float, renormalised (|lo| <= ulp(hi) / 2, |hi + lo - x| <= 2^-48 |x| for |x| >= 2^-102;
  *     smaller magnitudes lose lo gradually and become signed zeros below 2^-126; |x| >= 2^128 gives a
