@@ -906,6 +906,7 @@ int lmvd_create(const lmvd_config* cfg, void* stream, lmvd_ctx** out) {
   }
   if (!err) err = fft_prepare(c);
   if (!err) {
+    if (sizeof(cd) * TBUF_MAX * g.ny * g.pz * (g.nx / 2) <= TBUF_MAX_BYTES) c.tbuf_n = TBUF_MAX;
     // full layout if it takes at most 85% of the free device memory, else the lean one
     Carver probe{nullptr};
     carve(c, probe);

@@ -346,7 +346,7 @@ constexpr int FFT_MIN_X = 6, FFT_MIN_Z = 3;
 // memory as one asynchronous operation completing on an mbarrier, instead of one 16-byte load per thread
 // and element. The box lands row-major, i.e. as the interleaved layout the z-pass transforms work in.
 struct ZMaps {
-  CUtensorMap m[TBUF_FIELDS];  // one per field of the launch (z_inv: the spectral inputs; z_fwd: m[0] = T)
+  CUtensorMap m[TBUF_MAX];  // the spectral inputs, one per field of the launch
 };
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
     sh.top = 0;
   }
   __syncthreads();
-  if (threadIdx.x == 0 && LMVD_IN(f, TBUF_FIELDS)) {
+  if (threadIdx.x == 0 && LMVD_IN(f, TBUF_MAX)) {
     mbar_expect_tx(bar, (unsigned)(nz * COLS * sizeof(cfx)));
     for (int r = 0; r < nz; r += H) {
       const int pos = r < n2 ? r : pz - nz + r;
@@ -684,13 +684,13 @@ __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_fwd_dot3(FFTPlan
 }
 
 // ---------------------------------------------------------------- forward z-pass (truncate, scale)
-// T: [f][ny][pz][nx/2], read through maps.m[0] (all fields of the launch: planes f ny + j), its exponents te [f][ny]
+// T: [f][ny][pz][nx/2], read through the tensor map (all fields of the launch: planes f ny + j), its exponents te [f][ny]
 // [pz/2]; out: spectral fields [ny][nz][nxh]. Same interleaved layout as the inverse z-pass; kx = nx/2 and the kz
 // Nyquist row are written as zero. The last stage's middle outputs are the truncated kz. add (may be null, one field):
 // a spectral field added to the result.
 template <int EPT, int COLS>
 __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
-    k_fft_z_fwd(FFTPlan pl, Grid g, const __grid_constant__ ZMaps maps, const int* te, FieldsW out, const cd* add,
+    k_fft_z_fwd(FFTPlan pl, Grid g, const __grid_constant__ CUtensorMap map, const int* te, FieldsW out, const cd* add,
                 unsigned* flags) {
   grid_wait();
   extern __shared__ __align__(128) unsigned char sm_raw[];
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
   if (threadIdx.x == 0) {
     mbar_expect_tx(bar, (unsigned)(pz * COLS * sizeof(cfx)));
     for (int r = 0; r < pz; r += H)
-      if (LMVD_IN((r + H) * COLS - 1, pz * COLS)) tma_load_3d(a + (size_t)r * COLS, &maps.m[0], 2 * kx0, r, f * g.ny + j, bar);
+      if (LMVD_IN((r + H) * COLS - 1, pz * COLS)) tma_load_3d(a + (size_t)r * COLS, &map, 2 * kx0, r, f * g.ny + j, bar);
   }
   const bool first4 = EPT == 12 && pl.first4;
   int E[EPT], emin = INT_MAX;
@@ -939,20 +939,20 @@ static void z_inv_launch(Ctx& c, const FieldsC& fi, int n, size_t tstride, doubl
 static void z_fwd_launch(Ctx& c, int n, const FieldsW& fo, double fl, double by, const cd* add = nullptr) {
   const Grid& g = c.g;
   const FFTPlan& p = pick_plan(c.fz, c.fz6, (double)(g.nx / 2 + 1) * g.ny * n);
-  ZMaps maps;
-  if (!tile_map(&maps.m[0], c.tbuf, g.nx / 2, g.pz, (size_t)n * g.ny, p.batch, p.rows_t)) {
+  CUtensorMap map;
+  if (!tile_map(&map, c.tbuf, g.nx / 2, g.pz, (size_t)n * g.ny, p.batch, p.rows_t)) {
     map_failed(c);
     return;
   }
   const dim3 gz(cdiv(g.nx / 2 + 1, p.batch), g.ny, n);
   if (p.ept == 12 && p.batch == 4)
-    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 4>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, add,
+    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 4>), gz, threads(p), smem_bytes(p), p, g, map, c.texp, fo, add,
                 c.dflags);
   else if (p.ept == 12)
-    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 2>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, add,
+    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<12, 2>), gz, threads(p), smem_bytes(p), p, g, map, c.texp, fo, add,
                 c.dflags);
   else
-    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<6, 4>), gz, threads(p), smem_bytes(p), p, g, maps, c.texp, fo, add,
+    LMVD_LAUNCH(c, KC_FFT_Z_FWD, fl, by, (k_fft_z_fwd<6, 4>), gz, threads(p), smem_bytes(p), p, g, map, c.texp, fo, add,
                 c.dflags);
 }
 

@@ -53,7 +53,11 @@ constexpr int KMAX = 8;   // widest band (each side) of any y-system LU supporte
 // (transforms of more fields run in chunks), there are up to PW_FIELDS physical work fields, and the RHS
 // streams overwrite the first seven spectral value fields. When that layout would not leave room on the
 // device (768 x 769 x 768), lmvd_create uses the lean one: TBUF_LEAN and PW_LEAN fields.
-constexpr int TBUF_FIELDS = 4;
+// Where TBUF_MAX fields of the intermediate take at most TBUF_MAX_BYTES it holds those: the 8 and 9 fields of a substage's
+// two products are then transformed in one chunk. Steps at 4 / 10 fields: 32^3 1.688 / 1.647 ms (launches), 72 x 61 x 48
+// 2.505 / 2.475, 128^3 10.03 / 9.92 (fewer partly filled waves), 128 x 512 x 128 34.34 / 34.22, which is not worth 0.6 GB.
+constexpr int TBUF_FIELDS = 4, TBUF_MAX = 10;
+constexpr size_t TBUF_MAX_BYTES = (size_t)512 << 20;
 constexpr int PW_FIELDS = 9;
 constexpr int TBUF_LEAN = 2;
 constexpr int PW_LEAN = 6;
