@@ -70,7 +70,7 @@ def parse():
     ap.add_argument("--workload", default="rt512")
     ap.add_argument("--e2e-steps", type=int, default=2)
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--precision", type=int, default=0, help="0: FP64; 1: double-float evaluations around the transforms")
+    ap.add_argument("--precision", type=int, default=0, help="0: FP64; 1: double-float evaluations before the inverse transforms")
     ap.add_argument("--no-variant", action="store_true", help="skip timing the other precision")
     ap.add_argument("--no-adjoint", action="store_true", help="skip the adjoint/forward cost ratio")
     ap.add_argument("--adjoint-workload", default="rt128")

@@ -65,7 +65,7 @@ extern "C" {
  * kf          : fixed-point applications of L per substage (Sec. 3.2).
  * beta_n, beta_p: free parameters of the guesses of Eq. dzdt_guesses (paper: 0 and -4).
  * n_startup   : fixed-point iterations from dz/dt = 0 used by lmvd_set_state without history.
- * precision   : 0 = FP64; 1 = the B-spline evaluations before and after the transforms in
+ * precision   : 0 = FP64; 1 = the B-spline evaluations before the inverse transforms in
  *               double-float arithmetic on the FP32 units (pairs of floats, 48-bit significand,
  *               error-free TwoSum/TwoProd compensation), everything else (products, EOS, collocation,
  *               m^c and m2^d solves, RHS assembly, the RK update and the state) in FP64. In both the
@@ -219,8 +219,8 @@ int lmvd_inverse_transform_noalloc(int nx, int ny, int nz, const void* spec, dou
                                    void* cuda_stream);
 
 /* Self-test of the precision path's conversions (precision = 1; no paper counterpart). Its band
- * evaluations split each FP64 value into a double-float pair and round pairs back, with integer
- * operations only; this runs the same device code on caller arrays:
+ * evaluations split each FP64 value into a double-float pair with integer operations only, and a
+ * pair is rounded back likewise; this runs the same device code on caller arrays:
  *   (hi[i], lo[i]) = split of x[i]: hi the top 24 significand bits of x (truncated), lo the rest rounded
  *     to a float, renormalised (|lo| <= ulp(hi) / 2, |hi + lo - x| <= 2^-48 |x| for |x| >= 2^-102;
  *     smaller magnitudes lose lo gradually and become signed zeros below 2^-126; |x| >= 2^128 gives a

@@ -619,15 +619,11 @@ void enqueue_substage(Ctx& c, const Tape* tape) {
                             SolveReq{SolveJob{c.st[5], nullptr, c.st[5]}, li}, SolveReq{SolveJob{c.st[6], nullptr, c.st[6]}, li}});
   Fields7C stc{};
   for (int f = 0; f < 7; ++f) stc.p[f] = c.st[f];
-  if (cf.precision == 1) {
-    const dim3 grid(mode_blocks(g), row_chunks(g, g.ny + 1));
-    LMVD_LAUNCH_CALL(c, KC_RHS_EVAL, S * (4.0 * 6 * c.B1g.w + 4.0), 16.0 * 9 * S,
-                     launch_rhs_eval_df(cf.spline_order, grid, TPB_MODE, c.stream, g, c.B1g, c.B2g, c.Bs, stc, c.r_om,
-                                        c.r_phi, c.r_m));
-  } else
-    LMVD_LAUNCH(c, KC_RHS_EVAL, S * (4.0 * 6 * c.B1g.w + 4.0), 16.0 * 9 * S, k_rhs_eval,
-                dim3(mode_blocks(g), row_chunks(g, g.ny + 1)), TPB_MODE, 0,
-                g, c.B1g, c.B2g, c.Bs[0], c.Bs[1], c.Bs[2], c.Bs[3], stc, c.r_om, c.r_phi, c.r_m);
+  // FP64 in both precisions: the double-float form of these sums (six windows, 160 registers) was no faster at 256^3
+  // and 512^3 (1.36 / 1.36, 10.00 / 9.95 ms) and slower below (0.26 / 0.17 ms at 128^3)
+  LMVD_LAUNCH(c, KC_RHS_EVAL, S * (4.0 * 6 * c.B1g.w + 4.0), 16.0 * 9 * S, k_rhs_eval,
+              dim3(mode_blocks(g), row_chunks(g, g.ny + 1)), TPB_MODE, 0, g, c.B1g, c.B2g, c.Bs[0], c.Bs[1], c.Bs[2],
+              c.Bs[3], stc, c.r_om, c.r_phi, c.r_m);
   nvtxRangePop();
   nvtxRangePushA("step 6: RK2 update");
   // step 6: midpoint RK2, low-storage: (al, be) = (1/2, 0) at stage n, (1, -1/2) at stage '

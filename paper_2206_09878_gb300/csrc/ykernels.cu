@@ -80,12 +80,11 @@ __global__ void k_eval(Grid g, EvalJobs jobs) {
 }
 
 // ------------------------------------------------------------------ evaluations in double-float
-// The precision path (precision = 1) evaluates the B-spline sums that feed the inverse transforms and the
-// right-hand sides that follow the forward transforms in double-float on the FP32 pipe: the band entries
-// come as pairs (DBand.vf), each complex double input is split with integer operations, the products are
-// accumulated without renormalisation (error <= ~w 2^-48 of the sum of |terms|), and the result is
-// renormalised and rounded back to a double with integer operations. The per-mode multipliers (i k1,
-// 1/k^2, ...) are applied in double-float too, so these kernels issue no FP64 instruction per term.
+// The precision path (precision = 1) evaluates the B-spline sums that feed the inverse transforms in
+// double-float on the FP32 pipe: the band entries come as pairs (DBand.vf), each complex double input is split
+// with integer operations, the products are accumulated without renormalisation (error <= ~w 2^-48 of the sum
+// of |terms|), and the result is renormalised. The per-mode multipliers (i k1, 1/k^2, ...) are applied in
+// double-float too, so these kernels issue no FP64 instruction per term.
 
 // acc + b * x without renormalisation: TwoProd by FMA, TwoSum of the high parts, low parts summed
 __device__ __forceinline__ df dfma_lazy(df b, df x, df acc) {
@@ -103,9 +102,6 @@ __device__ __forceinline__ df drenorm(df a) {
   return df{s, e};
 }
 __device__ __forceinline__ cdf cd_to_cdf(cd x) { return cdf{df_from_double_int(x.re), df_from_double_int(x.im)}; }
-__device__ __forceinline__ cd cdf_to_cd(cdf x) {
-  return cd{df_to_double_int(drenorm(x.re)), df_to_double_int(drenorm(x.im))};
-}
 // The values these evaluations produce feed only the inverse transforms: they are stored as renormalised
 // pairs (cdf, the same 16 bytes as a complex double) and the z-pass converts the pairs to its fixed point
 // (fft_inverse, fft_inverse_mul with df_in), with fewer instructions than a double's bits need.
@@ -303,64 +299,6 @@ __global__ void __launch_bounds__(128) k_mc_values_df(Grid g, DBand Sg0, DBand S
   }
 }
 
-// k_rhs_eval in double-float; the k = 0 mean right-hand sides stay in FP64 (one mode). WB: band width of the
-// order-p space (B1g, B2g at g; Bs0..Bs3 at g*). Two sweeps: R_Omega2 (two windows), then R_phi2 (four).
-template <int WB>
-__global__ void __launch_bounds__(128) k_rhs_eval_df(Grid g, DBand B1g, DBand B2g, DBand Bs0, DBand Bs1, DBand Bs2,
-                                                     DBand Bs3, Fields7C st, cd* r_om, cd* r_phi, double* r_m) {
-  grid_wait();
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= (int)g.M) return;
-  const size_t M = g.M;
-  const int ny = g.ny;
-  int r0, r1;
-  row_range(ny + 1, blockIdx.y, gridDim.y, r0, r1);
-  if (m == 0 || is_nyquist(g, m)) {
-    for (int i = r0; i < r1; ++i) {
-      if (i < ny) r_om[(size_t)i * M + m] = mk(0, 0);
-      r_phi[(size_t)i * M + m] = mk(0, 0);
-      if (m == 0 && i < ny) {
-        r_m[i] = (band_row(B1g, i, st.p[1], M, 0) + band_row(B2g, i, st.p[2], M, 0)).re;
-        r_m[ny + i] = (band_row(B1g, i, st.p[4], M, 0) + band_row(B2g, i, st.p[5], M, 0)).re;
-      }
-    }
-    return;
-  }
-  {
-    DfWin<WB> w1, w2;
-    for (int i = r0; i < min(r1, ny); ++i) {
-      const int c = __ldg(B1g.c0 + i);
-      w1.seek(st.p[1], M, m, c, B1g.cols);
-      w2.seek(st.p[2], M, m, c, B2g.cols);
-      if (i + 1 < min(r1, ny)) {
-        const int cn = __ldg(B1g.c0 + i + 1);
-        w1.prefetch(st.p[1], M, m, cn, B1g.cols);
-        w2.prefetch(st.p[2], M, m, cn, B2g.cols);
-      }
-      const cdf a = cdf_add_lazy(w1.dot(B1g, i), w2.dot(B2g, i));
-      r_om[(size_t)i * M + m] = cdf_to_cd(cdf_add_lazy(a, cd_to_cdf(st.p[0][(size_t)i * M + m])));
-    }
-  }
-  DfWin<WB> w3, w4, w5, w6;
-  for (int i = r0; i < r1; ++i) {
-    const int c = __ldg(Bs0.c0 + i);
-    w3.seek(st.p[3], M, m, c, Bs0.cols);
-    w4.seek(st.p[4], M, m, c, Bs1.cols);
-    w5.seek(st.p[5], M, m, c, Bs2.cols);
-    w6.seek(st.p[6], M, m, c, Bs3.cols);
-    if (i + 1 < r1) {
-      const int cn = __ldg(Bs0.c0 + i + 1);
-      w3.prefetch(st.p[3], M, m, cn, Bs0.cols);
-      w4.prefetch(st.p[4], M, m, cn, Bs1.cols);
-      w5.prefetch(st.p[5], M, m, cn, Bs2.cols);
-      w6.prefetch(st.p[6], M, m, cn, Bs3.cols);
-    }
-    const cdf b = cdf_add_lazy(w3.dot(Bs0, i), w4.dot(Bs1, i));
-    const cdf d = cdf_add_lazy(w5.dot(Bs2, i), w6.dot(Bs3, i));
-    r_phi[(size_t)i * M + m] = cdf_to_cd(cdf_add_lazy(b, d));
-  }
-}
-
 // launchers for spline orders 4..8 (band widths 4..9); api.cu brackets them with its launch accounting
 void launch_eval_p1_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B0g, const DBand& B1g,
                        const DBand& B2g, const DBand& Sg0, const DBand& Sg1, const cd* z, const cd* om, const cd* m2,
@@ -387,15 +325,6 @@ void launch_mc_values_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid&
     case P: launch_next(k_mc_values_df<P + 1>, grid, tpb, 0, st, g, Sg0, Sg1, rtv, m2c, v1, v2, v3); break;
     LMVD_MV(4) LMVD_MV(5) LMVD_MV(6) LMVD_MV(7) LMVD_MV(8)
 #undef LMVD_MV
-  }
-}
-void launch_rhs_eval_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B1g, const DBand& B2g,
-                        const DBand* Bs, const Fields7C& stc, cd* r_om, cd* r_phi, double* r_m) {
-  switch (p) {
-#define LMVD_RE(P) \
-    case P: launch_next(k_rhs_eval_df<P>, grid, tpb, 0, st, g, B1g, B2g, Bs[0], Bs[1], Bs[2], Bs[3], stc, r_om, r_phi, r_m); break;
-    LMVD_RE(4) LMVD_RE(5) LMVD_RE(6) LMVD_RE(7) LMVD_RE(8)
-#undef LMVD_RE
   }
 }
 

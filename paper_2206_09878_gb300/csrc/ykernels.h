@@ -77,16 +77,14 @@ __global__ void k_eval_p1(Grid g, DBand B0g, DBand B1g, DBand B2g, DBand Sg0, DB
                           const cd* om, const cd* m2, const double* mm1, const double* mm3, Fields8 out);
 __global__ void k_eval(Grid g, EvalJobs jobs);
 // double-float evaluations of the precision path (same outputs as k_eval_p1, k_eval without accumulation and
-// k_rhs_eval), launched on st for spline orders p = 4..8 (band widths w = 4..9). The first two store their
-// values as double-float pairs (read by fft_inverse), the third FP64 values (for the FP64 RK update).
+// k_mc_values, stored as double-float pairs that fft_inverse reads), launched on st for spline orders p = 4..8
+// (band widths w = 4..9)
 void launch_eval_p1_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B0g, const DBand& B1g,
                        const DBand& B2g, const DBand& Sg0, const DBand& Sg1, const cd* z, const cd* om, const cd* m2,
                        const double* mm1, const double* mm3, const Fields8& out);
 void launch_eval_df(int w, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const EvalJobs& jobs);
 void launch_mc_values_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& Sg0, const DBand& Sg1,
                          const cd* rtv, const cd* m2c, cd* v1, cd* v2, cd* v3);
-void launch_rhs_eval_df(int p, dim3 grid, int tpb, cudaStream_t st, const Grid& g, const DBand& B1g, const DBand& B2g,
-                        const DBand* Bs, const Fields7C& stc, cd* r_om, cd* r_phi, double* r_m);
 __global__ void k_solve_cd(Grid g, DLU lu, SolveJobs jobs);
 __global__ void k_solve_piped(Grid g, const __grid_constant__ PipedJobs jobs);
 __global__ void k_mc_rhs(Grid g, DBand Bs1, const double* dstar, const cd* rt, cd* m2c);
