@@ -95,6 +95,16 @@ __device__ __forceinline__ void fx_butterfly(cfx (&v)[R], const FFTPlan& pl) {
   }
 }
 
+// A twiddle. The passes with 6 elements a thread use plain loads, so that a launch may overlap the kernel that wrote the
+// table (the allocation-free transform, 20.5 -> 18.5 us at 64 x 33 x 64). With 12 elements the choice is which spills less
+// and was measured: plain in the forward x-pass (3-field 256 x 129 x 256 analysis 500.0 -> 497.2 us), the read-only path
+// in the others (4-field 216 x 65 x 108 synthesis 170.9, plain 171.5 us).
+template <int SIGN, int EPT, int S>
+__device__ __forceinline__ int4 fx_tw(const int4* p) {
+  if constexpr (EPT == 12 && (S > 1 || SIGN > 0)) return __ldg(p);
+  else return *p;
+}
+
 // The sub-length L divides tpt (the radices before the last multiply to tpt), so a thread's butterflies share k = tt mod
 // L and their twiddles, which are fetched before the barrier.
 template <int SIGN, int R, int EPT, int S>
@@ -106,7 +116,7 @@ __device__ __forceinline__ void fx_stage(cfx* x, const FFTPlan& pl, int L, int t
   const int kt = k * (n / (L * R));
   int4 w[R];
 #pragma unroll
-  for (int q = 1; q < R; ++q) w[q] = __ldg(pl.tw + q * kt);
+  for (int q = 1; q < R; ++q) w[q] = fx_tw<SIGN, EPT, S>(pl.tw + q * kt);
   cfx v[NBT][R];
 #pragma unroll
   for (int j = 0; j < NBT; ++j)
@@ -182,7 +192,7 @@ __device__ __forceinline__ void fx_last(const cfx* x, const FFTPlan& pl, int tt,
   for (int q = 0; q < EPT; ++q) u[q] = LMVD_IN(tt + q * L, pl.n) ? x[(tt + q * L) * S] : cfx{0, 0};
   if (tt)
 #pragma unroll
-    for (int q = 1; q < EPT; ++q) u[q] = fx_mulw<SIGN>(u[q], __ldg(pl.tw + q * tt));
+    for (int q = 1; q < EPT; ++q) u[q] = fx_mulw<SIGN>(u[q], fx_tw<SIGN, EPT, S>(pl.tw + q * tt));
 #pragma unroll
   for (int b = 0; b < R; ++b) fx_bfly3<SIGN>(u[3 * b], u[(R + 3 * b) % EPT], u[(2 * R + 3 * b) % EPT], pl.s3);
 #pragma unroll
@@ -1179,10 +1189,10 @@ extern "C" int lmvd_inverse_transform_noalloc(int nx, int ny, int nz, const void
     ZMaps maps;
     if (!tile_map(&maps.m[0], fi.p[0], g.nxh, nz, ny, fz.batch, fz.rows_in)) return LMVD_ERR_CUDA;
     dim3 gz(cdiv(nx / 2, fz.batch), ny, 1);
-    // an ordinary launch: it reads the twiddles, which the kernel before may have written, through the read-only path
+    // an ordinary launch where the twiddles, which the kernel ahead may have written, come through the read-only path
     if (fz.ept == 12 && fz.batch == 4) k_fft_z_inv<cd, 12, 4><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, te, nullptr);
     else if (fz.ept == 12) k_fft_z_inv<cd, 12, 2><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, te, nullptr);
-    else k_fft_z_inv<cd, 6, 4><<<gz, threads(fz), smem_bytes(fz), st>>>(fz, g, maps, T, 0, te, nullptr);
+    else launch_next(k_fft_z_inv<cd, 6, 4>, gz, threads(fz), smem_bytes(fz), st, fz, g, maps, T, 0, te, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
     dim3 gx(cdiv(cdiv(g.pz, 2), fx.batch), ny, 1);
     if (fx.ept == 12) launch_next(k_fft_x_inv<12>, gx, threads(fx), smem_bytes(fx), st, fx, g, T, 0, te, fo, nullptr);

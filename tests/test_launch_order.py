@@ -39,3 +39,12 @@ def test_ordinary_kernels_are_launched_in_stream_order():
 
 def test_exponents_written_by_the_pass_ahead_use_plain_loads():
     assert not re.search(r"__ldg\(\s*(ej|te)\b", (CSRC / "fft.cu").read_text())
+
+
+def test_twiddles_of_an_overlapping_launch_use_plain_loads():
+    """The allocation-free transform's z-pass overlaps the kernel that writes its twiddles only in the instantiation
+    that reads them with plain loads (6 elements a thread)."""
+    text = (CSRC / "fft.cu").read_text()
+    assert len(re.findall(r"__ldg\(", text)) == 1 and "if constexpr (EPT == 12 && (S > 1 || SIGN > 0)) return __ldg(p);" in text
+    entry = text[text.index("lmvd_inverse_transform_noalloc(int nx"):]
+    assert re.findall(r"launch_next\((k_fft_z_inv<[^>]*>)", entry) == ["k_fft_z_inv<cd, 6, 4>"]
