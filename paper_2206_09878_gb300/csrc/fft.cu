@@ -19,11 +19,11 @@
 // Arithmetic: 64-bit fixed point with one exponent per 1D transform (fx.cuh), in both precisions. The
 // FP64 pipe retires 1.68 additions per clock per SM here, and transforms in complex double were bound by
 // it (85% busy); in fixed point the same passes run on the integer pipes (ALU 45-52%, multiply pipe
-// 50-60% busy), 5.3 times faster in FP64 arithmetic's place and 1.3 times faster than the double-float
-// transforms they replaced in the precision path: at 512 x 65 x 512, per substage, 100.1 ms (complex
-// double) and 25.2 ms (double-float) -> 18.8 ms. Physical fields and FP64 spectral fields are complex
-// double / double; the precision path's spectral inputs are double-float pairs; T is fixed point with an
-// array of exponents, so the conversions are at the ends only.
+// 50-60% busy), 5.4 times faster than in complex double and 1.4 times faster than in the double-float
+// arithmetic of the former precision path: at 512 x 65 x 512, per substage, 100.1 ms (complex double) and
+// 25.2 ms (double-float) -> 18.4 ms. Spectral fields are complex double (the precision path's inputs
+// double-float pairs) and physical fields double; T is fixed point with an array of exponents, so the
+// conversions are at the ends only.
 // Accuracy (rms error over rms result against a transform in extended precision, 2D inverse of white
 // noise / k^-2 spectra): 32^2: 4.9e-17 / 4.7e-17 (complex double: 2.1e-16 / 1.9e-16), 128 x 96: 7.7e-17 /
 // 4.9e-17 (2.5e-16 / 2.0e-16), 512^2: 2.3e-16 / 6.7e-17 (2.8e-16 / 2.3e-16).
