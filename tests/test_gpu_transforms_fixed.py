@@ -84,3 +84,30 @@ def test_non_finite_inputs_stay_in_their_plane(L, bad):
     kept = torch.isfinite(torch.view_as_real(back))[:, :, :nx // 2].flatten(2)
     assert not kept[3, 0].any() and kept[[i for i in range(ny) if i != 3]].all()
     ctx.close()
+
+
+# chunks of the intermediate: ten fields on grids where those take at most 512 MiB (16 x 10 x 16 and, just below, 256
+# x 62 x 256 with 465), four beyond (256 x 70 x 256: 525); field counts around both
+@pytest.mark.parametrize("nx,ny,nz,counts", [(16, 10, 16, (1, 4, 9, 10, 11, 21)), (256, 62, 256, (10, 11)),
+                                             (256, 70, 256, (4, 5, 9))])
+def test_chunks_of_fields(L, nx, ny, nz, counts):
+    """Fields of one call against the same fields one call each (another plan may be picked by their number, so the
+    results agree to the passes' rounding, not bit for bit)."""
+    gen = torch.Generator(device="cuda").manual_seed(nx + ny)
+    ctx = L.Context(L.lmvd_default_config(nx, ny, nz))
+    px, pz, nxh = 3 * nx // 2, 3 * nz // 2, nx // 2 + 1
+    for n in counts:
+        phys = torch.randn((n, ny, pz, px), generator=gen, dtype=torch.float64, device="cuda")
+        spec = torch.zeros((n, ny, nz, nxh), dtype=torch.complex128, device="cuda")
+        out = torch.zeros_like(phys)
+        one_s, one_p = torch.zeros_like(spec[0]), torch.zeros_like(phys[0])
+        torch.cuda.synchronize()
+        L.lmvd_forward_transform(ctx.h, phys, spec, n)
+        L.lmvd_inverse_transform(ctx.h, spec, out, n)
+        for f in range(n):
+            L.lmvd_forward_transform(ctx.h, phys[f], one_s, 1)
+            L.lmvd_inverse_transform(ctx.h, spec[f], one_p, 1)
+            ctx.synchronize()
+            assert (spec[f] - one_s).abs().max() <= 1e-13 * one_s.abs().max(), (n, f)
+            assert (out[f] - one_p).abs().max() <= 1e-13 * one_p.abs().max(), (n, f)
+    ctx.close()
