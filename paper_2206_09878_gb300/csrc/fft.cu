@@ -257,6 +257,15 @@ __device__ __forceinline__ void mag_add(FxMag& m, cd x) { m.add(x.re, x.im); }
 __device__ __forceinline__ void mag_add(FxMag& m, cdf x) { m.add(x.re, x.im); }
 template <class RAW>
 constexpr bool kIsDf = std::is_same<RAW, cdf>::value;
+template <int N>
+__device__ __forceinline__ int fx_any_bits(const cd (&raw)[N]) {
+  int any = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) any |= __double2loint(raw[i].re) | __double2loint(raw[i].im);
+  return any != 0;
+}
+template <int N>
+__device__ __forceinline__ int fx_any_bits(const cdf (&)[N]) { return 0; }
 
 // k of this thread's transform from the RAW values its threads hold (each counted `weight` times), all threads of
 // the CTA together; xe: see fx_rescale (0 on the usual path). One barrier.
@@ -266,6 +275,7 @@ __device__ __forceinline__ int fx_scale(RAW (&raw)[N], FxShared& sh, int slot, i
   FxMag m;
 #pragma unroll
   for (int i = 0; i < N; ++i) mag_add(m, raw[i]);
+  if (m.top == 0) m.top = fx_any_bits(raw);  // magnitudes below 2^-1042 have an empty high word
   float v = group_sum(m.sum, g, S);
   if ((tt & (g - 1)) == 0 && LMVD_IN(slot + (tt / g) * stride, FX_RED)) sh.red[slot + (tt / g) * stride] = v;
   xe = 0;
@@ -280,14 +290,16 @@ __device__ __forceinline__ int fx_scale(RAW (&raw)[N], FxShared& sh, int slot, i
   }
   float s = 0.f;
   for (int i = 0; i < np; ++i) s += sh.red[slot + i * stride];
-  return fx_exponent(weight * s);
+  return s == 0.f ? kFxZeroK : fx_exponent(weight * s);
 }
 // The intermediate T between the two passes of a transform stays in fixed point: 16 bytes per element and one
 // exponent E per transform of the first pass (a kx column of the inverse, a row pair of the forward one; the value is
-// X 2^-E), so neither side converts; kFxNan marks a transform with inf or nan in it. The second pass's exponent k is
-// at most the smallest E of its inputs (their own unit: a smaller one holds no information), so that its inputs only
-// shift right. Sums are formed from the high words in FP32, E in the range that the usual path gives.
-constexpr int kFxNan = INT_MIN, kFxMinE = -40, kFxMaxE = 165;
+// X 2^-E), so neither side converts; kFxNan marks a transform with inf or nan in it, kFxZero one of zeros (or of values
+// below 2^-126 of the largest one of its CTA). The second pass's exponent k is at most the smallest E of its inputs
+// (their own unit: a smaller one holds no information), so that its inputs only shift right; zeros have no unit and are
+// above every E, so that an empty column does not limit the others of its plane. Sums are formed from the high words in
+// FP32, E in the range that the usual path gives (up to 161, where fx_exponent ends too).
+constexpr int kFxNan = INT_MIN, kFxZero = 1 << 20, kFxMinE = -40, kFxMaxE = 161;
 __device__ __forceinline__ float fx_mag_hi(cfx x) {
   return fabsf(__int2float_rn((int)(x.re >> 32))) + fabsf(__int2float_rn((int)(x.im >> 32)));
 }
@@ -305,7 +317,7 @@ __device__ __forceinline__ int fx_scale_t(float mag, int& emin, FxShared& sh, in
   emin = __reduce_min_sync(warp_lanes(), emin);
   if ((threadIdx.x & 31) == 0) sh.emin[threadIdx.x >> 5] = emin;
   xe = 0;
-  const bool slow = __syncthreads_or(emin < kFxMinE || emin > kFxMaxE);
+  const bool slow = __syncthreads_or(emin < kFxMinE || emin > kFxMaxE && emin != kFxZero);
   const int nw = (blockDim.x + 31) >> 5;
   for (int w = 0; w < nw; ++w) emin = min(emin, sh.emin[w]);
   if (slow) {
@@ -324,9 +336,11 @@ __device__ __forceinline__ int fx_scale_t(float mag, int& emin, FxShared& sh, in
   for (int i = 0; i < np; ++i) s += sh.red[slot + i * stride];
   return min(fx_exponent(weight * s), emin);
 }
-// X 2^(k - E), rounded; d = E - k >= 0
+// X 2^(k - E), rounded to nearest; d = E - k >= 0. Beyond 62 places a magnitude of up to 2^62 becomes 0; the forward
+// pass's row sums may reach 2^62.7, which then become -1, an error below two units. (Without the rounding above 32 places
+// the columns of a decaying spectrum were off by half a unit on average, all in the same direction.)
 __device__ __forceinline__ cfx fx_align(cfx x, int d) {
-  const long long h = (long long)(unsigned long long)shl32(1u, d - 1);
+  const long long h = (long long)((unsigned long long)shl32(1u, min(d, 63) - 33) << 32 | shl32(1u, d - 1));
   return cfx{sar64(x.re + h, d), sar64(x.im + h, d)};
 }
 __device__ __forceinline__ cfx fx_convert(cd x, int k, float) { return cfx{fx_from(x.re, k), fx_from(x.im, k)}; }
@@ -410,7 +424,9 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
 }
 
 // The exponent a transform's fixed-point results are stored with (xe: fx_rescale's)
-__device__ __forceinline__ int fx_stored_exponent(int k, int xe) { return xe == kFxPoison ? kFxNan : k - xe; }
+__device__ __forceinline__ int fx_stored_exponent(int k, int xe) {
+  return xe == kFxPoison ? kFxNan : (k == kFxZeroK ? kFxZero : k - xe);
+}
 
 // Fixed-point inputs v of a transform in shared memory: through a first radix-4 stage in registers (v in the order of
 // fx_first4), or, for a plan without one, to the points tt + u tpt (v in that order), then the middle stages.
@@ -535,7 +551,7 @@ __device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, con
   const int* ej = te + ((size_t)f * g.ny + j) * h;
 #pragma unroll
   for (int u = 0; u < NP; ++u) {
-    E[u] = LMVD_IN(tt + u * tpt, h) ? ej[tt + u * tpt] : kFxMaxE;
+    E[u] = LMVD_IN(tt + u * tpt, h) ? ej[tt + u * tpt] : kFxZero;
     emin = min(emin, E[u]);
   }
   if (!mbar_wait_bounded(bar, flags)) return;
@@ -723,7 +739,7 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
 #pragma unroll
   for (int u = 0; u < EPT; ++u) {
     const int i = fx_point(u, first4, tt, tpt, pz >> 2);
-    E[u] = LMVD_IN(i, pz) ? ej[i >> 1] : kFxMaxE;
+    E[u] = LMVD_IN(i, pz) ? ej[i >> 1] : kFxZero;
     emin = min(emin, E[u]);
   }
   if (!mbar_wait_bounded(bar, flags)) return;

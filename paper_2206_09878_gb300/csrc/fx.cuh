@@ -95,7 +95,8 @@ __device__ __forceinline__ bool fx_out_of_range(const FxMag& m, bool df_in) {
   return !(m.sum < kFxHuge) || (m.sum < kFxTiny && m.top != 0) || (!df_in && m.top >= 0x47000000);
 }
 
-// k for the sum S: S 2^k <= 2^61.7 (sums truncate by < 2^-18)
+// k for the sum S: S 2^k <= 2^61.7 (sums truncate by < 2^-18); at most 161
+constexpr int kFxZeroK = 162;  // a transform of zeros: it has no exponent of its own (fx_stored_exponent)
 __device__ __forceinline__ int fx_exponent(float S) {
   S = fmaxf(S, kFxTiny);
   const int b = __float_as_int(S), e = (b >> 23) - 127;
@@ -123,8 +124,8 @@ __device__ __forceinline__ unsigned long long shl64(unsigned long long a, int n)
   asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
   return r;
 }
-// x 2^k (|x| 2^k < 2^62; a subnormal x becomes 0), rounded to nearest; a magnitude below 2^-33 of the largest
-// possible one is truncated toward zero
+// x 2^k (|x| 2^k < 2^62), rounded to nearest; a magnitude below 2^-33 of the largest possible one is truncated toward
+// zero. A subnormal x becomes 0: where a transform consists of such values fx_rescale has scaled them.
 __device__ __forceinline__ long long fx_from(double x, int k) {
   const int hi = __double2hiint(x), lo = __double2loint(x);
   const int e = (hi >> 20) & 0x7ff;
