@@ -72,10 +72,16 @@ __device__ __forceinline__ void fx_bfly4(cfx& v0, cfx& v1, cfx& v2, cfx& v3) {
   v2 = (a - s) + c;
   v3 = (a - t) - c;
 }
-template <int SIGN>
+// LAST: the last stage's. In the others the half of an odd t rounds up or down as v0 is odd or even, so that its error has
+// no direction of its own (rounded down, the three or four radix-3 stages of 432 to 648 modes put errors of 14 to 26 times
+// the rms into a few outputs); an even t stays exact. 4 fields of 216 x 65 x 108, six such stages in its two passes: 171.7
+// -> 174.8 us. In the last stage a half rounded down moves an output by one unit at most, and the rounding would cost
+// registers: 3 fields of 256 x 129 x 256 forward 498.2 -> 505.0 us.
+template <int SIGN, bool LAST>
 __device__ __forceinline__ void fx_bfly3(cfx& v0, cfx& v1, cfx& v2, int2 s3) {
   const cfx t = v1 + v2, d = v1 - v2;
-  const cfx m{v0.re - (t.re >> 1), v0.im - (t.im >> 1)};
+  const cfx m = LAST ? cfx{v0.re - (t.re >> 1), v0.im - (t.im >> 1)}
+                     : cfx{v0.re - ((t.re + (v0.re & 1)) >> 1), v0.im - ((t.im + (v0.im & 1)) >> 1)};
   const long long ur = fx_mulr(d.re, s3), ui = fx_mulr(d.im, s3);
   const cfx u = SIGN > 0 ? cfx{-ui, ur} : cfx{ui, -ur};  // (SIGN i sin(2 pi / 3)) (v1 - v2)
   v0 = v0 + t;
@@ -87,7 +93,7 @@ __device__ __forceinline__ void fx_butterfly(cfx (&v)[R], const FFTPlan& pl) {
   if constexpr (R == 4) {
     fx_bfly4<SIGN>(v[0], v[1], v[2], v[3]);
   } else if constexpr (R == 3) {
-    fx_bfly3<SIGN>(v[0], v[1], v[2], pl.s3);
+    fx_bfly3<SIGN, false>(v[0], v[1], v[2], pl.s3);
   } else {
     const cfx t = v[0];
     v[0] = t + v[1];
@@ -194,7 +200,7 @@ __device__ __forceinline__ void fx_last(const cfx* x, const FFTPlan& pl, int tt,
 #pragma unroll
     for (int q = 1; q < EPT; ++q) u[q] = fx_mulw<SIGN>(u[q], fx_tw<SIGN, EPT, S>(pl.tw + q * tt));
 #pragma unroll
-  for (int b = 0; b < R; ++b) fx_bfly3<SIGN>(u[3 * b], u[(R + 3 * b) % EPT], u[(2 * R + 3 * b) % EPT], pl.s3);
+  for (int b = 0; b < R; ++b) fx_bfly3<SIGN, true>(u[3 * b], u[(R + 3 * b) % EPT], u[(2 * R + 3 * b) % EPT], pl.s3);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     // u[(R a + 3 b) mod EPT] now holds (a', b) = (a, b)
