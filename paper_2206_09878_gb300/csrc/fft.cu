@@ -24,9 +24,14 @@
 // 25.2 ms (double-float) -> 18.4 ms. Spectral fields are complex double (the precision path's inputs
 // double-float pairs) and physical fields double; T is fixed point with an array of exponents, so the
 // conversions are at the ends only.
-// Accuracy (rms error over rms result against a transform in extended precision, 2D inverse of white
-// noise / k^-2 spectra): 32^2: 4.9e-17 / 4.7e-17 (complex double: 2.1e-16 / 1.9e-16), 128 x 96: 7.7e-17 /
-// 4.9e-17 (2.5e-16 / 2.0e-16), 512^2: 2.3e-16 / 6.7e-17 (2.8e-16 / 2.3e-16).
+// Accuracy (rms error over rms result against a transform in extended precision; 2D transforms of white noise, the
+// least and the most over amplitudes 1 .. 2, which the unit follows in one step; in parentheses complex double):
+//   modes           32^2              128^2             512^2             768^2             1024^2
+//   inverse   4.7-5.1e-17 (2.1e-16)  6.5-8.4e-17 (2.5)  1.4-2.5e-16 (2.8)  1.0-1.5e-16 (3.0)  1.3-1.7e-16 (3.0)
+//   forward   8.4-9.2e-17 (2.4e-16)  1.0-1.2e-16 (2.6)  1.9-2.8e-16 (2.9)  1.5-1.8e-16 (3.1)  1.6-2.2e-16 (3.0)
+// k^-2 spectra, inverse: 4.8e-17 (1.8e-16) at 32^2, 6.1e-17 (2.4e-16) at 512^2, 7.3e-17 (2.7e-16) at 1024^2.
+// Inputs whose sums leave the range of single precision (fx_out_of_range) or lie near its low end take a slow path: 4
+// fields of 512 x 65 x 512 at 1e-34 2.41 / 2.23 ms instead of 1.43 / 1.38 (complex double 7.8 / 8.6).
 #include <cuda.h>  // CUtensorMap and its enums (the encoder is reached through the runtime, no libcuda link)
 
 #include <climits>
@@ -72,16 +77,16 @@ __device__ __forceinline__ void fx_bfly4(cfx& v0, cfx& v1, cfx& v2, cfx& v3) {
   v2 = (a - s) + c;
   v3 = (a - t) - c;
 }
-// LAST: the last stage's. In the others the half of an odd t rounds up or down as v0 is odd or even, so that its error has
-// no direction of its own (rounded down, the three or four radix-3 stages of 432 to 648 modes put errors of 14 to 26 times
-// the rms into a few outputs); an even t stays exact. 4 fields of 216 x 65 x 108, six such stages in its two passes: 171.7
-// -> 174.8 us. In the last stage a half rounded down moves an output by one unit at most, and the rounding would cost
-// registers: 3 fields of 256 x 129 x 256 forward 498.2 -> 505.0 us.
-template <int SIGN, bool LAST>
+// FAIR: the half of an odd t rounds up or down as v0 is odd or even, so that its error has no direction of its own (rounded
+// down, the three or four radix-3 stages of 432 to 648 modes put errors of 14 to 26 times the rms into a few outputs); an
+// even t stays exact. 4 fields of 216 x 65 x 108, six such stages in its two passes: 171.7 -> 174.8 us. The last stage of
+// lengths without guard bits rounds down: that moves an output by 1.5 units on average, a tenth of the noise, and the
+// rounding would cost registers there: 3 fields of 256 x 129 x 256 forward 498.2 -> 505.0 us.
+template <int SIGN, bool FAIR>
 __device__ __forceinline__ void fx_bfly3(cfx& v0, cfx& v1, cfx& v2, int2 s3) {
   const cfx t = v1 + v2, d = v1 - v2;
-  const cfx m = LAST ? cfx{v0.re - (t.re >> 1), v0.im - (t.im >> 1)}
-                     : cfx{v0.re - ((t.re + (v0.re & 1)) >> 1), v0.im - ((t.im + (v0.im & 1)) >> 1)};
+  const cfx m = FAIR ? cfx{v0.re - ((t.re + (v0.re & 1)) >> 1), v0.im - ((t.im + (v0.im & 1)) >> 1)}
+                     : cfx{v0.re - (t.re >> 1), v0.im - (t.im >> 1)};
   const long long ur = fx_mulr(d.re, s3), ui = fx_mulr(d.im, s3);
   const cfx u = SIGN > 0 ? cfx{-ui, ur} : cfx{ui, -ur};  // (SIGN i sin(2 pi / 3)) (v1 - v2)
   v0 = v0 + t;
@@ -93,7 +98,7 @@ __device__ __forceinline__ void fx_butterfly(cfx (&v)[R], const FFTPlan& pl) {
   if constexpr (R == 4) {
     fx_bfly4<SIGN>(v[0], v[1], v[2], v[3]);
   } else if constexpr (R == 3) {
-    fx_bfly3<SIGN, false>(v[0], v[1], v[2], pl.s3);
+    fx_bfly3<SIGN, true>(v[0], v[1], v[2], pl.s3);
   } else {
     const cfx t = v[0];
     v[0] = t + v[1];
@@ -111,10 +116,34 @@ __device__ __forceinline__ int4 fx_tw(const int4* p) {
   else return *p;
 }
 
+// Guard bits (GUARD, lengths above kFxGuardLength). The unit follows the sum S of a transform's inputs, which grows like n
+// for a white input, while binary64's error hardly grows: above 768 points the noise, most of it from the rounding of the
+// inputs, would exceed it. But the first two stages add up at most 16 inputs, so their values carry e <= 2 more bits where
+// 16 times the largest input allows (white inputs; with a few large ones S is small already), and the third stage's
+// twiddles are 2^-e as large, so that its products round back to the unit. The noise of a 1536-point transform falls from
+// 17.5 units to 6.3, the error at 1024 x 1024 modes from 3.9-5.8e-16 to 1.3-1.7e-16 (inverse; forward 3.6-5.3e-16 to 1.6-2.2e-16;
+// complex double 3.0e-16). It costs registers and a tenth of the time: 4 fields of 768 x 33 x 768 1.99 / 1.93 -> 2.18 / 2.07 ms
+// (inverse / forward; complex double 9.9 / 10.8). Shorter lengths are as accurate without.
+constexpr int kFxGuardLength = 768, kFxGuardBits = 2, kFxGuardStage = 2;
+__device__ __forceinline__ int fx_guard(int most, int emin, int k) {  // most: see the callers
+  return max(0, min(min(most, emin - k), kFxGuardBits));
+}
+// the limbs of w 2^-e, e > 0; the low one toward zero, so that those of 1 and -1, whose products may end in a half, round
+// that toward zero and not always up
+__device__ __forceinline__ int2 fx_limbs_shift(int hi, int lo, int e) {
+  const int h = (hi >> e) + ((hi >> (e - 1)) & 1), rem = (int)((unsigned)hi - ((unsigned)h << e));
+  return make_int2(h, (int)((unsigned)rem << (31 - e)) + ((lo + (lo >> 31 & (1 << e) - 1)) >> e));
+}
+// x 2^-e, e > 0, rounded to nearest; a half goes up or down by a bit that the result does not hold (to even would favour
+// even results, whose lowest bits steer fx_bfly3)
+__device__ __forceinline__ long long fx_round(long long x, int e) {
+  return (x + ((1ll << (e - 1)) - 1 + ((x >> (e + 1)) & 1))) >> e;
+}
+
 // The sub-length L divides tpt (the radices before the last multiply to tpt), so a thread's butterflies share k = tt mod
-// L and their twiddles, which are fetched before the barrier.
-template <int SIGN, int R, int EPT, int S>
-__device__ __forceinline__ void fx_stage(cfx* x, const FFTPlan& pl, int L, int tt, int tpt) {
+// L and their twiddles, which are fetched before the barrier. SHIFT: the stage takes off e guard bits.
+template <int SIGN, int R, int EPT, int S, bool SHIFT>
+__device__ __forceinline__ void fx_stage(cfx* x, const FFTPlan& pl, int L, int tt, int tpt, int e) {
   constexpr int NBT = EPT / R;
   const int n = pl.n;
   const int nb = n / R;
@@ -123,6 +152,12 @@ __device__ __forceinline__ void fx_stage(cfx* x, const FFTPlan& pl, int L, int t
   int4 w[R];
 #pragma unroll
   for (int q = 1; q < R; ++q) w[q] = fx_tw<SIGN, EPT, S>(pl.tw + q * kt);
+  if (SHIFT && e)
+#pragma unroll
+    for (int q = 1; q < R; ++q) {
+      const int2 c = fx_limbs_shift(w[q].x, w[q].y, e), s = fx_limbs_shift(w[q].z, w[q].w, e);
+      w[q] = make_int4(c.x, c.y, s.x, s.y);
+    }
   cfx v[NBT][R];
 #pragma unroll
   for (int j = 0; j < NBT; ++j)
@@ -136,9 +171,10 @@ __device__ __forceinline__ void fx_stage(cfx* x, const FFTPlan& pl, int L, int t
 #pragma unroll
   for (int j = 0; j < NBT; ++j) {
     if (!LMVD_IN((tt - k) * R + k + j * tpt * R + (R - 1) * L, n)) continue;
-    if (k)  // (a product with w = 1 would not be exact)
+    if (k || SHIFT && e)  // (a product with w = 1 would not be exact)
 #pragma unroll
       for (int q = 1; q < R; ++q) v[j][q] = fx_mulw<SIGN>(v[j][q], w[q]);
+    if (SHIFT && e) v[j][0] = cfx{fx_round(v[j][0].re, e), fx_round(v[j][0].im, e)};
     fx_butterfly<SIGN, R>(v[j], pl);
 #pragma unroll
     for (int q = 0; q < R; ++q) y[(j * tpt * R + q * L) * S] = v[j][q];
@@ -161,35 +197,45 @@ __device__ __forceinline__ void fx_first4(cfx (&v)[12], cfx* x, const FFTPlan& p
   __syncthreads();
 }
 
-// Stages s0 .. nst - 2; returns when every point of the last stage's input is in x.
-template <int SIGN, int EPT, int S>
-__device__ __forceinline__ void fx_middle(cfx* x, const FFTPlan& pl, int s0, int tt, int tpt) {
+// Stages s0 .. nst - 2; returns when every point of the last stage's input is in x. e: the inputs' guard bits (a length above
+// kFxGuardLength has four of these stages).
+template <int SIGN, int EPT, int S, bool GUARD>
+__device__ __forceinline__ void fx_middle(cfx* x, const FFTPlan& pl, int s0, int tt, int tpt, int e) {
   int L = 1;
   unsigned code = pl.code;
   if (s0) {
     L = 4;
     code >>= 2;
   }
-  for (int s = s0; s < pl.nst - 1; ++s, code >>= 2) {
+  auto stage = [&](auto shift) {
+    constexpr bool SHIFT = decltype(shift)::value;
     const unsigned r2 = code & 3u;
     if (EPT == 12 && r2 == 0) {
-      fx_stage<SIGN, 4, EPT, S>(x, pl, L, tt, tpt);
+      fx_stage<SIGN, 4, EPT, S, SHIFT>(x, pl, L, tt, tpt, e);
       L *= 4;
     } else if (r2 == 1) {
-      fx_stage<SIGN, 2, EPT, S>(x, pl, L, tt, tpt);
+      fx_stage<SIGN, 2, EPT, S, SHIFT>(x, pl, L, tt, tpt, e);
       L *= 2;
     } else {
-      fx_stage<SIGN, 3, EPT, S>(x, pl, L, tt, tpt);
+      fx_stage<SIGN, 3, EPT, S, SHIFT>(x, pl, L, tt, tpt, e);
       L *= 3;
     }
+    code >>= 2;
+  };
+  int s = s0;
+  if constexpr (GUARD) {
+    for (; s < kFxGuardStage; ++s) stage(std::false_type{});
+    stage(std::true_type{});
+    ++s;
   }
+  for (; s < pl.nst - 1; ++s) stage(std::false_type{});
 }
 
 // Last stage: radix EPT, L = n / EPT = tpt; thread tt's butterfly reads and produces the points tt + q L. The EPT-point
 // transform is a prime-factor one (3 x 4 or 3 x 2): input q = (EPT / 3) a + 3 b, output q = 4 a' + s b' mod EPT
 // with s = 9 (EPT 12) or 3 (EPT 6), and no twiddles between its two parts. Against a radix-4 and a radix-3 stage
 // it saves an exchange through shared memory and a third of the two stages' twiddle products.
-template <int SIGN, int EPT, int S>
+template <int SIGN, int EPT, int S, bool GUARD>
 __device__ __forceinline__ void fx_last(const cfx* x, const FFTPlan& pl, int tt, cfx (&v)[EPT]) {
   constexpr int R = EPT / 3;
   const int L = pl.tpt;
@@ -200,7 +246,7 @@ __device__ __forceinline__ void fx_last(const cfx* x, const FFTPlan& pl, int tt,
 #pragma unroll
     for (int q = 1; q < EPT; ++q) u[q] = fx_mulw<SIGN>(u[q], fx_tw<SIGN, EPT, S>(pl.tw + q * tt));
 #pragma unroll
-  for (int b = 0; b < R; ++b) fx_bfly3<SIGN, true>(u[3 * b], u[(R + 3 * b) % EPT], u[(2 * R + 3 * b) % EPT], pl.s3);
+  for (int b = 0; b < R; ++b) fx_bfly3<SIGN, GUARD>(u[3 * b], u[(R + 3 * b) % EPT], u[(2 * R + 3 * b) % EPT], pl.s3);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     // u[(R a + 3 b) mod EPT] now holds (a', b) = (a, b)
@@ -223,6 +269,7 @@ struct FxShared {
   float red[FX_RED];
   int emin[8];
   int top;
+  int wtop[8];  // (GUARD) the warps' largest magnitudes
 };
 
 __device__ __forceinline__ unsigned warp_lanes() {  // the lanes of this warp (the last one may be partial)
@@ -273,17 +320,30 @@ __device__ __forceinline__ int fx_any_bits(const cd (&raw)[N]) {
 template <int N>
 __device__ __forceinline__ int fx_any_bits(const cdf (&)[N]) { return 0; }
 
-// k of this thread's transform from the RAW values its threads hold (each counted `weight` times), all threads of
-// the CTA together; xe: see fx_rescale (0 on the usual path). One barrier.
-template <class RAW, int N>
+// the CTA's largest of the threads' non-negative integers m, in two parts around a barrier
+__device__ __forceinline__ void fx_max_put(int m, FxShared& sh) {
+  m = __reduce_max_sync(warp_lanes(), m);
+  if ((threadIdx.x & 31) == 0) sh.wtop[threadIdx.x >> 5] = m;
+}
+__device__ __forceinline__ int fx_max_get(const FxShared& sh) {
+  int m = 0;
+  for (int w = 0; w < (int)(blockDim.x + 31) >> 5; ++w) m = max(m, sh.wtop[w]);
+  return m;
+}
+
+// k of this thread's transform from the RAW values its threads hold, all threads of the CTA together; xe: see fx_rescale
+// (0 on the usual path); e: the guard bits the inputs may carry beyond k (0 without GUARD): a magnitude with the high word
+// `top` is below 2^(t + 1), so 16 inputs' |re| + |im| stay below 2^(t + 6) and 2^(t + 6 + k + e) <= 2^61. One barrier.
+template <bool GUARD, class RAW, int N>
 __device__ __forceinline__ int fx_scale(RAW (&raw)[N], FxShared& sh, int slot, int np, int stride, int g, int S, int tt,
-                                        float weight, int& xe) {
+                                        int& xe, int& e) {
   FxMag m;
 #pragma unroll
   for (int i = 0; i < N; ++i) mag_add(m, raw[i]);
   if (m.top == 0) m.top = fx_any_bits(raw);  // magnitudes below 2^-1042 have an empty high word
   float v = group_sum(m.sum, g, S);
   if ((tt & (g - 1)) == 0 && LMVD_IN(slot + (tt / g) * stride, FX_RED)) sh.red[slot + (tt / g) * stride] = v;
+  if (GUARD) fx_max_put(m.top, sh);
   xe = 0;
   if (__syncthreads_or(fx_out_of_range(m, kIsDf<RAW>))) {
     xe = fx_rescale(raw, m.top, sh);
@@ -292,11 +352,15 @@ __device__ __forceinline__ int fx_scale(RAW (&raw)[N], FxShared& sh, int slot, i
     for (int i = 0; i < N; ++i) mag_add(r, raw[i]);
     v = group_sum(r.sum, g, S);
     if ((tt & (g - 1)) == 0 && LMVD_IN(slot + (tt / g) * stride, FX_RED)) sh.red[slot + (tt / g) * stride] = v;
+    if (GUARD) fx_max_put(r.top, sh);
     __syncthreads();
   }
   float s = 0.f;
   for (int i = 0; i < np; ++i) s += sh.red[slot + i * stride];
-  return s == 0.f ? kFxZeroK : fx_exponent(weight * s);
+  const int k = s == 0.f ? kFxZeroK : fx_exponent(s);
+  e = 0;
+  if (GUARD) e = fx_guard(55 - (kIsDf<RAW> ? (fx_max_get(sh) >> 23) - 127 : (fx_max_get(sh) >> 20) - 1023) - k, INT_MAX, k);
+  return k;
 }
 // The intermediate T between the two passes of a transform stays in fixed point: 16 bytes per element and one
 // exponent E per transform of the first pass (a kx column of the inverse, a row pair of the forward one; the value is
@@ -306,22 +370,23 @@ __device__ __forceinline__ int fx_scale(RAW (&raw)[N], FxShared& sh, int slot, i
 // above every E, so that an empty column does not limit the others of its plane. Sums are formed from the high words in
 // FP32, E in the range that the usual path gives (up to 161, where fx_exponent ends too).
 constexpr int kFxNan = INT_MIN, kFxZero = 1 << 20, kFxMinE = -40, kFxMaxE = 161;
-__device__ __forceinline__ float fx_mag_hi(cfx x) {
-  return fabsf(__int2float_rn((int)(x.re >> 32))) + fabsf(__int2float_rn((int)(x.im >> 32)));
-}
+__device__ __forceinline__ float fx_abs_hi(long long x) { return fabsf(__int2float_rn((int)(x >> 32))); }
+__device__ __forceinline__ float fx_mag_hi(cfx x) { return fx_abs_hi(x.re) + fx_abs_hi(x.im); }
 __device__ __forceinline__ float fx_pow2(int e) { return __int_as_float((e + 127) << 23); }  // -126 <= e <= 127
 // sum |X| 2^-E of inputs that share E (kFxMinE <= E; a sum at an E beyond kFxMaxE may read too large, never too small)
 __device__ __forceinline__ float fx_mag(float hi_sum, int E) { return hi_sum * 0x1p-32f * fx_pow2(max(64 - E, -126)); }
 
-// As fx_scale, for fixed-point inputs: per thread the sum `mag` of its inputs' magnitudes and the smallest E. On the
-// slow path E is first counted from the CTA's smallest (remag recomputes mag for the shifted E's).
-template <class Remag>
-__device__ __forceinline__ int fx_scale_t(float mag, int& emin, FxShared& sh, int slot, int np, int stride, int g, int S,
-                                          int tt, float weight, int& xe, Remag&& remag) {
+// As fx_scale, for fixed-point inputs: per thread the sum `mag` of its inputs' magnitudes (each |re| + |im|), the largest of
+// them `big` and the smallest E. On the slow path E is first counted from the CTA's smallest (remag recomputes mag and big
+// for the shifted E's).
+template <bool GUARD, class Remag>
+__device__ __forceinline__ int fx_scale_t(float mag, float big, int& emin, FxShared& sh, int slot, int np, int stride, int g,
+                                          int S, int tt, int& xe, int& e, Remag&& remag) {
   float v = group_sum(mag, g, S);
   if ((tt & (g - 1)) == 0 && LMVD_IN(slot + (tt / g) * stride, FX_RED)) sh.red[slot + (tt / g) * stride] = v;
   emin = __reduce_min_sync(warp_lanes(), emin);
   if ((threadIdx.x & 31) == 0) sh.emin[threadIdx.x >> 5] = emin;
+  if (GUARD) fx_max_put(__float_as_int(big), sh);
   xe = 0;
   const bool slow = __syncthreads_or(emin < kFxMinE || emin > kFxMaxE && emin != kFxZero);
   const int nw = (blockDim.x + 31) >> 5;
@@ -331,16 +396,20 @@ __device__ __forceinline__ int fx_scale_t(float mag, int& emin, FxShared& sh, in
       xe = kFxPoison;
     } else {
       xe = 61 - emin;  // E' = E + xe: the largest inputs are of the order of one
-      v = group_sum(remag(xe), g, S);
+      v = group_sum(remag(xe, big), g, S);
       __syncthreads();
       if ((tt & (g - 1)) == 0 && LMVD_IN(slot + (tt / g) * stride, FX_RED)) sh.red[slot + (tt / g) * stride] = v;
+      if (GUARD) fx_max_put(__float_as_int(big), sh);
       __syncthreads();
       emin = 61;
     }
   }
   float s = 0.f;
   for (int i = 0; i < np; ++i) s += sh.red[slot + i * stride];
-  return min(fx_exponent(weight * s), emin);
+  const int k = min(fx_exponent(s), emin);
+  e = 0;
+  if (GUARD) e = fx_guard(56 - ((fx_max_get(sh) >> 23) - 127) - k, emin, k);  // (as in fx_scale: `big` is a sum already)
+  return k;
 }
 // X 2^(k - E), rounded to nearest; d = E - k >= 0. Beyond 62 places a magnitude of up to 2^62 becomes 0; the forward
 // pass's row sums may reach 2^62.7, which then become -1, an error below two units. (Without the rounding above 32 places
@@ -436,12 +505,12 @@ __device__ __forceinline__ int fx_stored_exponent(int k, int xe) {
 
 // Fixed-point inputs v of a transform in shared memory: through a first radix-4 stage in registers (v in the order of
 // fx_first4), or, for a plan without one, to the points tt + u tpt (v in that order), then the middle stages.
-template <int SIGN, int EPT, int S>
-__device__ __forceinline__ void fx_run(cfx (&v)[EPT], cfx* x, const FFTPlan& pl, bool first4, int tt) {
+template <int SIGN, int EPT, int S, bool GUARD>
+__device__ __forceinline__ void fx_run(cfx (&v)[EPT], cfx* x, const FFTPlan& pl, bool first4, int tt, int e) {
   if constexpr (EPT == 12) {
     if (first4) {
       fx_first4<SIGN, S>(v, x, pl, tt, pl.tpt);
-      fx_middle<SIGN, EPT, S>(x, pl, 1, tt, pl.tpt);
+      fx_middle<SIGN, EPT, S, GUARD>(x, pl, 1, tt, pl.tpt, e);
       return;
     }
   }
@@ -449,7 +518,7 @@ __device__ __forceinline__ void fx_run(cfx (&v)[EPT], cfx* x, const FFTPlan& pl,
   for (int u = 0; u < EPT; ++u)
     if (LMVD_IN(tt + u * pl.tpt, pl.n)) x[(tt + u * pl.tpt) * S] = v[u];
   __syncthreads();
-  fx_middle<SIGN, EPT, S>(x, pl, 0, tt, pl.tpt);
+  fx_middle<SIGN, EPT, S, GUARD>(x, pl, 0, tt, pl.tpt, e);
 }
 // input point u of a thread, in the order fx_run expects (step: n / 4 with a first radix-4 stage)
 __device__ __forceinline__ int fx_point(int u, bool first4, int tt, int tpt, int step) {
@@ -494,21 +563,23 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
     const int i = fx_point(u, first4, tt, tpt, pz >> 2);
     raw[u] = kx < h && LMVD_IN(i, pz) && (i < lo || i >= hi) ? reinterpret_cast<const RAW*>(a)[i * COLS + c] : RAW{};
   }
-  int xe;
-  const int gz = pl.red_g, k = fx_scale(raw, sh, c, tpt / gz, COLS, gz, COLS, tt, 1.f, xe);
+  constexpr bool GUARD = COLS == 2;  // (the lengths of which 4 columns do not fit in a CTA)
+  static_assert(4 * kFxGuardLength == 12 * FFT_CTA_Z, "2 columns: above kFxGuardLength");
+  int xe, e;
+  const int gz = pl.red_g, k = fx_scale<GUARD>(raw, sh, c, tpt / gz, COLS, gz, COLS, tt, xe, e);
   {
     cfx v[EPT];
-    const float sa = fx_sa(k);
+    const float sa = fx_sa(k + e);
 #pragma unroll
     for (int u = 0; u < EPT; ++u) {
       const int i = fx_point(u, first4, tt, tpt, pz >> 2);
       v[u] = cfx{0, 0};
-      if (i < lo || i >= hi) v[u] = fx_convert(raw[u], k, sa);  // (whole warps skip the padding)
+      if (i < lo || i >= hi) v[u] = fx_convert(raw[u], k + e, sa);  // (whole warps skip the padding)
     }
-    fx_run<1, EPT, COLS>(v, a + c, pl, first4, tt);
+    fx_run<1, EPT, COLS, GUARD>(v, a + c, pl, first4, tt, e);
   }
   cfx v[EPT];
-  fx_last<1, EPT, COLS>(a + c, pl, tt, v);
+  fx_last<1, EPT, COLS, GUARD>(a + c, pl, tt, v);
   if (kx >= h) return;
   if (tt == 0) te[((size_t)f * g.ny + j) * h + kx] = fx_stored_exponent(k, xe);
   cfx* dst = T + f * tstride + (size_t)j * pz * h + kx;
@@ -521,7 +592,7 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
 // With MUL the epilogue stores w * phys instead of phys (w: a physical field of the same layout, one for all
 // fields of the launch): the product f'(z) dz/dt of the fixed point (Sec. 4.3) formed as the transform is
 // written, so neither dz/dt on the grid nor a separate product pass is needed. (pz is even: 6 divides it.)
-template <int EPT, bool MUL>
+template <int EPT, bool GUARD, bool MUL>
 __device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, const cfx* T, size_t tstride, const int* te,
                                            const FieldsRW& out, const double* wmul, unsigned* flags) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
@@ -562,7 +633,9 @@ __device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, con
   }
   if (!mbar_wait_bounded(bar, flags)) return;
   cfx raw[2 * NP];
-  float hs[NP], mag = 0.f;
+  // |re| + |im| of y[k] and y[px - k] add up to 2 (max(|Xa.re|, |Xb.im|) + max(|Xa.im|, |Xb.re|)); the sum of the four
+  // magnitudes is half a bit more (rms error of a white 1024 x 16 inverse at an unlucky amplitude: 5.3e-16)
+  float hs[NP], mag = 0.f, big = 0.f;
 #pragma unroll
   for (int u = 0; u < NP; ++u) {
     const int kk = tt + u * tpt;
@@ -570,21 +643,28 @@ __device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, con
     raw[2 * u] = in ? y[h + kk] : cfx{0, 0};
     raw[2 * u + 1] = in ? y[2 * h + kk] : cfx{0, 0};
     if (kk == 0) raw[2 * u].im = raw[2 * u + 1].im = 0;  // the kx = 0 coefficient of a real row is real
-    hs[u] = fx_mag_hi(raw[2 * u]) + fx_mag_hi(raw[2 * u + 1]);
-    mag += fx_mag(hs[u], E[u]);
+    hs[u] = 2.f * (fmaxf(fx_abs_hi(raw[2 * u].re), fx_abs_hi(raw[2 * u + 1].im)) +
+                   fmaxf(fx_abs_hi(raw[2 * u].im), fx_abs_hi(raw[2 * u + 1].re)));
+    const float y2 = fx_mag(hs[u], E[u]);
+    mag += y2;
+    big = fmaxf(big, y2);
   }
-  int xe;
+  int xe, e;
   const int gx = pl.red_g, np = tpt / gx;
-  const int k = fx_scale_t(mag, emin, sh, bt * np, np, 1, gx, 1, tt, 2.f, xe, [&](int s) {
-    float m = 0.f;
+  const int k = fx_scale_t<GUARD>(mag, big, emin, sh, bt * np, np, 1, gx, 1, tt, xe, e, [&](int s, float& b) {
+    float m = b = 0.f;
 #pragma unroll
-    for (int u = 0; u < NP; ++u) m += fx_mag(hs[u], E[u] += s);
+    for (int u = 0; u < NP; ++u) {
+      const float y2 = fx_mag(hs[u], E[u] += s);
+      m += y2;
+      b = fmaxf(b, y2);
+    }
     return m;
   });
 #pragma unroll
   for (int u = 0; u < NP; ++u) {
     const int kk = tt + u * tpt;
-    const cfx xa = fx_align(raw[2 * u], E[u] - k), xb = fx_align(raw[2 * u + 1], E[u] - k);
+    const cfx xa = fx_align(raw[2 * u], E[u] - k - e), xb = fx_align(raw[2 * u + 1], E[u] - k - e);
     if (!LMVD_IN(kk, h)) continue;
     if (kk == 0) {
       y[0] = cfx{xa.re, xb.re};
@@ -599,11 +679,11 @@ __device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, con
     if (LMVD_IN(h + tt + u * tpt, px)) y[h + tt + u * tpt] = cfx{0, 0};
   if (tt == 0 && LMVD_IN(2 * h, px)) y[2 * h] = cfx{0, 0};
   __syncthreads();
-  fx_middle<1, EPT, 1>(y, pl, 0, tt, tpt);
+  fx_middle<1, EPT, 1, GUARD>(y, pl, 0, tt, tpt, e);
   double* dst = reinterpret_cast<double*>(pick(out.p, f)) + (size_t)j * g.P + (size_t)za * px;
   const double* w = MUL ? wmul + (size_t)j * g.P + (size_t)za * px : nullptr;
   cfx v[EPT];
-  fx_last<1, EPT, 1>(y, pl, tt, v);
+  fx_last<1, EPT, 1, GUARD>(y, pl, tt, v);
   if (!live) return;
 #pragma unroll
   for (int q = 0; q < EPT; ++q) {
@@ -614,18 +694,18 @@ __device__ __forceinline__ void x_inv_body(const FFTPlan& pl, const Grid& g, con
     dst[px + x] = MUL ? w[px + x] * r.im : r.im;
   }
 }
-template <int EPT>
+template <int EPT, bool GUARD>
 __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_inv(FFTPlan pl, Grid g, const cfx* T, size_t tstride,
                                                                     const int* te, FieldsRW out, unsigned* flags) {
   grid_wait();
-  x_inv_body<EPT, false>(pl, g, T, tstride, te, out, nullptr, flags);
+  x_inv_body<EPT, GUARD, false>(pl, g, T, tstride, te, out, nullptr, flags);
 }
-template <int EPT>
+template <int EPT, bool GUARD>
 __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_inv_mul(FFTPlan pl, Grid g, const cfx* T, size_t tstride,
                                                                         const int* te, FieldsRW out, const double* wmul,
                                                                         unsigned* flags) {
   grid_wait();
-  x_inv_body<EPT, true>(pl, g, T, tstride, te, out, wmul, flags);
+  x_inv_body<EPT, GUARD, true>(pl, g, T, tstride, te, out, wmul, flags);
 }
 
 // ---------------------------------------------------------------- forward x-pass (r2c, 2 rows per transform)
@@ -637,7 +717,7 @@ struct Dot3 {
   const double* w[3];
   const double* m[3];
 };
-template <int EPT, bool DOT3>
+template <int EPT, bool GUARD, bool DOT3>
 __device__ __forceinline__ void x_fwd_body(const FFTPlan& pl, const Grid& g, const FieldsRC& in, cfx* T, size_t tstride,
                                            int* te, const Dot3& d) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
@@ -671,20 +751,20 @@ __device__ __forceinline__ void x_fwd_body(const FFTPlan& pl, const Grid& g, con
     raw[u] = v;
   }
   __syncthreads();  // sh.top
-  int xe;
+  int xe, e;
   // (the sums p + conj(m) = twice a row's coefficient formed at the end may reach 2^62.7: no product follows)
-  const int gx = pl.red_g, np = tpt / gx, k = fx_scale(raw, sh, bt * np, np, 1, gx, 1, tt, 1.f, xe);
+  const int gx = pl.red_g, np = tpt / gx, k = fx_scale<GUARD>(raw, sh, bt * np, np, 1, gx, 1, tt, xe, e);
   {
     cfx v[EPT];
 #pragma unroll
-    for (int u = 0; u < EPT; ++u) v[u] = fx_convert(raw[u], k, 0.f);
-    fx_run<-1, EPT, 1>(v, y, pl, first4, tt);
+    for (int u = 0; u < EPT; ++u) v[u] = fx_convert(raw[u], k + e, 0.f);
+    fx_run<-1, EPT, 1, GUARD>(v, y, pl, first4, tt, e);
   }
   // last stage: the retained kx are the outputs q < NP (kx = tt + q tpt) and q >= 2 NP (px - kx); a thread keeps the
   // first and stores the others for the thread that pairs them
   constexpr int NP = EPT / 3;
   cfx v[EPT];
-  fx_last<-1, EPT, 1>(y, pl, tt, v);
+  fx_last<-1, EPT, 1, GUARD>(y, pl, tt, v);
 #pragma unroll
   for (int q = 2 * NP; q < EPT; ++q)
     if (LMVD_IN(tt + q * tpt, px)) y[tt + q * tpt] = v[q];  // this thread's own inputs
@@ -702,17 +782,17 @@ __device__ __forceinline__ void x_fwd_body(const FFTPlan& pl, const Grid& g, con
     dst[h + kk] = cfx{p.im + m.im, m.re - p.re};
   }
 }
-template <int EPT>
+template <int EPT, bool GUARD>
 __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_fwd(FFTPlan pl, Grid g, FieldsRC in, cfx* T, size_t tstride,
                                                                     int* te) {
   grid_wait();
-  x_fwd_body<EPT, false>(pl, g, in, T, tstride, te, Dot3{});
+  x_fwd_body<EPT, GUARD, false>(pl, g, in, T, tstride, te, Dot3{});
 }
-template <int EPT>
+template <int EPT, bool GUARD>
 __global__ void __launch_bounds__(FFT_CTA_X, FFT_MIN_X) k_fft_x_fwd_dot3(FFTPlan pl, Grid g, cfx* T, size_t tstride, int* te,
                                                                          Dot3 d) {
   grid_wait();
-  x_fwd_body<EPT, true>(pl, g, FieldsRC{}, T, tstride, te, d);
+  x_fwd_body<EPT, GUARD, true>(pl, g, FieldsRC{}, T, tstride, te, d);
 }
 
 // ---------------------------------------------------------------- forward z-pass (truncate, scale)
@@ -750,25 +830,32 @@ __global__ void __launch_bounds__(FFT_CTA_Z, FFT_MIN_Z)
   }
   if (!mbar_wait_bounded(bar, flags)) return;
   cfx v[EPT];
-  float mag = 0.f;
+  float mag = 0.f, big = 0.f;
 #pragma unroll
   for (int u = 0; u < EPT; ++u) {
     const int i = fx_point(u, first4, tt, tpt, pz >> 2);
     v[u] = LMVD_IN(i, pz) ? a[i * COLS + c] : cfx{0, 0};
-    mag += fx_mag(fx_mag_hi(v[u]), E[u]);
+    const float z = fx_mag(fx_mag_hi(v[u]), E[u]);
+    mag += z;
+    big = fmaxf(big, z);
   }
-  int xe;
+  constexpr bool GUARD = COLS == 2;  // (as in the inverse z-pass)
+  int xe, e;
   const int gz = pl.red_g;
-  const int k = fx_scale_t(mag, emin, sh, c, tpt / gz, COLS, gz, COLS, tt, 1.f, xe, [&](int s) {
-    float m = 0.f;
+  const int k = fx_scale_t<GUARD>(mag, big, emin, sh, c, tpt / gz, COLS, gz, COLS, tt, xe, e, [&](int s, float& b) {
+    float m = b = 0.f;
 #pragma unroll
-    for (int u = 0; u < EPT; ++u) m += fx_mag(fx_mag_hi(v[u]), E[u] += s);
+    for (int u = 0; u < EPT; ++u) {
+      const float z = fx_mag(fx_mag_hi(v[u]), E[u] += s);
+      m += z;
+      b = fmaxf(b, z);
+    }
     return m;
   });
 #pragma unroll
-  for (int u = 0; u < EPT; ++u) v[u] = fx_align(v[u], E[u] - k);
-  fx_run<-1, EPT, COLS>(v, a + c, pl, first4, tt);
-  fx_last<-1, EPT, COLS>(a + c, pl, tt, v);
+  for (int u = 0; u < EPT; ++u) v[u] = fx_align(v[u], E[u] - k - e);
+  fx_run<-1, EPT, COLS, GUARD>(v, a + c, pl, first4, tt, e);
+  fx_last<-1, EPT, COLS, GUARD>(a + c, pl, tt, v);
   if (kx > h) return;
   cd* dst = pick(out.p, f) + (size_t)j * g.M + kx;
   // outputs q < NP (kz = tt + q tpt) and q >= 2 NP (kz = i - n2, row n2 + i; i = 0 is the Nyquist row)
@@ -882,6 +969,8 @@ static bool tile_map(CUtensorMap* m, const void* base, size_t cols, size_t rows,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+// the instantiation of an x-pass a plan runs (6 elements per thread: at most 768 points)
+#define FX_X_KERNEL(K, P) ((P).ept == 6 ? K<6, false> : (P).n > kFxGuardLength ? K<12, true> : K<12, false>)
 static unsigned threads(const FFTPlan& p) { return (unsigned)(p.batch * p.tpt); }
 
 // Every pass may take up to kFftSmemMax bytes of dynamic shared memory. The limit is a property of the
@@ -899,13 +988,14 @@ static bool smem_limit_z() {
   return smem_limit(k_fft_z_inv<cd, EPT, COLS>) && smem_limit(k_fft_z_inv<cdf, EPT, COLS>) &&
          smem_limit(k_fft_z_fwd<EPT, COLS>);
 }
-template <int EPT>
+template <int EPT, bool GUARD>
 static bool smem_limit_x() {
-  return smem_limit(k_fft_x_inv<EPT>) && smem_limit(k_fft_x_inv_mul<EPT>) && smem_limit(k_fft_x_fwd<EPT>) &&
-         smem_limit(k_fft_x_fwd_dot3<EPT>);
+  return smem_limit(k_fft_x_inv<EPT, GUARD>) && smem_limit(k_fft_x_inv_mul<EPT, GUARD>) &&
+         smem_limit(k_fft_x_fwd<EPT, GUARD>) && smem_limit(k_fft_x_fwd_dot3<EPT, GUARD>);
 }
 static int set_smem() {
-  return smem_limit_z<12, 4>() && smem_limit_z<12, 2>() && smem_limit_z<6, 4>() && smem_limit_x<12>() && smem_limit_x<6>()
+  return smem_limit_z<12, 4>() && smem_limit_z<12, 2>() && smem_limit_z<6, 4>() && smem_limit_x<12, false>() &&
+                 smem_limit_x<12, true>() && smem_limit_x<6, false>()
              ? LMVD_OK
              : LMVD_ERR_CUDA;
 }
@@ -1007,20 +1097,12 @@ static void inverse(Ctx& c, cd* const* in, double* const* out, int nf, bool df_i
     const FFTPlan& p = pick_plan(c.fx, c.fx6, 0.5 * g.pz * g.ny * n);
     dim3 gx(cdiv(cdiv(g.pz, 2), p.batch), g.ny, n);
     const double xfl = n * ny * ((g.pz + 1) / 2) * fft_flops(px), xby = n * ny * pz * (16.0 * h + 8.0 * px);
-    if (wmul) {  // the product with w in the epilogue: one more physical field read, one multiply per point
-      if (p.ept == 12)
-        LMVD_LAUNCH(c, KC_FFT_X_INV, xfl + n * ny * pz * px, xby + n * ny * pz * 8.0 * px, k_fft_x_inv_mul<12>, gx,
-                    threads(p), smem_bytes(p), p, g, c.tbuf, tstride, c.texp, fo, wmul, c.dflags);
-      else
-        LMVD_LAUNCH(c, KC_FFT_X_INV, xfl + n * ny * pz * px, xby + n * ny * pz * 8.0 * px, k_fft_x_inv_mul<6>, gx,
-                    threads(p), smem_bytes(p), p, g, c.tbuf, tstride, c.texp, fo, wmul, c.dflags);
-    } else if (p.ept == 12) {
-      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, k_fft_x_inv<12>, gx, threads(p), smem_bytes(p), p, g, c.tbuf,
+    if (wmul)  // the product with w in the epilogue: one more physical field read, one multiply per point
+      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl + n * ny * pz * px, xby + n * ny * pz * 8.0 * px, FX_X_KERNEL(k_fft_x_inv_mul, p), gx,
+                  threads(p), smem_bytes(p), p, g, c.tbuf, tstride, c.texp, fo, wmul, c.dflags);
+    else
+      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, FX_X_KERNEL(k_fft_x_inv, p), gx, threads(p), smem_bytes(p), p, g, c.tbuf,
                   tstride, c.texp, fo, c.dflags);
-    } else {
-      LMVD_LAUNCH(c, KC_FFT_X_INV, xfl, xby, k_fft_x_inv<6>, gx, threads(p), smem_bytes(p), p, g, c.tbuf,
-                  tstride, c.texp, fo, c.dflags);
-    }
   }
 }
 
@@ -1038,12 +1120,8 @@ void fft_forward(Ctx& c, double* const* in, cd* const* out, int nf) {
     const double h = g.nx / 2, ny = g.ny, pz = g.pz, px = g.px;
     const FFTPlan& p = pick_plan(c.fx, c.fx6, 0.5 * g.pz * g.ny * n);
     dim3 gx(cdiv(cdiv(g.pz, 2), p.batch), g.ny, n);
-    if (p.ept == 12)
-      LMVD_LAUNCH(c, KC_FFT_X_FWD, n * ny * ((g.pz + 1) / 2) * fft_flops(px), n * ny * pz * (16.0 * h + 8.0 * px),
-                  k_fft_x_fwd<12>, gx, threads(p), smem_bytes(p), p, g, fi, c.tbuf, tstride, c.texp);
-    else
-      LMVD_LAUNCH(c, KC_FFT_X_FWD, n * ny * ((g.pz + 1) / 2) * fft_flops(px), n * ny * pz * (16.0 * h + 8.0 * px),
-                  k_fft_x_fwd<6>, gx, threads(p), smem_bytes(p), p, g, fi, c.tbuf, tstride, c.texp);
+    LMVD_LAUNCH(c, KC_FFT_X_FWD, n * ny * ((g.pz + 1) / 2) * fft_flops(px), n * ny * pz * (16.0 * h + 8.0 * px),
+                FX_X_KERNEL(k_fft_x_fwd, p), gx, threads(p), smem_bytes(p), p, g, fi, c.tbuf, tstride, c.texp);
     z_fwd_launch(c, n, fo, n * ny * h * fft_flops(pz), n * ny * 16.0 * (pz * h + (double)g.nz * g.nxh));
   }
 }
@@ -1061,14 +1139,10 @@ void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, co
   fo.p[0] = out;
   const double h = g.nx / 2, ny = g.ny, pz = g.pz, px = g.px;
   const FFTPlan& p = pick_plan(c.fx, c.fx6, 0.5 * g.pz * g.ny * 1);
-    dim3 gx(cdiv(cdiv(g.pz, 2), p.batch), g.ny, 1);
+  const dim3 gx(cdiv(cdiv(g.pz, 2), p.batch), g.ny, 1);
   const double xfl = ny * ((g.pz + 1) / 2) * fft_flops(px) + 6.0 * ny * pz * px, xby = ny * pz * (16.0 * h + 48.0 * px);
-  if (p.ept == 12)
-    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, k_fft_x_fwd_dot3<12>, gx, threads(p), smem_bytes(p), p, g, c.tbuf,
-                tstride, c.texp, d);
-  else
-    LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, k_fft_x_fwd_dot3<6>, gx, threads(p), smem_bytes(p), p, g, c.tbuf,
-                tstride, c.texp, d);
+  LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, FX_X_KERNEL(k_fft_x_fwd_dot3, p), gx, threads(p), smem_bytes(p), p, g, c.tbuf, tstride,
+              c.texp, d);
   z_fwd_launch(c, 1, fo, ny * h * fft_flops(pz), ny * 16.0 * (pz * h + 2.0 * g.nz * g.nxh), add);
 }
 
@@ -1217,8 +1291,7 @@ extern "C" int lmvd_inverse_transform_noalloc(int nx, int ny, int nz, const void
     else launch_next(k_fft_z_inv<cd, 6, 4>, gz, threads(fz), smem_bytes(fz), st, fz, g, maps, T, 0, te, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
     dim3 gx(cdiv(cdiv(g.pz, 2), fx.batch), ny, 1);
-    if (fx.ept == 12) launch_next(k_fft_x_inv<12>, gx, threads(fx), smem_bytes(fx), st, fx, g, T, 0, te, fo, nullptr);
-    else launch_next(k_fft_x_inv<6>, gx, threads(fx), smem_bytes(fx), st, fx, g, T, 0, te, fo, nullptr);
+    launch_next(FX_X_KERNEL(k_fft_x_inv, fx), gx, threads(fx), smem_bytes(fx), st, fx, g, T, 0, te, fo, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LMVD_ERR_CUDA;
   }
   return LMVD_OK;

@@ -1,16 +1,17 @@
 // Block fixed-point arithmetic of the transforms: a complex value of one transform is a pair of 64-bit
 // integers X = x 2^k with one exponent k per transform.
 //
-// Why integers: GB300 retires 1.68 binary64 additions per clock per SM, but 62 64-bit integer additions and 62
+// Why integers: GB300 retires 1.68 binary64 additions per clock per SM, but 60 64-bit integer additions and 30
 // 32 x 32 + 64 -> 64 bit multiply-adds (measured, 8 independent chains per thread), so a transform in 64-bit
 // fixed point issues its arithmetic several times faster than one in binary64, and in fewer instructions than
 // one in double-float.
 // Why it is as accurate: the additions are exact, a twiddle product rounds to one unit, and k is as large as
 // the sum S = sum (|re| + |im|) of the transform's inputs allows: no partial sum of a transform exceeds S, so
-// with S 2^k <= 2^61.7 nothing overflows. The unit is then at most 2^-60.4 S <= 2^-60.4 sqrt(2 n) ||x||, that
-// is 2^-50.4 of the inputs' rms at n = 512, and rounding errors enter the result as noise of about half a
+// with S 2^k <= 2^61.7 nothing overflows. The unit is then at most 2^-60.7 S <= 2^-60.7 sqrt(2 n) ||x||, that
+// is 2^-50.7 of the inputs' rms at n = 512, and rounding errors enter the result as noise of about half a
 // unit times sqrt(n), where binary64 rounds every addition of every stage: measured against a transform in
-// extended precision, the error is below the binary64 transform's (figures in fft.cu).
+// extended precision, the error is below the binary64 transform's up to 768 points, and with guard bits beyond
+// (figures in fft.cu).
 #pragma once
 #include "df64.h"
 #include "lmvd_internal.h"

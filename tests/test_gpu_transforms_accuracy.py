@@ -71,3 +71,17 @@ def test_errors_do_not_pile_up(L, nx, nz, forward):
     (eight leaves a probability below 1e-9); a rounding with a mean adds up in a few outputs instead."""
     for e in errors(L, nx, nz, forward):
         assert e.max() <= 8 * np.sqrt(np.mean(e ** 2))
+
+
+# up to 768 points; above, where the first stages carry guard bits; both mixed; a small plan (6 points a thread)
+@pytest.mark.parametrize("forward", [False, True])
+@pytest.mark.parametrize("nx,nz", [(32, 32), (128, 96), (512, 512), (512, 16), (16, 512), (576, 576), (768, 768), (1024, 1024),
+                                   (1024, 16), (16, 1024), (648, 16), (16, 864), (864, 576)])
+def test_errors_are_below_those_of_binary64(L, nx, nz, forward):
+    """A binary64 radix-4/2/3 transform of white fields of these sizes has an rms error of 2.1e-16 to 3.5e-16 of the
+    result's rms (3.0e-16 at 1024 x 1024). A pass's unit is at most 2^-60.7 S with S = 1.6 n rms, and its noise at most 12.4
+    units at 768 points and 8 units with guard bits (a model of one transform): at most 2.1e-16 a pass at 768 points, 1.5e-16
+    above, 3.0e-16 for two."""
+    for e in errors(L, nx, nz, forward):
+        assert np.sqrt(np.mean(e ** 2)) <= 3.0e-16
+        assert e.max() <= 8 * 3.0e-16
