@@ -18,6 +18,7 @@ of all ranks over the slowest rank's time.
 """
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -37,10 +38,10 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # FP32 instructions (TwoSum-renormalised adds, FMA TwoProd products) per classic flop; the FP32 pipe issues
 # 152 SMs x 128 lanes x 2.07 GHz instructions per second.
 DF64_EQ_PEAK_TFLOPS = 152 * 128 * 2.07e9 / 10 / 1e12
-# The transforms compute in 64-bit fixed point on the integer pipes (csrc/fx.cuh), in both precisions. Their peak in
-# classic flops: a radix-2 butterfly (10 flops) takes one complex product of 12 multiply-adds 32 x 32 + 64 bits,
-# which the pipe retires at 30 lanes per clock per SM (measured), the slower of its pipes.
-FIXED_EQ_PEAK_TFLOPS = 152 * 30 / 12 * 10 * 2.07e9 / 1e12
+# The transforms compute in 64-bit fixed point on the integer pipes (csrc/fx.cuh), in both precisions. Their bound is the
+# pipe that retires multiply-adds 32 x 32 + 64 bits at 30 lanes per clock per SM (measured with 8 independent chains per
+# thread, profiles/issue_rates_fp64_fp32_gb300.md).
+MULTIPLY_ADD_RATE = 152 * 30 * 2.07e9
 # Measured DRAM bytes (read + write) of the dominant kernel class over its algorithmic bytes, from one ncu
 # capture of a smaller case with the same transform length (512 x 33 x 512: 768-point x-transforms), keyed by
 # (precision, kernel class, transform length). The class fft_x_inverse holds k_fft_x_inv (19045-19423 B per
@@ -297,6 +298,28 @@ def traffic_per_launch(fp, kernel, grid, alg_bytes_per_launch):
     return frac * alg_bytes_per_launch
 
 
+def fixed_point_madds(n):
+    """Multiply-adds 32 x 32 + 64 bits per point that a fixed-point transform of length n issues, by the radices of its
+    plan (csrc/fft.cu make_plan: 4s, 2s, 3s, then a last stage of 12 or 6): 12 per twiddle product, of which a stage of
+    radix r has (r - 1) / r per point (the first stage none), and 2 per point in a radix-3 butterfly."""
+    last = 12 if n % 12 == 0 else 6
+    m, radices = n // last, []
+    for r in ((4, 2, 3) if last == 12 else (2, 3)):
+        while m % r == 0:
+            radices.append(r)
+            m //= r
+    assert m == 1 and n % last == 0, n
+    total = 0.0
+    for i, r in enumerate(radices + [last]):
+        total += 12.0 * (r - 1) / r * (i > 0) + 2.0 * (r % 3 == 0)
+    return total
+
+
+def fixed_point_peak(n):
+    """Classic flops per second (5 n log2 n per transform, in TFLOP/s) at which the multiply pipe would be full."""
+    return MULTIPLY_ADD_RATE / fixed_point_madds(n) * 5.0 * math.log2(n) / 1e12
+
+
 def class_table(prof, steps):
     """Per kernel class and step: time, launches, algorithmic TFLOP/s and GB/s, and the GB/s as a fraction
     of the measured HBM copy bandwidth (prof: class -> (ms, launches, flops, bytes) over `steps` steps)."""
@@ -339,11 +362,12 @@ def roofline_of(prof, ms_step_total, fp, grid, rates=None):
                                             "lanes x 2.07 GHz / 10 FP32 instructions per classic flop")
     fixed = {}
     if top.startswith("fft"):
-        fixed = {"fixed_point_peak": FIXED_EQ_PEAK_TFLOPS,
-                 "fixed_point_frac": achieved / FIXED_EQ_PEAK_TFLOPS if achieved else None}
+        n = 3 * (grid[0] if top.startswith("fft_x") else grid[2]) // 2
+        fixed = {"fixed_point_peak": fixed_point_peak(n),
+                 "fixed_point_frac": achieved / fixed_point_peak(n) if achieved else None}
         note += ("; the transforms run in 64-bit fixed point on the integer pipes, so this fraction may exceed 1: "
-                 "fixed_point_frac is against the integer multiply pipe (12 multiply-adds per radix-2 butterfly of 10 "
-                 "flops, 30 lanes per clock per SM measured, 152 SMs, 2.07 GHz)")
+                 "fixed_point_frac is against the integer multiply pipe (%g multiply-adds per point of a transform of "
+                 "%d, 30 lanes per clock per SM measured, 152 SMs, 2.07 GHz)" % (fixed_point_madds(n), n))
     return {"kernel": top, "bound": "alu", **fixed, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak if achieved else None,
             "traffic": traffic_per_launch(fp, top, grid, tby / tn if tn else None),
