@@ -613,7 +613,7 @@ def run_cuda(args):
         dist.init_process_group("nccl", device_id=torch.device("cuda", local))
     w, config = workload_config(args.workload)
     config["parallelism"] = "replicas%d" % ws if ws > 1 else "single"
-    config["precision"] = ("FP64 throughout" if args.precision == 0 else
+    config["precision"] = ("FP64, transforms in 64-bit fixed point" if args.precision == 0 else
                            "double-float band evaluations, fixed-point transforms, FP64 elsewhere")
     npts = w["nx"] * w["ny"] * w["nz"]
     stream = torch.cuda.Stream()
@@ -647,7 +647,7 @@ def run_cuda(args):
         _, v2 = aggregate(r2["ms"], npts * args.steps, ws, device="cuda")
         errs = {k: rel_err(f2[k], final[k]) for k in ("z", "om", "m2")}
         out["variant"] = {
-            "precision": ("FP64 throughout" if other == 0 else
+            "precision": ("FP64, transforms in 64-bit fixed point" if other == 0 else
                           "double-float (2 x FP32, error-free transformations) band evaluations, fixed-point "
                           "transforms, FP64 products / solves / RHS / update"),
             "value": v2, "unit": UNIT, "ms_per_step": r2["ms"] / args.steps, "clocks": r2["clocks"],

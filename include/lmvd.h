@@ -69,8 +69,9 @@ extern "C" {
  *               double-float arithmetic on the FP32 units (pairs of floats, 48-bit significand,
  *               error-free TwoSum/TwoProd compensation), everything else (products, EOS, collocation,
  *               m^c and m2^d solves, RHS assembly, the RK update and the state) in FP64. In both the
- *               transforms compute in 64-bit fixed point with one exponent per 1D transform, with
- *               rounding errors below those of a binary64 FFT.
+ *               transforms compute in 64-bit fixed point with one exponent per 1D transform; their rms
+ *               rounding error is 0.05 to 0.3 of 1e-15 of the result's rms (a binary64 FFT's 0.2 to 0.3),
+ *               measured on white fields from 32 x 32 to 1024 x 1024 modes.
  * bc_mode     : boundary rows at y0 and y1. 0 = no-slip walls: Omega2 = 0, m2^d = dm2^d/dy = 0,
  *               m2^c = 0, <m1> = <m3> = 0, dz/dy = 0, <m2^c>(y1) = 0.
  *               1 = the paper's potential matching (Sec. 4.5, Eq. bc_both, md_bc) for a domain
@@ -80,8 +81,9 @@ extern "C" {
  *               boundary rows first and last in each per-mode system and factor it without pivoting.
  * memory_layout: 0 = automatic (the full layout unless its workspace would take more than 85% of the
  *               free device memory), 1 = full, 2 = lean (6 instead of 9 physical work fields, the products
- *               of the RHS formed in three batches instead of one, a 2-field instead of 4-field transform
- *               intermediate: the same results in about 35 GB less at 768 x 769 x 768).
+ *               of the RHS formed in three batches instead of one, a transform intermediate of 2 fields instead
+ *               of 4, or of 10 on grids where those take at most 512 MB: the same results, to the transforms'
+ *               rounding, in about 35 GB less at 768 x 769 x 768).
  */
 typedef struct {
   int nx, ny, nz, spline_order;
@@ -179,7 +181,8 @@ int lmvd_get_field(lmvd_ctx* ctx, int which, void* out);
 size_t lmvd_field_bytes(const lmvd_ctx* ctx, int which);
 
 /* Fourier synthesis / analysis with the 3/2 rule (Eq. disc_f; Sec. 4.4: nonlinear terms are formed
- * on the physical grid), always in FP64, on the context's grid and stream, using its workspace.
+ * on the physical grid), FP64 in and out in both precisions, on the context's grid and stream, using its
+ * workspace.
  * spec: nfields consecutive spectral arrays [ny][nz][nx/2+1] complex128 holding values at the ny
  *       collocation points (not B-spline coefficients); Nyquist slots are ignored on input and
  *       written as zero on output.

@@ -754,8 +754,8 @@ int adjoint_impl(Ctx& c) {
   // step 5: RHS streams, collocation solves, transforms, products of pass 2
   St7 stw{};
   for (int q = 0; q < 7; ++q) stw.p[q] = A.st[q];
-  LMVD_LAUNCH(c, KC_RHS_EVAL, 0, 0, k_adj_rhs_eval, dim3(mblocks(g), row_chunks(g, ny)), TPB, 0, g, A.B1gT, A.B2gT, A.BsT[0], A.BsT[1],
-              A.BsT[2], A.BsT[3], A.rom, A.rphi, A.rm, stw);
+  LMVD_LAUNCH(c, KC_RHS_EVAL, 0, 0, k_adj_rhs_eval, dim3(mblocks(g), row_chunks(g, ny)), TPB, 0, g, A.B1gT, A.B2gT,
+              A.BsT[0], A.BsT[1], A.BsT[2], A.BsT[3], A.rom, A.rphi, A.rm, stw);
   solve_T_jobs(c, KC_SOLVE, c.lu_interp,
                {SolveTJob{A.st[1], A.st[1], 0, ny - 1}, SolveTJob{A.st[2], A.st[2], 0, ny - 1},
                 SolveTJob{A.st[3], A.st[3], 0, ny - 1}, SolveTJob{A.st[4], A.st[4], 0, ny - 1},
@@ -827,8 +827,8 @@ int pass1_T(Ctx& c, AdjWork& A) {
   Sv8 w8{};
   for (int q = 0; q < 8; ++q) v8.p[q] = w8.p[q] = A.sv[q];
   LMVD_LAUNCH(c, KC_EVAL_P1, 0, 0, k_adj_p1_combine, dim3(mblocks(g), row_chunks(g, g.ny)), TPB, 0, g, w8);
-  LMVD_LAUNCH(c, KC_EVAL_P1, 0, 0, k_adj_eval_p1, dim3(mblocks(g), row_chunks(g, g.ny)), TPB, 0, g, A.B0gT, A.B1gT, A.B2gT, A.Sg0T, A.Sg1T, v8,
-              A.z, A.om, A.m2, A.mm1, A.mm3);
+  LMVD_LAUNCH(c, KC_EVAL_P1, 0, 0, k_adj_eval_p1, dim3(mblocks(g), row_chunks(g, g.ny)), TPB, 0, g, A.B0gT, A.B1gT,
+              A.B2gT, A.Sg0T, A.Sg1T, v8, A.z, A.om, A.m2, A.mm1, A.mm3);
   // lmvd_set_state zeroes these entries of the state, so the substage does not depend on them
   LMVD_LAUNCH(c, KC_MISC, 0, 0, k_sanitize, eblocks(S), 256, 0, g, g.ny, A.z, 0);
   LMVD_LAUNCH(c, KC_MISC, 0, 0, k_sanitize, eblocks(S), 256, 0, g, g.ny, A.om, 1);

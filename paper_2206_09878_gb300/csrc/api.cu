@@ -431,6 +431,7 @@ void physical_pass_1(Ctx& c, double* const* zp = nullptr) {
   double* fin[1] = {c.pw[5]};
   cd* fout[1] = {c.sv[SV_RZ]};
   fft_forward(c, fin, fout, 1);
+  // its coefficients, for lmvd_get_field alone: the fixed point adds the values kept in sv[SV_RZ]
   solve_interp(c, SolveJob{c.sv[SV_RZ], nullptr, c.Rz});
 }
 
@@ -875,8 +876,6 @@ int lmvd_create(const lmvd_config* cfg, void* stream, lmvd_ctx** out) {
     for (int d = 0; d < 4 && !err; ++d) err = upload_band(c, Bs[d], c.Bs[d]);
     if (!err) err = upload_band(c, Sg0, c.Sg0);
     if (!err) err = upload_band(c, Sg1, c.Sg1);
-    if (!err) err = upload_band(c, Ss0, c.Ss0);
-    if (!err) err = upload_band(c, Ss2, c.Ss2);
     if (!err) err = upload(c, ds, &c.dstar);
     if (!err) err = upload(c, greville_quadrature(kb, B0g), &c.wq);
     // shared LUs: interpolation / Dirichlet (values at g) and Neumann (dz/dy rows at the walls)

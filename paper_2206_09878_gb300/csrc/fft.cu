@@ -108,8 +108,9 @@ __device__ __forceinline__ void fx_butterfly(cfx (&v)[R], const FFTPlan& pl) {
 
 // A twiddle. The passes with 6 elements a thread use plain loads, so that a launch may overlap the kernel that wrote the
 // table (the allocation-free transform, 20.5 -> 18.5 us at 64 x 33 x 64). With 12 elements the choice is which spills less
-// and was measured: plain in the forward x-pass (3-field 256 x 129 x 256 analysis 500.0 -> 497.2 us), the read-only path
-// in the others (4-field 216 x 65 x 108 synthesis 170.9, plain 171.5 us).
+// (bytes, read-only / plain: forward x-pass 136 / 120, inverse z-pass 124 / 140, forward z-pass 116 / 124, inverse x-pass
+// 64 / 64), a difference of half a percent: plain in the forward x-pass (3-field 256 x 129 x 256 analysis 500.0 -> 497.2 us), the
+// read-only path in the others (4-field 216 x 65 x 108 synthesis 170.9, plain 171.5 us).
 template <int SIGN, int EPT, int S>
 __device__ __forceinline__ int4 fx_tw(const int4* p) {
   if constexpr (EPT == 12 && (S > 1 || SIGN > 0)) return __ldg(p);
@@ -121,9 +122,9 @@ __device__ __forceinline__ int4 fx_tw(const int4* p) {
 // inputs, would exceed it. But the first two stages add up at most 16 inputs, so their values carry e <= 2 more bits where
 // 16 times the largest input allows (white inputs; with a few large ones S is small already), and the third stage's
 // twiddles are 2^-e as large, so that its products round back to the unit. The noise of a 1536-point transform falls from
-// 17.5 units to 6.3, the error at 1024 x 1024 modes from 3.9-5.8e-16 to 1.3-1.7e-16 (inverse; forward 3.6-5.3e-16 to 1.6-2.2e-16;
-// complex double 3.0e-16). It costs registers and a tenth of the time: 4 fields of 768 x 33 x 768 1.99 / 1.93 -> 2.18 / 2.07 ms
-// (inverse / forward; complex double 9.9 / 10.8). Shorter lengths are as accurate without.
+// 17.5 units to 6.3, the error at 1024 x 1024 modes from 3.9-5.8e-16 to 1.3-1.7e-16 (inverse) and from 3.6-5.3e-16 to
+// 1.6-2.2e-16 (forward; complex double 3.0e-16). It costs registers and a tenth of the time: 4 fields of 768 x 33 x 768
+// 1.99 / 1.93 -> 2.18 / 2.07 ms (inverse / forward; complex double 9.9 / 10.8). Shorter lengths are as accurate without.
 constexpr int kFxGuardLength = 768, kFxGuardBits = 2, kFxGuardStage = 2;
 __device__ __forceinline__ int fx_guard(int most, int emin, int k) {  // most: see the callers
   return max(0, min(min(most, emin - k), kFxGuardBits));
@@ -197,8 +198,8 @@ __device__ __forceinline__ void fx_first4(cfx (&v)[12], cfx* x, const FFTPlan& p
   __syncthreads();
 }
 
-// Stages s0 .. nst - 2; returns when every point of the last stage's input is in x. e: the inputs' guard bits (a length above
-// kFxGuardLength has four of these stages).
+// Stages s0 .. nst - 2; returns when every point of the last stage's input is in x. e: the inputs' guard bits (a length
+// above kFxGuardLength has four of these stages).
 template <int SIGN, int EPT, int S, bool GUARD>
 __device__ __forceinline__ void fx_middle(cfx* x, const FFTPlan& pl, int s0, int tt, int tpt, int e) {
   int L = 1;
@@ -1141,8 +1142,8 @@ void fft_forward_dot3(Ctx& c, const double* const* w, const double* const* m, co
   const FFTPlan& p = pick_plan(c.fx, c.fx6, 0.5 * g.pz * g.ny * 1);
   const dim3 gx(cdiv(cdiv(g.pz, 2), p.batch), g.ny, 1);
   const double xfl = ny * ((g.pz + 1) / 2) * fft_flops(px) + 6.0 * ny * pz * px, xby = ny * pz * (16.0 * h + 48.0 * px);
-  LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, FX_X_KERNEL(k_fft_x_fwd_dot3, p), gx, threads(p), smem_bytes(p), p, g, c.tbuf, tstride,
-              c.texp, d);
+  LMVD_LAUNCH(c, KC_FFT_X_FWD, xfl, xby, FX_X_KERNEL(k_fft_x_fwd_dot3, p), gx, threads(p), smem_bytes(p), p, g, c.tbuf,
+              tstride, c.texp, d);
   z_fwd_launch(c, 1, fo, ny * h * fft_flops(pz), ny * 16.0 * (pz * h + 2.0 * g.nz * g.nxh), add);
 }
 

@@ -8,7 +8,7 @@
 // Why it is as accurate: the additions are exact, a twiddle product rounds to one unit, and k is as large as
 // the sum S = sum (|re| + |im|) of the transform's inputs allows: no partial sum of a transform exceeds S, so
 // with S 2^k <= 2^61.7 nothing overflows. The unit is then at most 2^-60.7 S <= 2^-60.7 sqrt(2 n) ||x||, that
-// is 2^-50.7 of the inputs' rms at n = 512, and rounding errors enter the result as noise of about half a
+// is 2^-51.2 of the inputs' rms at n = 512, and rounding errors enter the result as noise of about half a
 // unit times sqrt(n), where binary64 rounds every addition of every stage: measured against a transform in
 // extended precision, the error is below the binary64 transform's up to 768 points, and with guard bits beyond
 // (figures in fft.cu).

@@ -154,10 +154,10 @@ __host__ __device__ inline void row_range(int rows, int c, int nc, int& r0, int&
   r1 = (int)((long long)rows * (c + 1) / nc);
 }
 
-// Row chunks for the evaluation kernels: about 2^17 threads when the grid has few
-// Fourier modes (more repeat the per-mode FP64 work of a chunk's start: 1% of a substage at 128 modes), at least 2 rows per thread. (With 8 a thread's rows were the time of a launch on the smallest grids: one
-// warp's FP64 instruction takes 64 cycles whatever else runs. 32 x 33 x 32: pass-1 evaluation 58 -> 27 us, right-hand
-// sides 76 -> 24 us.)
+// Row chunks for the evaluation kernels: about 2^17 threads when the grid has few Fourier modes (more repeat the
+// per-mode FP64 work of a chunk's start: 1% of a substage at 128 modes), at least 2 rows per thread. (With 8 a
+// thread's rows were the time of a launch on the smallest grids: one warp's FP64 instruction takes 64 cycles
+// whatever else runs. 32 x 33 x 32: pass-1 evaluation 58 -> 27 us, right-hand sides 76 -> 24 us.)
 inline unsigned row_chunks(const Grid& g, int rows) {
   const size_t want = (((size_t)1 << 17) + g.M - 1) / g.M;
   const size_t cap = (size_t)(rows / 2 > 1 ? rows / 2 : 1);
@@ -253,7 +253,7 @@ struct Ctx {
   int status = 0;
 
   // operators
-  DBand B0g, B1g, B2g, Bs[4], Sg0, Sg1, Ss0, Ss2;
+  DBand B0g, B1g, B2g, Bs[4], Sg0, Sg1;
   double* dstar = nullptr;  // ny entries: (D* c)_i = dstar[i] (c_{i+1} - c_i)
   DLU lu_interp, lu_neumann, lu_mc, lu_md;
   DLU lu_means;  // lu_interp (walls) or lu_neumann (potential matching): not owned
