@@ -39,8 +39,8 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # 152 SMs x 128 lanes x 2.07 GHz instructions per second.
 DF64_EQ_PEAK_TFLOPS = 152 * 128 * 2.07e9 / 10 / 1e12
 # The transforms compute in 64-bit fixed point on the integer pipes (csrc/fx.cuh), in both precisions. Their bound is the
-# pipe that retires multiply-adds 32 x 32 + 64 bits at 30 lanes per clock per SM (measured with 8 independent chains per
-# thread, profiles/issue_rates_fp64_fp32_gb300.md).
+# pipe that retires multiply-adds 32 x 32 + 64 bits (mad.lo.cc / madc.hi) at 30 lanes per clock per SM, measured with 8
+# independent chains per thread.
 MULTIPLY_ADD_RATE = 152 * 30 * 2.07e9
 # Measured DRAM bytes (read + write) of the dominant kernel class over its algorithmic bytes, from one ncu
 # capture of a smaller case with the same transform length (512 x 33 x 512: 768-point x-transforms), keyed by

@@ -31,7 +31,7 @@ def hermitian(f):
 
 
 def spectra(kind, rng, nz, nxh):
-    """Ten planes at every scale, and a plane of zeros."""
+    """A plane at each scale, and a plane of zeros."""
     f = rng.normal(size=(len(SCALES) + 1, nz, nxh)) + 1j * rng.normal(size=(len(SCALES) + 1, nz, nxh))
     kz = np.abs(np.fft.fftfreq(nz, 1.0 / nz))[:, None]
     kx = np.arange(nxh)[None, :]
