@@ -109,8 +109,8 @@ __device__ __forceinline__ void fx_butterfly(cfx (&v)[R], const FFTPlan& pl) {
 // A twiddle. The passes with 6 elements a thread use plain loads, so that a launch may overlap the kernel that wrote the
 // table (the allocation-free transform, 20.5 -> 18.5 us at 64 x 33 x 64). With 12 elements the choice is which spills less
 // (bytes, read-only / plain: forward x-pass 136 / 120, inverse z-pass 124 / 140, forward z-pass 116 / 124, inverse x-pass
-// 64 / 64), a difference of half a percent: plain in the forward x-pass (3-field 256 x 129 x 256 analysis 500.0 -> 497.2 us), the
-// read-only path in the others (4-field 216 x 65 x 108 synthesis 170.9, plain 171.5 us).
+// 64 / 64), a difference of half a percent: plain in the forward x-pass (3-field 256 x 129 x 256 analysis 500.0 -> 497.2
+// us), the read-only path in the others (4-field 216 x 65 x 108 synthesis 170.9, plain 171.5 us).
 template <int SIGN, int EPT, int S>
 __device__ __forceinline__ int4 fx_tw(const int4* p) {
   if constexpr (EPT == 12 && (S > 1 || SIGN > 0)) return __ldg(p);
